@@ -45,6 +45,7 @@ constexpr int PF_KEYS = 128;                        // keys per block
 constexpr int PF_PAGES = PF_KEYS / KV_BLOCK;        // 8
 constexpr int PF_NK = 2;                            // key ring depth
 constexpr int PF_NV = 2;                            // value ring depth
+constexpr int PF_ONE_WAVE = 128;                    // CTAs that are certainly resident at once (one per SM of a B200's 148, in pairs)
 constexpr int PF_KS = 2;                            // CTAs that share a tile's key blocks (the cluster size)
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -74,9 +75,14 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   using L = PfLayout<HD>;
   constexpr int TPT = 128 / GROUP;                  // tokens per tile
   constexpr int KSTEPS = HD / 16;
-  griddep_launch_dependents();
+  // The next kernel may start its prologue early only where every cluster is resident at once.  With clusters still to
+  // be placed it must not: its CTAs (and those of the kernel behind it, which need no shared memory) take single SMs as
+  // they become free, while a cluster needs two at the same time.
+  if (gridDim.x * gridDim.y <= PF_ONE_WAVE) griddep_launch_dependents();
   griddep_wait();                                   // q and the chunk's own keys / values come from the kernel before
-  const int tile = blockIdx.x / PF_KS, rank = blockIdx.x % PF_KS, g = blockIdx.y;
+  // heads fastest, the last tiles (the most key blocks) first: with more clusters than the SMs hold, the short ones
+  // fill the last wave
+  const int tile = (int)gridDim.y - 1 - (int)blockIdx.y, rank = blockIdx.x % PF_KS, g = blockIdx.x / PF_KS;
   const int row0 = tile * TPT;                      // first chunk row of the tile
   // the tile's last active row decides how many key blocks there are
   int last = -1;
@@ -469,7 +475,7 @@ cudaError_t launch_attention_prefill(const CUtensorMap &tmK, const CUtensorMap &
   if (group * kv.n_kv != nq) return cudaErrorInvalidValue;
   if (group != 1 && group != 2 && group != 4 && group != 8) return cudaErrorInvalidValue;
   const int tpt = 128 / group;
-  const dim3 grid(((rows.R + tpt - 1) / tpt) * PF_KS, kv.n_kv);
+  const dim3 grid(kv.n_kv * PF_KS, (rows.R + tpt - 1) / tpt);
 #define CORUN_PF_CASE(HD_, G_) \
   if (kv.hd == HD_ && group == G_) return pf_launch<HD_, G_>(grid, st, tmK, tmV, q, rows, nq, kv, out_hi, out_lo, d_status);
   CORUN_PF_CASE(128, 1) CORUN_PF_CASE(128, 2) CORUN_PF_CASE(128, 4) CORUN_PF_CASE(128, 8)

@@ -72,8 +72,20 @@ struct Program {
   int *tab_uk = nullptr, *tab_uv = nullptr;
   GemmPlan p_uk, p_uv, p_gu_d, p_down_d;
   bool has_layers = false, has_lm = false;
+  // Prefill of long prompts: up to `cap` rows at a time (R: the rows of the chunk at hand), the projections on pairs of
+  // SMs (gemm_pair.cu); their results are plain matrices, the SwiGLU is in the gate / up GEMM's epilogue.
+  bool pair = false;
+  int cap = 0;
+  GemmPairPlan b_qkv, b_o, b_gu, b_down;
   std::vector<void *> allocs;
 };
+
+// Prompts of up to PREFILL_SMALL tokens run through the fixed chunk program (its GEMMs cut K over the SMs: few rows
+// leave most SMs without a tile otherwise), longer ones through the program of PREFILL_BIG rows.  Which one depends on
+// the prompt's own length only, so a prompt's values do not depend on what is prefilled with it.  Measured on the
+// Qwen3-8B layer: 256 rows 192 us of GEMMs in the chunk program, 293 us on pairs of SMs; 512 rows 384 against 359; 1024
+// rows 766 against 531; 2048 rows 1532 against 1010 (hence chunks as large as the buffers allow).
+constexpr int PREFILL_SMALL = 256, PREFILL_BIG = 2048;
 
 }  // namespace
 
@@ -89,6 +101,7 @@ struct corun_engine {
   const bf16 *embed = nullptr, *lm_head = nullptr, *final_norm = nullptr;
   std::vector<const bf16 *> attn_norm, mlp_norm;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
+  std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down;   // boxes of 128 rows: the GEMMs on pairs of SMs
   std::vector<CUtensorMap> tm_gu_half;     // dense gate / up matrices with the box of the GEMM with SwiGLU in its epilogue
   std::vector<CUtensorMap> tm_k, tm_v;   // per layer: the pages as rows of head_dim halfs (keys and values alike)
   std::vector<CUtensorMap> tm_k4;        // the same memory as [8-token group][64-dim half][8 tokens][64 dims]: one box per (page, head) tile
@@ -131,7 +144,7 @@ struct corun_engine {
   int *h_out_tokens = nullptr, *h_status = nullptr;
   int *h_rows = nullptr;          // prefill row metadata staging [5][chunk]
   bool staged_valid = false, in_flight = false;
-  Program dec, pre, lm1;
+  Program dec, pre, big, lm1;
   // prefill-only per-row sampling arrays (length 1)
   float *d_pf_temp = nullptr, *d_pf_top_p = nullptr;
   uint64_t *d_pf_seed = nullptr;
@@ -312,6 +325,38 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
   return CORUN_OK;
 }
 
+// The program of long prompts (dense feed-forward, grouped-query attention): buffers for `cap` rows.
+int program_create_big(corun_engine *e, Program &P, int cap) {
+  const corun_shape &s = e->sh;
+  const int H = s.hidden, QD = s.n_q_heads * s.head_dim, KD = s.n_kv_heads * s.head_dim, F = s.ffn, QKVN = QD + 2 * KD;
+  P.pair = true;
+  P.R = P.cap = P.BN = cap;
+  P.has_layers = true;
+  auto &A = P.allocs;
+  const size_t c = (size_t)cap;
+  RC(dmalloc(A, &P.xn_hi, c * H));
+  RC(dmalloc(A, &P.xn_lo, c * H));
+  RC(dmalloc(A, &P.row_token, c));
+  RC(dmalloc(A, &P.row_pos, c));
+  RC(dmalloc(A, &P.row_active, c));
+  RC(dmalloc(A, &P.row_slot, c));
+  RC(dmalloc(A, &P.h, c * H));
+  RC(dmalloc(A, &P.q, c * QD));
+  RC(dmalloc(A, &P.qkv_out, c * QKVN));
+  RC(dmalloc(A, &P.o_out, c * H));
+  RC(dmalloc(A, &P.down_out, c * H));
+  RC(dmalloc(A, &P.ao_hi, c * QD));
+  RC(dmalloc(A, &P.ao_lo, c * QD));
+  RC(dmalloc(A, &P.ff_hi, c * F));
+  RC(dmalloc(A, &P.ff_lo, c * F));
+  RC(dmalloc(A, &P.plain_tiles, (size_t)((QKVN > H ? QKVN : H) / GEMM_TILE_N + 1)));
+  RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, cap, P.qkv_out, e->num_sms));
+  RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, cap, P.o_out, e->num_sms));
+  RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, cap, P.ff_hi, P.ff_lo, e->num_sms));
+  RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, cap, P.down_out, e->num_sms));
+  return CORUN_OK;
+}
+
 void program_destroy(Program &P) {
   gemm_plan_destroy(&P.p_qkv);
   gemm_plan_destroy(&P.p_o);
@@ -335,9 +380,14 @@ KvLayout kv_layout(const corun_engine *e) {
 
 // The result of a layer's feed-forward part as the next kernel reads it: the down GEMM's partials, or (grouped
 // Mixture-of-Experts form) the combined plain matrix.
+GemmOut plain_out(const Program &P, const float *m, int N) {
+  return GemmOut{m, nullptr, P.plain_tiles, P.plain_tiles, N, 0, P.BN};
+}
+
 bool dense_layer(const corun_engine *e, int layer) { return e->mla && e->moe_E && layer < e->first_dense; }
 
 GemmOut ffn_out(const corun_engine *e, const Program &P, int layer) {
+  if (P.pair) return plain_out(P, P.down_out, e->sh.hidden);
   if (dense_layer(e, layer)) return P.p_down_d.out();
   if (P.grouped) return GemmOut{P.down_out, nullptr, P.plain_tiles, P.plain_tiles, P.p_down.N, P.p_down.KB, P.BN};
   return P.p_down.out();
@@ -369,6 +419,19 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
     GemmOut prev = ffn_out(e, P, l > 0 ? l - 1 : 0);
     STAGE(launch_resid_norm(P.h, s.hidden, e->embed, rows, l == 0 ? nullptr : &prev, e->attn_norm[l], s.rms_eps,
                             P.xn_hi, P.xn_lo, e->st));
+    if (P.pair) {
+      // long prompts: projections on pairs of SMs, plain results
+      STAGE(gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st));
+      STAGE(launch_qkv_post_plain(P.qkv_out, rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
+      STAGE(launch_attention_prefill(e->tm_k[l], e->tm_v[l], P.q, rows, s.n_q_heads, kv, P.ao_hi, P.ao_lo, e->d_status, e->st));
+      STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
+      const GemmOut o = plain_out(P, P.o_out, s.hidden);
+      STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
+      STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st));
+      STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st));
+      n += 8;
+      continue;
+    }
     STAGE(gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, tr(4 * l + 0), true));
     if (e->mla) {
       // cache append and query parts -> q_lat = W_uk^T q_nope per head -> absorbed attention over the row's latent
@@ -654,11 +717,12 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     if (fit < e->pool_blocks) e->pool_blocks = fit / e->kv_run * e->kv_run;
     if (e->pool_blocks < e->kv_run) return fail(CORUN_ENOMEM);
   }
-  e->chunk = 256;
+  e->chunk = PREFILL_SMALL;
+  bool one_chunk_size = false;                      // the environment asks for chunks of its own size, for every prompt
   if (const char *c = getenv("CORUN_ATTN_WHOLE_PAIRS")) e->whole_pairs = atoi(c) != 0;   // ablation only
   if (const char *c = getenv("CORUN_PREFILL_CHUNK")) {
     const int v = atoi(c);
-    if (v >= 16 && v <= 256 && v % 16 == 0) e->chunk = v;
+    if (v >= 16 && v <= 256 && v % 16 == 0) { e->chunk = v; one_chunk_size = true; }
   }
   e->embed = (const bf16 *)w->embed;
   e->lm_head = (const bf16 *)w->lm_head;
@@ -685,6 +749,12 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     }
     if ((rc = gemm_encode_map(&e->tm_gu[l], moe ? moe->gate_up[l] : w->wgate_up[l], 2 * F, H, GEMM_TILE_N))) return fail(rc);
     if ((rc = gemm_encode_map(&e->tm_down[l], moe ? moe->down[l] : w->wdown[l], H, F, GEMM_TILE_N))) return fail(rc);
+    if (!moe && !mla) {
+      if (e->tb_qkv.empty()) { e->tb_qkv.resize(s.n_layers); e->tb_o.resize(s.n_layers); e->tb_gu.resize(s.n_layers); e->tb_down.resize(s.n_layers); }
+      if ((rc = gemm_encode_map(&e->tb_qkv[l], w->wqkv[l], qkv_rows, H, 128)) || (rc = gemm_encode_map(&e->tb_o[l], w->wo[l], H, QD, 128)) ||
+          (rc = gemm_encode_map(&e->tb_gu[l], w->wgate_up[l], 2 * F, H, 128)) || (rc = gemm_encode_map(&e->tb_down[l], w->wdown[l], H, F, 128)))
+        return fail(rc);
+    }
     if (!moe && (rc = gemm_encode_map(&e->tm_gu_half[l], w->wgate_up[l], 2 * F, H, gemm_swiglu_half(F, e->num_sms)))) return fail(rc);
     if (moe && moe_half && (rc = gemm_encode_map(&e->tm_gu_half[l], moe->gate_up[l], 2 * F, H, moe_half))) return fail(rc);
   }
@@ -782,7 +852,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   if (cudaMallocHost(&e->h_active, B) != cudaSuccess || cudaMallocHost(&e->h_seeds, B * sizeof(uint64_t)) != cudaSuccess ||
       cudaMallocHost(&e->h_out_tokens, B * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&e->h_status, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&e->h_rows, (size_t)5 * e->chunk * sizeof(int)) != cudaSuccess)
+      cudaMallocHost(&e->h_rows, (size_t)5 * PREFILL_BIG * sizeof(int)) != cudaSuccess)
     return fail(CORUN_ENOMEM);
   memset(e->h_active, 0, B);
   memset(e->h_seeds, 0, B * sizeof(uint64_t));
@@ -806,6 +876,10 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   // a prefill chunk is filled from row 0: the host says which blocks of rows it reaches (prefill_run)
   for (GemmPlan *pl : {&e->pre.p_qkv, &e->pre.p_o, &e->pre.p_gu, &e->pre.p_down, &e->pre.p_gu_d, &e->pre.p_down_d})
     pl->row_blocks = e->pre.row_blocks;
+  if (!mla && !moe && !one_chunk_size && max_context > PREFILL_SMALL) {
+    const int cap = max_context < PREFILL_BIG ? (max_context + 255) / 256 * 256 : PREFILL_BIG;
+    if ((rc = program_create_big(e, e->big, cap))) return fail(rc);
+  }
   if ((rc = program_create(e, e->lm1, 1, false, true))) return fail(rc);
 
   // the allocations above were cleared and filled through the legacy stream, which the engine's
@@ -851,6 +925,7 @@ void corun_destroy(corun_engine *e) {
   if (e->graph) cudaGraphDestroy(e->graph);
   program_destroy(e->dec);
   program_destroy(e->pre);
+  program_destroy(e->big);
   program_destroy(e->lm1);
   for (void *p : e->allocs) cudaFree(p);
   if (e->h_active) cudaFreeHost(e->h_active);
@@ -877,9 +952,9 @@ struct PfReq {
 
 // Final norm -> LM head (one row) -> sample with R(seed, 0) for the request whose last prompt token is row
 // `row` of the chunk that has just run; the logits go to the slot's place among the prefill logits.
-int prefill_finish_row(corun_engine *e, int row, PfReq &r) {
+int prefill_finish_row(corun_engine *e, const Program &P, int row, PfReq &r) {
   const corun_shape &s = e->sh;
-  Program &P = e->pre, &L = e->lm1;
+  Program &L = e->lm1;
   GemmOut prev = ffn_out(e, P, s.n_layers - 1);
   prev.direct += (size_t)row * prev.N;
   if (prev.ws) prev.ws += (size_t)row * GEMM_TILE_N;
@@ -904,13 +979,14 @@ int prefill_finish_row(corun_engine *e, int row, PfReq &r) {
   return CORUN_OK;
 }
 
-// Prefill of one or several requests through the fixed-shape prefill program (chunks of `chunk` rows).  The
+// Prefill of one or several requests through one prefill program: the chunk program (chunks of `chunk` rows) or the
+// one of long prompts (chunks of up to its `cap` rows, launched for the rows they hold).  The
 // rows of a chunk are dealt in request order; every piece of a request starts on a tile boundary of the
 // prefill attention kernel (a tile's rows share one slot), so a chunk may hold pieces of several requests.
 // Every kernel of the program treats its rows independently of each other and of where they sit in the
 // chunk, and attention reads all keys -- the chunk's own too -- from the cache, so a request's values do not
 // depend on how its prompt is cut into pieces nor on what else shares its chunks.
-int prefill_run(corun_engine *e, PfReq *reqs, int n_req);
+int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req);
 
 int prefill_many(corun_engine *e, PfReq *reqs, int n_req) {
   RC(sync_stream(e));
@@ -919,7 +995,19 @@ int prefill_many(corun_engine *e, PfReq *reqs, int n_req) {
   if (need > e->free_blocks.size()) return CORUN_ENOSPACE;
   int rc = CORUN_OK;
   for (int i = 0; i < n_req && rc == CORUN_OK; ++i) rc = reserve_blocks(e, reqs[i].slot, reqs[i].reserve);
-  if (rc == CORUN_OK) rc = prefill_run(e, reqs, n_req);
+  std::vector<PfReq *> small, big;                  // by the prompt's own length
+  for (int i = 0; i < n_req; ++i) (e->big.pair && reqs[i].n > PREFILL_SMALL ? big : small).push_back(&reqs[i]);
+  if (rc == CORUN_OK && !small.empty()) rc = prefill_run(e, e->pre, small.data(), (int)small.size());
+  if (rc == CORUN_OK && !big.empty()) rc = prefill_run(e, e->big, big.data(), (int)big.size());
+  for (int i = 0; i < n_req && rc == CORUN_OK; ++i) {
+    const PfReq &q = reqs[i];
+    rc = set_slot_state(e, q.slot, 1, q.n, 1, q.first, q.smp.temperature, q.smp.top_p);
+    if (rc != CORUN_OK) break;
+    e->in_use[q.slot] = 1;
+    e->ctx[q.slot] = q.n;
+    e->reserve[q.slot] = q.reserve;
+    e->step[q.slot] = 1;
+  }
   if (rc != CORUN_OK)                               // nothing was admitted: the pages go back to the pool
     for (int i = 0; i < n_req; ++i) {
       std::vector<int> &mine = e->slot_blocks[reqs[i].slot];
@@ -930,36 +1018,39 @@ int prefill_many(corun_engine *e, PfReq *reqs, int n_req) {
   return rc;
 }
 
-int prefill_run(corun_engine *e, PfReq *reqs, int n_req) {
+int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
   const corun_shape &s = e->sh;
-  Program &P = e->pre;
-  const int CH = e->chunk;
+  const int CH = P.pair ? P.cap : e->chunk;
   int unit = 128 / (s.n_q_heads / s.n_kv_heads);    // tokens per attention tile
   if (e->mla) unit = 16;                            // no query tiles there: every row is on its own
   if (unit > CH || CH % unit) unit = CH;
   int *tok = e->h_rows, *pos = tok + CH, *act = pos + CH, *slt = act + CH, *blocks = slt + CH;
   std::vector<std::pair<int, int>> fins;           // (request, chunk row of its last prompt token)
-  int fill = 0, pad_slot = reqs[0].slot;
+  int fill = 0, pad_slot = reqs[0]->slot;
   auto run_chunk = [&]() -> int {
-    for (int i = fill; i < CH; ++i) { tok[i] = 0; pos[i] = 0; act[i] = 0; slt[i] = pad_slot; }
-    CK(cudaMemcpyAsync(P.row_token, tok, CH * sizeof(int), cudaMemcpyHostToDevice, e->st));
-    CK(cudaMemcpyAsync(P.row_pos, pos, CH * sizeof(int), cudaMemcpyHostToDevice, e->st));
-    CK(cudaMemcpyAsync(P.row_active, act, CH * sizeof(int), cudaMemcpyHostToDevice, e->st));
-    CK(cudaMemcpyAsync(P.row_slot, slt, CH * sizeof(int), cudaMemcpyHostToDevice, e->st));
+    const int rows_n = P.pair ? fill : CH;
+    if (P.pair) P.R = fill;
+    for (int i = fill; i < rows_n; ++i) { tok[i] = 0; pos[i] = 0; act[i] = 0; slt[i] = pad_slot; }
+    CK(cudaMemcpyAsync(P.row_token, tok, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
+    CK(cudaMemcpyAsync(P.row_pos, pos, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
+    CK(cudaMemcpyAsync(P.row_active, act, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
+    CK(cudaMemcpyAsync(P.row_slot, slt, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
     // the chunk's rows are filled from row 0: the GEMMs leave out the blocks of rows behind the last one in use
     // (blocks of 64 rows up to 128 padded rows, of 128 rows above)
-    const int blk = P.BN <= 128 ? 64 : 128;
-    blocks[0] = (fill > 0 ? 1 : 0) | (fill > blk ? 2 : 0);
-    CK(cudaMemcpyAsync(P.row_blocks, blocks, sizeof(int), cudaMemcpyHostToDevice, e->st));
+    if (!P.pair) {
+      const int blk = P.BN <= 128 ? 64 : 128;
+      blocks[0] = (fill > 0 ? 1 : 0) | (fill > blk ? 2 : 0);
+      CK(cudaMemcpyAsync(P.row_blocks, blocks, sizeof(int), cudaMemcpyHostToDevice, e->st));
+    }
     RC(run_layers(e, P, nullptr));
-    for (auto &f : fins) RC(prefill_finish_row(e, f.second, reqs[f.first]));
+    for (auto &f : fins) RC(prefill_finish_row(e, P, f.second, *reqs[f.first]));
     CK(cudaStreamSynchronize(e->st));   // the staging arrays are reused by the next chunk
     fins.clear();
     fill = 0;
     return CORUN_OK;
   };
   for (int r = 0; r < n_req; ++r) {
-    const PfReq &q = reqs[r];
+    const PfReq &q = *reqs[r];
     for (int done = 0; done < q.n;) {
       while (fill % unit) { tok[fill] = 0; pos[fill] = 0; act[fill] = 0; slt[fill] = pad_slot; ++fill; }   // rest of the tile before
       if (fill == CH) RC(run_chunk());
@@ -980,16 +1071,7 @@ int prefill_run(corun_engine *e, PfReq *reqs, int n_req) {
   if (fill > 0 || !fins.empty()) RC(run_chunk());
   CK(cudaMemcpyAsync(e->h_status, e->d_status, sizeof(int), cudaMemcpyDeviceToHost, e->st));
   CK(cudaStreamSynchronize(e->st));
-  RC(check_status(e));
-  for (int i = 0; i < n_req; ++i) {
-    PfReq &q = reqs[i];
-    RC(set_slot_state(e, q.slot, 1, q.n, 1, q.first, q.smp.temperature, q.smp.top_p));
-    e->in_use[q.slot] = 1;
-    e->ctx[q.slot] = q.n;
-    e->reserve[q.slot] = q.reserve;
-    e->step[q.slot] = 1;
-  }
-  return CORUN_OK;
+  return check_status(e);
 }
 
 }  // namespace

@@ -171,6 +171,23 @@ int tma_encode_fp16_4d(CUtensorMap *m, const void *base, const unsigned long lon
 // The same with 2 to 5 dimensions (dims / box: nd values, strides: nd - 1 byte strides of dimensions 1 ..).
 int tma_encode_fp16_nd(CUtensorMap *m, const void *base, int nd, const unsigned long long *dims, const unsigned long long *strides,
                        const unsigned *box);
+// ---- many rows (gemm_pair.cu): tiles of 256 rows x 256 weight rows, one per pair of SMs, whole K, no partials ----
+struct GemmPairPlan {
+  CUtensorMap tmHi, tmLo, tmOut, tmOut2;
+  int N = 0, K = 0, cap = 0, pairs = 0, n_tiles = 0;   // weight rows, reduction length, rows the buffers hold
+  bool swiglu = false;
+  float *out = nullptr;              // not owned
+};
+// out [cap, N] fp32 = X W^T for activations Xhi / Xlo [cap, K] (N % 8 == 0).
+int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, int num_sms);
+// W is [2F, K] (F gate rows, then F up rows; F % 8 == 0): out_hi / out_lo [cap, F] = silu(gate) * up as a bf16 hi/lo pair.
+int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,
+                                 __nv_bfloat16 *out_lo, int num_sms);
+int gemm_pair_prepare();             // opts the kernels into their shared-memory size (idempotent)
+// Rows 0 .. R-1 (R <= cap).  tmW: the weight matrix with a box of 128 rows (gemm_encode_map(.., 128)).
+cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st);
+// Tensor map for TMA stores of tiles of 32 rows x 128 bytes into a [rows, cols] row-major matrix (fp32 or bf16), 128-byte swizzle.
+int tma_encode_store_2d(CUtensorMap *m, const void *base, int is_fp32, unsigned long long rows, int cols);
 // direct[r, n] = gemm_load(r, n) for every tile that has partials (makes `direct` a plain matrix).
 cudaError_t gemm_fixup_launch(const GemmPlan &p, cudaStream_t st, bool pdl = false);
 

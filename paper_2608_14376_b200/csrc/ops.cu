@@ -132,6 +132,59 @@ qkv_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, int
   }
 }
 
+// The same for many rows from a plain matrix: bound by the L2 / HBM traffic (at 1024 rows of Qwen3-8B 25 MB read, 25 MB
+// written).  A thread takes four consecutive rotation indices of one head, (i .. i + 3) and their partners half a head
+// on: 16-byte loads and q stores, 8-byte cache stores, where the kernel above moves 4 and 2 bytes per access.
+constexpr int QKV_PLAIN_THREADS = 256;
+__global__ void __launch_bounds__(QKV_PLAIN_THREADS)
+qkv_post_plain_kernel(const float *__restrict__ qkv, Rows rows, const float2 *__restrict__ rope_tab, int nq, KvLayout kv, int layer,
+                      float *__restrict__ q_out, int *status) {
+  griddep_launch_dependents();
+  griddep_wait();
+  qkv = after_wait(qkv);                            // no load through it may move up across the wait
+  const int hd = kv.hd, half = hd >> 1, nkv = kv.n_kv, per_head = half / 4;
+  const int r = blockIdx.y, u = blockIdx.x * QKV_PLAIN_THREADS + threadIdx.x;
+  const int head = u / per_head, i = (u - head * per_head) * 4;
+  if (head >= nq + 2 * nkv) return;
+  if (head >= nq && rows.active[r] == 0) return;   // padding rows write no cache
+  const int pos = rows.pos[r];
+  const float *src = qkv + (size_t)r * (nq + 2 * nkv) * hd + head * hd + i;
+  float4 a = *reinterpret_cast<const float4 *>(src), b = *reinterpret_cast<const float4 *>(src + half);
+  if (head < nq + nkv) {
+    const float4 t0 = *reinterpret_cast<const float4 *>(rope_tab + (size_t)pos * half + i);      // (cos, sin) twice
+    const float4 t1 = *reinterpret_cast<const float4 *>(rope_tab + (size_t)pos * half + i + 2);
+    const float4 x = a, y = b;
+    a = make_float4(x.x * t0.x - y.x * t0.y, x.y * t0.z - y.y * t0.w, x.z * t1.x - y.z * t1.y, x.w * t1.z - y.w * t1.w);
+    b = make_float4(x.x * t0.y + y.x * t0.x, x.y * t0.w + y.y * t0.z, x.z * t1.y + y.z * t1.x, x.w * t1.w + y.w * t1.z);
+  }
+  if (head < nq) {
+    float *q = q_out + (size_t)r * nq * hd + head * hd + i;
+    *reinterpret_cast<float4 *>(q) = a;
+    *reinterpret_cast<float4 *>(q + half) = b;
+    return;
+  }
+#ifdef CORUN_CHECKED
+  if (!check_slot_pos(rows.slot[r], kv.n_slots, pos, kv.max_blocks, KV_BLOCK)) {   // the write is skipped
+    atomicCAS(status, 0, DEV_BAD_INDEX);
+    return;
+  }
+#endif
+  const int blk = kv.block_table[(size_t)rows.slot[r] * kv.max_blocks + pos / KV_BLOCK];
+#ifdef CORUN_CHECKED
+  if (!check_page(blk, kv.pool_blocks)) {
+    atomicCAS(status, 0, DEV_BAD_INDEX);
+    return;
+  }
+#endif
+  __half *page = kv.pool + (size_t)layer * kv.layer_stride + (size_t)blk * 2 * nkv * KV_BLOCK * hd;
+  const int tok = pos % KV_BLOCK;
+  __half *dst = head < nq + nkv ? page + kv_k_off(hd, head - nq, tok, i) : page + kv_v_off(nkv, hd, head - nq - nkv, tok, i);
+  const __half2 oa[2] = {__floats2half2_rn(a.x, a.y), __floats2half2_rn(a.z, a.w)};
+  const __half2 ob[2] = {__floats2half2_rn(b.x, b.y), __floats2half2_rn(b.z, b.w)};
+  *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(oa);
+  *reinterpret_cast<uint2 *>(dst + half) = *reinterpret_cast<const uint2 *>(ob);
+}
+
 // ---------------------------------------------------------------- SwiGLU
 __global__ void __launch_bounds__(256)
 swiglu_kernel(GemmOut gu, int F, __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo) {
@@ -874,6 +927,13 @@ cudaError_t launch_qkv_post(const GemmOut &qkv, const Rows &rows, const float2 *
                             int layer, float *q_out, int *d_status, cudaStream_t st) {
   return launch_k(qkv_post_kernel, dim3(nq + 2 * kv.n_kv, rows.R), dim3(kv.hd / 2), 0, st, true, qkv, rows, rope_tab, nq,
                   kv, layer, q_out, d_status);
+}
+
+cudaError_t launch_qkv_post_plain(const float *qkv, const Rows &rows, const float2 *rope_tab, int nq, const KvLayout &kv,
+                                  int layer, float *q_out, int *d_status, cudaStream_t st) {
+  const int units = (nq + 2 * kv.n_kv) * (kv.hd / 8);
+  return launch_k(qkv_post_plain_kernel, dim3((units + QKV_PLAIN_THREADS - 1) / QKV_PLAIN_THREADS, rows.R), dim3(QKV_PLAIN_THREADS), 0, st,
+                  true, qkv, rows, rope_tab, nq, kv, layer, q_out, d_status);
 }
 
 cudaError_t launch_swiglu(const GemmOut &gu, int R, int F, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, cudaStream_t st) {
