@@ -76,7 +76,9 @@ struct Program {
   // SMs (gemm_pair.cu); their results are plain matrices, the SwiGLU is in the gate / up GEMM's epilogue.
   bool pair = false;
   int cap = 0;
-  GemmPairPlan b_qkv, b_o, b_gu, b_down;
+  GemmPairPlan b_qkv, b_o, b_gu, b_down, b_router;
+  float *router_out = nullptr;
+  uint32_t *moe_mask = nullptr;
   std::vector<void *> allocs;
 };
 
@@ -86,6 +88,9 @@ struct Program {
 // Qwen3-8B layer: 256 rows 192 us of GEMMs in the chunk program, 293 us on pairs of SMs; 512 rows 384 against 359; 1024
 // rows 766 against 531; 2048 rows 1532 against 1010 (hence chunks as large as the buffers allow).
 constexpr int PREFILL_SMALL = 256, PREFILL_BIG = 2048;
+// Rows of a long prompt's chunk that the latent attention takes at a time (its partial results are kept per row).
+constexpr int MLA_ROWS = 256;
+static_assert(PREFILL_BIG <= MOE_MANY_ROWS, "a chunk of a long prompt is grouped in one go");
 
 }  // namespace
 
@@ -101,7 +106,7 @@ struct corun_engine {
   const bf16 *embed = nullptr, *lm_head = nullptr, *final_norm = nullptr;
   std::vector<const bf16 *> attn_norm, mlp_norm;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
-  std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down;   // boxes of 128 rows: the GEMMs on pairs of SMs
+  std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down, tb_router;   // boxes of 128 rows: the GEMMs on pairs of SMs
   std::vector<CUtensorMap> tm_gu_half;     // dense gate / up matrices with the box of the GEMM with SwiGLU in its epilogue
   std::vector<CUtensorMap> tm_k, tm_v;   // per layer: the pages as rows of head_dim halfs (keys and values alike)
   std::vector<CUtensorMap> tm_k4;        // the same memory as [8-token group][64-dim half][8 tokens][64 dims]: one box per (page, head) tile
@@ -177,6 +182,9 @@ int dmalloc(std::vector<void *> &keep, T **p, size_t n, bool zero = true) {
 
 int pad16(int x) { return (x + 15) / 16 * 16; }
 
+void mla_group_table(std::vector<int> &t, int nh, int rows_per_head, int BG, int R, int w_rows, int count_at);
+int program_create_groups(corun_engine *e, Program &P, int R);
+
 // fuse_swiglu: the gate / up GEMM writes silu(gate) * up itself (dense feed-forward, up to 128 padded rows: the
 // decode program while it is bound by the weight stream; whole tiles on fewer CTAs would cost a prefill chunk,
 // which is bound by the tensor pipe, a third of its gate / up rate).
@@ -231,14 +239,9 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
       RC(dmalloc(A, &P.mla_po, (size_t)mla_part_o_floats(R, md.nh, md.rank, e->max_ctx)));
       RC(dmalloc(A, &P.tab_uk, (size_t)n_groups * 3 + 1));
       RC(dmalloc(A, &P.tab_uv, (size_t)n_groups * 3 + 1));
-      std::vector<int> tk((size_t)n_groups * 3 + 1), tv((size_t)n_groups * 3 + 1);
-      tk[(size_t)n_groups * 3] = tv[(size_t)n_groups * 3] = n_groups;   // all groups are in use
-      for (int g = 0; g < n_groups; ++g) {          // group = (head, block of BG rows): its weight rows, rows in use
-        const int h = g / (P.RPH / BG), rb = g % (P.RPH / BG);
-        const int valid = R - rb * BG < BG ? (R - rb * BG > 0 ? R - rb * BG : 0) : BG;
-        tk[3 * g] = h * md.rank; tk[3 * g + 1] = 0; tk[3 * g + 2] = valid;
-        tv[3 * g] = h * (md.nope + md.vh); tv[3 * g + 1] = 0; tv[3 * g + 2] = valid;
-      }
+      std::vector<int> tk, tv;                      // all groups are in use
+      mla_group_table(tk, md.nh, P.RPH, BG, R, md.rank, 3 * n_groups);
+      mla_group_table(tv, md.nh, P.RPH, BG, R, md.nope + md.vh, 3 * n_groups);
       CK(cudaMemcpy(P.tab_uk, tk.data(), tk.size() * sizeof(int), cudaMemcpyHostToDevice));
       CK(cudaMemcpy(P.tab_uv, tv.data(), tv.size() * sizeof(int), cudaMemcpyHostToDevice));
       RC(gemm_plan_create_grouped(&P.p_uk, e->w_ukT, (long long)md.nh * md.rank, md.nope, md.rank, md.nope, P.qn_hi, P.qn_lo, n_groups,
@@ -286,35 +289,8 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
       if (grouped && (2 * e->moe_F) % GEMM_TILE_N == 0 && H % GEMM_TILE_N == 0) {
         // prefill chunks: every row through every expert would be (E + S) / top_k times the MMA work, which a
         // chunk of 256 rows does pay for; the rows of an expert are gathered into blocks of 64 instead
-        const int Fm = e->moe_F;
-        MoeGroups &g = P.grp;
-        g.n_groups_max = moe_max_groups(R, e->moe_E, e->moe_S, e->moe_K);
-        const size_t slots = (size_t)g.n_groups_max * MOE_GROUP_ROWS;
-        RC(dmalloc(A, &g.tab_up, (size_t)g.n_groups_max * 3 + 1));
-        RC(dmalloc(A, &g.tab_down, (size_t)g.n_groups_max * 3 + 1));
-        RC(dmalloc(A, &g.group_expert, (size_t)g.n_groups_max));
-        RC(dmalloc(A, &g.slot_row, slots));
-        RC(dmalloc(A, &g.slot_of, (size_t)R * NB));
-        RC(dmalloc(A, &g.slot_w, slots));
-        RC(dmalloc(A, &P.xg_hi, slots * H));
-        RC(dmalloc(A, &P.xg_lo, slots * H));
-        RC(dmalloc(A, &P.hg_hi, slots * Fm));
-        RC(dmalloc(A, &P.hg_lo, slots * Fm));
-        RC(dmalloc(A, &P.gug_out, slots * 2 * Fm));
-        RC(dmalloc(A, &P.yg_out, slots * H));
         RC(dmalloc(A, &P.plain_tiles, (size_t)(H / GEMM_TILE_N + 1)));
-        // gate / up per group with the routing weight and the SwiGLU in the epilogue where a tile width divides the
-        // experts' width, else fp32 sums and a kernel of its own
-        const int half = gemm_swiglu_blocks_half(Fm, NB, e->num_sms);
-        if (half)
-          RC(gemm_plan_create_grouped_swiglu(&P.p_gug, e->w0_gu, (long long)NB * 2 * Fm, Fm, H, half, P.xg_hi, P.xg_lo, g.n_groups_max,
-                                             MOE_GROUP_ROWS, P.hg_hi, P.hg_lo, g.slot_w, g.tab_up, e->num_sms));
-        else
-          RC(gemm_plan_create_grouped(&P.p_gug, e->w0_gu, (long long)NB * 2 * Fm, H, 2 * Fm, H, P.xg_hi, P.xg_lo, g.n_groups_max,
-                                      MOE_GROUP_ROWS, P.gug_out, g.tab_up, e->num_sms));
-        RC(gemm_plan_create_grouped(&P.p_dng, e->w0_down, H, NB * Fm, H, Fm, P.hg_hi, P.hg_lo, g.n_groups_max, MOE_GROUP_ROWS,
-                                    P.yg_out, g.tab_down, e->num_sms));
-        P.grouped = true;
+        RC(program_create_groups(e, P, R));
       }
     }
   }
@@ -325,10 +301,62 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
   return CORUN_OK;
 }
 
-// The program of long prompts (dense feed-forward, grouped-query attention): buffers for `cap` rows.
+// Group table of the up-projections of a latent attention layer with rows_per_head rows per head, R of them in use:
+// group = (head, block of BG rows): its first weight row, its first weight k-block, its rows; at count_at the number of
+// groups.
+void mla_group_table(std::vector<int> &t, int nh, int rows_per_head, int BG, int R, int w_rows, int count_at) {
+  t.assign((size_t)count_at + 1, 0);
+  const int per_head = rows_per_head / BG, n = nh * per_head;
+  for (int g = 0; g < n; ++g) {
+    const int h = g / per_head, rb = g % per_head, left = R - rb * BG;
+    t[3 * g] = h * w_rows;
+    t[3 * g + 2] = left < 0 ? 0 : left < BG ? left : BG;
+  }
+  t[count_at] = n;
+}
+
+// Buffers and plans of the experts' grouped form for up to R rows.
+int program_create_groups(corun_engine *e, Program &P, int R) {
+  const int Fm = e->moe_F, NB = e->moe_E + e->moe_S, H = e->sh.hidden;
+  auto &A = P.allocs;
+  MoeGroups &g = P.grp;
+  g.n_groups_max = moe_max_groups(R, e->moe_E, e->moe_S, e->moe_K);
+  const size_t slots = (size_t)g.n_groups_max * MOE_GROUP_ROWS;
+  RC(dmalloc(A, &g.tab_up, (size_t)g.n_groups_max * 3 + 1));
+  RC(dmalloc(A, &g.tab_down, (size_t)g.n_groups_max * 3 + 1));
+  RC(dmalloc(A, &g.group_expert, (size_t)g.n_groups_max));
+  RC(dmalloc(A, &g.slot_row, slots));
+  RC(dmalloc(A, &g.slot_of, (size_t)R * NB));
+  RC(dmalloc(A, &g.slot_w, slots));
+  RC(dmalloc(A, &P.xg_hi, slots * H));
+  RC(dmalloc(A, &P.xg_lo, slots * H));
+  RC(dmalloc(A, &P.hg_hi, slots * Fm));
+  RC(dmalloc(A, &P.hg_lo, slots * Fm));
+  RC(dmalloc(A, &P.yg_out, slots * H));
+  // gate / up per group with the routing weight and the SwiGLU in the epilogue where a tile width divides the
+  // experts' width, else fp32 sums and a kernel of its own
+  const int half = gemm_swiglu_blocks_half(Fm, NB, e->num_sms);
+  if (half) {
+    RC(gemm_plan_create_grouped_swiglu(&P.p_gug, e->w0_gu, (long long)NB * 2 * Fm, Fm, H, half, P.xg_hi, P.xg_lo, g.n_groups_max,
+                                       MOE_GROUP_ROWS, P.hg_hi, P.hg_lo, g.slot_w, g.tab_up, e->num_sms));
+  } else {
+    RC(dmalloc(A, &P.gug_out, slots * 2 * Fm));
+    RC(gemm_plan_create_grouped(&P.p_gug, e->w0_gu, (long long)NB * 2 * Fm, H, 2 * Fm, H, P.xg_hi, P.xg_lo, g.n_groups_max,
+                                MOE_GROUP_ROWS, P.gug_out, g.tab_up, e->num_sms));
+  }
+  RC(gemm_plan_create_grouped(&P.p_dng, e->w0_down, H, NB * Fm, H, Fm, P.hg_hi, P.hg_lo, g.n_groups_max, MOE_GROUP_ROWS,
+                              P.yg_out, g.tab_down, e->num_sms));
+  P.grouped = true;
+  return CORUN_OK;
+}
+
+// The program of long prompts: buffers for `cap` rows.
 int program_create_big(corun_engine *e, Program &P, int cap) {
   const corun_shape &s = e->sh;
-  const int H = s.hidden, QD = s.n_q_heads * s.head_dim, KD = s.n_kv_heads * s.head_dim, F = s.ffn, QKVN = QD + 2 * KD;
+  const MlaDims &md = e->md;
+  const int H = s.hidden, QD = s.n_q_heads * s.head_dim, KD = s.n_kv_heads * s.head_dim;
+  const int QKVN = e->mla ? md.nh * (md.nope + md.rope) + md.rank + md.rope : QD + 2 * KD;
+  const int F = e->moe_E ? e->dense_ffn : s.ffn;    // width of the dense feed-forward layers, 0: there are none
   P.pair = true;
   P.R = P.cap = P.BN = cap;
   P.has_layers = true;
@@ -341,19 +369,64 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   RC(dmalloc(A, &P.row_active, c));
   RC(dmalloc(A, &P.row_slot, c));
   RC(dmalloc(A, &P.h, c * H));
-  RC(dmalloc(A, &P.q, c * QD));
   RC(dmalloc(A, &P.qkv_out, c * QKVN));
   RC(dmalloc(A, &P.o_out, c * H));
   RC(dmalloc(A, &P.down_out, c * H));
   RC(dmalloc(A, &P.ao_hi, c * QD));
   RC(dmalloc(A, &P.ao_lo, c * QD));
-  RC(dmalloc(A, &P.ff_hi, c * F));
-  RC(dmalloc(A, &P.ff_lo, c * F));
   RC(dmalloc(A, &P.plain_tiles, (size_t)((QKVN > H ? QKVN : H) / GEMM_TILE_N + 1)));
   RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, cap, P.qkv_out, e->num_sms));
   RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, cap, P.o_out, e->num_sms));
-  RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, cap, P.ff_hi, P.ff_lo, e->num_sms));
-  RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, cap, P.down_out, e->num_sms));
+  if (F > 0) {
+    RC(dmalloc(A, &P.ff_hi, c * F));
+    RC(dmalloc(A, &P.ff_lo, c * F));
+    RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, cap, P.ff_hi, P.ff_lo, e->num_sms));
+    RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, cap, P.down_out, e->num_sms));
+  }
+  if (!e->mla) {
+    RC(dmalloc(A, &P.q, c * QD));
+  } else {
+    const size_t hr = (size_t)md.nh * cap;          // rows of the head-major matrices (cap is a multiple of 64)
+    const int n_groups = md.nh * (cap / 64);
+    RC(dmalloc(A, &P.qn_hi, hr * md.nope));
+    RC(dmalloc(A, &P.qn_lo, hr * md.nope));
+    RC(dmalloc(A, &P.q_lat, hr * md.rank));
+    RC(dmalloc(A, &P.q_rope, c * md.nh * md.rope));
+    RC(dmalloc(A, &P.ol_hi, hr * md.rank));
+    RC(dmalloc(A, &P.ol_lo, hr * md.rank));
+    RC(dmalloc(A, &P.uv_out, hr * (md.nope + md.vh)));
+    RC(dmalloc(A, &P.mla_ml, (size_t)mla_part_ml_floats(MLA_ROWS, md.nh, e->max_ctx) / 2));
+    RC(dmalloc(A, &P.mla_po, (size_t)mla_part_o_floats(MLA_ROWS, md.nh, md.rank, e->max_ctx)));
+    RC(dmalloc(A, &P.tab_uk, (size_t)n_groups * 3 + 1));
+    RC(dmalloc(A, &P.tab_uv, (size_t)n_groups * 3 + 1));
+    RC(gemm_plan_create_grouped(&P.p_uk, e->w_ukT, (long long)md.nh * md.rank, md.nope, md.rank, md.nope, P.qn_hi, P.qn_lo, n_groups,
+                                64, P.q_lat, P.tab_uk, e->num_sms));
+    RC(gemm_plan_create_grouped(&P.p_uv, e->w0_uv, (long long)md.nh * (md.nope + md.vh), md.rank, md.nope + md.vh, md.rank, P.ol_hi,
+                                P.ol_lo, n_groups, 64, P.uv_out, P.tab_uv, e->num_sms));
+    P.p_uk.keep_div = P.p_uv.keep_div = -1;         // the tables are copied ahead of a chunk's kernels (set_mla_rows)
+  }
+  if (e->moe_E) {
+    RC(dmalloc(A, &P.moe_w, c * (e->moe_E + e->moe_S)));
+    RC(dmalloc(A, &P.router_out, c * e->moe_E));
+    RC(dmalloc(A, &P.moe_mask, (size_t)(e->moe_E + e->moe_S) * (MOE_MANY_ROWS / 32)));
+    RC(gemm_pair_plan_create(&P.b_router, e->moe_E, H, P.xn_hi, P.xn_lo, cap, P.router_out, e->num_sms));
+    RC(program_create_groups(e, P, cap));
+  }
+  return CORUN_OK;
+}
+
+// (long prompts) lays the head-major matrices out for a chunk of R rows: whole blocks of 64 per head, one behind the other.
+int set_mla_rows(corun_engine *e, Program &P, int R) {
+  const MlaDims &md = e->md;
+  const int rph = (R + 63) / 64 * 64, count_at = md.nh * (P.cap / 64) * 3;
+  P.RPH = rph;
+  std::vector<int> t;
+  mla_group_table(t, md.nh, rph, 64, R, md.rank, count_at);
+  CK(cudaMemcpyAsync(P.tab_uk, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice, e->st));
+  CK(cudaStreamSynchronize(e->st));                 // `t` is pageable and reused
+  mla_group_table(t, md.nh, rph, 64, R, md.nope + md.vh, count_at);
+  CK(cudaMemcpyAsync(P.tab_uv, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice, e->st));
+  CK(cudaStreamSynchronize(e->st));
   return CORUN_OK;
 }
 
@@ -422,14 +495,48 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
     if (P.pair) {
       // long prompts: projections on pairs of SMs, plain results
       STAGE(gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st));
-      STAGE(launch_qkv_post_plain(P.qkv_out, rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
-      STAGE(launch_attention_prefill(e->tm_k[l], e->tm_v[l], P.q, rows, s.n_q_heads, kv, P.ao_hi, P.ao_lo, e->d_status, e->st));
+      if (e->mla) {
+        const MlaDims &md = e->md;
+        const MlaCache cache{e->kv_pool + (size_t)l * e->layer_stride, e->d_block_table, e->max_blocks, e->B, (long long)e->pool_blocks, e->kv_run};
+        STAGE(launch_mla_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi, P.qn_lo,
+                              P.q_rope, e->d_status, e->st));
+        STAGE(gemm_launch(P.p_uk, &e->tm_uk[l], e->d_status, e->st, nullptr, true));
+        for (int r0 = 0; r0 < P.R; r0 += MLA_ROWS) {
+          const int nr = P.R - r0 < MLA_ROWS ? P.R - r0 : MLA_ROWS;
+          const Rows part{P.row_token + r0, P.row_pos + r0, P.row_active + r0, P.row_slot + r0, nr};
+          STAGE(launch_mla_attention(e->tm_c[l], e->tm_cv[l], P.q_lat + (size_t)r0 * md.rank, md.rank, (long long)P.RPH * md.rank,
+                                     P.q_rope + (size_t)r0 * md.nh * md.rope, e->d_block_table, e->max_blocks, nullptr, &part, nr, md,
+                                     1.0f / sqrtf((float)(md.nope + md.rope)), e->mla_splits, P.mla_ml, P.mla_po, nullptr,
+                                     P.ol_hi + (size_t)r0 * md.rank, P.ol_lo + (size_t)r0 * md.rank, P.RPH, e->num_sms, e->d_status, true,
+                                     e->st, e->kv_run));
+        }
+        STAGE(gemm_launch(P.p_uv, &e->tm_uv[l], e->d_status, e->st, nullptr, true));
+        STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
+      } else {
+        STAGE(launch_qkv_post_plain(P.qkv_out, rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
+        STAGE(launch_attention_prefill(e->tm_k[l], e->tm_v[l], P.q, rows, s.n_q_heads, kv, P.ao_hi, P.ao_lo, e->d_status, e->st));
+      }
       STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
       const GemmOut o = plain_out(P, P.o_out, s.hidden);
       STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
-      STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st));
-      STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st));
-      n += 8;
+      if (e->moe_E && !dense_layer(e, l)) {
+        const int NB = e->moe_E + e->moe_S;
+        STAGE(gemm_pair_launch(P.b_router, e->tb_router[l], P.R, e->d_status, e->st));
+        STAGE(launch_moe_route(P.router_out, P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, e->st));
+        STAGE(launch_moe_group_many(P.moe_w, P.row_active, P.R, e->moe_E, e->moe_S, e->moe_F, P.moe_mask, P.grp, e->st));
+        STAGE(launch_moe_gather(P.xn_hi, P.xn_lo, s.hidden, P.grp, P.xg_hi, P.xg_lo, e->st));
+        if (P.p_gug.sw_hi) {
+          STAGE(gemm_launch(P.p_gug, &e->tm_gu_half[l], e->d_status, e->st, nullptr, true));
+        } else {
+          STAGE(gemm_launch(P.p_gug, &e->tm_gu[l], e->d_status, e->st, nullptr, true));
+          STAGE(launch_moe_swiglu_grouped(P.gug_out, P.moe_w, NB, e->moe_F, P.grp, P.hg_hi, P.hg_lo, e->st));
+        }
+        STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
+        STAGE(launch_moe_combine(P.yg_out, P.row_active, P.R, NB, s.hidden, P.grp, P.down_out, e->st));
+      } else {
+        STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st));
+        STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st));
+      }
       continue;
     }
     STAGE(gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, tr(4 * l + 0), true));
@@ -728,6 +835,11 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   e->lm_head = (const bf16 *)w->lm_head;
   e->final_norm = (const bf16 *)w->final_norm;
   const int H = s.hidden, QD = s.n_q_heads * s.head_dim, KD = s.n_kv_heads * s.head_dim, F = s.ffn;
+  // long prompts get a program of their own where their projections and experts have a form for many rows
+  const bool big_ok = !one_chunk_size && max_context > PREFILL_SMALL &&
+                      (!moe || (moe->n_experts % 8 == 0 && (2 * moe->expert_ffn) % GEMM_TILE_N == 0 && H % GEMM_TILE_N == 0 &&
+                                !getenv("CORUN_MOE_PREFILL_DENSE")));
+  const int big_cap = !big_ok ? 0 : max_context < PREFILL_BIG ? (max_context + 255) / 256 * 256 : PREFILL_BIG;
   e->tm_qkv.resize(s.n_layers);
   e->tm_o.resize(s.n_layers);
   e->tm_gu.resize(s.n_layers);
@@ -741,6 +853,17 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     const int qkv_rows = mla ? s.n_q_heads * (mla->qk_nope + mla->qk_rope) + mla->kv_lora_rank + mla->qk_rope : QD + 2 * KD;
     if ((rc = gemm_encode_map(&e->tm_qkv[l], w->wqkv[l], qkv_rows, H, GEMM_TILE_N))) return fail(rc);
     if ((rc = gemm_encode_map(&e->tm_o[l], w->wo[l], H, QD, GEMM_TILE_N))) return fail(rc);
+    if (big_cap) {                                  // the program of long prompts
+      if (e->tb_qkv.empty())
+        for (auto *v : {&e->tb_qkv, &e->tb_o, &e->tb_gu, &e->tb_down, &e->tb_router}) v->resize(s.n_layers);
+      const bool experts = moe && l >= first_dense;
+      const int Fd = moe ? dense_ffn : F;
+      if ((rc = gemm_encode_map(&e->tb_qkv[l], w->wqkv[l], qkv_rows, H, 128)) || (rc = gemm_encode_map(&e->tb_o[l], w->wo[l], H, QD, 128)))
+        return fail(rc);
+      if (experts ? (rc = gemm_encode_map(&e->tb_router[l], moe->router[l], moe->n_experts, H, 128))
+                  : ((rc = gemm_encode_map(&e->tb_gu[l], w->wgate_up[l], 2 * Fd, H, 128)) || (rc = gemm_encode_map(&e->tb_down[l], w->wdown[l], H, Fd, 128))))
+        return fail(rc);
+    }
     if (moe && l < first_dense) {                   // a dense feed-forward layer of a decoder with expert layers
       if (e->tm_gu_d.empty()) { e->tm_gu_d.resize(s.n_layers); e->tm_down_d.resize(s.n_layers); }
       if ((rc = gemm_encode_map(&e->tm_gu_d[l], w->wgate_up[l], 2 * dense_ffn, H, GEMM_TILE_N))) return fail(rc);
@@ -749,12 +872,6 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     }
     if ((rc = gemm_encode_map(&e->tm_gu[l], moe ? moe->gate_up[l] : w->wgate_up[l], 2 * F, H, GEMM_TILE_N))) return fail(rc);
     if ((rc = gemm_encode_map(&e->tm_down[l], moe ? moe->down[l] : w->wdown[l], H, F, GEMM_TILE_N))) return fail(rc);
-    if (!moe && !mla) {
-      if (e->tb_qkv.empty()) { e->tb_qkv.resize(s.n_layers); e->tb_o.resize(s.n_layers); e->tb_gu.resize(s.n_layers); e->tb_down.resize(s.n_layers); }
-      if ((rc = gemm_encode_map(&e->tb_qkv[l], w->wqkv[l], qkv_rows, H, 128)) || (rc = gemm_encode_map(&e->tb_o[l], w->wo[l], H, QD, 128)) ||
-          (rc = gemm_encode_map(&e->tb_gu[l], w->wgate_up[l], 2 * F, H, 128)) || (rc = gemm_encode_map(&e->tb_down[l], w->wdown[l], H, F, 128)))
-        return fail(rc);
-    }
     if (!moe && (rc = gemm_encode_map(&e->tm_gu_half[l], w->wgate_up[l], 2 * F, H, gemm_swiglu_half(F, e->num_sms)))) return fail(rc);
     if (moe && moe_half && (rc = gemm_encode_map(&e->tm_gu_half[l], moe->gate_up[l], 2 * F, H, moe_half))) return fail(rc);
   }
@@ -876,10 +993,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   // a prefill chunk is filled from row 0: the host says which blocks of rows it reaches (prefill_run)
   for (GemmPlan *pl : {&e->pre.p_qkv, &e->pre.p_o, &e->pre.p_gu, &e->pre.p_down, &e->pre.p_gu_d, &e->pre.p_down_d})
     pl->row_blocks = e->pre.row_blocks;
-  if (!mla && !moe && !one_chunk_size && max_context > PREFILL_SMALL) {
-    const int cap = max_context < PREFILL_BIG ? (max_context + 255) / 256 * 256 : PREFILL_BIG;
-    if ((rc = program_create_big(e, e->big, cap))) return fail(rc);
-  }
+  if (big_cap && (rc = program_create_big(e, e->big, big_cap))) return fail(rc);
   if ((rc = program_create(e, e->lm1, 1, false, true))) return fail(rc);
 
   // the allocations above were cleared and filled through the legacy stream, which the engine's
@@ -1029,7 +1143,10 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
   int fill = 0, pad_slot = reqs[0]->slot;
   auto run_chunk = [&]() -> int {
     const int rows_n = P.pair ? fill : CH;
-    if (P.pair) P.R = fill;
+    if (P.pair) {
+      P.R = fill;
+      if (e->mla) RC(set_mla_rows(e, P, fill));
+    }
     for (int i = fill; i < rows_n; ++i) { tok[i] = 0; pos[i] = 0; act[i] = 0; slt[i] = pad_slot; }
     CK(cudaMemcpyAsync(P.row_token, tok, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
     CK(cudaMemcpyAsync(P.row_pos, pos, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));

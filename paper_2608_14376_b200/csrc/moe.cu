@@ -284,6 +284,112 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_kernel(const floa
   }
 }
 
+// ---- many rows (up to MOE_MANY_ROWS): the kernel above reads the whole table w[r, e] in every CTA, 1 MB at 2048 rows and
+// 128 experts.  Here a first kernel turns it into one bit per (expert, row), 32 KB in all, which every CTA of the second
+// reads, and the second hands out the slots of all its rows at once.
+constexpr int MOE_MASK_WORDS = MOE_MANY_ROWS / 32;
+
+__global__ void __launch_bounds__(256) moe_mask_kernel(const float *__restrict__ w, const int *__restrict__ active, int R, int NB,
+                                                       uint32_t *__restrict__ mask) {
+  griddep_launch_dependents();
+  griddep_wait();
+  w = after_wait(w); active = after_wait(active);
+  const int r0 = (int)blockIdx.x * 32;
+  for (int e = (int)threadIdx.x; e < NB; e += 256) {
+    uint32_t m = 0u;
+#pragma unroll 8
+    for (int i = 0; i < 32; ++i) {
+      const int r = r0 + i;
+      if (r < R && active[r] != 0 && w[(size_t)r * NB + e] != 0.f) m |= 1u << i;
+    }
+    mask[e * MOE_MASK_WORDS + (int)blockIdx.x] = m;
+  }
+}
+
+__global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_many_kernel(const float *__restrict__ w, const uint32_t *__restrict__ mask, int R,
+                                                                           int NB, int E, int F, MoeGroups g) {
+  griddep_launch_dependents();
+  __shared__ int cnt[MOE_MAX_EXPERTS + 8];
+  __shared__ uint32_t own[MOE_MASK_WORDS];
+  __shared__ int own_before[MOE_MASK_WORDS];         // the expert's rows before a word
+  __shared__ int first_s, total_s;
+  const int e = (int)blockIdx.x, tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int words = (R + 31) / 32;
+  griddep_wait();
+  w = after_wait(w); mask = after_wait(mask);
+  for (int ee = warp; ee < NB; ee += MOE_GROUP_THREADS / 32) {
+    const uint32_t a = lane < words ? mask[ee * MOE_MASK_WORDS + lane] : 0u, b = lane + 32 < words ? mask[ee * MOE_MASK_WORDS + lane + 32] : 0u;
+    const int na = __popc(a), nb = __popc(b);
+    int ia = na, ib = nb;                            // inclusive sums over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int xa = __shfl_up_sync(0xffffffffu, ia, o), xb = __shfl_up_sync(0xffffffffu, ib, o);
+      if (lane >= o) { ia += xa; ib += xb; }
+    }
+    const int all_a = __shfl_sync(0xffffffffu, ia, 31), all_b = __shfl_sync(0xffffffffu, ib, 31);
+    if (lane == 0) cnt[ee] = all_a + all_b;
+    if (ee == e) {
+      own[lane] = a; own[lane + 32] = b;
+      own_before[lane] = ia - na; own_before[lane + 32] = all_a + ib - nb;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int before = 0, all = 0;
+    for (int ee = lane; ee < NB; ee += 32) {
+      const int n = (cnt[ee] + MOE_GROUP_ROWS - 1) / MOE_GROUP_ROWS;
+      all += n;
+      if (ee < e) before += n;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      before += __shfl_xor_sync(0xffffffffu, before, o);
+      all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+    if (lane == 0) { first_s = before; total_s = all < g.n_groups_max ? all : g.n_groups_max; }
+  }
+  __syncthreads();
+  const int first = first_s, used = total_s;
+  if (e == 0) {
+    for (int u = used + tid; u < g.n_groups_max; u += MOE_GROUP_THREADS) {   // groups nobody needs
+      g.tab_up[3 * u + 2] = 0;
+      g.tab_down[3 * u + 2] = 0;
+    }
+    if (tid == 0) g.tab_up[3 * g.n_groups_max] = g.tab_down[3 * g.n_groups_max] = used;   // what the GEMMs walk
+  }
+  const int n_groups = (cnt[e] + MOE_GROUP_ROWS - 1) / MOE_GROUP_ROWS;
+  for (int k = tid; k < n_groups; k += MOE_GROUP_THREADS) {
+    const int u = first + k;
+    if (u >= g.n_groups_max) break;                 // cannot happen: n_groups_max bounds the sum
+    const int rows = min(MOE_GROUP_ROWS, cnt[e] - k * MOE_GROUP_ROWS);
+    g.tab_up[3 * u] = e * 2 * F; g.tab_up[3 * u + 1] = 0; g.tab_up[3 * u + 2] = rows;
+    g.tab_down[3 * u] = 0; g.tab_down[3 * u + 1] = e * F / GEMM_BLOCK_K; g.tab_down[3 * u + 2] = rows;
+    g.group_expert[u] = e;
+  }
+  for (int r = tid; r < R; r += MOE_GROUP_THREADS) {
+    const uint32_t m = own[r >> 5], bit = 1u << (r & 31);
+    int slot = -1;
+    if (m & bit) {
+      slot = first * MOE_GROUP_ROWS + own_before[r >> 5] + __popc(m & (bit - 1u));
+      g.slot_row[slot] = r;
+      g.slot_w[slot] = w[(size_t)r * NB + e];
+    }
+    g.slot_of[(size_t)e * R + r] = slot;
+  }
+}
+
+// Routing of many rows: one warp per row.
+__global__ void __launch_bounds__(256) moe_route_kernel(const float *__restrict__ logits, int R, int E, int S, int top_k, int renormalize,
+                                                        float *__restrict__ w) {
+  griddep_launch_dependents();
+  griddep_wait();
+  logits = after_wait(logits);
+  const int r = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (r >= R) return;
+  const float *row = logits + (size_t)r * E;
+  moe_route_row([&](int e) { return row[e]; }, r, lane, E, S, top_k, renormalize, w, nullptr, nullptr);
+}
+
 // The gathered activation rows: one warp per slot of the groups in use (all of a row's loads requested before the
 // first store).  H % 256 == 0 up to 4096, else eight 16-byte pieces per lane at a time.
 __global__ void __launch_bounds__(256) moe_gather_kernel(const bf16 *__restrict__ x_hi, const bf16 *__restrict__ x_lo, int H,
@@ -381,6 +487,18 @@ cudaError_t launch_moe_group(const float *w, const int *active, int R, int E, in
                              cudaStream_t st) {
   if (E + S > MOE_MAX_EXPERTS + 8 || F % GEMM_BLOCK_K || R > 256) return cudaErrorInvalidValue;
   return launch_k(moe_group_kernel, dim3(E + S), dim3(MOE_GROUP_THREADS), 0, st, true, w, active, R, E + S, E, F, g);
+}
+
+cudaError_t launch_moe_group_many(const float *w, const int *active, int R, int E, int S, int F, uint32_t *mask, const MoeGroups &g,
+                                  cudaStream_t st) {
+  if (E + S > MOE_MAX_EXPERTS + 8 || F % GEMM_BLOCK_K || R > MOE_MANY_ROWS) return cudaErrorInvalidValue;
+  cudaError_t e = launch_k(moe_mask_kernel, dim3((R + 31) / 32), dim3(256), 0, st, true, w, active, R, E + S, mask);
+  if (e != cudaSuccess) return e;
+  return launch_k(moe_group_many_kernel, dim3(E + S), dim3(MOE_GROUP_THREADS), 0, st, true, w, mask, R, E + S, E, F, g);
+}
+
+cudaError_t launch_moe_route(const float *logits, int R, int E, int S, int top_k, int renormalize, float *w, cudaStream_t st) {
+  return launch_k(moe_route_kernel, dim3((R + 7) / 8), dim3(256), 0, st, true, logits, R, E, S, top_k, renormalize, w);
 }
 
 cudaError_t launch_moe_gather(const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_lo, int H, const MoeGroups &g,

@@ -21,6 +21,7 @@ cudaError_t launch_moe_swiglu(const GemmOut &gu, const float *w, int R, int F, i
 
 // ---- grouped form (prefill chunks): every expert's rows gathered into blocks of MOE_GROUP_ROWS rows ----
 constexpr int MOE_GROUP_ROWS = 64;
+constexpr int MOE_MANY_ROWS = 2048;   // most rows of the many-rows forms below
 // Most groups a chunk of R rows can need: one per expert plus one per full block of selected (row, expert) pairs.
 inline int moe_max_groups(int R, int E, int S, int top_k) { return E + S + R * (top_k + S) / MOE_GROUP_ROWS; }
 
@@ -40,6 +41,11 @@ struct MoeGroups {
 // active[r] == 0 are left out.  w: the routing weights [R][E + S] of launch_moe_route.  One CTA.
 cudaError_t launch_moe_group(const float *w, const int *active, int R, int E, int S, int F, const MoeGroups &g,
                              cudaStream_t st);
+// The same for up to MOE_MANY_ROWS rows in two kernels (prefill of long prompts).  mask: [E + S][MOE_MANY_ROWS / 32] words.
+cudaError_t launch_moe_group_many(const float *w, const int *active, int R, int E, int S, int F, uint32_t *mask, const MoeGroups &g,
+                                  cudaStream_t st);
+// Routing of many rows from their router logits [R, E] (fp32, computed by a GEMM): as launch_moe_router otherwise.
+cudaError_t launch_moe_route(const float *logits, int R, int E, int S, int top_k, int renormalize, float *w, cudaStream_t st);
 // xg[slot, :] = x[slot_row[slot], :] for both halves of the activations (bf16, H values per row).
 cudaError_t launch_moe_gather(const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_lo, int H, const MoeGroups &g,
                               __nv_bfloat16 *xg_hi, __nv_bfloat16 *xg_lo, cudaStream_t st);
