@@ -53,3 +53,58 @@ def test_long_prompts_alone_and_sharing_chunks(tiny, lens):
     assert list(e.prefill_batch(slots, prompts, res, 0.7, 0.95, seeds)) == first
     assert after() == alone
     e.close()
+
+
+@pytest.mark.parametrize("arch", ["moe", "mla"])
+@pytest.mark.parametrize("lens", [[257, 30, 383], [2049, 300]])
+def test_long_prompts_through_expert_layers(orc, arch, lens):
+    """The same for decoders with expert layers (rows grouped by expert over a whole chunk; 2049 tokens: several groups of an
+    expert, and a chunk of one row behind a full one) and for latent attention (blocks of 64 rows per head)."""
+    from paper_2608_14376_b200 import corun
+
+    B = 4
+    mla = dict(kv_lora_rank=256, qk_nope=128, qk_rope=32, v_head=128, first_dense=1)
+    moe = dict(n_experts=16, top_k=3, expert_ffn=128, n_shared=1, renormalize=arch == "moe")
+    if arch == "mla":
+        sh = synth.ModelShape(2, 256, 4, 4, 128, 384, 1024, 1e-6, 10000.0)
+        w, m = synth.make_mla_weights_numpy(sh, mla, seed=4)
+    else:
+        sh = synth.ModelShape(2, 256, 4, 2, 64, 64, 1024, 1e-6, 10000.0)
+        w, m = synth.make_weights_numpy(sh, seed=4), None
+    ex = synth.make_moe_numpy(sh, seed=4, **moe)
+    model = orc.Model(orc.Shape(**sh.dict()), w, moe=ex, **(dict(mla=m) if m else {}))
+    kw = dict(moe=synth.moe_numpy_to_torch(ex, "cuda"))
+    if m:
+        wt, kw["mla"] = synth.mla_numpy_to_torch(w, m, "cuda")
+        kw["kv_block"] = 64
+    else:
+        wt = synth.weights_numpy_to_torch(w, "cuda")
+    prompts = synth.make_prompts(sh.vocab, lens, seed=900 + lens[0])
+    slots = [2, 0, 3][:len(lens)]
+    seeds = np.array([synth.request_seed(i) for i in range(len(lens))], np.uint64)
+    res = [n + 4 for n in lens]
+    e = corun.Engine(sh, wt, B, max(res), **kw)
+
+    def after():
+        active = np.zeros(B, np.uint8); active[slots] = 1
+        sd = np.zeros(B, np.uint64); sd[slots] = seeds
+        out = [e.logits(s).tobytes() for s in slots]
+        for s, n in zip(slots, lens):
+            k, v = e.kv_read(s, sh.n_layers - 1, 0, n)
+            out.append(k.tobytes() + (v.tobytes() if v is not None else b""))
+        out.append(e.decode_step(active, sd).tobytes())
+        return out + [e.logits(s).tobytes() for s in slots]
+
+    first = [e.prefill(s, p, r, 0.7, 0.95, seed=int(sd)) for s, p, r, sd in zip(slots, prompts, res, seeds)]
+    for s, p in zip(slots, prompts):
+        if arch == "mla" and len(p) > 400:               # its oracle decompresses every cached token for every row: minutes
+            continue
+        r = orc.Request(model, p, 1, max_T=len(p) + 4)
+        r.prefill()
+        assert np.abs(e.logits(s) - r.logits).max() <= TOL
+    alone = after()
+    for s in slots:
+        e.release(s)
+    assert list(e.prefill_batch(slots, prompts, res, 0.7, 0.95, seeds)) == first
+    assert after() == alone
+    e.close()
