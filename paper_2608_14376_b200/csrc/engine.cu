@@ -513,7 +513,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         STAGE(gemm_launch(P.p_uv, &e->tm_uv[l], e->d_status, e->st, nullptr, true));
         STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
       } else {
-        STAGE(launch_qkv_post_plain(P.qkv_out, rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
+        STAGE(launch_qkv_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
         STAGE(launch_attention_prefill(e->tm_k[l], e->tm_v[l], P.q, rows, s.n_q_heads, kv, P.ao_hi, P.ao_lo, e->d_status, e->st));
       }
       STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));

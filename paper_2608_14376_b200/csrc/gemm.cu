@@ -638,7 +638,9 @@ int gemm_plan_fill(GemmPlan *p, const void *W, int N, int K, const void *Xhi, co
   // SMs left out): no CTA then crosses a tile boundary, so none has two epilogues in a row, and above 128
   // rows -- where the two row blocks of a tile fill TMEM and the epilogue of a segment cannot overlap the MMAs
   // of the next -- none stops in the middle of its range.
-  const int per_tile = p->grid >= 2 * p->n_tiles ? p->grid / p->n_tiles : 0;
+  // At least four k-blocks per CTA: with fewer, the consumer's extra partials cost more than the shorter stream saves.
+  int per_tile = p->grid >= 2 * p->n_tiles ? p->grid / p->n_tiles : 0;
+  if (per_tile > 2 && per_tile > (p->KB + 3) / 4) per_tile = p->KB > 8 ? (p->KB + 3) / 4 : 2;
   if (per_tile) p->grid = per_tile * p->n_tiles;
   if (total * (long long)p->grid >= (1ll << 31)) return CORUN_EINVAL;
   const size_t stage = (size_t)W_TILE_BYTES + gemm_x_stage_bytes(BN);

@@ -85,9 +85,10 @@ resid_norm_kernel(float *__restrict__ h, int H, const __nv_bfloat16 *__restrict_
 }
 
 // ---------------------------------------------------------------- RoPE + KV append
-// One CTA per (head, row): heads 0..nq-1 are q, nq..nq+nkv-1 are k, the rest are v; hd/2 threads.
+// Few rows: one CTA per (head, row), two values per thread, so that the many small loads of the GEMM's partials are spread
+// over thousands of threads (64 rows of the Qwen3-8B layer: 3.4 us less per layer than four values per thread).  Heads 0..nq-1 are q, nq..nq+nkv-1 are k, the rest are v; hd/2 threads.
 __global__ void __launch_bounds__(64)
-qkv_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, int nq, KvLayout kv, int layer,
+qkv_post_few_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, int nq, KvLayout kv, int layer,
                 float *__restrict__ q_out, int *status) {
   griddep_launch_dependents();
   griddep_wait();
@@ -132,24 +133,32 @@ qkv_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, int
   }
 }
 
-// The same for many rows from a plain matrix: bound by the L2 / HBM traffic (at 1024 rows of Qwen3-8B 25 MB read, 25 MB
-// written).  A thread takes four consecutive rotation indices of one head, (i .. i + 3) and their partners half a head
-// on: 16-byte loads and q stores, 8-byte cache stores, where the kernel above moves 4 and 2 bytes per access.
-constexpr int QKV_PLAIN_THREADS = 256;
-__global__ void __launch_bounds__(QKV_PLAIN_THREADS)
-qkv_post_plain_kernel(const float *__restrict__ qkv, Rows rows, const float2 *__restrict__ rope_tab, int nq, KvLayout kv, int layer,
-                      float *__restrict__ q_out, int *status) {
+// Many rows: a thread takes four consecutive rotation indices of one head, (i .. i + 3) and their partners half a head on: 16-byte loads
+// and q stores, 8-byte cache stores.  Bound by L2 / HBM traffic (PLAIN: prefill of long prompts, a plain matrix: at 1024
+// rows of Qwen3-8B 25 MB read, 25 MB written; 256 rows with partials: 11 us less per layer than the kernel above).
+constexpr int QKV_THREADS = 128, QKV_FEW_ROWS = 64;
+template <bool PLAIN>
+__global__ void __launch_bounds__(QKV_THREADS)
+qkv_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, int nq, KvLayout kv, int layer,
+                float *__restrict__ q_out, int *status) {
   griddep_launch_dependents();
   griddep_wait();
-  qkv = after_wait(qkv);                            // no load through it may move up across the wait
   const int hd = kv.hd, half = hd >> 1, nkv = kv.n_kv, per_head = half / 4;
-  const int r = blockIdx.y, u = blockIdx.x * QKV_PLAIN_THREADS + threadIdx.x;
+  const int r = blockIdx.y, u = blockIdx.x * QKV_THREADS + threadIdx.x;
   const int head = u / per_head, i = (u - head * per_head) * 4;
   if (head >= nq + 2 * nkv) return;
   if (head >= nq && rows.active[r] == 0) return;   // padding rows write no cache
   const int pos = rows.pos[r];
-  const float *src = qkv + (size_t)r * (nq + 2 * nkv) * hd + head * hd + i;
-  float4 a = *reinterpret_cast<const float4 *>(src), b = *reinterpret_cast<const float4 *>(src + half);
+  const int col = head * hd + i;                   // q, k and v heads are contiguous in the GEMM output
+  float4 a, b;
+  if (PLAIN) {
+    const float *src = after_wait(qkv.direct) + (size_t)r * qkv.N + col;
+    a = *reinterpret_cast<const float4 *>(src);
+    b = *reinterpret_cast<const float4 *>(src + half);
+  } else {
+    a = gemm_load4(qkv, r, col);
+    b = gemm_load4(qkv, r, col + half);
+  }
   if (head < nq + nkv) {
     const float4 t0 = *reinterpret_cast<const float4 *>(rope_tab + (size_t)pos * half + i);      // (cos, sin) twice
     const float4 t1 = *reinterpret_cast<const float4 *>(rope_tab + (size_t)pos * half + i + 2);
@@ -925,15 +934,12 @@ cudaError_t launch_resid_norm(float *h, int H, const __nv_bfloat16 *embed, const
 
 cudaError_t launch_qkv_post(const GemmOut &qkv, const Rows &rows, const float2 *rope_tab, int nq, const KvLayout &kv,
                             int layer, float *q_out, int *d_status, cudaStream_t st) {
-  return launch_k(qkv_post_kernel, dim3(nq + 2 * kv.n_kv, rows.R), dim3(kv.hd / 2), 0, st, true, qkv, rows, rope_tab, nq,
+  if (rows.R <= QKV_FEW_ROWS)
+    return launch_k(qkv_post_few_kernel, dim3(nq + 2 * kv.n_kv, rows.R), dim3(kv.hd / 2), 0, st, true, qkv, rows, rope_tab, nq, kv, layer,
+                    q_out, d_status);
+  const dim3 grid(((nq + 2 * kv.n_kv) * (kv.hd / 8) + QKV_THREADS - 1) / QKV_THREADS, rows.R);
+  return launch_k(qkv.ws ? qkv_post_kernel<false> : qkv_post_kernel<true>, grid, dim3(QKV_THREADS), 0, st, true, qkv, rows, rope_tab, nq,
                   kv, layer, q_out, d_status);
-}
-
-cudaError_t launch_qkv_post_plain(const float *qkv, const Rows &rows, const float2 *rope_tab, int nq, const KvLayout &kv,
-                                  int layer, float *q_out, int *d_status, cudaStream_t st) {
-  const int units = (nq + 2 * kv.n_kv) * (kv.hd / 8);
-  return launch_k(qkv_post_plain_kernel, dim3((units + QKV_PLAIN_THREADS - 1) / QKV_PLAIN_THREADS, rows.R), dim3(QKV_PLAIN_THREADS), 0, st,
-                  true, qkv, rows, rope_tab, nq, kv, layer, q_out, d_status);
 }
 
 cudaError_t launch_swiglu(const GemmOut &gu, int R, int F, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, cudaStream_t st) {
