@@ -55,6 +55,12 @@ struct Program {
   // Mixture-of-Experts feed-forward layers: p_gu / p_down are then the GEMMs over all experts' gate / up rows
   // and over the concatenated hidden activations; moe_w the rows' routing weights
   float *moe_w = nullptr;
+  // selected-experts form (decode up to 64 rows): only the experts that a row selected are streamed; p_gug / p_dng are its
+  // GEMMs, hg / yg hold [expert][BN] rows, moe_sel every row's experts.  Measured per step, 12 layers of the Qwen3-30B-A3B
+  // shape, against every row through every expert: 1 row of 1 3.15 -> 1.24 ms, 16 of 32 3.54 -> 2.72, 40 of 64
+  // 3.94 -> 3.87, 64 of 64 (nearly all experts selected) 4.26 -> 4.28.
+  bool select = false;
+  int *moe_sel = nullptr;
   // grouped form of the experts' GEMMs (prefill chunks: the rows of an expert gathered into blocks of 64)
   bool grouped = false;
   MoeGroups grp{};
@@ -252,12 +258,17 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
     }
     RC(dmalloc(A, &P.qkv_out, (size_t)R * QKVN));
     RC(dmalloc(A, &P.o_out, (size_t)R * H));
-    RC(dmalloc(A, &P.gu_out, (size_t)R * 2 * Fmax));
+    // expert layers up to 64 rows: all rows with every expert that one of them selected
+    const int NBx = e->moe_E + e->moe_S, half_x = e->moe_E ? gemm_swiglu_blocks_half(e->moe_F, NBx, e->num_sms) : 0;
+    P.select = fuse_swiglu && e->moe_E && P.BN <= 64 && half_x && H % GEMM_TILE_N == 0 && NBx <= GEMM_MAX_SELECT &&
+               !getenv("CORUN_MOE_DECODE_DENSE");
+    const int Fbuf = P.select ? (Fd > 64 ? Fd : 64) : Fmax;   // the selected-experts form has buffers of its own
+    RC(dmalloc(A, &P.gu_out, (size_t)R * 2 * Fbuf));
     RC(dmalloc(A, &P.down_out, (size_t)R * H));
     RC(dmalloc(A, &P.ao_hi, (size_t)P.BN * QD));
     RC(dmalloc(A, &P.ao_lo, (size_t)P.BN * QD));
-    RC(dmalloc(A, &P.ff_hi, (size_t)P.BN * Fmax));
-    RC(dmalloc(A, &P.ff_lo, (size_t)P.BN * Fmax));
+    RC(dmalloc(A, &P.ff_hi, (size_t)P.BN * Fbuf));
+    RC(dmalloc(A, &P.ff_lo, (size_t)P.BN * Fbuf));
     if (e->mla && e->moe_E && e->first_dense > 0) {   // the dense feed-forward layers of a decoder with expert layers
       RC(gemm_plan_create(&P.p_gu_d, e->w0_gu_d, 2 * Fd, H, P.xn_hi, P.xn_lo, R, P.BN, P.gu_out, P.ws, e->num_sms));
       RC(gemm_plan_create(&P.p_down_d, e->w0_down_d, H, Fd, P.ff_hi, P.ff_lo, R, P.BN, P.down_out, P.ws, e->num_sms));
@@ -270,12 +281,24 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
     // SwiGLU kernel measured faster: the epilogue would write zeros for every pair that was not selected)
     const bool moe_fused = fuse_swiglu && e->moe_E && P.BN > 64 && P.BN <= 128 &&
                            gemm_swiglu_blocks_half(e->moe_F, e->moe_E + e->moe_S, e->num_sms) > 0;
-    if (fuse_swiglu && !e->moe_E && P.BN <= 128)
+    if (P.select) {
+      const int nb = e->moe_E + e->moe_S, per_row = e->moe_K + e->moe_S, Fm = e->moe_F;
+      RC(dmalloc(A, &P.moe_w, (size_t)R * nb));
+      RC(dmalloc(A, &P.moe_sel, (size_t)R * per_row));
+      RC(dmalloc(A, &P.hg_hi, (size_t)nb * P.BN * Fm));
+      RC(dmalloc(A, &P.hg_lo, (size_t)nb * P.BN * Fm));
+      RC(dmalloc(A, &P.yg_out, (size_t)nb * P.BN * H));
+      RC(dmalloc(A, &P.plain_tiles, (size_t)(H / GEMM_TILE_N + 1)));
+      RC(gemm_plan_create_select_up(&P.p_gug, e->w0_gu, nb, Fm, H, half_x, P.xn_hi, P.xn_lo, R, P.BN, P.hg_hi, P.hg_lo, P.moe_w, P.moe_sel,
+                                    R * per_row, e->num_sms));
+      RC(gemm_plan_create_select_down(&P.p_dng, e->w0_down, nb, H, Fm, P.hg_hi, P.hg_lo, R, P.BN, P.yg_out, P.moe_w, P.moe_sel,
+                                      R * per_row, e->num_sms));
+    } else if (fuse_swiglu && !e->moe_E && P.BN <= 128)
       RC(gemm_plan_create_swiglu(&P.p_gu, e->w0_gu, F, H, P.xn_hi, P.xn_lo, R, P.BN, P.ff_hi, P.ff_lo, e->num_sms));
     else if (!moe_fused)
       RC(gemm_plan_create(&P.p_gu, e->w0_gu, 2 * F, H, P.xn_hi, P.xn_lo, R, P.BN, P.gu_out, P.ws, e->num_sms));
-    RC(gemm_plan_create(&P.p_down, e->w0_down, H, F, P.ff_hi, P.ff_lo, R, P.BN, P.down_out, P.ws, e->num_sms));
-    if (e->moe_E) {
+    if (!P.select) RC(gemm_plan_create(&P.p_down, e->w0_down, H, F, P.ff_hi, P.ff_lo, R, P.BN, P.down_out, P.ws, e->num_sms));
+    if (e->moe_E && !P.select) {
       const int NB = e->moe_E + e->moe_S;
       RC(dmalloc(A, &P.moe_w, (size_t)R * NB));
       if (moe_fused)
@@ -462,7 +485,7 @@ bool dense_layer(const corun_engine *e, int layer) { return e->mla && e->moe_E &
 GemmOut ffn_out(const corun_engine *e, const Program &P, int layer) {
   if (P.pair) return plain_out(P, P.down_out, e->sh.hidden);
   if (dense_layer(e, layer)) return P.p_down_d.out();
-  if (P.grouped) return GemmOut{P.down_out, nullptr, P.plain_tiles, P.plain_tiles, P.p_down.N, P.p_down.KB, P.BN};
+  if (P.grouped || P.select) return plain_out(P, P.down_out, e->sh.hidden);
   return P.p_down.out();
 }
 
@@ -588,6 +611,16 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
       STAGE(launch_moe_combine(P.yg_out, P.row_active, P.R, NB, s.hidden, P.grp, P.down_out, e->st));
       n += 13 + (&P == &e->dec ? 1 : 0);
+      continue;
+    } else if (P.select) {
+      // router -> top-k weights and the rows' experts -> gate / up with routing weight and SwiGLU, then down, per selected
+      // expert for all rows -> the row's experts summed in ascending expert id
+      STAGE(launch_moe_router(P.xn_hi, P.xn_lo, s.hidden, e->router[l], P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, nullptr,
+                              nullptr, e->st, P.row_active, P.moe_sel));
+      STAGE(gemm_launch(P.p_gug, &e->tm_gu_half[l], e->d_status, e->st, nullptr, true));
+      STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
+      STAGE(launch_moe_combine_select(P.yg_out, P.moe_sel, e->moe_K + e->moe_S, P.BN, P.R, s.hidden, P.down_out, e->st));
+      n += 10 + (&P == &e->dec ? 1 : 0);
       continue;
     } else if (e->moe_E) {
       // router -> top-k weights -> all experts' gate / up (rows that did not select a tile's expert are not
@@ -1479,14 +1512,19 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
         // launched as in the step's graph: with programmatic stream serialization
         case 0: ce = gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, nullptr, true); break;
         case 1: ce = gemm_launch(P.p_o, &e->tm_o[l], e->d_status, e->st, nullptr, true); break;
-        case 2: if (P.grouped && !dense_layer(e, l)) {   // the groups of the last step's last layer
+        case 2: if ((P.grouped || P.select) && !dense_layer(e, l)) {   // the groups of the last step's last layer
                   ce = gemm_launch(P.p_gug, P.p_gug.sw_hi ? &e->tm_gu_half[l] : &e->tm_gu[l], e->d_status, e->st, nullptr, true);
                   if (ce == cudaSuccess && !P.p_gug.sw_hi)
                     ce = launch_moe_swiglu_grouped(P.gug_out, P.moe_w, e->moe_E + e->moe_S, e->moe_F, P.grp, P.hg_hi, P.hg_lo, e->st);
                   break;
                 }
                 ce = gemm_launch(P.p_gu, P.p_gu.sw_hi ? &e->tm_gu_half[l] : &e->tm_gu[l], e->d_status, e->st, nullptr, true); break;
-        case 3: if (P.grouped && !dense_layer(e, l)) {   // per-group down GEMM + the sum over a row's experts
+        case 3: if (P.select && !dense_layer(e, l)) {    // down GEMM per selected expert + the sum over a row's experts
+                  ce = gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true);
+                  if (ce == cudaSuccess) ce = launch_moe_combine_select(P.yg_out, P.moe_sel, e->moe_K + e->moe_S, P.BN, P.R, s.hidden, P.down_out, e->st);
+                  break;
+                }
+                if (P.grouped && !dense_layer(e, l)) {   // per-group down GEMM + the sum over a row's experts
                   ce = gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true);
                   if (ce == cudaSuccess) ce = launch_moe_combine(P.yg_out, P.row_active, P.R, e->moe_E + e->moe_S, s.hidden, P.grp, P.down_out, e->st);
                   break;
@@ -1516,7 +1554,7 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
                   break;
                 }
                 ce = launch_qkv_post(P.p_qkv.out(), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st); break;
-        case 8: if (P.p_gu.sw_hi || P.grouped) break;   // no such kernel: the SwiGLU is in the GEMM's epilogue (grouped form: timed with kind 2)
+        case 8: if (P.p_gu.sw_hi || P.grouped || P.select) break;   // no such kernel: the SwiGLU is in the GEMM's epilogue (grouped form: timed with kind 2)
                 ce = e->moe_E ? launch_moe_swiglu(P.p_gu.out(), P.moe_w, P.R, e->moe_F, e->moe_E + e->moe_S, P.ff_hi, P.ff_lo, e->st)
                               : launch_swiglu(P.p_gu.out(), P.R, s.ffn, P.ff_hi, P.ff_lo, e->st);
                 break;
@@ -1533,7 +1571,7 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
                  if (ce == cudaSuccess) ce = launch_moe_gather(P.xn_hi, P.xn_lo, s.hidden, P.grp, P.xg_hi, P.xg_lo, e->st);
                  break;
         case 12: ce = launch_moe_router(P.xn_hi, P.xn_lo, s.hidden, e->router[l], P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm,
-                                        P.moe_w, nullptr, nullptr, e->st);
+                                        P.moe_w, nullptr, nullptr, e->st, P.row_active, P.moe_sel);
                  break;
       }
     }
@@ -1558,6 +1596,7 @@ int corun_debug_gemm_trace(corun_engine *e, int32_t kind, int32_t layer, uint64_
   const CUtensorMap *tm[5] = {&e->tm_qkv[layer], &e->tm_o[layer], P.p_gu.sw_hi ? &e->tm_gu_half[layer] : &e->tm_gu[layer],
                               &e->tm_down[layer], nullptr};
   const GemmPlan &p = *pl[kind];
+  if (!p.grid) return CORUN_EINVAL;                 // expert layers in their grouped or selected form
   unsigned long long *d = nullptr;
   if (cudaMalloc(&d, (size_t)p.grid * 8 * sizeof(unsigned long long)) != cudaSuccess) return CORUN_ENOMEM;
   cudaError_t ce = cudaMemsetAsync(d, 0, (size_t)p.grid * 8 * sizeof(unsigned long long), e->st);

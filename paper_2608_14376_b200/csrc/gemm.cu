@@ -55,7 +55,12 @@ constexpr uint32_t A_BLOCK_BYTES = GEMM_ROW_BLOCK * GEMM_BLOCK_K * 2;      // 16
 // earlier kernel of the step, or null = both) says which blocks exist this step: an absent block is neither loaded
 // nor multiplied nor stored (its output rows keep what they held: nobody reads rows without a request).  A row's
 // value does not depend on which blocks exist.
-template <bool MASKED, bool STACKED, bool GROUPED, bool SWIGLU, int NSB = 1>
+// SELECT (with STACKED, GROUPED; the experts of up to 64 rows): the groups are the experts that at least one row
+// selected, all rows of the step together (no gathering: they fit one A tile).  group_tab holds keep_div ints, the
+// selected experts of every row (< 0: none); every CTA makes the ascending list of them itself.  Expert e's weight rows
+// start at e * N (SWIGLU) or its k-blocks at e * KB, its rows of the intermediate and of the output at e * BN; row_keep is
+// the table of routing weights [rows][keep_pitch], and only rows that selected the expert are stored.
+template <bool MASKED, bool STACKED, bool GROUPED, bool SWIGLU, int NSB = 1, bool SELECT = false>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                     const __grid_constant__ CUtensorMap tmLo, float *__restrict__ direct, float *__restrict__ ws,
@@ -74,6 +79,9 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   __shared__ __align__(8) uint64_t tmem_empty_bar[2];
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
+  __shared__ uint32_t sel_bits[SELECT ? GEMM_MAX_SELECT / 32 : 1];   // SELECT: which experts have a row
+  __shared__ unsigned short sel_list[SELECT ? GEMM_MAX_SELECT : 1];  // and their list, ascending
+  __shared__ int sel_n;
   __shared__ float xch[2][64 * 33];   // stacked epilogue: W*hi and W*lo of 64 rows x 32 columns (row pitch 33: no bank conflicts)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -86,6 +94,13 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       g_tile = tile;
       g_id = t / tiles_per_group;
       g_j = t - g_id * tiles_per_group;
+      if (SELECT) {
+        g_id = sel_list[g_id];
+        g_wrow = SWIGLU ? g_id * N : 0;
+        g_wk = SWIGLU ? 0 : g_id * KB;
+        g_rows = R;
+        return;
+      }
       g_wrow = group_tab[3 * g_id];
       g_wk = group_tab[3 * g_id + 1];
       g_rows = group_tab[3 * g_id + 2];
@@ -165,7 +180,29 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   // GROUPED: the CTA walks the tiles cta, cta + grid, ... of the groups in use (their number follows the table's
   // keep_pitch entries), every tile whole; the flat range counts the k-blocks of those tiles.
   int k0, k1;
-  if (GROUPED) {
+  if (SELECT) {
+    if (threadIdx.x < GEMM_MAX_SELECT / 32) sel_bits[threadIdx.x] = 0u;
+    __syncthreads();
+    griddep_wait();
+    for (int i = (int)threadIdx.x; i < keep_div; i += GEMM_THREADS) {
+      const int e = *reinterpret_cast<const volatile int *>(group_tab + i);
+      if (e >= 0) atomicOr(&sel_bits[e >> 5], 1u << (e & 31));
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int n = 0;
+      for (int w = 0; w < GEMM_MAX_SELECT / 32; ++w) {
+        const uint32_t m = sel_bits[w];
+        if ((m >> lane) & 1u) sel_list[n + __popc(m & ((1u << lane) - 1u))] = (unsigned short)(w * 32 + lane);
+        n += __popc(m);
+      }
+      if (lane == 0) sel_n = n;
+    }
+    __syncthreads();
+    const int used = sel_n * tiles_per_group;
+    k0 = 0;
+    k1 = cta < used ? (used - cta + (int)gridDim.x - 1) / (int)gridDim.x * KB : 0;
+  } else if (GROUPED) {
     if (keep_div >= 0) griddep_wait();              // the group table comes from an earlier kernel (keep_div < 0: it is fixed)
     const int used = min(group_tab[3 * keep_pitch], keep_pitch) * tiles_per_group;
     k0 = 0;
@@ -219,8 +256,9 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
               tma_load_2d(dst + w_tile_bytes + lo_off + (uint32_t)b * A_BLOCK_BYTES, &tmLo, kb * GEMM_BLOCK_K, GEMM_ROW_BLOCK * b, fb, pol_x);
             }
         } else {
-          tma_load_2d(dst + w_tile_bytes, &tmHi, kb * GEMM_BLOCK_K, GROUPED ? g_id * BN : 0, fb, pol_x);
-          tma_load_2d(dst + w_tile_bytes + lo_off, &tmLo, kb * GEMM_BLOCK_K, GROUPED ? g_id * BN : 0, fb, pol_x);
+          const int y = GROUPED && !(SELECT && SWIGLU) ? g_id * BN : 0;   // (SELECT: every expert's gate / up reads the step's rows)
+          tma_load_2d(dst + w_tile_bytes, &tmHi, kb * GEMM_BLOCK_K, y, fb, pol_x);
+          tma_load_2d(dst + w_tile_bytes + lo_off, &tmLo, kb * GEMM_BLOCK_K, y, fb, pol_x);
         }
       };
       for (int it = 0; it < n_pre; ++it) {
@@ -375,7 +413,9 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
                     float y[4] = {silu_mul(gt[i][0], s0), silu_mul(gt[i][1], s1), silu_mul(gt[i][2], s2),
                                   silu_mul(gt[i][3], s3)};
                     if (MASKED || GROUPED) {           // the row's routing weight for this expert; 0: not selected
-                      const float wgt = GROUPED ? row_keep[sw_row0 + r] : row_keep[(size_t)(rb0 + r) * keep_pitch + blk];
+                      const float wgt = SELECT ? row_keep[(size_t)r * keep_pitch + g_id]
+                                               : GROUPED ? row_keep[sw_row0 + r] : row_keep[(size_t)(rb0 + r) * keep_pitch + blk];
+                      if (SELECT && wgt == 0.f) continue;   // nobody reads the row's values for this expert
 #pragma unroll
                       for (int q = 0; q < 4; ++q) y[q] = wgt != 0.f ? wgt * y[q] : 0.f;
                     }
@@ -447,7 +487,8 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int r = i * 16 + srow;
-          row_on[i] = r < rows_valid && (!MASKED || rb0 + r >= R || keep[(size_t)(rb0 + r) * keep_pitch] != 0.f);
+          row_on[i] = r < rows_valid && (!MASKED || rb0 + r >= R || keep[(size_t)(rb0 + r) * keep_pitch] != 0.f) &&
+                      (!SELECT || row_keep[(size_t)r * keep_pitch + g_id] != 0.f);
         }
         for (int c0 = 0; c0 < GEMM_TILE_N; c0 += 32) {
           if (whole && n0 + c0 >= N) break;          // columns beyond the matrix (last tile); uniform
@@ -901,6 +942,25 @@ int gemm_plan_create_grouped_swiglu(GemmPlan *p, const void *W, long long w_rows
   return CORUN_OK;
 }
 
+int gemm_plan_create_select_up(GemmPlan *p, const void *W, int NB, int F, int K, int half, const void *Xhi, const void *Xlo, int R, int BN,
+                               __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, const float *w, const int *sel, int n_sel, int num_sms) {
+  if (NB > GEMM_MAX_SELECT) return CORUN_EINVAL;
+  int rc = gemm_plan_create_grouped_swiglu(p, W, (long long)NB * 2 * F, F, K, half, Xhi, Xlo, NB, BN, out_hi, out_lo, w, sel, num_sms);
+  if (rc) return rc;
+  p->R = R; p->keep_pitch = NB; p->keep_div = n_sel; p->select = true;
+  if ((rc = tma_encode_2d(&p->tmHi, Xhi, 0, (unsigned long long)BN, K, BN, GEMM_BLOCK_K)) != 0) return rc;   // one set of rows
+  return tma_encode_2d(&p->tmLo, Xlo, 0, (unsigned long long)BN, K, BN, GEMM_BLOCK_K);
+}
+
+int gemm_plan_create_select_down(GemmPlan *p, const void *W, int NB, int N, int F, const void *Xhi, const void *Xlo, int R, int BN,
+                                 float *direct, const float *w, const int *sel, int n_sel, int num_sms) {
+  if (NB > GEMM_MAX_SELECT) return CORUN_EINVAL;
+  const int rc = gemm_plan_create_grouped(p, W, N, NB * F, N, F, Xhi, Xlo, NB, BN, direct, sel, num_sms);
+  if (rc) return rc;
+  p->R = R; p->row_keep = w; p->keep_pitch = NB; p->keep_div = n_sel; p->select = true;
+  return CORUN_OK;
+}
+
 cudaError_t gemm_prepare_kernel() {
   cudaError_t e = cudaFuncSetAttribute(gemm_streamk_kernel<false, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_streamk_kernel<false, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
@@ -916,6 +976,8 @@ cudaError_t gemm_prepare_kernel() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_streamk_kernel<true, true, false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_streamk_kernel<false, true, false, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_streamk_kernel<true, true, false, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_streamk_kernel<false, true, true, true, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_streamk_kernel<false, true, true, false, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
   return e;
 }
 
@@ -937,6 +999,7 @@ cudaError_t gemm_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int 
     if (p.sw_hi) return masked ? go(gemm_streamk_kernel<true, true, false, true, 2>) : go(gemm_streamk_kernel<false, true, false, true, 2>);
     return masked ? go(gemm_streamk_kernel<true, true, false, false, 2>) : go(gemm_streamk_kernel<false, true, false, false, 2>);
   }
+  if (p.select) return p.sw_hi ? go(gemm_streamk_kernel<false, true, true, true, 1, true>) : go(gemm_streamk_kernel<false, true, true, false, 1, true>);
   if (p.group_tab && p.sw_hi) return go(gemm_streamk_kernel<false, true, true, true>);
   if (p.sw_hi && masked) return stacked ? go(gemm_streamk_kernel<true, true, false, true>) : go(gemm_streamk_kernel<true, false, false, true>);
   if (p.sw_hi) return stacked ? go(gemm_streamk_kernel<false, true, false, true>) : go(gemm_streamk_kernel<false, false, false, true>);

@@ -23,6 +23,7 @@ extern int g_last_cuda_error;
 constexpr int GEMM_TILE_N = 256;   // weight rows per tile (the MMA's N)
 constexpr int GEMM_ROW_BLOCK = 128; // activation rows per MMA (the MMA's M)
 constexpr int GEMM_BLOCK_K = 64;   // bf16 elements per k-block (= one 128-byte swizzle row)
+constexpr int GEMM_MAX_SELECT = 288;  // experts of a selected-experts GEMM
 constexpr int GEMM_THREADS = 192;  // warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue
 
 // What a consumer kernel needs to read a GEMM result.
@@ -92,6 +93,7 @@ struct GemmPlan {
                                      // then ONE more int: the number of groups in use (the first ones);
                                      // keep_div = -1 tells the kernel that no kernel of the same stream writes it
   int tiles_per_group = 0;
+  bool select = false;               // gemm_plan_create_select_*: group_tab holds the rows' experts, keep_div ints
   // Gate / up GEMM with SwiGLU in the epilogue (gemm_plan_create_swiglu): the bf16 hi/lo output [BN, N / 2].
   __nv_bfloat16 *sw_hi = nullptr, *sw_lo = nullptr;
   int sw_half = 0;                   // gate rows (= up rows) per tile
@@ -125,6 +127,15 @@ int gemm_plan_create_grouped(GemmPlan *p, const void *W, long long w_rows, int w
 int gemm_plan_create_grouped_swiglu(GemmPlan *p, const void *W, long long w_rows, int F, int K, int half, const void *Xhi,
                                     const void *Xlo, int n_groups, int BN, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo,
                                     const float *row_scale, const int *group_tab, int num_sms);
+// The experts of a Mixture-of-Experts layer for up to BN <= 64 rows, all rows of the step together per expert: only the
+// experts that a row selected are loaded and multiplied.  sel: n_sel ints, every row's experts (< 0: none); w: the routing
+// weights [R][NB].  up: W [NB * 2F, K] -> out_hi / out_lo [NB * BN, F], row e * BN + r = w[r, e] * silu(gate) * up (tiles
+// of `half` gate rows as above).  down: W [N, NB * F] -> direct [NB * BN, N], row e * BN + r.  Rows that did not select
+// the expert keep what they held.
+int gemm_plan_create_select_up(GemmPlan *p, const void *W, int NB, int F, int K, int half, const void *Xhi, const void *Xlo, int R, int BN,
+                               __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, const float *w, const int *sel, int n_sel, int num_sms);
+int gemm_plan_create_select_down(GemmPlan *p, const void *W, int NB, int N, int F, const void *Xhi, const void *Xlo, int R, int BN,
+                                 float *direct, const float *w, const int *sel, int n_sel, int num_sms);
 // Gate / up GEMM with the SwiGLU in its epilogue: W is [2F, K] (F gate rows, then F up rows; F % 8 == 0);
 // out_hi / out_lo [BN, F] receive silu(gate) * up of rows 0 .. R-1 as a bf16 hi/lo pair.  A tile is
 // gemm_swiglu_half(F, num_sms) gate rows with the up rows of the same outputs, and every CTA owns whole tiles

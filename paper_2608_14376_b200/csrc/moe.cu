@@ -43,7 +43,8 @@ __device__ __forceinline__ void moe_split(float x, bf16 &hi, bf16 &lo) {
 // w[r, 0 .. E + S): p_e for the selected experts, 0 for the others, 1 for the shared ones.
 template <typename LoadLogit>
 __device__ __forceinline__ void moe_route_row(LoadLogit load, int r, int lane, int E, int S, int top_k, int renormalize,
-                                              float *__restrict__ w, int *__restrict__ experts, float *__restrict__ probs) {
+                                              float *__restrict__ w, int *__restrict__ experts, float *__restrict__ probs,
+                                              int *__restrict__ sel = nullptr, bool on = true) {
   constexpr int PER = MOE_MAX_EXPERTS / 32;
   float z[PER];
   float mx = -CUDART_INF_F;
@@ -99,6 +100,15 @@ __device__ __forceinline__ void moe_route_row(LoadLogit load, int r, int lane, i
       if (experts) experts[(size_t)r * top_k + k] = ids[k];
       if (probs) probs[(size_t)r * top_k + k] = p;
     }
+  if (sel) {                                         // every lane knows all ids: lane k places the k-th
+    int *out = sel + (size_t)r * (top_k + S);
+    for (int k = 0; k < top_k; ++k) {
+      int place = 0;
+      for (int j = 0; j < top_k; ++j) place += ids[j] < ids[k] ? 1 : 0;
+      if (lane == k) out[place] = on ? ids[k] : -1;
+    }
+    for (int s = lane; s < S; s += 32) out[top_k + s] = on ? E + s : -1;
+  }
 }
 
 // Router of one row per CTA: logits = Wr x on the CUDA cores (E dot products of H terms: far too little for a
@@ -110,7 +120,8 @@ constexpr int ROUTER_THREADS = 1024;
 __global__ void __launch_bounds__(ROUTER_THREADS) moe_router_kernel(const bf16 *__restrict__ x_hi, const bf16 *__restrict__ x_lo, int H,
                                                                     const bf16 *__restrict__ Wr, int E, int S, int top_k,
                                                                     int renormalize, float *__restrict__ w,
-                                                                    int *__restrict__ experts, float *__restrict__ probs) {
+                                                                    int *__restrict__ experts, float *__restrict__ probs,
+                                                                    const int *active, int *__restrict__ sel) {
   griddep_launch_dependents();
   extern __shared__ float xs[];                      // the row as fp32 [H]
   __shared__ float logit[MOE_MAX_EXPERTS];
@@ -149,7 +160,8 @@ __global__ void __launch_bounds__(ROUTER_THREADS) moe_router_kernel(const bf16 *
     if (lane == 0) logit[e] = acc;
   }
   __syncthreads();
-  if (warp == 0) moe_route_row([&](int e) { return logit[e]; }, r, lane, E, S, top_k, renormalize, w, experts, probs);
+  if (warp == 0) moe_route_row([&](int e) { return logit[e]; }, r, lane, E, S, top_k, renormalize, w, experts, probs, sel,
+                               !sel || active[r] != 0);
 }
 
 // h[r, e*F + f] = w[r, e] * silu(gate) * up as a bf16 hi/lo pair; zeros where w[r, e] == 0 (nothing is read
@@ -442,6 +454,28 @@ __global__ void __launch_bounds__(256) moe_swiglu_grouped_kernel(const float *__
   }
 }
 
+// Selected-experts form: y[r, :] = the sum of the row's experts in ascending id; their rows sit at e * BN + r.
+__global__ void __launch_bounds__(256) moe_combine_select_kernel(const float *__restrict__ yg, const int *__restrict__ sel, int n_per_row,
+                                                                 int BN, int H, float *__restrict__ y) {
+  griddep_launch_dependents();
+  griddep_wait();
+  yg = after_wait(yg); sel = after_wait(sel);
+  const int r = blockIdx.y, i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  const int *mine = sel + (size_t)r * n_per_row;
+  if (i >= H || mine[0] < 0) return;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k0 = 0; k0 < n_per_row; k0 += 8) {        // eight loads in flight; the additions stay in ascending order
+    float4 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k0 + k < n_per_row) v[k] = *reinterpret_cast<const float4 *>(yg + ((size_t)mine[k0 + k] * BN + r) * H + i);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k0 + k < n_per_row) { acc.x += v[k].x; acc.y += v[k].y; acc.z += v[k].z; acc.w += v[k].w; }
+  }
+  *reinterpret_cast<float4 *>(y + (size_t)r * H + i) = acc;
+}
+
 __global__ void __launch_bounds__(256) moe_combine_kernel(const float *__restrict__ yg, const int *__restrict__ active, int NB,
                                                           int H, MoeGroups g, float *__restrict__ y) {
   griddep_launch_dependents();
@@ -519,9 +553,13 @@ cudaError_t launch_moe_combine(const float *yg, const int *active, int R, int n_
 }
 
 cudaError_t launch_moe_router(const bf16 *x_hi, const bf16 *x_lo, int H, const bf16 *Wr, int R, int E, int S, int top_k,
-                              int renormalize, float *w, int *experts, float *probs, cudaStream_t st) {
+                              int renormalize, float *w, int *experts, float *probs, cudaStream_t st, const int *active, int *sel) {
   return launch_k(moe_router_kernel, dim3(R), dim3(ROUTER_THREADS), (size_t)H * sizeof(float), st, true, x_hi, x_lo, H, Wr, E, S, top_k,
-                  renormalize, w, experts, probs);
+                  renormalize, w, experts, probs, active, sel);
+}
+
+cudaError_t launch_moe_combine_select(const float *yg, const int *sel, int n_per_row, int BN, int R, int H, float *y, cudaStream_t st) {
+  return launch_k(moe_combine_select_kernel, dim3((H / 4 + 255) / 256, R), dim3(256), 0, st, true, yg, sel, n_per_row, BN, H, y);
 }
 
 cudaError_t launch_moe_swiglu(const GemmOut &gu, const float *w, int R, int F, int n_blocks, __nv_bfloat16 *out_hi,
