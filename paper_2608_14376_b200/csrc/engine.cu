@@ -78,24 +78,29 @@ struct Program {
   int *tab_uk = nullptr, *tab_uv = nullptr;
   GemmPlan p_uk, p_uv, p_gu_d, p_down_d;
   bool has_layers = false, has_lm = false;
-  // Prefill of long prompts: up to `cap` rows at a time (R: the rows of the chunk at hand), the projections on pairs of
-  // SMs (gemm_pair.cu); their results are plain matrices, the SwiGLU is in the gate / up GEMM's epilogue.
+  // Prefill: up to `cap` rows at a time (R: the rows of the chunk at hand).  Long prompts: the projections on pairs of SMs
+  // (gemm_pair.cu), their results plain matrices, the SwiGLU in the gate / up GEMM's epilogue.  Short prompts (shorts): the
+  // dense projections in blocks of SHORT_ROWS rows through the decode GEMM (s_*: one plan per block, blocks of 64 rows
+  // without a row left out), the token-wise kernels behind a projection block by block; attention and experts over all
+  // rows as for long ones.
   bool pair = false;
   int cap = 0;
+  bool shorts = false;
+  std::vector<GemmPlan> s_qkv, s_o, s_gu, s_down;
   GemmPairPlan b_qkv, b_o, b_gu, b_down, b_router;
   float *router_out = nullptr;
   uint32_t *moe_mask = nullptr;
   std::vector<void *> allocs;
 };
 
-// Prompts of up to PREFILL_SMALL tokens run through the fixed chunk program (its GEMMs cut K over the SMs: few rows
-// leave most SMs without a tile otherwise), longer ones through the program of PREFILL_BIG rows.  Which one depends on
-// the prompt's own length only, so a prompt's values do not depend on what is prefilled with it.  Measured on the
-// Qwen3-8B layer: 256 rows 192 us of GEMMs in the chunk program, 293 us on pairs of SMs; 512 rows 384 against 359; 1024
-// rows 766 against 531; 2048 rows 1532 against 1010 (hence chunks as large as the buffers allow).
+// Prompts of up to PREFILL_SMALL tokens are short (Program::shorts), longer ones long.  Which one depends on the prompt's
+// own length only, so a prompt's values do not depend on what is prefilled with it.  Measured, GEMMs of the Qwen3-8B layer:
+// 64 rows 82 us and 128 rows 110 us in blocks of SHORT_ROWS; 256 rows 293 us, 512 rows 359, 1024 rows 531, 2048 rows 1010
+// on pairs of SMs (hence chunks as large as the buffers allow).
 constexpr int PREFILL_SMALL = 256, PREFILL_BIG = 2048;
 // Rows of a long prompt's chunk that the latent attention takes at a time (its partial results are kept per row).
 constexpr int MLA_ROWS = 256;
+constexpr int SHORT_ROWS = 128;
 static_assert(PREFILL_BIG <= MOE_MANY_ROWS, "a chunk of a long prompt is grouped in one go");
 
 }  // namespace
@@ -113,6 +118,7 @@ struct corun_engine {
   std::vector<const bf16 *> attn_norm, mlp_norm;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
   std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down, tb_router;   // boxes of 128 rows: the GEMMs on pairs of SMs
+  std::vector<CUtensorMap> tb_gu_half;     // dense layers of a decoder with expert layers: the box of the GEMM with SwiGLU
   std::vector<CUtensorMap> tm_gu_half;     // dense gate / up matrices with the box of the GEMM with SwiGLU in its epilogue
   std::vector<CUtensorMap> tm_k, tm_v;   // per layer: the pages as rows of head_dim halfs (keys and values alike)
   std::vector<CUtensorMap> tm_k4;        // the same memory as [8-token group][64-dim half][8 tokens][64 dims]: one box per (page, head) tile
@@ -153,10 +159,12 @@ struct corun_engine {
   uint8_t *h_active = nullptr;
   uint64_t *h_seeds = nullptr;
   int *h_out_tokens = nullptr, *h_status = nullptr;
-  int *h_rows = nullptr;          // prefill row metadata staging [5][chunk]
+  int *h_rows = nullptr;          // prefill staging: rows [4][chunk], blocks of rows, group tables of the latent projections
+  int *h_table = nullptr;         // [B][max_blocks]: the block table as it was last sent (a slot's row changes only while it is free)
+  int *h_first = nullptr;         // [B]: first tokens of a prefill call's requests
   bool staged_valid = false, in_flight = false;
   Program dec, pre, big, lm1;
-  // prefill-only per-row sampling arrays (length 1)
+  // prefill-only per-row sampling arrays (length FINISH_ROWS)
   float *d_pf_temp = nullptr, *d_pf_top_p = nullptr;
   uint64_t *d_pf_seed = nullptr;
   int *d_pf_step = nullptr, *d_pf_one = nullptr, *d_pf_tok = nullptr;
@@ -387,10 +395,8 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   const size_t c = (size_t)cap;
   RC(dmalloc(A, &P.xn_hi, c * H));
   RC(dmalloc(A, &P.xn_lo, c * H));
-  RC(dmalloc(A, &P.row_token, c));
-  RC(dmalloc(A, &P.row_pos, c));
-  RC(dmalloc(A, &P.row_active, c));
-  RC(dmalloc(A, &P.row_slot, c));
+  RC(dmalloc(A, &P.row_token, 4 * c));              // token | position | active | slot, as many rows as the chunk at hand has
+  RC(dmalloc(A, &P.row_blocks, c / SHORT_ROWS));
   RC(dmalloc(A, &P.h, c * H));
   RC(dmalloc(A, &P.qkv_out, c * QKVN));
   RC(dmalloc(A, &P.o_out, c * H));
@@ -398,13 +404,32 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   RC(dmalloc(A, &P.ao_hi, c * QD));
   RC(dmalloc(A, &P.ao_lo, c * QD));
   RC(dmalloc(A, &P.plain_tiles, (size_t)((QKVN > H ? QKVN : H) / GEMM_TILE_N + 1)));
+  const int n_blk = cap / SHORT_ROWS;               // cap is a multiple of 256
+  RC(dmalloc(A, &P.ws, gemm_ws_floats(e->num_sms, SHORT_ROWS)));
+  for (auto *v : {&P.s_qkv, &P.s_o, &P.s_gu, &P.s_down}) v->resize((size_t)n_blk);
+  RC(gemm_plan_create(&P.s_qkv[0], e->w0_qkv, QKVN, H, P.xn_hi, P.xn_lo, SHORT_ROWS, SHORT_ROWS, P.qkv_out, P.ws, e->num_sms));
+  RC(gemm_plan_create(&P.s_o[0], e->w0_o, H, QD, P.ao_hi, P.ao_lo, SHORT_ROWS, SHORT_ROWS, P.o_out, P.ws, e->num_sms));
   RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, cap, P.qkv_out, e->num_sms));
   RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, cap, P.o_out, e->num_sms));
   if (F > 0) {
     RC(dmalloc(A, &P.ff_hi, c * F));
     RC(dmalloc(A, &P.ff_lo, c * F));
+    RC(gemm_plan_create_swiglu(&P.s_gu[0], e->moe_E ? e->w0_gu_d : e->w0_gu, F, H, P.xn_hi, P.xn_lo, SHORT_ROWS, SHORT_ROWS, P.ff_hi, P.ff_lo,
+                               e->num_sms));
+    RC(gemm_plan_create(&P.s_down[0], e->moe_E ? e->w0_down_d : e->w0_down, H, F, P.ff_hi, P.ff_lo, SHORT_ROWS, SHORT_ROWS, P.down_out, P.ws,
+                        e->num_sms));
     RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, cap, P.ff_hi, P.ff_lo, e->num_sms));
     RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, cap, P.down_out, e->num_sms));
+  }
+  for (int b = n_blk - 1; b >= 0; --b) {            // (block 0 last: the others are copies of it)
+    const size_t r0 = (size_t)b * SHORT_ROWS;
+    const int *rb = P.row_blocks + b;
+    RC(gemm_plan_rebase(&P.s_qkv[b], P.s_qkv[0], P.xn_hi + r0 * H, P.xn_lo + r0 * H, P.qkv_out + r0 * QKVN, nullptr, nullptr, rb));
+    RC(gemm_plan_rebase(&P.s_o[b], P.s_o[0], P.ao_hi + r0 * QD, P.ao_lo + r0 * QD, P.o_out + r0 * H, nullptr, nullptr, rb));
+    if (F > 0) {
+      RC(gemm_plan_rebase(&P.s_gu[b], P.s_gu[0], P.xn_hi + r0 * H, P.xn_lo + r0 * H, nullptr, P.ff_hi + r0 * F, P.ff_lo + r0 * F, rb));
+      RC(gemm_plan_rebase(&P.s_down[b], P.s_down[0], P.ff_hi + r0 * F, P.ff_lo + r0 * F, P.down_out + r0 * H, nullptr, nullptr, rb));
+    }
   }
   if (!e->mla) {
     RC(dmalloc(A, &P.q, c * QD));
@@ -438,18 +463,18 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   return CORUN_OK;
 }
 
-// (long prompts) lays the head-major matrices out for a chunk of R rows: whole blocks of 64 per head, one behind the other.
-int set_mla_rows(corun_engine *e, Program &P, int R) {
+// (prefill) lays the head-major matrices out for a chunk of R rows: whole blocks of 64 per head, one behind the other.
+// stage: pinned memory for the two group tables, not touched again before the stream has drained.
+int set_mla_rows(corun_engine *e, Program &P, int R, int *stage) {
   const MlaDims &md = e->md;
   const int rph = (R + 63) / 64 * 64, count_at = md.nh * (P.cap / 64) * 3;
   P.RPH = rph;
   std::vector<int> t;
-  mla_group_table(t, md.nh, rph, 64, R, md.rank, count_at);
-  CK(cudaMemcpyAsync(P.tab_uk, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice, e->st));
-  CK(cudaStreamSynchronize(e->st));                 // `t` is pageable and reused
-  mla_group_table(t, md.nh, rph, 64, R, md.nope + md.vh, count_at);
-  CK(cudaMemcpyAsync(P.tab_uv, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice, e->st));
-  CK(cudaStreamSynchronize(e->st));
+  for (int k = 0; k < 2; ++k) {
+    mla_group_table(t, md.nh, rph, 64, R, k == 0 ? md.rank : md.nope + md.vh, count_at);
+    memcpy(stage + k * t.size(), t.data(), t.size() * sizeof(int));
+    CK(cudaMemcpyAsync(k == 0 ? P.tab_uk : P.tab_uv, stage + k * t.size(), t.size() * sizeof(int), cudaMemcpyHostToDevice, e->st));
+  }
   return CORUN_OK;
 }
 
@@ -465,6 +490,8 @@ void program_destroy(Program &P) {
   gemm_plan_destroy(&P.p_uv);
   gemm_plan_destroy(&P.p_gu_d);
   gemm_plan_destroy(&P.p_down_d);
+  for (auto *v : {&P.s_qkv, &P.s_o, &P.s_gu, &P.s_down})
+    if (!v->empty()) gemm_plan_destroy(&(*v)[0]);   // the others share its tables
   for (void *p : P.allocs) cudaFree(p);
   P.allocs.clear();
 }
@@ -489,7 +516,7 @@ GemmOut ffn_out(const corun_engine *e, const Program &P, int layer) {
   return P.p_down.out();
 }
 
-// Enqueues embed -> all layers (ends with the last down GEMM).  Counts launches.
+// Enqueues embed -> all layers (ends with the last down GEMM; prefill: with the final norm of every row).  Counts launches.
 int run_layers(corun_engine *e, Program &P, int *launches) {
   const corun_shape &s = e->sh;
   const Rows rows{P.row_token, P.row_pos, P.row_active, P.row_slot, P.R};
@@ -511,18 +538,35 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
     CK(call);                                         \
     ++stage;                                          \
   } while (0)
+  bool normed = false;                              // the layer's input has been normalised behind the layer before
+  const int QD = s.n_q_heads * s.head_dim;
+  // (short prompts) the blocks of the chunk: first row, and the rows of it as token-wise kernels take them
+  const int n_blk = P.shorts ? (P.R + SHORT_ROWS - 1) / SHORT_ROWS : 0;
+  auto block_rows = [&](int b) {
+    const int r0 = b * SHORT_ROWS, left = P.R - r0;
+    return Rows{P.row_token + r0, P.row_pos + r0, P.row_active + r0, P.row_slot + r0, left < SHORT_ROWS ? left : SHORT_ROWS};
+  };
   for (int l = 0; l < s.n_layers; ++l) {
     GemmOut prev = ffn_out(e, P, l > 0 ? l - 1 : 0);
-    STAGE(launch_resid_norm(P.h, s.hidden, e->embed, rows, l == 0 ? nullptr : &prev, e->attn_norm[l], s.rms_eps,
-                            P.xn_hi, P.xn_lo, e->st));
+    if (!normed)
+      STAGE(launch_resid_norm(P.h, s.hidden, e->embed, rows, l == 0 ? nullptr : &prev, e->attn_norm[l], s.rms_eps,
+                              P.xn_hi, P.xn_lo, e->st));
+    normed = false;
     if (P.pair) {
-      // long prompts: projections on pairs of SMs, plain results
-      STAGE(gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st));
+      // prefill; long prompts: projections on pairs of SMs, plain results
+      if (!P.shorts) STAGE(gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st));
       if (e->mla) {
         const MlaDims &md = e->md;
         const MlaCache cache{e->kv_pool + (size_t)l * e->layer_stride, e->d_block_table, e->max_blocks, e->B, (long long)e->pool_blocks, e->kv_run};
-        STAGE(launch_mla_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi, P.qn_lo,
-                              P.q_rope, e->d_status, e->st));
+        if (!P.shorts)
+          STAGE(launch_mla_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi,
+                                P.qn_lo, P.q_rope, e->d_status, e->st));
+        for (int b = 0; b < n_blk; ++b) {
+          const size_t r0 = (size_t)b * SHORT_ROWS;
+          STAGE(gemm_launch(P.s_qkv[b], &e->tm_qkv[l], e->d_status, e->st, nullptr, true));
+          STAGE(launch_mla_post(P.s_qkv[b].out(), block_rows(b), e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi + r0 * md.nope,
+                                P.qn_lo + r0 * md.nope, P.q_rope + r0 * md.nh * md.rope, e->d_status, e->st));
+        }
         STAGE(gemm_launch(P.p_uk, &e->tm_uk[l], e->d_status, e->st, nullptr, true));
         for (int r0 = 0; r0 < P.R; r0 += MLA_ROWS) {
           const int nr = P.R - r0 < MLA_ROWS ? P.R - r0 : MLA_ROWS;
@@ -536,13 +580,35 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         STAGE(gemm_launch(P.p_uv, &e->tm_uv[l], e->d_status, e->st, nullptr, true));
         STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
       } else {
-        STAGE(launch_qkv_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
+        if (!P.shorts) STAGE(launch_qkv_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
+        for (int b = 0; b < n_blk; ++b) {
+          STAGE(gemm_launch(P.s_qkv[b], &e->tm_qkv[l], e->d_status, e->st, nullptr, true));
+          STAGE(launch_qkv_post(P.s_qkv[b].out(), block_rows(b), e->d_rope, s.n_q_heads, kv, l, P.q + (size_t)b * SHORT_ROWS * QD, e->d_status,
+                                e->st));
+        }
         STAGE(launch_attention_prefill(e->tm_k[l], e->tm_v[l], P.q, rows, s.n_q_heads, kv, P.ao_hi, P.ao_lo, e->d_status, e->st));
       }
-      STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
-      const GemmOut o = plain_out(P, P.o_out, s.hidden);
-      STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
-      if (e->moe_E && !dense_layer(e, l)) {
+      if (!P.shorts) {
+        STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
+        const GemmOut o = plain_out(P, P.o_out, s.hidden);
+        STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
+      }
+      const bool experts = e->moe_E && !dense_layer(e, l);
+      const bf16 *next_norm = l + 1 < s.n_layers ? e->attn_norm[l + 1] : e->final_norm;
+      for (int b = 0; b < n_blk; ++b) {             // (short prompts) the rest of a dense layer, block by block
+        const size_t o0 = (size_t)b * SHORT_ROWS * s.hidden;
+        const Rows br = block_rows(b);
+        STAGE(gemm_launch(P.s_o[b], &e->tm_o[l], e->d_status, e->st, nullptr, true));
+        const GemmOut o = P.s_o[b].out();
+        STAGE(launch_resid_norm(P.h + o0, s.hidden, nullptr, br, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi + o0, P.xn_lo + o0, e->st));
+        if (experts) continue;
+        STAGE(gemm_launch(P.s_gu[b], e->moe_E ? &e->tb_gu_half[l] : &e->tm_gu_half[l], e->d_status, e->st, nullptr, true));
+        STAGE(gemm_launch(P.s_down[b], e->moe_E ? &e->tm_down_d[l] : &e->tm_down[l], e->d_status, e->st, nullptr, true));
+        const GemmOut d = P.s_down[b].out();
+        STAGE(launch_resid_norm(P.h + o0, s.hidden, nullptr, br, &d, next_norm, s.rms_eps, P.xn_hi + o0, P.xn_lo + o0, e->st));
+      }
+      normed = P.shorts && !experts;
+      if (experts) {
         const int NB = e->moe_E + e->moe_S;
         STAGE(gemm_pair_launch(P.b_router, e->tb_router[l], P.R, e->d_status, e->st));
         STAGE(launch_moe_route(P.router_out, P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, e->st));
@@ -556,7 +622,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         }
         STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
         STAGE(launch_moe_combine(P.yg_out, P.row_active, P.R, NB, s.hidden, P.grp, P.down_out, e->st));
-      } else {
+      } else if (!P.shorts) {
         STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st));
         STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st));
       }
@@ -646,6 +712,10 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
     STAGE(gemm_launch(P.p_down, &e->tm_down[l], e->d_status, e->st, tr(4 * l + 3), true));
     n += 9 + (&P == &e->dec ? 1 : 0);   // decode attention is two kernels (splits, combine)
   }
+  if (&P != &e->dec && !normed) {                   // prefill: the final norm
+    const GemmOut last = ffn_out(e, P, s.n_layers - 1);
+    STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &last, e->final_norm, s.rms_eps, P.xn_hi, P.xn_lo, e->st));
+  }
 #undef STAGE
   if (launches) *launches += n;
   return CORUN_OK;
@@ -699,26 +769,20 @@ int reserve_blocks(corun_engine *e, int slot, int reserve_len) {
   if ((size_t)need > e->free_blocks.size()) return CORUN_ENOSPACE;
   std::vector<int> &mine = e->slot_blocks[slot];
   mine.clear();
-  std::vector<int> row(e->max_blocks, 0);
+  int *row = e->h_table + (size_t)slot * e->max_blocks;   // pinned; the last copy from it has completed: the slot was free
+  memset(row, 0, (size_t)e->max_blocks * sizeof(int));
   for (int i = 0; i < need; ++i) {
     mine.push_back(e->free_blocks.back());
     e->free_blocks.pop_back();
     for (int j = 0; j < e->kv_run && i * e->kv_run + j < e->max_blocks; ++j) row[i * e->kv_run + j] = mine.back() * e->kv_run + j;
   }
-  CK(cudaMemcpyAsync(e->d_block_table + (size_t)slot * e->max_blocks, row.data(), e->max_blocks * sizeof(int),
-                     cudaMemcpyHostToDevice, e->st));
-  CK(cudaStreamSynchronize(e->st));   // `row` is pageable and local
+  CK(cudaMemcpyAsync(e->d_block_table + (size_t)slot * e->max_blocks, row, e->max_blocks * sizeof(int), cudaMemcpyHostToDevice, e->st));
   return CORUN_OK;
 }
 
 int set_slot_state(corun_engine *e, int slot, int in_use, int ctx, int step, int pending, float temp, float top_p) {
-  CK(cudaMemcpyAsync(e->d_in_use + slot, &in_use, sizeof(int), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_ctx + slot, &ctx, sizeof(int), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_step + slot, &step, sizeof(int), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_pending + slot, &pending, sizeof(int), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_temp + slot, &temp, sizeof(float), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_top_p + slot, &top_p, sizeof(float), cudaMemcpyHostToDevice, e->st));
-  CK(cudaStreamSynchronize(e->st));
+  CK(launch_set_slot(SlotArrays{e->d_in_use, e->d_ctx, e->d_step, e->d_pending, e->d_temp, e->d_top_p}, slot, in_use, ctx, step, pending,
+                     temp, top_p, e->st));
   return CORUN_OK;
 }
 
@@ -868,11 +932,13 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   e->lm_head = (const bf16 *)w->lm_head;
   e->final_norm = (const bf16 *)w->final_norm;
   const int H = s.hidden, QD = s.n_q_heads * s.head_dim, KD = s.n_kv_heads * s.head_dim, F = s.ffn;
-  // long prompts get a program of their own where their projections and experts have a form for many rows
-  const bool big_ok = !one_chunk_size && max_context > PREFILL_SMALL &&
+  // prefill runs through the program of many rows where their projections and experts have a form for many rows
+  const bool big_ok = !one_chunk_size &&
                       (!moe || (moe->n_experts % 8 == 0 && (2 * moe->expert_ffn) % GEMM_TILE_N == 0 && H % GEMM_TILE_N == 0 &&
                                 !getenv("CORUN_MOE_PREFILL_DENSE")));
-  const int big_cap = !big_ok ? 0 : max_context < PREFILL_BIG ? (max_context + 255) / 256 * 256 : PREFILL_BIG;
+  // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG
+  const long long big_rows = (long long)B * ((max_context + 127) / 128 * 128);
+  const int big_cap = !big_ok ? 0 : big_rows < PREFILL_BIG ? (int)((big_rows + 255) / 256 * 256) : PREFILL_BIG;
   e->tm_qkv.resize(s.n_layers);
   e->tm_o.resize(s.n_layers);
   e->tm_gu.resize(s.n_layers);
@@ -886,15 +952,16 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     const int qkv_rows = mla ? s.n_q_heads * (mla->qk_nope + mla->qk_rope) + mla->kv_lora_rank + mla->qk_rope : QD + 2 * KD;
     if ((rc = gemm_encode_map(&e->tm_qkv[l], w->wqkv[l], qkv_rows, H, GEMM_TILE_N))) return fail(rc);
     if ((rc = gemm_encode_map(&e->tm_o[l], w->wo[l], H, QD, GEMM_TILE_N))) return fail(rc);
-    if (big_cap) {                                  // the program of long prompts
+    if (big_cap) {                                  // the program of many rows
       if (e->tb_qkv.empty())
-        for (auto *v : {&e->tb_qkv, &e->tb_o, &e->tb_gu, &e->tb_down, &e->tb_router}) v->resize(s.n_layers);
+        for (auto *v : {&e->tb_qkv, &e->tb_o, &e->tb_gu, &e->tb_down, &e->tb_router, &e->tb_gu_half}) v->resize(s.n_layers);
       const bool experts = moe && l >= first_dense;
       const int Fd = moe ? dense_ffn : F;
       if ((rc = gemm_encode_map(&e->tb_qkv[l], w->wqkv[l], qkv_rows, H, 128)) || (rc = gemm_encode_map(&e->tb_o[l], w->wo[l], H, QD, 128)))
         return fail(rc);
       if (experts ? (rc = gemm_encode_map(&e->tb_router[l], moe->router[l], moe->n_experts, H, 128))
-                  : ((rc = gemm_encode_map(&e->tb_gu[l], w->wgate_up[l], 2 * Fd, H, 128)) || (rc = gemm_encode_map(&e->tb_down[l], w->wdown[l], H, Fd, 128))))
+                  : ((moe && (rc = gemm_encode_map(&e->tb_gu_half[l], w->wgate_up[l], 2 * Fd, H, gemm_swiglu_half(Fd, e->num_sms)))) ||
+                     (rc = gemm_encode_map(&e->tb_gu[l], w->wgate_up[l], 2 * Fd, H, 128)) || (rc = gemm_encode_map(&e->tb_down[l], w->wdown[l], H, Fd, 128))))
         return fail(rc);
     }
     if (moe && l < first_dense) {                   // a dense feed-forward layer of a decoder with expert layers
@@ -971,9 +1038,10 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   if ((rc = dmalloc(A, &e->d_in_use, B)) || (rc = dmalloc(A, &e->d_ctx, B)) || (rc = dmalloc(A, &e->d_step, B)) ||
       (rc = dmalloc(A, &e->d_pending, B)) || (rc = dmalloc(A, &e->d_temp, B)) || (rc = dmalloc(A, &e->d_top_p, B)) ||
       (rc = dmalloc(A, &e->d_seeds, B)) || (rc = dmalloc(A, &e->d_active, B)) || (rc = dmalloc(A, &e->d_out_tokens, B)) ||
-      (rc = dmalloc(A, &e->d_status, 1)) || (rc = dmalloc(A, &e->d_pf_temp, 1)) || (rc = dmalloc(A, &e->d_pf_top_p, 1)) ||
-      (rc = dmalloc(A, &e->d_pf_seed, 1)) || (rc = dmalloc(A, &e->d_pf_step, 1)) || (rc = dmalloc(A, &e->d_pf_one, 1)) ||
-      (rc = dmalloc(A, &e->d_pf_tok, 1)) || (rc = dmalloc(A, &e->pf_logits, (size_t)B * s.vocab)))
+      (rc = dmalloc(A, &e->d_status, 1)) || (rc = dmalloc(A, &e->d_pf_temp, FINISH_ROWS)) ||
+      (rc = dmalloc(A, &e->d_pf_top_p, FINISH_ROWS)) || (rc = dmalloc(A, &e->d_pf_seed, FINISH_ROWS)) ||
+      (rc = dmalloc(A, &e->d_pf_step, FINISH_ROWS)) || (rc = dmalloc(A, &e->d_pf_one, FINISH_ROWS)) ||
+      (rc = dmalloc(A, &e->d_pf_tok, FINISH_ROWS)) || (rc = dmalloc(A, &e->pf_logits, (size_t)B * s.vocab)))
     return fail(rc);
   e->logits_row.assign((size_t)B, -1);
   {
@@ -988,8 +1056,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     if ((rc = dmalloc(A, &e->d_rope, tab.size(), false))) return fail(rc);
     if (cudaMemcpy(e->d_rope, tab.data(), tab.size() * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
       return fail(CORUN_ECUDA);
-    const int one = 1;
-    if (cudaMemcpy(e->d_pf_one, &one, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return fail(CORUN_ECUDA);
+    const std::vector<int> ones(FINISH_ROWS, 1);
+    if (cudaMemcpy(e->d_pf_one, ones.data(), FINISH_ROWS * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return fail(CORUN_ECUDA);
   }
   const int64_t n_runs = e->pool_blocks / e->kv_run;
   e->free_blocks.resize((size_t)n_runs);
@@ -1002,7 +1070,9 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   if (cudaMallocHost(&e->h_active, B) != cudaSuccess || cudaMallocHost(&e->h_seeds, B * sizeof(uint64_t)) != cudaSuccess ||
       cudaMallocHost(&e->h_out_tokens, B * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&e->h_status, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&e->h_rows, (size_t)5 * PREFILL_BIG * sizeof(int)) != cudaSuccess)
+      cudaMallocHost(&e->h_table, (size_t)B * e->max_blocks * sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&e->h_first, B * sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&e->h_rows, ((size_t)4 * PREFILL_BIG + 64 + 2 * (16 * (PREFILL_BIG / 64) * 3 + 1)) * sizeof(int)) != cudaSuccess)
     return fail(CORUN_ENOMEM);
   memset(e->h_active, 0, B);
   memset(e->h_seeds, 0, B * sizeof(uint64_t));
@@ -1022,12 +1092,12 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   // rows each above); the GEMMs leave the others out (the one-row program has one block)
   for (GemmPlan *pl : {&e->dec.p_qkv, &e->dec.p_o, &e->dec.p_gu, &e->dec.p_down, &e->dec.p_lm, &e->dec.p_gu_d, &e->dec.p_down_d})
     pl->row_blocks = e->dec.row_blocks;
-  if ((rc = program_create(e, e->pre, e->chunk, true, false, e->moe_E > 0 && !getenv("CORUN_MOE_PREFILL_DENSE")))) return fail(rc);
+  if (!big_cap && (rc = program_create(e, e->pre, e->chunk, true, false, e->moe_E > 0 && !getenv("CORUN_MOE_PREFILL_DENSE")))) return fail(rc);
   // a prefill chunk is filled from row 0: the host says which blocks of rows it reaches (prefill_run)
   for (GemmPlan *pl : {&e->pre.p_qkv, &e->pre.p_o, &e->pre.p_gu, &e->pre.p_down, &e->pre.p_gu_d, &e->pre.p_down_d})
     pl->row_blocks = e->pre.row_blocks;
   if (big_cap && (rc = program_create_big(e, e->big, big_cap))) return fail(rc);
-  if ((rc = program_create(e, e->lm1, 1, false, true))) return fail(rc);
+  if ((rc = program_create(e, e->lm1, FINISH_ROWS, false, true))) return fail(rc);
 
   // the allocations above were cleared and filled through the legacy stream, which the engine's
   // stream does not wait for: drain the device once before the first launch
@@ -1080,6 +1150,8 @@ void corun_destroy(corun_engine *e) {
   if (e->h_out_tokens) cudaFreeHost(e->h_out_tokens);
   if (e->h_status) cudaFreeHost(e->h_status);
   if (e->h_rows) cudaFreeHost(e->h_rows);
+  if (e->h_table) cudaFreeHost(e->h_table);
+  if (e->h_first) cudaFreeHost(e->h_first);
   if (e->own_stream) cudaStreamDestroy(e->st);
   delete e;
 }
@@ -1097,37 +1169,39 @@ struct PfReq {
   int first;
 };
 
-// Final norm -> LM head (one row) -> sample with R(seed, 0) for the request whose last prompt token is row
-// `row` of the chunk that has just run; the logits go to the slot's place among the prefill logits.
-int prefill_finish_row(corun_engine *e, const Program &P, int row, PfReq &r) {
+// LM head -> sample with R(seed, 0) for up to FINISH_ROWS requests whose last prompt tokens are rows of the chunk that has
+// just run (the final norm is in P.xn); the logits go to the slots' places among the prefill logits, the tokens to h_first
+// (valid once the stream has drained).  A row's logits do not depend on the other rows of the product.
+int prefill_finish(corun_engine *e, const Program &P, const std::pair<int, int> *fins, int n, PfReq *const *reqs) {
   const corun_shape &s = e->sh;
   Program &L = e->lm1;
-  GemmOut prev = ffn_out(e, P, s.n_layers - 1);
-  prev.direct += (size_t)row * prev.N;
-  if (prev.ws) prev.ws += (size_t)row * GEMM_TILE_N;
-  const Rows one{P.row_token + row, P.row_pos + row, P.row_active + row, P.row_slot + row, 1};
-  CK(launch_resid_norm(P.h + (size_t)row * s.hidden, s.hidden, nullptr, one, &prev, e->final_norm, s.rms_eps, L.xn_hi,
-                       L.xn_lo, e->st));
+  FinishRows f{};
+  f.n = n;
+  for (int i = 0; i < n; ++i) {
+    const PfReq &r = *reqs[fins[i].first];
+    f.row[i] = fins[i].second;
+    f.temp[i] = r.smp.temperature;
+    f.top_p[i] = r.smp.top_p;
+    f.seed[i] = r.seed;
+  }
+  CK(launch_finish_rows(f, P.xn_hi, P.xn_lo, s.hidden, L.xn_hi, L.xn_lo, e->d_pf_temp, e->d_pf_top_p, e->d_pf_seed, e->st));
   CK(gemm_launch(L.p_lm, nullptr, e->d_status, e->st));
-  CK(gemm_fixup_launch(L.p_lm, e->st));
-  const int zero = 0;
-  CK(cudaMemcpyAsync(e->d_pf_temp, &r.smp.temperature, sizeof(float), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_pf_top_p, &r.smp.top_p, sizeof(float), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_pf_seed, &r.seed, sizeof(uint64_t), cudaMemcpyHostToDevice, e->st));
-  CK(cudaMemcpyAsync(e->d_pf_step, &zero, sizeof(int), cudaMemcpyHostToDevice, e->st));
+  CK(gemm_fixup_launch(L.p_lm, e->st, true, n));
   SampleArgs sa{L.logits, s.vocab, e->d_pf_one, e->d_pf_temp, e->d_pf_top_p, e->d_pf_seed, e->d_pf_step, nullptr,
                 e->d_pf_tok};
-  CK(launch_sampler(sa, 1, e->st));
-  CK(cudaMemcpyAsync(e->pf_logits + (size_t)r.slot * s.vocab, L.logits, (size_t)s.vocab * sizeof(float),
-                     cudaMemcpyDeviceToDevice, e->st));
-  e->logits_row[(size_t)r.slot] = -1;              // corun_get_logits: the prefill's logits until the slot decodes
-  CK(cudaMemcpyAsync(&r.first, e->d_pf_tok, sizeof(int), cudaMemcpyDeviceToHost, e->st));
-  CK(cudaStreamSynchronize(e->st));   // the one-row buffers and the sampling staging serve the next request
+  CK(launch_sampler(sa, n, e->st, true));
+  for (int i = 0; i < n; ++i) {
+    const PfReq &r = *reqs[fins[i].first];
+    CK(cudaMemcpyAsync(e->pf_logits + (size_t)r.slot * s.vocab, L.logits + (size_t)i * s.vocab, (size_t)s.vocab * sizeof(float),
+                       cudaMemcpyDeviceToDevice, e->st));
+    CK(cudaMemcpyAsync(e->h_first + r.slot, e->d_pf_tok + i, sizeof(int), cudaMemcpyDeviceToHost, e->st));
+    e->logits_row[(size_t)r.slot] = -1;            // corun_get_logits: the prefill's logits until the slot decodes
+  }
   return CORUN_OK;
 }
 
-// Prefill of one or several requests through one prefill program: the chunk program (chunks of `chunk` rows) or the
-// one of long prompts (chunks of up to its `cap` rows, launched for the rows they hold).  The
+// Prefill of one or several requests, all short or all long, through the program of many rows (chunks of up to its `cap`
+// rows, launched for the rows they hold) or, where an engine has none, the chunk program (chunks of `chunk` rows).  The
 // rows of a chunk are dealt in request order; every piece of a request starts on a tile boundary of the
 // prefill attention kernel (a tile's rows share one slot), so a chunk may hold pieces of several requests.
 // Every kernel of the program treats its rows independently of each other and of where they sit in the
@@ -1142,12 +1216,16 @@ int prefill_many(corun_engine *e, PfReq *reqs, int n_req) {
   if (need > e->free_blocks.size()) return CORUN_ENOSPACE;
   int rc = CORUN_OK;
   for (int i = 0; i < n_req && rc == CORUN_OK; ++i) rc = reserve_blocks(e, reqs[i].slot, reqs[i].reserve);
-  std::vector<PfReq *> small, big;                  // by the prompt's own length
-  for (int i = 0; i < n_req; ++i) (e->big.pair && reqs[i].n > PREFILL_SMALL ? big : small).push_back(&reqs[i]);
-  if (rc == CORUN_OK && !small.empty()) rc = prefill_run(e, e->pre, small.data(), (int)small.size());
-  if (rc == CORUN_OK && !big.empty()) rc = prefill_run(e, e->big, big.data(), (int)big.size());
+  std::vector<PfReq *> part[2];                     // short and long, by the prompt's own length
+  for (int i = 0; i < n_req; ++i) part[e->big.pair && reqs[i].n > PREFILL_SMALL ? 1 : 0].push_back(&reqs[i]);
+  for (int k = 0; k < 2 && rc == CORUN_OK; ++k) {
+    if (part[k].empty()) continue;
+    e->big.shorts = k == 0;
+    rc = prefill_run(e, e->big.pair ? e->big : e->pre, part[k].data(), (int)part[k].size());   // (the chunk program takes any length)
+  }
   for (int i = 0; i < n_req && rc == CORUN_OK; ++i) {
-    const PfReq &q = reqs[i];
+    PfReq &q = reqs[i];
+    q.first = e->h_first[q.slot];
     rc = set_slot_state(e, q.slot, 1, q.n, 1, q.first, q.smp.temperature, q.smp.top_p);
     if (rc != CORUN_OK) break;
     e->in_use[q.slot] = 1;
@@ -1171,29 +1249,45 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
   int unit = 128 / (s.n_q_heads / s.n_kv_heads);    // tokens per attention tile
   if (e->mla) unit = 16;                            // no query tiles there: every row is on its own
   if (unit > CH || CH % unit) unit = CH;
-  int *tok = e->h_rows, *pos = tok + CH, *act = pos + CH, *slt = act + CH, *blocks = slt + CH;
+  std::vector<int> tok((size_t)CH), pos((size_t)CH), act((size_t)CH), slt((size_t)CH);
   std::vector<std::pair<int, int>> fins;           // (request, chunk row of its last prompt token)
   int fill = 0, pad_slot = reqs[0]->slot;
   auto run_chunk = [&]() -> int {
     const int rows_n = P.pair ? fill : CH;
+    for (int i = fill; i < rows_n; ++i) { tok[i] = 0; pos[i] = 0; act[i] = 0; slt[i] = pad_slot; }
+    int *h = e->h_rows;                             // pinned: token | position | active | slot of the chunk's rows
+    const size_t bytes = (size_t)rows_n * sizeof(int);
+    memcpy(h, tok.data(), bytes);
+    memcpy(h + rows_n, pos.data(), bytes);
+    memcpy(h + 2 * rows_n, act.data(), bytes);
+    memcpy(h + 3 * rows_n, slt.data(), bytes);
+    int *blocks = h + 4 * PREFILL_BIG, *tabs = blocks + 64;
     if (P.pair) {
       P.R = fill;
-      if (e->mla) RC(set_mla_rows(e, P, fill));
-    }
-    for (int i = fill; i < rows_n; ++i) { tok[i] = 0; pos[i] = 0; act[i] = 0; slt[i] = pad_slot; }
-    CK(cudaMemcpyAsync(P.row_token, tok, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
-    CK(cudaMemcpyAsync(P.row_pos, pos, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
-    CK(cudaMemcpyAsync(P.row_active, act, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
-    CK(cudaMemcpyAsync(P.row_slot, slt, rows_n * sizeof(int), cudaMemcpyHostToDevice, e->st));
-    // the chunk's rows are filled from row 0: the GEMMs leave out the blocks of rows behind the last one in use
-    // (blocks of 64 rows up to 128 padded rows, of 128 rows above)
-    if (!P.pair) {
+      P.row_pos = P.row_token + fill;
+      P.row_active = P.row_pos + fill;
+      P.row_slot = P.row_active + fill;
+      CK(cudaMemcpyAsync(P.row_token, h, 4 * bytes, cudaMemcpyHostToDevice, e->st));
+      if (e->mla) RC(set_mla_rows(e, P, fill, tabs));
+      if (P.shorts) {                               // which blocks of 64 rows exist
+        const int nb = (fill + SHORT_ROWS - 1) / SHORT_ROWS;
+        for (int b = 0; b < nb; ++b) blocks[b] = 1 | (fill > b * SHORT_ROWS + 64 ? 2 : 0);
+        CK(cudaMemcpyAsync(P.row_blocks, blocks, nb * sizeof(int), cudaMemcpyHostToDevice, e->st));
+      }
+    } else {
+      CK(cudaMemcpyAsync(P.row_token, h, bytes, cudaMemcpyHostToDevice, e->st));
+      CK(cudaMemcpyAsync(P.row_pos, h + rows_n, bytes, cudaMemcpyHostToDevice, e->st));
+      CK(cudaMemcpyAsync(P.row_active, h + 2 * rows_n, bytes, cudaMemcpyHostToDevice, e->st));
+      CK(cudaMemcpyAsync(P.row_slot, h + 3 * rows_n, bytes, cudaMemcpyHostToDevice, e->st));
+      // the chunk's rows are filled from row 0: the GEMMs leave out the blocks of rows behind the last one in use
+      // (blocks of 64 rows up to 128 padded rows, of 128 rows above)
       const int blk = P.BN <= 128 ? 64 : 128;
       blocks[0] = (fill > 0 ? 1 : 0) | (fill > blk ? 2 : 0);
       CK(cudaMemcpyAsync(P.row_blocks, blocks, sizeof(int), cudaMemcpyHostToDevice, e->st));
     }
     RC(run_layers(e, P, nullptr));
-    for (auto &f : fins) RC(prefill_finish_row(e, P, f.second, *reqs[f.first]));
+    for (size_t i = 0; i < fins.size(); i += FINISH_ROWS)
+      RC(prefill_finish(e, P, &fins[i], (int)(fins.size() - i < FINISH_ROWS ? fins.size() - i : FINISH_ROWS), reqs));
     CK(cudaStreamSynchronize(e->st));   // the staging arrays are reused by the next chunk
     fins.clear();
     fill = 0;

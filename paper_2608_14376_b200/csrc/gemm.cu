@@ -1008,9 +1008,21 @@ cudaError_t gemm_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int 
   return stacked ? go(gemm_streamk_kernel<false, true, false, false>) : go(gemm_streamk_kernel<false, false, false, false>);
 }
 
-cudaError_t gemm_fixup_launch(const GemmPlan &p, cudaStream_t st, bool pdl) {
+int gemm_plan_rebase(GemmPlan *q, const GemmPlan &p, const void *Xhi, const void *Xlo, float *direct, __nv_bfloat16 *sw_hi,
+                     __nv_bfloat16 *sw_lo, const int *row_blocks) {
+  *q = p;
+  q->direct = direct;
+  q->sw_hi = sw_hi;
+  q->sw_lo = sw_lo;
+  q->row_blocks = row_blocks;
+  int rc;
+  if ((rc = gemm_encode_map(&q->tmHi, Xhi, p.BN, p.K, gemm_x_box_rows(p.BN))) != 0) return rc;
+  return gemm_encode_map(&q->tmLo, Xlo, p.BN, p.K, gemm_x_box_rows(p.BN));
+}
+
+cudaError_t gemm_fixup_launch(const GemmPlan &p, cudaStream_t st, bool pdl, int rows) {
   if (p.n_split_tiles == 0) return cudaSuccess;
-  return launch_k(gemm_fixup_kernel, dim3(p.n_split_tiles, p.R), dim3(GEMM_TILE_N), 0, st, pdl, p.out(), p.direct,
+  return launch_k(gemm_fixup_kernel, dim3(p.n_split_tiles, rows ? rows : p.R), dim3(GEMM_TILE_N), 0, st, pdl, p.out(), p.direct,
                   p.d_split_tiles);
 }
 

@@ -871,6 +871,25 @@ __global__ void advance_kernel(const int *slot_row, const int *row_active, const
   __threadfence_system();
 }
 
+__global__ void __launch_bounds__(256)
+finish_rows_kernel(const __grid_constant__ FinishRows f, const __nv_bfloat16 *__restrict__ x_hi, const __nv_bfloat16 *__restrict__ x_lo, int H,
+                   __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, float *temp, float *top_p, uint64_t *seed) {
+  const int i = blockIdx.x;
+  if (threadIdx.x == 0) { temp[i] = f.temp[i]; top_p[i] = f.top_p[i]; seed[i] = f.seed[i]; }
+  const uint4 *sh = reinterpret_cast<const uint4 *>(x_hi + (size_t)f.row[i] * H), *sl = reinterpret_cast<const uint4 *>(x_lo + (size_t)f.row[i] * H);
+  uint4 *dh = reinterpret_cast<uint4 *>(out_hi + (size_t)i * H), *dl = reinterpret_cast<uint4 *>(out_lo + (size_t)i * H);
+  for (int k = threadIdx.x; k < H / 8; k += 256) { dh[k] = sh[k]; dl[k] = sl[k]; }
+}
+
+__global__ void set_slot_kernel(SlotArrays a, int slot, int in_use, int ctx, int step, int pending, float temp, float top_p) {
+  a.in_use[slot] = in_use;
+  a.ctx[slot] = ctx;
+  a.step[slot] = step;
+  a.pending[slot] = pending;
+  a.temp[slot] = temp;
+  a.top_p[slot] = top_p;
+}
+
 __global__ void kv_copy_kernel(KvLayout kv, int layer, int slot, int pos0, int n, float *k, float *v, int write) {
   const int KD = kv.n_kv * kv.hd;
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -976,6 +995,18 @@ cudaError_t launch_sampler(const SampleArgs &a, int R, cudaStream_t st, bool pdl
   cfg.attrs = attr;
   cfg.numAttrs = (pdl && g_use_pdl) ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, sampler_kernel, a);
+}
+
+cudaError_t launch_finish_rows(const FinishRows &f, const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_lo, int H, __nv_bfloat16 *out_hi,
+                               __nv_bfloat16 *out_lo, float *temp, float *top_p, uint64_t *seed, cudaStream_t st) {
+  finish_rows_kernel<<<f.n, 256, 0, st>>>(f, x_hi, x_lo, H, out_hi, out_lo, temp, top_p, seed);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_set_slot(const SlotArrays &a, int slot, int in_use, int ctx, int step, int pending, float temp, float top_p,
+                            cudaStream_t st) {
+  set_slot_kernel<<<1, 1, 0, st>>>(a, slot, in_use, ctx, step, pending, temp, top_p);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_prepare_rows(const uint8_t *active_mask, const uint64_t *seeds_in, uint64_t *seeds_out, const int *in_use,

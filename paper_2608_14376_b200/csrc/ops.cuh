@@ -107,6 +107,19 @@ cudaError_t launch_kv_copy(const KvLayout &kv, int layer, int slot, int pos0, in
                            cudaStream_t st);
 // fills cached positions [0, n) of every layer of a slot with seeded N(0, std^2) values (bench set-up)
 cudaError_t launch_kv_fill(const KvLayout &kv, int n_layers, int slot, int n, float std, uint64_t seed, cudaStream_t st);
+// ---- the end of a prefill: the final rows of up to FINISH_ROWS requests, and a slot's state, by value (no copies)
+constexpr int FINISH_ROWS = 16;
+struct FinishRows {
+  int n, row[FINISH_ROWS];
+  float temp[FINISH_ROWS], top_p[FINISH_ROWS];
+  uint64_t seed[FINISH_ROWS];
+};
+// out[i, :] = x[f.row[i], :] for both halves (H % 8 == 0) and the rows' sampling arguments to device arrays.
+cudaError_t launch_finish_rows(const FinishRows &f, const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_lo, int H, __nv_bfloat16 *out_hi,
+                               __nv_bfloat16 *out_lo, float *temp, float *top_p, uint64_t *seed, cudaStream_t st);
+struct SlotArrays { int *in_use, *ctx, *step, *pending; float *temp, *top_p; };
+cudaError_t launch_set_slot(const SlotArrays &a, int slot, int in_use, int ctx, int step, int pending, float temp, float top_p,
+                            cudaStream_t st);
 cudaError_t launch_variate(uint64_t seed, uint64_t t, uint32_t *out, cudaStream_t st);
 
 }  // namespace corun
