@@ -38,6 +38,20 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
+// Device memory of one owner, handed out from a few blocks: an allocation of a few MB or more costs 0.35 ms whatever its
+// size, and an engine has some sixty buffers.
+struct DevMem {
+  std::vector<void *> blocks;
+  char *cur = nullptr;
+  size_t left = 0, next = (size_t)32 << 20;
+  void release() {
+    for (void *p : blocks) cudaFree(p);
+    blocks.clear();
+    cur = nullptr;
+    left = 0;
+  }
+};
+
 // Buffers and GEMM plans of the row program at one fixed row count.
 struct Program {
   int R = 0, BN = 0;
@@ -90,7 +104,7 @@ struct Program {
   GemmPairPlan b_qkv, b_o, b_gu, b_down, b_router;
   float *router_out = nullptr;
   uint32_t *moe_mask = nullptr;
-  std::vector<void *> allocs;
+  DevMem allocs;
 };
 
 // Prompts of up to PREFILL_SMALL tokens are short (Program::shorts), longer ones long.  Which one depends on the prompt's
@@ -155,7 +169,8 @@ struct corun_engine {
   int *d_out_tokens = nullptr, *d_status = nullptr;
   // slot state: host mirrors
   std::vector<int> in_use, ctx, reserve, step;
-  // pinned staging
+  // pinned staging (one allocation)
+  void *h_pinned = nullptr;
   uint8_t *h_active = nullptr;
   uint64_t *h_seeds = nullptr;
   int *h_out_tokens = nullptr, *h_status = nullptr;
@@ -174,7 +189,7 @@ struct corun_engine {
   unsigned long long *step_trace = nullptr;   // debug (CORUN_TRACE_STEP=1): GEMM timelines of a whole step
   int stop_after = -1;            // debug: eager decode stops after this many stages of layer 0
   int decode_launches = 0;
-  std::vector<void *> allocs;
+  DevMem allocs;
 };
 
 namespace {
@@ -191,6 +206,36 @@ int dmalloc(std::vector<void *> &keep, T **p, size_t n, bool zero = true) {
   keep.push_back(q);
   if (zero && cudaMemset(q, 0, n * sizeof(T)) != cudaSuccess) return CORUN_ECUDA;
   *p = (T *)q;
+  return CORUN_OK;
+}
+
+template <typename T>
+int dmalloc(DevMem &m, T **p, size_t n, bool zero = true) {
+  const size_t bytes = ((n ? n : 1) * sizeof(T) + 1023) / 1024 * 1024;
+  if (bytes > m.left) {
+    size_t want = m.next;
+    if (bytes >= want) want = bytes;
+    else if (m.next < ((size_t)256 << 20)) m.next *= 2;
+    void *q = nullptr;
+    cudaError_t e = cudaMalloc(&q, want);
+    if (e != cudaSuccess && want > bytes) { cudaGetLastError(); e = cudaMalloc(&q, want = bytes); }   // no room for a whole block
+    if (e != cudaSuccess) {
+      g_last_cuda_error = (int)e;
+      return CORUN_ENOMEM;
+    }
+    m.blocks.push_back(q);
+    if (want == bytes) {                            // a block of its own: the current one goes on
+      if (zero && cudaMemset(q, 0, bytes) != cudaSuccess) return CORUN_ECUDA;
+      *p = (T *)q;
+      return CORUN_OK;
+    }
+    m.cur = (char *)q;
+    m.left = want;
+  }
+  if (zero && cudaMemset(m.cur, 0, bytes) != cudaSuccess) return CORUN_ECUDA;
+  *p = (T *)m.cur;
+  m.cur += bytes;
+  m.left -= bytes;
   return CORUN_OK;
 }
 
@@ -492,8 +537,7 @@ void program_destroy(Program &P) {
   gemm_plan_destroy(&P.p_down_d);
   for (auto *v : {&P.s_qkv, &P.s_o, &P.s_gu, &P.s_down})
     if (!v->empty()) gemm_plan_destroy(&(*v)[0]);   // the others share its tables
-  for (void *p : P.allocs) cudaFree(p);
-  P.allocs.clear();
+  P.allocs.release();
 }
 
 KvLayout kv_layout(const corun_engine *e) {
@@ -1048,9 +1092,11 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     // cos/sin of pos * theta^(-2i/hd), evaluated in fp64 on the host (hd: the rotated width)
     const int rot = mla ? mla->qk_rope : s.head_dim, half = rot / 2;
     std::vector<float2> tab((size_t)max_context * half);
+    std::vector<double> freq((size_t)half);
+    for (int i = 0; i < half; ++i) freq[(size_t)i] = std::pow((double)s.rope_theta, -2.0 * (double)i / (double)rot);
     for (int p = 0; p < max_context; ++p)
       for (int i = 0; i < half; ++i) {
-        const double ang = (double)p * std::pow((double)s.rope_theta, -2.0 * (double)i / (double)rot);
+        const double ang = (double)p * freq[(size_t)i];
         tab[(size_t)p * half + i] = make_float2((float)std::cos(ang), (float)std::sin(ang));
       }
     if ((rc = dmalloc(A, &e->d_rope, tab.size(), false))) return fail(rc);
@@ -1067,13 +1113,23 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   e->ctx.assign(B, 0);
   e->reserve.assign(B, 0);
   e->step.assign(B, 0);
-  if (cudaMallocHost(&e->h_active, B) != cudaSuccess || cudaMallocHost(&e->h_seeds, B * sizeof(uint64_t)) != cudaSuccess ||
-      cudaMallocHost(&e->h_out_tokens, B * sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&e->h_status, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&e->h_table, (size_t)B * e->max_blocks * sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&e->h_first, B * sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&e->h_rows, ((size_t)4 * PREFILL_BIG + 64 + 2 * (16 * (PREFILL_BIG / 64) * 3 + 1)) * sizeof(int)) != cudaSuccess)
-    return fail(CORUN_ENOMEM);
+  {
+    // all pinned staging in one allocation (each costs milliseconds)
+    size_t off = 0;
+    auto place = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
+    const size_t o_active = place(B), o_seeds = place(B * sizeof(uint64_t)), o_tok = place(B * sizeof(int)), o_status = place(sizeof(int)),
+                 o_first = place(B * sizeof(int)), o_table = place((size_t)B * e->max_blocks * sizeof(int)),
+                 o_rows = place(((size_t)4 * PREFILL_BIG + 64 + 2 * (16 * (PREFILL_BIG / 64) * 3 + 1)) * sizeof(int));
+    if (cudaMallocHost(&e->h_pinned, off) != cudaSuccess) return fail(CORUN_ENOMEM);
+    char *h = (char *)e->h_pinned;
+    e->h_active = (uint8_t *)(h + o_active);
+    e->h_seeds = (uint64_t *)(h + o_seeds);
+    e->h_out_tokens = (int *)(h + o_tok);
+    e->h_status = (int *)(h + o_status);
+    e->h_first = (int *)(h + o_first);
+    e->h_table = (int *)(h + o_table);
+    e->h_rows = (int *)(h + o_rows);
+  }
   memset(e->h_active, 0, B);
   memset(e->h_seeds, 0, B * sizeof(uint64_t));
   *e->h_status = 0;
@@ -1144,14 +1200,8 @@ void corun_destroy(corun_engine *e) {
   program_destroy(e->pre);
   program_destroy(e->big);
   program_destroy(e->lm1);
-  for (void *p : e->allocs) cudaFree(p);
-  if (e->h_active) cudaFreeHost(e->h_active);
-  if (e->h_seeds) cudaFreeHost(e->h_seeds);
-  if (e->h_out_tokens) cudaFreeHost(e->h_out_tokens);
-  if (e->h_status) cudaFreeHost(e->h_status);
-  if (e->h_rows) cudaFreeHost(e->h_rows);
-  if (e->h_table) cudaFreeHost(e->h_table);
-  if (e->h_first) cudaFreeHost(e->h_first);
+  e->allocs.release();
+  if (e->h_pinned) cudaFreeHost(e->h_pinned);
   if (e->own_stream) cudaStreamDestroy(e->st);
   delete e;
 }
