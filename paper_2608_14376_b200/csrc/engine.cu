@@ -102,16 +102,16 @@ struct Program {
   bool shorts = false;
   std::vector<GemmPlan> s_qkv, s_o, s_gu, s_down;
   GemmPairPlan b_qkv, b_o, b_gu, b_down, b_router;
-  float *router_out = nullptr;
+  float *router_out = nullptr, *pair_part = nullptr;
   uint32_t *moe_mask = nullptr;
   DevMem allocs;
 };
 
 // Prompts of up to PREFILL_SMALL tokens are short (Program::shorts), longer ones long.  Which one depends on the prompt's
 // own length only, so a prompt's values do not depend on what is prefilled with it.  Measured, GEMMs of the Qwen3-8B layer:
-// 64 rows 82 us and 128 rows 110 us in blocks of SHORT_ROWS; 256 rows 293 us, 512 rows 359, 1024 rows 531, 2048 rows 1010
-// on pairs of SMs (hence chunks as large as the buffers allow).
-constexpr int PREFILL_SMALL = 256, PREFILL_BIG = 2048;
+// 64 rows 82 us and 128 rows 110 us in a block of SHORT_ROWS; 256 rows 179 us (two blocks: 220), 512 rows 299, 1024 rows
+// 543, 2048 rows 1049 on pairs of SMs (hence chunks as large as the buffers allow).
+constexpr int PREFILL_SMALL = 128, PREFILL_BIG = 2048;
 // Rows of a long prompt's chunk that the latent attention takes at a time (its partial results are kept per row).
 constexpr int MLA_ROWS = 256;
 constexpr int SHORT_ROWS = 128;
@@ -131,7 +131,7 @@ struct corun_engine {
   const bf16 *embed = nullptr, *lm_head = nullptr, *final_norm = nullptr;
   std::vector<const bf16 *> attn_norm, mlp_norm;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
-  std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down, tb_router;   // boxes of 128 rows: the GEMMs on pairs of SMs
+  std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down, tb_router, tb_gu96;   // boxes of 128 rows (96): the GEMMs on pairs of SMs
   std::vector<CUtensorMap> tb_gu_half;     // dense layers of a decoder with expert layers: the box of the GEMM with SwiGLU
   std::vector<CUtensorMap> tm_gu_half;     // dense gate / up matrices with the box of the GEMM with SwiGLU in its epilogue
   std::vector<CUtensorMap> tm_k, tm_v;   // per layer: the pages as rows of head_dim halfs (keys and values alike)
@@ -454,8 +454,14 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   for (auto *v : {&P.s_qkv, &P.s_o, &P.s_gu, &P.s_down}) v->resize((size_t)n_blk);
   RC(gemm_plan_create(&P.s_qkv[0], e->w0_qkv, QKVN, H, P.xn_hi, P.xn_lo, SHORT_ROWS, SHORT_ROWS, P.qkv_out, P.ws, e->num_sms));
   RC(gemm_plan_create(&P.s_o[0], e->w0_o, H, QD, P.ao_hi, P.ao_lo, SHORT_ROWS, SHORT_ROWS, P.o_out, P.ws, e->num_sms));
-  RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, cap, P.qkv_out, e->num_sms));
-  RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, cap, P.o_out, e->num_sms));
+  // partial matrices of an unfilled wave: consumed by the next kernel of the stream, so one buffer serves all
+  size_t part = (size_t)gemm_pair_slices(QKVN, H, e->num_sms) * QKVN;
+  const size_t part_o = (size_t)gemm_pair_slices(H, QD, e->num_sms) * H, part_d = F > 0 ? (size_t)gemm_pair_slices(H, F, e->num_sms) * H : 0,
+               part_r = e->moe_E ? (size_t)gemm_pair_slices(e->moe_E, H, e->num_sms) * e->moe_E : 0;
+  for (size_t x : {part_o, part_d, part_r}) part = x > part ? x : part;
+  RC(dmalloc(A, &P.pair_part, part * c, false));
+  RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, cap, P.qkv_out, P.pair_part, e->num_sms));
+  RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, cap, P.o_out, P.pair_part, e->num_sms));
   if (F > 0) {
     RC(dmalloc(A, &P.ff_hi, c * F));
     RC(dmalloc(A, &P.ff_lo, c * F));
@@ -464,7 +470,7 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
     RC(gemm_plan_create(&P.s_down[0], e->moe_E ? e->w0_down_d : e->w0_down, H, F, P.ff_hi, P.ff_lo, SHORT_ROWS, SHORT_ROWS, P.down_out, P.ws,
                         e->num_sms));
     RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, cap, P.ff_hi, P.ff_lo, e->num_sms));
-    RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, cap, P.down_out, e->num_sms));
+    RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, cap, P.down_out, P.pair_part, e->num_sms));
   }
   for (int b = n_blk - 1; b >= 0; --b) {            // (block 0 last: the others are copies of it)
     const size_t r0 = (size_t)b * SHORT_ROWS;
@@ -502,7 +508,7 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
     RC(dmalloc(A, &P.moe_w, c * (e->moe_E + e->moe_S)));
     RC(dmalloc(A, &P.router_out, c * e->moe_E));
     RC(dmalloc(A, &P.moe_mask, (size_t)(e->moe_E + e->moe_S) * (MOE_MANY_ROWS / 32)));
-    RC(gemm_pair_plan_create(&P.b_router, e->moe_E, H, P.xn_hi, P.xn_lo, cap, P.router_out, e->num_sms));
+    RC(gemm_pair_plan_create(&P.b_router, e->moe_E, H, P.xn_hi, P.xn_lo, cap, P.router_out, P.pair_part, e->num_sms));
     RC(program_create_groups(e, P, cap));
   }
   return CORUN_OK;
@@ -548,13 +554,13 @@ KvLayout kv_layout(const corun_engine *e) {
 // The result of a layer's feed-forward part as the next kernel reads it: the down GEMM's partials, or (grouped
 // Mixture-of-Experts form) the combined plain matrix.
 GemmOut plain_out(const Program &P, const float *m, int N) {
-  return GemmOut{m, nullptr, P.plain_tiles, P.plain_tiles, N, 0, P.BN};
+  return GemmOut{m, nullptr, P.plain_tiles, P.plain_tiles, N, 0, P.BN, 0, 0, 0};
 }
 
 bool dense_layer(const corun_engine *e, int layer) { return e->mla && e->moe_E && layer < e->first_dense; }
 
 GemmOut ffn_out(const corun_engine *e, const Program &P, int layer) {
-  if (P.pair) return plain_out(P, P.down_out, e->sh.hidden);
+  if (P.pair) return P.grouped && !dense_layer(e, layer) ? plain_out(P, P.down_out, e->sh.hidden) : gemm_pair_out(P.b_down, P.R, P.plain_tiles);
   if (dense_layer(e, layer)) return P.p_down_d.out();
   if (P.grouped || P.select) return plain_out(P, P.down_out, e->sh.hidden);
   return P.p_down.out();
@@ -603,7 +609,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         const MlaDims &md = e->md;
         const MlaCache cache{e->kv_pool + (size_t)l * e->layer_stride, e->d_block_table, e->max_blocks, e->B, (long long)e->pool_blocks, e->kv_run};
         if (!P.shorts)
-          STAGE(launch_mla_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi,
+          STAGE(launch_mla_post(gemm_pair_out(P.b_qkv, P.R, P.plain_tiles), rows, e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi,
                                 P.qn_lo, P.q_rope, e->d_status, e->st));
         for (int b = 0; b < n_blk; ++b) {
           const size_t r0 = (size_t)b * SHORT_ROWS;
@@ -624,7 +630,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         STAGE(gemm_launch(P.p_uv, &e->tm_uv[l], e->d_status, e->st, nullptr, true));
         STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
       } else {
-        if (!P.shorts) STAGE(launch_qkv_post(plain_out(P, P.qkv_out, P.b_qkv.N), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
+        if (!P.shorts) STAGE(launch_qkv_post(gemm_pair_out(P.b_qkv, P.R, P.plain_tiles), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
         for (int b = 0; b < n_blk; ++b) {
           STAGE(gemm_launch(P.s_qkv[b], &e->tm_qkv[l], e->d_status, e->st, nullptr, true));
           STAGE(launch_qkv_post(P.s_qkv[b].out(), block_rows(b), e->d_rope, s.n_q_heads, kv, l, P.q + (size_t)b * SHORT_ROWS * QD, e->d_status,
@@ -634,7 +640,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       }
       if (!P.shorts) {
         STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
-        const GemmOut o = plain_out(P, P.o_out, s.hidden);
+        const GemmOut o = gemm_pair_out(P.b_o, P.R, P.plain_tiles);
         STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
       }
       const bool experts = e->moe_E && !dense_layer(e, l);
@@ -655,7 +661,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       if (experts) {
         const int NB = e->moe_E + e->moe_S;
         STAGE(gemm_pair_launch(P.b_router, e->tb_router[l], P.R, e->d_status, e->st));
-        STAGE(launch_moe_route(P.router_out, P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, e->st));
+        STAGE(launch_moe_route(gemm_pair_out(P.b_router, P.R, P.plain_tiles), P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, e->st));
         STAGE(launch_moe_group_many(P.moe_w, P.row_active, P.R, e->moe_E, e->moe_S, e->moe_F, P.moe_mask, P.grp, e->st));
         STAGE(launch_moe_gather(P.xn_hi, P.xn_lo, s.hidden, P.grp, P.xg_hi, P.xg_lo, e->st));
         if (P.p_gug.sw_hi) {
@@ -667,7 +673,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
         STAGE(launch_moe_combine(P.yg_out, P.row_active, P.R, NB, s.hidden, P.grp, P.down_out, e->st));
       } else if (!P.shorts) {
-        STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st));
+        STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st, &e->tb_gu96[l]));
         STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st));
       }
       continue;
@@ -965,7 +971,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     if (fit < e->pool_blocks) e->pool_blocks = fit / e->kv_run * e->kv_run;
     if (e->pool_blocks < e->kv_run) return fail(CORUN_ENOMEM);
   }
-  e->chunk = PREFILL_SMALL;
+  e->chunk = 256;
   bool one_chunk_size = false;                      // the environment asks for chunks of its own size, for every prompt
   if (const char *c = getenv("CORUN_ATTN_WHOLE_PAIRS")) e->whole_pairs = atoi(c) != 0;   // ablation only
   if (const char *c = getenv("CORUN_PREFILL_CHUNK")) {
@@ -998,13 +1004,14 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     if ((rc = gemm_encode_map(&e->tm_o[l], w->wo[l], H, QD, GEMM_TILE_N))) return fail(rc);
     if (big_cap) {                                  // the program of many rows
       if (e->tb_qkv.empty())
-        for (auto *v : {&e->tb_qkv, &e->tb_o, &e->tb_gu, &e->tb_down, &e->tb_router, &e->tb_gu_half}) v->resize(s.n_layers);
+        for (auto *v : {&e->tb_qkv, &e->tb_o, &e->tb_gu, &e->tb_down, &e->tb_router, &e->tb_gu_half, &e->tb_gu96}) v->resize(s.n_layers);
       const bool experts = moe && l >= first_dense;
       const int Fd = moe ? dense_ffn : F;
       if ((rc = gemm_encode_map(&e->tb_qkv[l], w->wqkv[l], qkv_rows, H, 128)) || (rc = gemm_encode_map(&e->tb_o[l], w->wo[l], H, QD, 128)))
         return fail(rc);
       if (experts ? (rc = gemm_encode_map(&e->tb_router[l], moe->router[l], moe->n_experts, H, 128))
                   : ((moe && (rc = gemm_encode_map(&e->tb_gu_half[l], w->wgate_up[l], 2 * Fd, H, gemm_swiglu_half(Fd, e->num_sms)))) ||
+                     (rc = gemm_encode_map(&e->tb_gu96[l], w->wgate_up[l], 2 * Fd, H, 96)) ||
                      (rc = gemm_encode_map(&e->tb_gu[l], w->wgate_up[l], 2 * Fd, H, 128)) || (rc = gemm_encode_map(&e->tb_down[l], w->wdown[l], H, Fd, 128))))
         return fail(rc);
     }

@@ -618,10 +618,11 @@ int tma_encode_store_2d(CUtensorMap *m, const void *base, int is_fp32, unsigned 
   if (((uintptr_t)base & 15u) || (cols * eb) % 16 || rows < 1) return CORUN_EINVAL;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)cols * eb};
-  cuuint32_t box[2] = {(cuuint32_t)(128 / eb), 32};
+  cuuint32_t box[2] = {32, 32};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(m, is_fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims,
-                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, is_fp32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                   CU_TENSOR_MAP_L2_PROMOTION_NONE,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) g_last_cuda_error = 100000 + (int)r;
   return r == CUDA_SUCCESS ? CORUN_OK : CORUN_ECUDA;

@@ -33,7 +33,32 @@ struct GemmOut {
   const int *tile_first; // [n_tiles] 2 * (first CTA touching the tile) + (the slot that CTA used for it)
   const int *tile_cend;  // [n_tiles] last CTA touching the tile (every later CTA used slot 0)
   int N, KB, BN;
+  // Result of gemm_pair.cu (row_tiles > 0): tiles [256 rows x 256 columns], row tiles fastest; the first `whole` are in
+  // `direct`, the others in `ws`, `slices` partial matrices [BN, N] behind one another.
+  int row_tiles, whole, slices;
 };
+
+// Values of a gemm_pair.cu result, the slices added in ascending order.
+__device__ __forceinline__ float gemm_load_pair(const GemmOut &g, int r, int n) {
+  const size_t o = (size_t)r * g.N + n;
+  if ((n / GEMM_TILE_N) * g.row_tiles + r / 256 < g.whole) return g.direct[o];
+  float acc = g.ws[o];
+  for (int s = 1; s < g.slices; ++s) acc += g.ws[(size_t)s * g.BN * g.N + o];
+  return acc;
+}
+__device__ __forceinline__ float4 gemm_load_pair4(const GemmOut &g, int r, int n) {
+  const size_t o = (size_t)r * g.N + n;
+  if ((n / GEMM_TILE_N) * g.row_tiles + r / 256 < g.whole) return *reinterpret_cast<const float4 *>(g.direct + o);
+  float4 v[8];                                      // at most eight slices, all requested together
+#pragma unroll
+  for (int s = 0; s < 8; ++s)
+    if (s < g.slices) v[s] = *reinterpret_cast<const float4 *>(g.ws + (size_t)s * g.BN * g.N + o);
+  float4 acc = v[0];
+#pragma unroll
+  for (int s = 1; s < 8; ++s)
+    if (s < g.slices) { acc.x += v[s].x; acc.y += v[s].y; acc.z += v[s].z; acc.w += v[s].w; }
+  return acc;
+}
 
 // Value (r, n) of a GEMM result, partials added in ascending CTA order.
 __device__ __forceinline__ float gemm_load(const GemmOut &g, int r, int n) {
@@ -51,6 +76,7 @@ __device__ __forceinline__ float gemm_load(const GemmOut &g, int r, int n) {
 // Four consecutive values (n % 4 == 0, N % 4 == 0) with the same summation order as gemm_load.
 // Loads are issued four partials at a time; an absent partial contributes +0.0f.
 __device__ __forceinline__ float4 gemm_load4(const GemmOut &g, int r, int n) {
+  if (g.row_tiles) return gemm_load_pair4(g, r, n);
   const int t = n / GEMM_TILE_N, col = n % GEMM_TILE_N;
   const int f = g.tile_first[t], c0 = f >> 1, c1 = g.tile_cend[t];
   if (c0 == c1) return *reinterpret_cast<const float4 *>(g.direct + (size_t)r * g.N + n);
@@ -186,18 +212,26 @@ int tma_encode_fp16_nd(CUtensorMap *m, const void *base, int nd, const unsigned 
 struct GemmPairPlan {
   CUtensorMap tmHi, tmLo, tmOut, tmOut2;
   int N = 0, K = 0, cap = 0, pairs = 0, n_tiles = 0;   // weight rows, reduction length, rows the buffers hold
+  int slices = 1;                    // cuts of K (gemm_pair_slices)
   bool swiglu = false;
-  float *out = nullptr;              // not owned
+  float *out = nullptr, *part = nullptr;   // not owned
 };
-// out [cap, N] fp32 = X W^T for activations Xhi / Xlo [cap, K] (N % 8 == 0).
-int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, int num_sms);
+// Into how many slices K is cut: a function of the matrix and the GPU, never of the rows.
+int gemm_pair_slices(int N, int K, int num_sms);
+// X W^T for activations Xhi / Xlo [cap, K] (N % 8 == 0) -> out [cap, N] fp32 and, for the tiles of an unfilled wave, part
+// [slices][cap][N] (null: one slice).  Read through gemm_pair_out(p, R, zeros).
+int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms);
+GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles);
+cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st);   // makes `out` a plain matrix
 // W is [2F, K] (F gate rows, then F up rows; F % 8 == 0): out_hi / out_lo [cap, F] = silu(gate) * up as a bf16 hi/lo pair.
 int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,
                                  __nv_bfloat16 *out_lo, int num_sms);
 int gemm_pair_prepare();             // opts the kernels into their shared-memory size (idempotent)
-// Rows 0 .. R-1 (R <= cap).  tmW: the weight matrix with a box of 128 rows (gemm_encode_map(.., 128)).
-cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st);
-// Tensor map for TMA stores of tiles of 32 rows x 128 bytes into a [rows, cols] row-major matrix (fp32 or bf16), 128-byte swizzle.
+// Rows 0 .. R-1 (R <= cap).  tmW: the weight matrix with a box of 128 rows (gemm_encode_map(.., 128)); tmW96 (swiglu): the
+// same with 96 rows, taken where it shortens the waves.
+cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st,
+                             const CUtensorMap *tmW96 = nullptr);
+// Tensor map for TMA stores of tiles of 32 rows x 32 columns into a [rows, cols] row-major matrix (fp32: 128-byte swizzle; bf16: 64).
 int tma_encode_store_2d(CUtensorMap *m, const void *base, int is_fp32, unsigned long long rows, int cols);
 // direct[r, n] = gemm_load(r, n) for every tile that has partials (makes `direct` a plain matrix).
 cudaError_t gemm_fixup_launch(const GemmPlan &p, cudaStream_t st, bool pdl = false, int rows = 0);   // rows: the first ones (0: p.R)

@@ -1,4 +1,4 @@
-// tcgen05 GEMM for many activation rows (prompts beyond one small chunk): two SMs work as a pair on one tile.
+// tcgen05 GEMM for many activation rows (long prompts, decode steps above 128 rows): two SMs work as a pair on one tile.
 #include <cudaTypedefs.h>
 
 #include "../../include/corun.h"
@@ -10,13 +10,14 @@ namespace corun {
 
 namespace {
 
-constexpr int PG_THREADS = 192;                     // warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue
+constexpr int PG_THREADS = 320;                     // warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue
+constexpr int PG_EPI = 8;                           // epilogue warps: two per TMEM lane quarter, half of the columns each
 constexpr int PG_STAGES = 4;
 constexpr uint32_t PG_X_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: a CTA's 128 activation rows, hi or lo
 constexpr uint32_t PG_W_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: a CTA's half of the 256 weight rows
 constexpr uint32_t PG_STAGE_BYTES = 2 * PG_X_BYTES + PG_W_BYTES;
-constexpr uint32_t PG_OUT_BYTES = 32 * 128;                  // one staging tile of the epilogue: 32 rows x 128 bytes
-constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + 4 * 2 * PG_OUT_BYTES;
+constexpr uint32_t PG_OUT_BYTES = 32 * 128;                  // an epilogue warp's staging tile: 32 rows x 32 fp32 (or hi and lo of 32 bf16)
+constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + PG_EPI * PG_OUT_BYTES;
 
 // out[r, n] = sum_k W[n, k] * (Xhi[r, k] + Xlo[r, k]) for tiles of 256 rows x 256 weight rows.
 //
@@ -27,8 +28,12 @@ constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + 4 * 2 * P
 // rows) would need 64 and be bound by what the L2 delivers into an SM.  hi and lo go into the same accumulator,
 // k-slice by k-slice.  Two accumulators of 256 columns alternate, so that a tile's epilogue overlaps the next tile.
 //
-// A tile's sum runs over the whole of K in one accumulator whatever the number of rows, the tile order or the grid:
-// a row's result depends on its own activations only, not on its place among the rows nor on their number.
+// K is cut into `slices` (a function of N, K and the number of SMs): a slice is summed in one accumulator, the slices in
+// ascending order in fp32.  A pair that has a whole tile does both itself (the running sum in the epilogue's registers);
+// the tiles that do not fill a wave of the pairs are dealt out slice by slice, each leaving a partial matrix, and the
+// consumer adds them in the same order (gemm_load_pair4).  So a row's result depends on its own activations only, not on
+// its place among the rows nor on their number: 256 rows of the Qwen3-8B QKV projection are 24 tiles, 72 units of a third
+// of K each for 74 pairs (43 us as 24 whole tiles).
 //
 // Launched in plain stream order (no programmatic launch): a pair's two SMs are taken and left together, never while a
 // CTA of a neighbouring kernel of the stream is on one of them.
@@ -36,13 +41,14 @@ constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + 4 * 2 * P
 // The tiles are walked row tile first (pair p takes tiles p, p + pairs, ...), so that the pairs that run at the same
 // time share weight tiles in L2 and the weights are read from HBM once.
 //
-// SWIGLU: W is a gate / up matrix ([2F, K]); a tile is 128 gate rows (first CTA) and the up rows of the same outputs
-// (second CTA), and the epilogue writes silu(gate) * up as the bf16 hi/lo pair the down GEMM reads.
+// SWIGLU: W is a gate / up matrix ([2F, K]); a tile is `half` gate rows (first CTA) and the up rows of the same outputs
+// (second CTA), whole K, and the epilogue writes silu(gate) * up as the bf16 hi/lo pair the down GEMM reads.
 template <bool SWIGLU>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                  const __grid_constant__ CUtensorMap tmLo, const __grid_constant__ CUtensorMap tmOut,
-                 const __grid_constant__ CUtensorMap tmOut2, int R, int N, int KB, int row_tiles, int n_tiles, int *status) {
+                 const __grid_constant__ CUtensorMap tmOut2, int R, int N, int KB, int row_tiles, int whole, int units, int slices,
+                 int half, int cap, int *status) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[PG_STAGES];      // used in the first CTA: both CTAs' loads of a stage
   __shared__ __align__(8) uint64_t empty_bar[PG_STAGES];     // in each CTA: the MMAs have read the stage
@@ -54,7 +60,6 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int tiles = row_tiles * n_tiles;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
   if (threadIdx.x == 0) {
@@ -65,7 +70,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&tmem_full_bar[a]), 1);
-      mbar_init(smem_u32(&tmem_empty_bar[a]), 256);
+      mbar_init(smem_u32(&tmem_empty_bar[a]), 2 * 32 * PG_EPI);
     }
     fence_mbar_init();
     fence_proxy_async();
@@ -73,7 +78,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     prefetch_tensormap(&tmHi);
     prefetch_tensormap(&tmLo);
     prefetch_tensormap(&tmOut);
-    if (SWIGLU) prefetch_tensormap(&tmOut2);
+    prefetch_tensormap(&tmOut2);
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(&tmem_base_s), 512);   // (the permit is given back at the end: see there)
   tc_fence_before();
@@ -84,38 +89,45 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   volatile int *abort_p = &abort_flag;
   int fail = 0;
 
+  // Work unit u: a whole tile (all slices in turn), or one slice of a tile beyond the `whole` first ones.
+  struct Unit { int tile, s0, s1; };
+  auto unit = [&](int u) {
+    if (u < whole) return Unit{u, 0, slices};
+    const int v = u - whole, t = v / slices, sl = v - t * slices;
+    return Unit{whole + t, sl, sl + 1};
+  };
+  auto cut = [&](int sl) { return sl * KB / slices; };       // first k-block of a slice
+
   if (warp == 0) {
     if (lane == 0) {
       // ---------------- TMA producer (both CTAs; the bytes count on the first CTA's barrier) ----------------
       const uint64_t pol_w = l2_policy_evict_first();        // a weight tile is used by the row tiles that run now
       const uint64_t pol_x = l2_policy_evict_last();
-      auto load_w = [&](int it, int tile, int kb) {
-        const int s = it % PG_STAGES, nt = tile / row_tiles;
-        const uint32_t fb = smem_u32(&full_bar[s]);
-        if (rank == 0) mbar_arrive_expect_tx(fb, 2 * PG_STAGE_BYTES);
-        const int y = SWIGLU ? nt * 128 + rank * (N >> 1) : nt * GEMM_TILE_N + rank * 128;
-        tma_load_2d_pair(base + (uint32_t)s * PG_STAGE_BYTES + 2 * PG_X_BYTES, &tmW, kb * GEMM_BLOCK_K, y, cluster_map(fb, 0), pol_w);
-      };
-      auto load_x = [&](int it, int tile, int kb) {
-        const int s = it % PG_STAGES, y = (tile % row_tiles) * 256 + rank * 128;
-        const uint32_t fb = cluster_map(smem_u32(&full_bar[s]), 0), dst = base + (uint32_t)s * PG_STAGE_BYTES;
-        tma_load_2d_pair(dst, &tmHi, kb * GEMM_BLOCK_K, y, fb, pol_x);
-        tma_load_2d_pair(dst + PG_X_BYTES, &tmLo, kb * GEMM_BLOCK_K, y, fb, pol_x);
-      };
+      const uint32_t stage_tx = 2u * (2 * PG_X_BYTES + (uint32_t)half * 128u);
       int it = 0;
-      for (int tile = pair; tile < tiles && !fail; tile += n_pairs)
-        for (int kb = 0; kb < KB; ++kb, ++it) {
-          if (!mbar_wait(smem_u32(&empty_bar[it % PG_STAGES]), ((uint32_t)(it / PG_STAGES) & 1u) ^ 1u, abort_p)) {
+      for (int u = pair; u < units && !fail; u += n_pairs) {
+        const Unit un = unit(u);
+        const int nt = un.tile / row_tiles, yx = (un.tile % row_tiles) * 256 + rank * 128;
+        const int yw = SWIGLU ? nt * half + rank * (N >> 1) : nt * GEMM_TILE_N + rank * 128;
+        const int kb1 = cut(un.s1);
+        for (int kb = cut(un.s0); kb < kb1; ++kb, ++it) {
+          const int s = it % PG_STAGES;
+          if (!mbar_wait(smem_u32(&empty_bar[s]), ((uint32_t)(it / PG_STAGES) & 1u) ^ 1u, abort_p)) {
             fail = DEV_TIMEOUT_PRODUCER;
             break;
           }
-          load_w(it, tile, kb);
-          load_x(it, tile, kb);
+          const uint32_t fb = smem_u32(&full_bar[s]), dst = base + (uint32_t)s * PG_STAGE_BYTES;
+          if (rank == 0) mbar_arrive_expect_tx(fb, stage_tx);
+          const uint32_t fb0 = cluster_map(fb, 0);
+          tma_load_2d_pair(dst + 2 * PG_X_BYTES, &tmW, kb * GEMM_BLOCK_K, yw, fb0, pol_w);
+          tma_load_2d_pair(dst, &tmHi, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
+          tma_load_2d_pair(dst + PG_X_BYTES, &tmLo, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
         }
+      }
       // every stage's last release has arrived before this CTA may end: an arrival of the pair's MMAs must not find the
       // shared memory given to another CTA
       for (int i = 0; i < PG_STAGES && !fail; ++i) {
-        const int last = it - 1 - i;                // the it-th last use of the ring
+        const int last = it - 1 - i;
         if (last < 0) break;
         if (!mbar_wait(smem_u32(&empty_bar[last % PG_STAGES]), (uint32_t)(last / PG_STAGES) & 1u, abort_p)) fail = DEV_TIMEOUT_PRODUCER;
       }
@@ -123,106 +135,125 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
       // ---------------- MMA issuer (first CTA) ----------------
-      // kind::f16: D fp32, A and B bf16, both K-major, N = 256, M = 256 over the pair
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GEMM_TILE_N >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      // kind::f16: D fp32, A and B bf16, both K-major, N = 2 * half, M = 256 over the pair
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * half >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
       int it = 0, seg = 0;
-      for (int tile = pair; tile < tiles && !fail; tile += n_pairs, ++seg) {
-        const int acc = seg & 1;
-        if (!mbar_wait(smem_u32(&tmem_empty_bar[acc]), ((uint32_t)(seg >> 1) & 1u) ^ 1u, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
-        tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)acc * GEMM_TILE_N;
-        for (int kb = 0; kb < KB; ++kb, ++it) {
-          const int s = it % PG_STAGES;
-          if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(it / PG_STAGES) & 1u, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
+      for (int u = pair; u < units && !fail; u += n_pairs) {
+        const Unit un = unit(u);
+        for (int sl = un.s0; sl < un.s1 && !fail; ++sl, ++seg) {
+          const int acc = seg & 1;
+          if (!mbar_wait(smem_u32(&tmem_empty_bar[acc]), ((uint32_t)(seg >> 1) & 1u) ^ 1u, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
           tc_fence_after();
-          const uint32_t st = base + (uint32_t)s * PG_STAGE_BYTES;
-          const uint64_t hi = umma_desc_sw128(st), lo = umma_desc_sw128(st + PG_X_BYTES), w = umma_desc_sw128(st + 2 * PG_X_BYTES);
+          const uint32_t d = tmem_base + (uint32_t)acc * GEMM_TILE_N;
+          const int kb0 = cut(sl), kb1 = cut(sl + 1);
+          for (int kb = kb0; kb < kb1; ++kb, ++it) {
+            const int s = it % PG_STAGES;
+            if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(it / PG_STAGES) & 1u, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
+            tc_fence_after();
+            const uint32_t st = base + (uint32_t)s * PG_STAGE_BYTES;
+            const uint64_t hi = umma_desc_sw128(st), lo = umma_desc_sw128(st + PG_X_BYTES), w = umma_desc_sw128(st + 2 * PG_X_BYTES);
 #pragma unroll
-          for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
-            const uint64_t adv = (uint64_t)(k * 2);
-            umma_bf16_pair(d, hi + adv, w + adv, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-            umma_bf16_pair(d, lo + adv, w + adv, idesc, 1u);
+            for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
+              const uint64_t adv = (uint64_t)(k * 2);
+              umma_bf16_pair(d, hi + adv, w + adv, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+              umma_bf16_pair(d, lo + adv, w + adv, idesc, 1u);
+            }
+            umma_commit_pair(smem_u32(&empty_bar[s]));
           }
-          umma_commit_pair(smem_u32(&empty_bar[s]));
+          if (!fail) umma_commit_pair(smem_u32(&tmem_full_bar[acc]));
         }
-        if (!fail) umma_commit_pair(smem_u32(&tmem_full_bar[acc]));
       }
     }
   } else {
     // ---------------- epilogue: TMEM -> registers -> swizzled staging tile -> TMA store ----------------
-    const int lane_base = (warp & 3) * 32;
-    const uint32_t stg = base + PG_STAGES * PG_STAGE_BYTES + (uint32_t)(warp - 2) * 2 * PG_OUT_BYTES;
+    const int lane_base = (warp & 3) * 32, grp = (warp - 2) >> 2;   // lane quarter; half of the columns
+    const uint32_t stg = base + PG_STAGES * PG_STAGE_BYTES + (uint32_t)(warp - 2) * PG_OUT_BYTES;
     uint8_t *stg_p = smem_raw + (stg - smem_u32(smem_raw));
-    const uint32_t swz = (uint32_t)(lane & 7);
-    int seg = 0, buf = 0;                           // buf: the staging tile of the next store (they alternate)
-    for (int tile = pair; tile < tiles; tile += n_pairs, ++seg) {
-      const int acc = seg & 1, nt = tile / row_tiles;
-      const int row0 = (tile % row_tiles) * 256 + rank * 128 + lane_base;   // this warp's 32 rows
-      bool ok = mbar_wait(smem_u32(&tmem_full_bar[acc]), (uint32_t)(seg >> 1) & 1u, abort_p);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) { fail = DEV_TIMEOUT_EPILOGUE; break; }
-      tc_fence_after();
-      const uint32_t ta = tmem_base + (uint32_t)acc * GEMM_TILE_N + ((uint32_t)lane_base << 16);
-      if (row0 < R) {                               // warp-uniform
-        if (SWIGLU) {
-          for (int c0 = 0; c0 < 128; c0 += 64) {
-            const int col = nt * 128 + c0;
-            if (col >= (N >> 1)) break;
-            if (lane == 0) bulk_wait_read<0>();     // the staging tiles have been read
-            __syncwarp();
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              uint32_t g[32], u[32];
-              tmem_ld32(ta + (uint32_t)(c0 + 32 * half), g);
-              tmem_ld32(ta + (uint32_t)(128 + c0 + 32 * half), u);
+    const uint32_t lane_off = (uint32_t)lane_base << 16;
+    int seg = 0;
+    bool ok = true;
+    for (int u = pair; u < units && ok; u += n_pairs) {
+      const Unit un = unit(u);
+      const int nt = un.tile / row_tiles;
+      const int row0 = (un.tile % row_tiles) * 256 + rank * 128 + lane_base;   // this warp's 32 rows
+      float sum[128];                               // (not SWIGLU) this thread's row, 128 columns
+      for (int sl = un.s0; sl < un.s1; ++sl, ++seg) {
+        const int acc = seg & 1;
+        ok = mbar_wait(smem_u32(&tmem_full_bar[acc]), (uint32_t)(seg >> 1) & 1u, abort_p);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) { fail = DEV_TIMEOUT_EPILOGUE; break; }
+        tc_fence_after();
+        const uint32_t ta = tmem_base + (uint32_t)acc * GEMM_TILE_N + lane_off;
+        if (row0 < R) {                             // warp-uniform
+          if (SWIGLU) {
+            for (int c0 = grp * 32; c0 < half; c0 += 64) {
+              const int col = nt * half + c0;
+              if (col >= (N >> 1)) break;
+              uint32_t g[32], up[32];
+              tmem_ld32(ta + (uint32_t)c0, g);
+              tmem_ld32(ta + (uint32_t)(half + c0), up);
+              if (lane == 0) bulk_wait_read<0>();   // the staging tile has been read
+              __syncwarp();
               tmem_ld_wait();
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {         // 16 bytes = 8 outputs
+              for (int q = 0; q < 4; ++q) {         // 16 bytes = 8 outputs; 64-byte rows, 64-byte swizzle
                 __nv_bfloat16 a[8], b[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                   const float gt = __uint_as_float(g[8 * q + j]);
-                  const float y = gt / (1.f + expf(-gt)) * __uint_as_float(u[8 * q + j]);
+                  const float y = gt / (1.f + expf(-gt)) * __uint_as_float(up[8 * q + j]);
                   a[j] = __float2bfloat16_rn(y);
                   b[j] = __float2bfloat16_rn(y - __bfloat162float(a[j]));
                 }
-                const uint32_t off = (uint32_t)lane * 128 + (((uint32_t)(4 * half + q) ^ swz) << 4);
+                const uint32_t off = (uint32_t)lane * 64 + (((uint32_t)q ^ (((uint32_t)lane >> 1) & 3u)) << 4);
                 *reinterpret_cast<uint4 *>(stg_p + off) = *reinterpret_cast<const uint4 *>(a);
-                *reinterpret_cast<uint4 *>(stg_p + PG_OUT_BYTES + off) = *reinterpret_cast<const uint4 *>(b);
+                *reinterpret_cast<uint4 *>(stg_p + PG_OUT_BYTES / 2 + off) = *reinterpret_cast<const uint4 *>(b);
+              }
+              fence_proxy_async();
+              __syncwarp();
+              if (lane == 0) {
+                tma_store_2d(&tmOut, stg, col, row0);
+                tma_store_2d(&tmOut2, stg + PG_OUT_BYTES / 2, col, row0);
+                bulk_commit();
               }
             }
-            fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) {
-              tma_store_2d(&tmOut, stg, col, row0);
-              tma_store_2d(&tmOut2, stg + PG_OUT_BYTES, col, row0);
-              bulk_commit();
+          } else {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {          // (8 columns at a time: 128 running sums leave few registers)
+              uint32_t v[8];
+              tmem_ld8(ta + (uint32_t)(grp * 128 + q * 8), v);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 8; ++j) sum[8 * q + j] = (sl == un.s0 ? 0.f : sum[8 * q + j]) + __uint_as_float(v[j]);
             }
           }
-        } else {
-          for (int c0 = 0; c0 < GEMM_TILE_N; c0 += 32, buf ^= 1) {
-            const int col = nt * GEMM_TILE_N + c0;
-            if (col >= N) break;
-            uint32_t v[32];
-            tmem_ld32(ta + (uint32_t)c0, v);
-            if (lane == 0) bulk_wait_read<1>();     // the store before the last one has read this staging tile
-            __syncwarp();
-            tmem_ld_wait();
+        }
+        tc_fence_before();
+        mbar_arrive_cluster(cluster_map(smem_u32(&tmem_empty_bar[acc]), 0));
+      }
+      if (!SWIGLU && ok && row0 < R) {
+        // a whole tile goes to the output, a slice to its partial matrix
+        const bool part = u >= whole;
+        const int y = part ? un.s0 * cap + row0 : row0;
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-              *reinterpret_cast<uint4 *>(stg_p + buf * PG_OUT_BYTES + lane * 128 + (((uint32_t)q ^ swz) << 4)) =
-                  make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int q = 0; q < 4; ++q) {
+          const int col = nt * GEMM_TILE_N + grp * 128 + q * 32;
+          if (col < N) {
+            if (lane == 0) bulk_wait_read<0>();
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+              *reinterpret_cast<float4 *>(stg_p + lane * 128 + (((uint32_t)c ^ ((uint32_t)lane & 7u)) << 4)) =
+                  make_float4(sum[32 * q + 4 * c], sum[32 * q + 4 * c + 1], sum[32 * q + 4 * c + 2], sum[32 * q + 4 * c + 3]);
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) {
-              tma_store_2d(&tmOut, stg + (uint32_t)buf * PG_OUT_BYTES, col, row0);
+              tma_store_2d(part ? &tmOut2 : &tmOut, stg, col, y);
               bulk_commit();
             }
           }
         }
       }
-      tc_fence_before();
-      mbar_arrive_cluster(cluster_map(smem_u32(&tmem_empty_bar[acc]), 0));
     }
     if (lane == 0) bulk_wait<0>();                  // the stores have been performed before the kernel ends
   }
@@ -241,17 +272,88 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
 }
 
+// The tiles that were left as partial matrices, added up in place (for consumers that read a plain matrix).
+__global__ void __launch_bounds__(256) gemm_pair_fixup_kernel(GemmOut g, float *direct, int first_tile) {
+  griddep_launch_dependents();
+  griddep_wait();
+  const int t = first_tile + blockIdx.x, r = (t % g.row_tiles) * 256 + blockIdx.y, n = (t / g.row_tiles) * GEMM_TILE_N + threadIdx.x;
+  if (n < g.N && r < g.BN) direct[(size_t)r * g.N + n] = gemm_load_pair(g, r, n);
+}
+
+// How a launch over R rows divides its tiles: the first `whole` as whole tiles, the others slice by slice where that
+// shortens the last wave.
+struct PairShape { int row_tiles, whole, units, half; };
+PairShape pair_shape(const GemmPairPlan &p, int R, bool narrow) {
+  PairShape q{};
+  q.row_tiles = (R + 255) / 256;
+  q.half = 128;
+  int n_tiles = p.n_tiles;
+  if (p.swiglu && narrow) {
+    // tiles of 96 outputs where their waves are shorter by a tenth or more (256 rows of the Qwen3-8B gate / up: two of 96
+    // against two of 128, 79 us against 114; 2048 rows would gain 4 % of the waves and re-read a third more activations)
+    const int F = p.N / 2, t128 = q.row_tiles * ((F + 127) / 128), t96 = q.row_tiles * ((F + 95) / 96);
+    if ((t96 + p.pairs - 1) / p.pairs * 96 * 10 < (t128 + p.pairs - 1) / p.pairs * 128 * 9) { q.half = 96; n_tiles = (F + 95) / 96; }
+  }
+  const int tiles = q.row_tiles * n_tiles;
+  q.whole = tiles;
+  q.units = tiles;
+  if (p.slices > 1) {
+    const int full = tiles / p.pairs * p.pairs, tail = tiles - full;
+    // worth it where the time of the last wave that is saved (0.8 us per k-block) exceeds what writing and reading the
+    // partials costs (0.5 MB per slice of a tile at 5 TB/s): 16 of 16 tiles of the Qwen3-8B O projection at 256 rows 51 -> 21
+    // us, not 54 of 128 at 2048 rows
+    const int parts = (tail * p.slices + p.pairs - 1) / p.pairs;
+    const float saved = 0.8f * (float)(p.K / GEMM_BLOCK_K) * (float)(p.slices - parts) / (float)p.slices;
+    if (tail && saved > 0.1f * (float)(tail * p.slices)) {
+      q.whole = full;
+      q.units = full + tail * p.slices;
+    }
+  }
+  return q;
+}
+
 }  // namespace
 
-int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, int num_sms) {
+int gemm_pair_slices(int N, int K, int num_sms) {
+  const int n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N, kb = K / GEMM_BLOCK_K, pairs = num_sms / 2;
+  int s = pairs / n_tiles;                          // one row tile in one wave
+  if (s < 1) s = 4;                                 // more tiles than pairs: the slices serve the last wave only
+  if (s > 8) s = 8;
+  while (s > 1 && kb / s < 8) --s;                  // a slice of fewer than 8 k-blocks costs more than it shortens
+  return s;
+}
+
+int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms) {
   if (N <= 0 || N % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out || num_sms < 2) return CORUN_EINVAL;
-  p->N = N; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = false; p->out = out;
+  p->N = N; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = false; p->out = out; p->part = part;
   p->n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N;
+  p->slices = part ? gemm_pair_slices(N, K, num_sms) : 1;
   int rc;
   if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
   if ((rc = tma_encode_store_2d(&p->tmOut, out, 1, cap, N)) != 0) return rc;
-  p->tmOut2 = p->tmOut;
+  if (p->slices > 1) {
+    if ((rc = tma_encode_store_2d(&p->tmOut2, part, 1, (unsigned long long)p->slices * cap, N)) != 0) return rc;
+  } else {
+    p->tmOut2 = p->tmOut;
+  }
   return gemm_pair_prepare();
+}
+
+GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles) {
+  const PairShape q = pair_shape(p, R, false);
+  GemmOut g{p.out, p.part, zero_tiles, zero_tiles, p.N, 0, p.cap};
+  g.row_tiles = q.row_tiles;
+  g.whole = q.whole;
+  g.slices = p.slices;
+  return g;
+}
+
+cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st) {
+  const PairShape q = pair_shape(p, R, false);
+  const int tiles = q.row_tiles * p.n_tiles;
+  if (q.whole == tiles) return cudaSuccess;
+  return launch_k(gemm_pair_fixup_kernel, dim3(tiles - q.whole, R < 256 ? R : 256), dim3(256), 0, st, true, gemm_pair_out(p, R, nullptr), p.out,
+                  q.whole);
 }
 
 int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,
@@ -259,6 +361,7 @@ int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi,
   if (F <= 0 || F % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out_hi || !out_lo || num_sms < 2) return CORUN_EINVAL;
   p->N = 2 * F; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = true; p->out = nullptr;
   p->n_tiles = (F + 127) / 128;
+  p->slices = 1;
   int rc;
   if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
   if ((rc = tma_encode_store_2d(&p->tmOut, out_hi, 0, cap, F)) != 0 || (rc = tma_encode_store_2d(&p->tmOut2, out_lo, 0, cap, F)) != 0)
@@ -273,13 +376,13 @@ int gemm_pair_prepare() {
   return CORUN_OK;
 }
 
-cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st) {
+cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st, const CUtensorMap *tmW96) {
   if (R < 1 || R > p.cap) return cudaErrorInvalidValue;
-  const int row_tiles = (R + 255) / 256, tiles = row_tiles * p.n_tiles;
-  const int pairs = tiles < p.pairs ? tiles : p.pairs;
+  const PairShape q = pair_shape(p, R, tmW96 != nullptr);
+  const int pairs = q.units < p.pairs ? q.units : p.pairs;
   auto go = [&](auto kernel) {
-    return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2, R, p.N,
-                    p.K / GEMM_BLOCK_K, row_tiles, p.n_tiles, d_status);
+    return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, q.half == 96 ? *tmW96 : tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2,
+                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, q.half, p.cap, d_status);
   };
   return p.swiglu ? go(gemm_pair_kernel<true>) : go(gemm_pair_kernel<false>);
 }

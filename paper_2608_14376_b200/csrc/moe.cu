@@ -391,15 +391,15 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_many_kernel(const
 }
 
 // Routing of many rows: one warp per row.
-__global__ void __launch_bounds__(256) moe_route_kernel(const float *__restrict__ logits, int R, int E, int S, int top_k, int renormalize,
+__global__ void __launch_bounds__(256) moe_route_kernel(GemmOut logits, int R, int E, int S, int top_k, int renormalize,
                                                         float *__restrict__ w) {
   griddep_launch_dependents();
   griddep_wait();
-  logits = after_wait(logits);
+  logits.direct = after_wait(logits.direct);
+  logits.ws = after_wait(logits.ws);
   const int r = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= R) return;
-  const float *row = logits + (size_t)r * E;
-  moe_route_row([&](int e) { return row[e]; }, r, lane, E, S, top_k, renormalize, w, nullptr, nullptr);
+  moe_route_row([&](int e) { return gemm_load_pair(logits, r, e); }, r, lane, E, S, top_k, renormalize, w, nullptr, nullptr);
 }
 
 // The gathered activation rows: one warp per slot of the groups in use (all of a row's loads requested before the
@@ -531,7 +531,7 @@ cudaError_t launch_moe_group_many(const float *w, const int *active, int R, int 
   return launch_k(moe_group_many_kernel, dim3(E + S), dim3(MOE_GROUP_THREADS), 0, st, true, w, mask, R, E + S, E, F, g);
 }
 
-cudaError_t launch_moe_route(const float *logits, int R, int E, int S, int top_k, int renormalize, float *w, cudaStream_t st) {
+cudaError_t launch_moe_route(const GemmOut &logits, int R, int E, int S, int top_k, int renormalize, float *w, cudaStream_t st) {
   return launch_k(moe_route_kernel, dim3((R + 7) / 8), dim3(256), 0, st, true, logits, R, E, S, top_k, renormalize, w);
 }
 

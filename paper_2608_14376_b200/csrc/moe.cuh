@@ -49,8 +49,8 @@ cudaError_t launch_moe_group(const float *w, const int *active, int R, int E, in
 // The same for up to MOE_MANY_ROWS rows in two kernels (prefill of long prompts).  mask: [E + S][MOE_MANY_ROWS / 32] words.
 cudaError_t launch_moe_group_many(const float *w, const int *active, int R, int E, int S, int F, uint32_t *mask, const MoeGroups &g,
                                   cudaStream_t st);
-// Routing of many rows from their router logits [R, E] (fp32, computed by a GEMM): as launch_moe_router otherwise.
-cudaError_t launch_moe_route(const float *logits, int R, int E, int S, int top_k, int renormalize, float *w, cudaStream_t st);
+// Routing of many rows from their router logits (a gemm_pair.cu result [R, E]): as launch_moe_router otherwise.
+cudaError_t launch_moe_route(const GemmOut &logits, int R, int E, int S, int top_k, int renormalize, float *w, cudaStream_t st);
 // xg[slot, :] = x[slot_row[slot], :] for both halves of the activations (bf16, H values per row).
 cudaError_t launch_moe_gather(const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_lo, int H, const MoeGroups &g,
                               __nv_bfloat16 *xg_hi, __nv_bfloat16 *xg_lo, cudaStream_t st);

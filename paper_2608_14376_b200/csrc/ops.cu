@@ -134,7 +134,7 @@ qkv_post_few_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab,
 }
 
 // Many rows: a thread takes four consecutive rotation indices of one head, (i .. i + 3) and their partners half a head on: 16-byte loads
-// and q stores, 8-byte cache stores.  Bound by L2 / HBM traffic (PLAIN: prefill of long prompts, a plain matrix: at 1024
+// and q stores, 8-byte cache stores.  Bound by L2 / HBM traffic (PLAIN: a gemm_pair.cu result: at 1024
 // rows of Qwen3-8B 25 MB read, 25 MB written; 256 rows with partials: 11 us less per layer than the kernel above).
 constexpr int QKV_THREADS = 128, QKV_FEW_ROWS = 64;
 template <bool PLAIN>
@@ -152,9 +152,10 @@ qkv_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, int
   const int col = head * hd + i;                   // q, k and v heads are contiguous in the GEMM output
   float4 a, b;
   if (PLAIN) {
-    const float *src = after_wait(qkv.direct) + (size_t)r * qkv.N + col;
-    a = *reinterpret_cast<const float4 *>(src);
-    b = *reinterpret_cast<const float4 *>(src + half);
+    qkv.direct = after_wait(qkv.direct);
+    qkv.ws = after_wait(qkv.ws);
+    a = gemm_load_pair4(qkv, r, col);
+    b = gemm_load_pair4(qkv, r, col + half);
   } else {
     a = gemm_load4(qkv, r, col);
     b = gemm_load4(qkv, r, col + half);
@@ -953,11 +954,11 @@ cudaError_t launch_resid_norm(float *h, int H, const __nv_bfloat16 *embed, const
 
 cudaError_t launch_qkv_post(const GemmOut &qkv, const Rows &rows, const float2 *rope_tab, int nq, const KvLayout &kv,
                             int layer, float *q_out, int *d_status, cudaStream_t st) {
-  if (rows.R <= QKV_FEW_ROWS)
+  if (rows.R <= QKV_FEW_ROWS && !qkv.row_tiles)
     return launch_k(qkv_post_few_kernel, dim3(nq + 2 * kv.n_kv, rows.R), dim3(kv.hd / 2), 0, st, true, qkv, rows, rope_tab, nq, kv, layer,
                     q_out, d_status);
   const dim3 grid(((nq + 2 * kv.n_kv) * (kv.hd / 8) + QKV_THREADS - 1) / QKV_THREADS, rows.R);
-  return launch_k(qkv.ws ? qkv_post_kernel<false> : qkv_post_kernel<true>, grid, dim3(QKV_THREADS), 0, st, true, qkv, rows, rope_tab, nq,
+  return launch_k(qkv.row_tiles ? qkv_post_kernel<true> : qkv_post_kernel<false>, grid, dim3(QKV_THREADS), 0, st, true, qkv, rows, rope_tab, nq,
                   kv, layer, q_out, d_status);
 }
 

@@ -108,3 +108,41 @@ def test_long_prompts_through_expert_layers(orc, arch, lens):
     assert list(e.prefill_batch(slots, prompts, res, 0.7, 0.95, seeds)) == first
     assert after() == alone
     e.close()
+
+
+@pytest.mark.parametrize("lens", [[257, 300, 4], [1500, 513], [2048, 260]])
+def test_slices_of_the_projections_give_the_same_bytes_in_any_chunk(orc, lens):
+    """Hidden 1024 / FFN 3072: K is cut into 2 (projections) and 6 (down) slices, which a pair of SMs adds up itself for
+    whole tiles and leaves as partial matrices for the tiles of an unfilled wave; how many there are depends on the rows
+    of the chunk, so alone and sharing chunks take different ways to the same bytes."""
+    from paper_2608_14376_b200 import corun
+
+    B = 4
+    sh = synth.ModelShape(2, 1024, 8, 2, 128, 3072, 1024, 1e-6, 10000.0)
+    w = synth.make_weights_numpy(sh, seed=6)
+    model = orc.Model(orc.Shape(**sh.dict()), w)
+    prompts = synth.make_prompts(sh.vocab, lens, seed=40 + lens[0])
+    slots = [1, 3, 0][:len(lens)]
+    seeds = np.array([synth.request_seed(i) for i in range(len(lens))], np.uint64)
+    res = [n + 2 for n in lens]
+    e = corun.Engine(sh, synth.weights_numpy_to_torch(w, "cuda"), B, max(res))
+
+    def after():
+        out = [e.logits(s).tobytes() for s in slots]
+        for s, n in zip(slots, lens):
+            k, v = e.kv_read(s, sh.n_layers - 1, 0, n)
+            out.append(k.tobytes() + v.tobytes())
+        return out
+
+    first = [e.prefill(s, p, r, 0.7, 0.95, seed=int(sd)) for s, p, r, sd in zip(slots, prompts, res, seeds)]
+    for s, p in zip(slots, prompts):
+        if len(p) <= 600:
+            r = orc.Request(model, p, 1, max_T=len(p) + 2)
+            r.prefill()
+            assert np.abs(e.logits(s) - r.logits).max() <= TOL
+    alone = after()
+    for s in slots:
+        e.release(s)
+    assert list(e.prefill_batch(slots, prompts, res, 0.7, 0.95, seeds)) == first
+    assert after() == alone
+    e.close()
