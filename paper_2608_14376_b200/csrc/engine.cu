@@ -99,6 +99,11 @@ struct Program {
   // rows as for long ones.
   bool pair = false;
   int cap = 0;
+  // Decode above 128 rows (wide): the dense projections and the LM head on pairs of SMs too.  Per Qwen3-8B layer at 256 rows
+  // 248 us of GEMMs (hi and lo of two row blocks per weight tile on one SM each, two stages of shared memory) and 17 us of
+  // SwiGLU, against 179 us.
+  bool wide = false;
+  GemmPairPlan b_lm;
   bool shorts = false;
   std::vector<GemmPlan> s_qkv, s_o, s_gu, s_down;
   GemmPairPlan b_qkv, b_o, b_gu, b_down, b_router;
@@ -132,6 +137,7 @@ struct corun_engine {
   std::vector<const bf16 *> attn_norm, mlp_norm;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
   std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down, tb_router, tb_gu96;   // boxes of 128 rows (96): the GEMMs on pairs of SMs
+  CUtensorMap tb_lm;
   std::vector<CUtensorMap> tb_gu_half;     // dense layers of a decoder with expert layers: the box of the GEMM with SwiGLU
   std::vector<CUtensorMap> tm_gu_half;     // dense gate / up matrices with the box of the GEMM with SwiGLU in its epilogue
   std::vector<CUtensorMap> tm_k, tm_v;   // per layer: the pages as rows of head_dim halfs (keys and values alike)
@@ -259,10 +265,12 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
   P.BN = pad16(R);
   P.has_layers = layers;
   P.has_lm = lm;
+  P.wide = layers && lm && P.BN > 128 && V % 8 == 0;
+  const int RB = P.wide ? 256 : P.BN, RR = P.wide ? 256 : R;   // rows of the projections' inputs and outputs
   auto &A = P.allocs;
-  RC(dmalloc(A, &P.xn_hi, (size_t)P.BN * H));
-  RC(dmalloc(A, &P.xn_lo, (size_t)P.BN * H));
-  RC(dmalloc(A, &P.ws, gemm_ws_floats(e->num_sms, P.BN)));
+  RC(dmalloc(A, &P.xn_hi, (size_t)RB * H));
+  RC(dmalloc(A, &P.xn_lo, (size_t)RB * H));
+  if (!P.wide || e->moe_E) RC(dmalloc(A, &P.ws, gemm_ws_floats(e->num_sms, P.BN)));
   RC(dmalloc(A, &P.row_token, R));
   RC(dmalloc(A, &P.row_pos, R));
   RC(dmalloc(A, &P.row_active, R));
@@ -309,26 +317,43 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
                                   P.ol_lo, n_groups, BG, P.uv_out, P.tab_uv, e->num_sms));
       P.p_uk.keep_div = P.p_uv.keep_div = -1;       // the tables are written once, here: the kernels need not wait for them
     }
-    RC(dmalloc(A, &P.qkv_out, (size_t)R * QKVN));
-    RC(dmalloc(A, &P.o_out, (size_t)R * H));
+    RC(dmalloc(A, &P.qkv_out, (size_t)RR * QKVN));
+    RC(dmalloc(A, &P.o_out, (size_t)RR * H));
     // expert layers up to 64 rows: all rows with every expert that one of them selected
     const int NBx = e->moe_E + e->moe_S, half_x = e->moe_E ? gemm_swiglu_blocks_half(e->moe_F, NBx, e->num_sms) : 0;
     P.select = fuse_swiglu && e->moe_E && P.BN <= 64 && half_x && H % GEMM_TILE_N == 0 && NBx <= GEMM_MAX_SELECT &&
                !getenv("CORUN_MOE_DECODE_DENSE");
-    const int Fbuf = P.select ? (Fd > 64 ? Fd : 64) : Fmax;   // the selected-experts form has buffers of its own
+    const bool groups = grouped && e->moe_E && !P.select && (2 * e->moe_F) % GEMM_TILE_N == 0 && H % GEMM_TILE_N == 0;
+    const int Fbuf = P.select || groups ? (Fd > 64 ? Fd : 64) : Fmax;   // those forms have buffers of their own
     RC(dmalloc(A, &P.gu_out, (size_t)R * 2 * Fbuf));
-    RC(dmalloc(A, &P.down_out, (size_t)R * H));
-    RC(dmalloc(A, &P.ao_hi, (size_t)P.BN * QD));
-    RC(dmalloc(A, &P.ao_lo, (size_t)P.BN * QD));
-    RC(dmalloc(A, &P.ff_hi, (size_t)P.BN * Fbuf));
-    RC(dmalloc(A, &P.ff_lo, (size_t)P.BN * Fbuf));
+    RC(dmalloc(A, &P.down_out, (size_t)RR * H));
+    RC(dmalloc(A, &P.ao_hi, (size_t)RB * QD));
+    RC(dmalloc(A, &P.ao_lo, (size_t)RB * QD));
+    RC(dmalloc(A, &P.ff_hi, (size_t)RB * Fbuf));
+    RC(dmalloc(A, &P.ff_lo, (size_t)RB * Fbuf));
     if (e->mla && e->moe_E && e->first_dense > 0) {   // the dense feed-forward layers of a decoder with expert layers
       RC(gemm_plan_create(&P.p_gu_d, e->w0_gu_d, 2 * Fd, H, P.xn_hi, P.xn_lo, R, P.BN, P.gu_out, P.ws, e->num_sms));
       RC(gemm_plan_create(&P.p_down_d, e->w0_down_d, H, Fd, P.ff_hi, P.ff_lo, R, P.BN, P.down_out, P.ws, e->num_sms));
     }
     // the plans carry layer 0's weights; the per-layer tensor maps override them at launch
-    RC(gemm_plan_create(&P.p_qkv, e->w0_qkv, QKVN, H, P.xn_hi, P.xn_lo, R, P.BN, P.qkv_out, P.ws, e->num_sms));
-    RC(gemm_plan_create(&P.p_o, e->w0_o, H, QD, P.ao_hi, P.ao_lo, R, P.BN, P.o_out, P.ws, e->num_sms));
+    if (P.wide) {
+      const bool ffn = !e->moe_E;
+      size_t part = gemm_pair_part_floats(QKVN, H, 256, e->num_sms);
+      for (size_t x : {gemm_pair_part_floats(H, QD, 256, e->num_sms), ffn ? gemm_pair_part_floats(H, F, 256, e->num_sms) : 0,
+                       gemm_pair_part_floats(V, H, 256, e->num_sms)})
+        part = x > part ? x : part;
+      RC(dmalloc(A, &P.pair_part, part, false));
+      if (!P.plain_tiles) RC(dmalloc(A, &P.plain_tiles, (size_t)((QKVN > V ? QKVN : V) / GEMM_TILE_N + 1)));
+      RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, 256, P.qkv_out, P.pair_part, e->num_sms));
+      RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, 256, P.o_out, P.pair_part, e->num_sms));
+      if (ffn) {
+        RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, 256, P.ff_hi, P.ff_lo, e->num_sms));
+        RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, 256, P.down_out, P.pair_part, e->num_sms));
+      }
+    } else {
+      RC(gemm_plan_create(&P.p_qkv, e->w0_qkv, QKVN, H, P.xn_hi, P.xn_lo, R, P.BN, P.qkv_out, P.ws, e->num_sms));
+      RC(gemm_plan_create(&P.p_o, e->w0_o, H, QD, P.ao_hi, P.ao_lo, R, P.BN, P.o_out, P.ws, e->num_sms));
+    }
     // expert layers without groups: the routing weight and the SwiGLU in the epilogue of the GEMM over all experts'
     // gate / up rows (65..128 rows, where the grouped form below does not apply; up to 64 rows the masked store plus a
     // SwiGLU kernel measured faster: the epilogue would write zeros for every pair that was not selected)
@@ -346,15 +371,18 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
                                     R * per_row, e->num_sms));
       RC(gemm_plan_create_select_down(&P.p_dng, e->w0_down, nb, H, Fm, P.hg_hi, P.hg_lo, R, P.BN, P.yg_out, P.moe_w, P.moe_sel,
                                       R * per_row, e->num_sms));
+    } else if (groups || (P.wide && !e->moe_E)) {
+      // their GEMMs are made below / above
     } else if (fuse_swiglu && !e->moe_E && P.BN <= 128)
       RC(gemm_plan_create_swiglu(&P.p_gu, e->w0_gu, F, H, P.xn_hi, P.xn_lo, R, P.BN, P.ff_hi, P.ff_lo, e->num_sms));
     else if (!moe_fused)
       RC(gemm_plan_create(&P.p_gu, e->w0_gu, 2 * F, H, P.xn_hi, P.xn_lo, R, P.BN, P.gu_out, P.ws, e->num_sms));
-    if (!P.select) RC(gemm_plan_create(&P.p_down, e->w0_down, H, F, P.ff_hi, P.ff_lo, R, P.BN, P.down_out, P.ws, e->num_sms));
+    if (!P.select && !groups && !(P.wide && !e->moe_E)) RC(gemm_plan_create(&P.p_down, e->w0_down, H, F, P.ff_hi, P.ff_lo, R, P.BN, P.down_out, P.ws, e->num_sms));
     if (e->moe_E && !P.select) {
       const int NB = e->moe_E + e->moe_S;
       RC(dmalloc(A, &P.moe_w, (size_t)R * NB));
-      if (moe_fused)
+      if (groups) {
+      } else if (moe_fused)
         RC(gemm_plan_create_swiglu_blocks(&P.p_gu, e->w0_gu, NB, e->moe_F, H, P.xn_hi, P.xn_lo, R, P.BN, P.ff_hi, P.ff_lo, P.moe_w,
                                           e->num_sms));
       else if ((2 * e->moe_F) % GEMM_TILE_N == 0) {   // a weight tile belongs to one expert: rows that did not
@@ -362,16 +390,17 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
         P.p_gu.keep_pitch = NB;
         P.p_gu.keep_div = 2 * e->moe_F / GEMM_TILE_N;
       }
-      if (grouped && (2 * e->moe_F) % GEMM_TILE_N == 0 && H % GEMM_TILE_N == 0) {
+      if (groups) {
         // prefill chunks: every row through every expert would be (E + S) / top_k times the MMA work, which a
         // chunk of 256 rows does pay for; the rows of an expert are gathered into blocks of 64 instead
-        RC(dmalloc(A, &P.plain_tiles, (size_t)(H / GEMM_TILE_N + 1)));
+        if (!P.plain_tiles) RC(dmalloc(A, &P.plain_tiles, (size_t)(H / GEMM_TILE_N + 1)));
         RC(program_create_groups(e, P, R));
       }
     }
   }
   if (lm) {
-    RC(dmalloc(A, &P.logits, (size_t)R * V));
+    RC(dmalloc(A, &P.logits, (size_t)RR * V));
+    if (P.wide) return gemm_pair_plan_create(&P.b_lm, V, H, P.xn_hi, P.xn_lo, 256, P.logits, P.pair_part, e->num_sms);
     RC(gemm_plan_create(&P.p_lm, e->lm_head, V, H, P.xn_hi, P.xn_lo, R, P.BN, P.logits, P.ws, e->num_sms));
   }
   return CORUN_OK;
@@ -454,12 +483,12 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   for (auto *v : {&P.s_qkv, &P.s_o, &P.s_gu, &P.s_down}) v->resize((size_t)n_blk);
   RC(gemm_plan_create(&P.s_qkv[0], e->w0_qkv, QKVN, H, P.xn_hi, P.xn_lo, SHORT_ROWS, SHORT_ROWS, P.qkv_out, P.ws, e->num_sms));
   RC(gemm_plan_create(&P.s_o[0], e->w0_o, H, QD, P.ao_hi, P.ao_lo, SHORT_ROWS, SHORT_ROWS, P.o_out, P.ws, e->num_sms));
-  // partial matrices of an unfilled wave: consumed by the next kernel of the stream, so one buffer serves all
-  size_t part = (size_t)gemm_pair_slices(QKVN, H, e->num_sms) * QKVN;
-  const size_t part_o = (size_t)gemm_pair_slices(H, QD, e->num_sms) * H, part_d = F > 0 ? (size_t)gemm_pair_slices(H, F, e->num_sms) * H : 0,
-               part_r = e->moe_E ? (size_t)gemm_pair_slices(e->moe_E, H, e->num_sms) * e->moe_E : 0;
-  for (size_t x : {part_o, part_d, part_r}) part = x > part ? x : part;
-  RC(dmalloc(A, &P.pair_part, part * c, false));
+  // partial tiles of an unfilled wave: consumed by the next kernel of the stream, so one buffer serves all
+  size_t part = gemm_pair_part_floats(QKVN, H, cap, e->num_sms);
+  for (size_t x : {gemm_pair_part_floats(H, QD, cap, e->num_sms), F > 0 ? gemm_pair_part_floats(H, F, cap, e->num_sms) : 0,
+                   e->moe_E ? gemm_pair_part_floats(e->moe_E, H, cap, e->num_sms) : 0})
+    part = x > part ? x : part;
+  RC(dmalloc(A, &P.pair_part, part, false));
   RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, cap, P.qkv_out, P.pair_part, e->num_sms));
   RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, cap, P.o_out, P.pair_part, e->num_sms));
   if (F > 0) {
@@ -562,6 +591,7 @@ bool dense_layer(const corun_engine *e, int layer) { return e->mla && e->moe_E &
 GemmOut ffn_out(const corun_engine *e, const Program &P, int layer) {
   if (P.pair) return P.grouped && !dense_layer(e, layer) ? plain_out(P, P.down_out, e->sh.hidden) : gemm_pair_out(P.b_down, P.R, P.plain_tiles);
   if (dense_layer(e, layer)) return P.p_down_d.out();
+  if (P.wide && !e->moe_E) return gemm_pair_out(P.b_down, P.R, P.plain_tiles);
   if (P.grouped || P.select) return plain_out(P, P.down_out, e->sh.hidden);
   return P.p_down.out();
 }
@@ -678,13 +708,15 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       }
       continue;
     }
-    STAGE(gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, tr(4 * l + 0), true));
+    if (P.wide) STAGE(gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st));
+    else STAGE(gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, tr(4 * l + 0), true));
+    const GemmOut qkv = P.wide ? gemm_pair_out(P.b_qkv, P.R, P.plain_tiles) : P.p_qkv.out();
     if (e->mla) {
       // cache append and query parts -> q_lat = W_uk^T q_nope per head -> absorbed attention over the row's latent
       // pages (decode rows and prefill rows alike) -> [. | o] = W_kv_b o_lat per head -> the value part, split
       const MlaDims &md = e->md;
       const MlaCache cache{e->kv_pool + (size_t)l * e->layer_stride, e->d_block_table, e->max_blocks, e->B, (long long)e->pool_blocks, e->kv_run};
-      STAGE(launch_mla_post(P.p_qkv.out(), rows, e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi, P.qn_lo, P.q_rope,
+      STAGE(launch_mla_post(qkv, rows, e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi, P.qn_lo, P.q_rope,
                             e->d_status, e->st));
       STAGE(gemm_launch(P.p_uk, &e->tm_uk[l], e->d_status, e->st, nullptr, true));
       STAGE(launch_mla_attention(e->tm_c[l], e->tm_cv[l], P.q_lat, md.rank, (long long)P.RPH * md.rank, P.q_rope, e->d_block_table,
@@ -694,14 +726,15 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
       n += 3 + (&P == &e->dec ? 0 : 1);               // beyond the count below: two grouped GEMMs, the split, and in prefill too a second attention kernel
     } else {
-    STAGE(launch_qkv_post(P.p_qkv.out(), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
+    STAGE(launch_qkv_post(qkv, rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
     // (the decode kernel takes the one-box-per-tile view of the pages, the prefill kernel the row view)
     STAGE(launch_attention(&P == &e->dec ? e->tm_k4[l] : e->tm_k[l], &P == &e->dec ? e->tm_k4[l] : e->tm_v[l], P.q, rows, s.n_q_heads, kv, l, e->max_splits, P.att_work, P.att_n_work,
                            e->num_sms, P.part_acc, P.part_ml, P.att_pool + l, P.ao_hi, P.ao_lo, &P == &e->dec ? (e->whole_pairs ? 2 : 0) : 1,
                            e->d_status, e->st));
     }
-    STAGE(gemm_launch(P.p_o, &e->tm_o[l], e->d_status, e->st, tr(4 * l + 1), true));
-    GemmOut o = P.p_o.out();
+    if (P.wide) STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
+    else STAGE(gemm_launch(P.p_o, &e->tm_o[l], e->d_status, e->st, tr(4 * l + 1), true));
+    GemmOut o = P.wide ? gemm_pair_out(P.b_o, P.R, P.plain_tiles) : P.p_o.out();
     STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
     if (dense_layer(e, l)) {
       STAGE(gemm_launch(P.p_gu_d, &e->tm_gu_d[l], e->d_status, e->st, nullptr, true));
@@ -750,6 +783,11 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         STAGE(launch_moe_swiglu(P.p_gu.out(), P.moe_w, P.R, e->moe_F, e->moe_E + e->moe_S, P.ff_hi, P.ff_lo, e->st));
         n += 1;
       }
+    } else if (P.wide) {
+      STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st, &e->tb_gu96[l]));
+      STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st));
+      n += 9;
+      continue;
     } else {
       if (P.p_gu.sw_hi) {                             // SwiGLU in the GEMM's epilogue
         STAGE(gemm_launch(P.p_gu, &e->tm_gu_half[l], e->d_status, e->st, tr(4 * l + 2), true));
@@ -771,6 +809,17 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
   return CORUN_OK;
 }
 
+int launch_lm_head(corun_engine *e, const Program &P) {
+  if (P.wide) {
+    CK(gemm_pair_launch(P.b_lm, e->tb_lm, P.R, e->d_status, e->st));
+    CK(gemm_pair_fixup_launch(P.b_lm, P.R, e->st));
+  } else {
+    CK(gemm_launch(P.p_lm, nullptr, e->d_status, e->st, nullptr, true));
+    CK(gemm_fixup_launch(P.p_lm, e->st, true));
+  }
+  return CORUN_OK;
+}
+
 // One decode iteration on the stream (what the graph captures).
 int enqueue_decode_body(corun_engine *e, int *launches) {
   Program &P = e->dec;
@@ -787,13 +836,12 @@ int enqueue_decode_body(corun_engine *e, int *launches) {
     const Rows rows{P.row_token, P.row_pos, P.row_active, P.row_slot, P.R};
     GemmOut prev = ffn_out(e, P, s.n_layers - 1);
     CK(launch_resid_norm(P.h, s.hidden, nullptr, rows, &prev, e->final_norm, s.rms_eps, P.xn_hi, P.xn_lo, e->st));
-    CK(gemm_launch(P.p_lm, nullptr, e->d_status, e->st, nullptr, true));
-    CK(gemm_fixup_launch(P.p_lm, e->st, true));
+    RC(launch_lm_head(e, P));
     SampleArgs sa{P.logits, s.vocab, P.do_sample, P.row_temp, P.row_top_p, e->d_seeds, P.row_step, nullptr, P.sampled};   // all by row
     CK(launch_sampler(sa, P.R, e->st, true));
     CK(launch_advance(P.slot_row, P.row_active, P.sampled, e->B, e->d_ctx, e->d_step, e->d_pending, e->h_out_tokens, e->d_status, e->h_status,
                       e->st));
-    n += 4 + (P.p_lm.n_split_tiles ? 1 : 0);
+    n += 4 + (P.wide ? gemm_pair_has_parts(P.b_lm, P.R) : P.p_lm.n_split_tiles ? 1 : 0);
   }
   if (e->eager && e->stop_after >= 0)            // (debug) no last kernel ran: fetch the status word the plain way
     CK(cudaMemcpyAsync(e->h_status, e->d_status, sizeof(int), cudaMemcpyDeviceToHost, e->st));
@@ -989,6 +1037,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG
   const long long big_rows = (long long)B * ((max_context + 127) / 128 * 128);
   const int big_cap = !big_ok ? 0 : big_rows < PREFILL_BIG ? (int)((big_rows + 255) / 256 * 256) : PREFILL_BIG;
+  const bool wide = pad16(B) > 128;                 // decode on pairs of SMs (Program::wide)
+  if (wide && gemm_encode_map(&e->tb_lm, w->lm_head, s.vocab, H, 128)) return fail(CORUN_EINVAL);
   e->tm_qkv.resize(s.n_layers);
   e->tm_o.resize(s.n_layers);
   e->tm_gu.resize(s.n_layers);
@@ -1002,7 +1052,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     const int qkv_rows = mla ? s.n_q_heads * (mla->qk_nope + mla->qk_rope) + mla->kv_lora_rank + mla->qk_rope : QD + 2 * KD;
     if ((rc = gemm_encode_map(&e->tm_qkv[l], w->wqkv[l], qkv_rows, H, GEMM_TILE_N))) return fail(rc);
     if ((rc = gemm_encode_map(&e->tm_o[l], w->wo[l], H, QD, GEMM_TILE_N))) return fail(rc);
-    if (big_cap) {                                  // the program of many rows
+    if (big_cap || wide) {                          // the programs of many rows
       if (e->tb_qkv.empty())
         for (auto *v : {&e->tb_qkv, &e->tb_o, &e->tb_gu, &e->tb_down, &e->tb_router, &e->tb_gu_half, &e->tb_gu96}) v->resize(s.n_layers);
       const bool experts = moe && l >= first_dense;
@@ -1153,6 +1203,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   if ((rc = program_create(e, e->dec, B, true, true, dec_grouped, true))) return fail(rc);
   // the decode step's first kernel says which blocks of rows hold a request (64 rows each up to 128 padded rows, 128
   // rows each above); the GEMMs leave the others out (the one-row program has one block)
+  for (GemmPairPlan *pl : {&e->dec.b_qkv, &e->dec.b_o, &e->dec.b_gu, &e->dec.b_down, &e->dec.b_lm}) pl->row_blocks = e->dec.row_blocks;
   for (GemmPlan *pl : {&e->dec.p_qkv, &e->dec.p_o, &e->dec.p_gu, &e->dec.p_down, &e->dec.p_lm, &e->dec.p_gu_d, &e->dec.p_down_d})
     pl->row_blocks = e->dec.row_blocks;
   if (!big_cap && (rc = program_create(e, e->pre, e->chunk, true, false, e->moe_E > 0 && !getenv("CORUN_MOE_PREFILL_DENSE")))) return fail(rc);
@@ -1661,14 +1712,17 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
                             (long long)e->pool_blocks, e->kv_run};
       switch (kind) {
         // launched as in the step's graph: with programmatic stream serialization
-        case 0: ce = gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, nullptr, true); break;
-        case 1: ce = gemm_launch(P.p_o, &e->tm_o[l], e->d_status, e->st, nullptr, true); break;
+        case 0: if (P.wide) { ce = gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st); break; }
+                ce = gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, nullptr, true); break;
+        case 1: if (P.wide) { ce = gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st); break; }
+                ce = gemm_launch(P.p_o, &e->tm_o[l], e->d_status, e->st, nullptr, true); break;
         case 2: if ((P.grouped || P.select) && !dense_layer(e, l)) {   // the groups of the last step's last layer
                   ce = gemm_launch(P.p_gug, P.p_gug.sw_hi ? &e->tm_gu_half[l] : &e->tm_gu[l], e->d_status, e->st, nullptr, true);
                   if (ce == cudaSuccess && !P.p_gug.sw_hi)
                     ce = launch_moe_swiglu_grouped(P.gug_out, P.moe_w, e->moe_E + e->moe_S, e->moe_F, P.grp, P.hg_hi, P.hg_lo, e->st);
                   break;
                 }
+                if (P.wide && !e->moe_E) { ce = gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st, &e->tb_gu96[l]); break; }
                 ce = gemm_launch(P.p_gu, P.p_gu.sw_hi ? &e->tm_gu_half[l] : &e->tm_gu[l], e->d_status, e->st, nullptr, true); break;
         case 3: if (P.select && !dense_layer(e, l)) {    // down GEMM per selected expert + the sum over a row's experts
                   ce = gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true);
@@ -1680,9 +1734,9 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
                   if (ce == cudaSuccess) ce = launch_moe_combine(P.yg_out, P.row_active, P.R, e->moe_E + e->moe_S, s.hidden, P.grp, P.down_out, e->st);
                   break;
                 }
+                if (P.wide && !e->moe_E) { ce = gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st); break; }
                 ce = gemm_launch(P.p_down, &e->tm_down[l], e->d_status, e->st, nullptr, true); break;
-        case 4: ce = gemm_launch(P.p_lm, nullptr, e->d_status, e->st, nullptr, true);
-                if (ce == cudaSuccess) ce = gemm_fixup_launch(P.p_lm, e->st);
+        case 4: ce = launch_lm_head(e, P) == CORUN_OK ? cudaSuccess : cudaErrorUnknown;
                 break;
         case 5: if (e->mla) {
                   ce = launch_mla_attention(e->tm_c[l], e->tm_cv[l], P.q_lat, e->md.rank, (long long)P.RPH * e->md.rank, P.q_rope,
@@ -1700,12 +1754,12 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
         case 6: ce = launch_resid_norm(P.h, s.hidden, nullptr, rows, &prev, e->attn_norm[l], s.rms_eps, P.xn_hi,
                                        P.xn_lo, e->st); break;
         case 7: if (e->mla) {   // (re-appends the rows' current positions: the same values)
-                  ce = launch_mla_post(P.p_qkv.out(), rows, e->d_rope, e->md, e->kv_norm[l], s.rms_eps, mcache, P.RPH, P.qn_hi, P.qn_lo,
+                  ce = launch_mla_post(P.wide ? gemm_pair_out(P.b_qkv, P.R, P.plain_tiles) : P.p_qkv.out(), rows, e->d_rope, e->md, e->kv_norm[l], s.rms_eps, mcache, P.RPH, P.qn_hi, P.qn_lo,
                                        P.q_rope, e->d_status, e->st);
                   break;
                 }
-                ce = launch_qkv_post(P.p_qkv.out(), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st); break;
-        case 8: if (P.p_gu.sw_hi || P.grouped || P.select) break;   // no such kernel: the SwiGLU is in the GEMM's epilogue (grouped form: timed with kind 2)
+                ce = launch_qkv_post(P.wide ? gemm_pair_out(P.b_qkv, P.R, P.plain_tiles) : P.p_qkv.out(), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st); break;
+        case 8: if (P.p_gu.sw_hi || P.grouped || P.select || (P.wide && !e->moe_E)) break;   // no such kernel: the SwiGLU is in the GEMM's epilogue (grouped form: timed with kind 2)
                 ce = e->moe_E ? launch_moe_swiglu(P.p_gu.out(), P.moe_w, P.R, e->moe_F, e->moe_E + e->moe_S, P.ff_hi, P.ff_lo, e->st)
                               : launch_swiglu(P.p_gu.out(), P.R, s.ffn, P.ff_hi, P.ff_lo, e->st);
                 break;

@@ -34,25 +34,30 @@ struct GemmOut {
   const int *tile_cend;  // [n_tiles] last CTA touching the tile (every later CTA used slot 0)
   int N, KB, BN;
   // Result of gemm_pair.cu (row_tiles > 0): tiles [256 rows x 256 columns], row tiles fastest; the first `whole` are in
-  // `direct`, the others in `ws`, `slices` partial matrices [BN, N] behind one another.
+  // `direct`, the others in `ws`, tile after tile as `slices` partial tiles [256][256].
   int row_tiles, whole, slices;
 };
 
 // Values of a gemm_pair.cu result, the slices added in ascending order.
+__device__ __forceinline__ const float *gemm_pair_at(const GemmOut &g, int tile, int r, int n) {
+  return g.ws + ((size_t)(tile - g.whole) * g.slices * 256 + (r & 255)) * GEMM_TILE_N + n % GEMM_TILE_N;
+}
 __device__ __forceinline__ float gemm_load_pair(const GemmOut &g, int r, int n) {
-  const size_t o = (size_t)r * g.N + n;
-  if ((n / GEMM_TILE_N) * g.row_tiles + r / 256 < g.whole) return g.direct[o];
-  float acc = g.ws[o];
-  for (int s = 1; s < g.slices; ++s) acc += g.ws[(size_t)s * g.BN * g.N + o];
+  const int tile = (n / GEMM_TILE_N) * g.row_tiles + r / 256;
+  if (tile < g.whole) return g.direct[(size_t)r * g.N + n];
+  const float *p = gemm_pair_at(g, tile, r, n);
+  float acc = p[0];
+  for (int s = 1; s < g.slices; ++s) acc += p[(size_t)s * 256 * GEMM_TILE_N];
   return acc;
 }
 __device__ __forceinline__ float4 gemm_load_pair4(const GemmOut &g, int r, int n) {
-  const size_t o = (size_t)r * g.N + n;
-  if ((n / GEMM_TILE_N) * g.row_tiles + r / 256 < g.whole) return *reinterpret_cast<const float4 *>(g.direct + o);
+  const int tile = (n / GEMM_TILE_N) * g.row_tiles + r / 256;
+  if (tile < g.whole) return *reinterpret_cast<const float4 *>(g.direct + (size_t)r * g.N + n);
+  const float *p = gemm_pair_at(g, tile, r, n);
   float4 v[8];                                      // at most eight slices, all requested together
 #pragma unroll
   for (int s = 0; s < 8; ++s)
-    if (s < g.slices) v[s] = *reinterpret_cast<const float4 *>(g.ws + (size_t)s * g.BN * g.N + o);
+    if (s < g.slices) v[s] = *reinterpret_cast<const float4 *>(p + (size_t)s * 256 * GEMM_TILE_N);
   float4 acc = v[0];
 #pragma unroll
   for (int s = 1; s < 8; ++s)
@@ -215,13 +220,18 @@ struct GemmPairPlan {
   int slices = 1;                    // cuts of K (gemm_pair_slices)
   bool swiglu = false;
   float *out = nullptr, *part = nullptr;   // not owned
+  const int *row_blocks = nullptr;   // device, not owned (cap 256): bit 1 = rows 128 .. hold a request; null = they do
 };
 // Into how many slices K is cut: a function of the matrix and the GPU, never of the rows.
 int gemm_pair_slices(int N, int K, int num_sms);
+// Floats of partial tiles that launches over up to cap rows leave (the next kernel of the stream consumes them, so one
+// buffer serves all plans of a program).
+size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms);
 // X W^T for activations Xhi / Xlo [cap, K] (N % 8 == 0) -> out [cap, N] fp32 and, for the tiles of an unfilled wave, part
-// [slices][cap][N] (null: one slice).  Read through gemm_pair_out(p, R, zeros).
+// (gemm_pair_part_floats; null: one slice).  Read through gemm_pair_out(p, R, zeros).
 int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms);
 GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles);
+int gemm_pair_has_parts(const GemmPairPlan &p, int R);   // 1 if some of the result of R rows is left in partial matrices
 cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st);   // makes `out` a plain matrix
 // W is [2F, K] (F gate rows, then F up rows; F % 8 == 0): out_hi / out_lo [cap, F] = silu(gate) * up as a bf16 hi/lo pair.
 int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,

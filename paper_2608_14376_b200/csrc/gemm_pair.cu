@@ -48,7 +48,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                  const __grid_constant__ CUtensorMap tmLo, const __grid_constant__ CUtensorMap tmOut,
                  const __grid_constant__ CUtensorMap tmOut2, int R, int N, int KB, int row_tiles, int whole, int units, int slices,
-                 int half, int cap, int *status) {
+                 int half, int *status, const int *row_blocks) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[PG_STAGES];      // used in the first CTA: both CTAs' loads of a stage
   __shared__ __align__(8) uint64_t empty_bar[PG_STAGES];     // in each CTA: the MMAs have read the stage
@@ -62,6 +62,17 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
+  // (decode) the step's requests are in the first rows: without one in rows 128 .. the second CTA's activations are zeros,
+  // neither loaded nor stored (200 against 100 requests in 256 rows: what is saved is L2 traffic and power)
+  const bool upper = !row_blocks || (*reinterpret_cast<const volatile int *>(row_blocks) & 2);
+  if (!upper && R > 128) R = 128;
+  if (!upper && rank == 1) {
+    for (int s = 0; s < PG_STAGES; ++s) {
+      uint4 *z = reinterpret_cast<uint4 *>(smem_raw + (base - smem_u32(smem_raw)) + s * PG_STAGE_BYTES);
+      for (uint32_t i = threadIdx.x; i < 2 * PG_X_BYTES / 16; i += PG_THREADS) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    fence_proxy_async();
+  }
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < PG_STAGES; ++s) {
@@ -103,7 +114,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       // ---------------- TMA producer (both CTAs; the bytes count on the first CTA's barrier) ----------------
       const uint64_t pol_w = l2_policy_evict_first();        // a weight tile is used by the row tiles that run now
       const uint64_t pol_x = l2_policy_evict_last();
-      const uint32_t stage_tx = 2u * (2 * PG_X_BYTES + (uint32_t)half * 128u);
+      const uint32_t stage_tx = 2u * (uint32_t)half * 128u + (upper ? 2u : 1u) * 2u * PG_X_BYTES;
       int it = 0;
       for (int u = pair; u < units && !fail; u += n_pairs) {
         const Unit un = unit(u);
@@ -120,8 +131,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           if (rank == 0) mbar_arrive_expect_tx(fb, stage_tx);
           const uint32_t fb0 = cluster_map(fb, 0);
           tma_load_2d_pair(dst + 2 * PG_X_BYTES, &tmW, kb * GEMM_BLOCK_K, yw, fb0, pol_w);
-          tma_load_2d_pair(dst, &tmHi, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
-          tma_load_2d_pair(dst + PG_X_BYTES, &tmLo, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
+          if (rank == 0 || upper) {
+            tma_load_2d_pair(dst, &tmHi, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
+            tma_load_2d_pair(dst + PG_X_BYTES, &tmLo, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
+          }
         }
       }
       // every stage's last release has arrived before this CTA may end: an arrival of the pair's MMAs must not find the
@@ -234,7 +247,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       if (!SWIGLU && ok && row0 < R) {
         // a whole tile goes to the output, a slice to its partial matrix
         const bool part = u >= whole;
-        const int y = part ? un.s0 * cap + row0 : row0;
+        const int y = part ? ((un.tile - whole) * slices + un.s0) * 256 + rank * 128 + lane_base : row0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int col = nt * GEMM_TILE_N + grp * 128 + q * 32;
@@ -248,7 +261,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) {
-              tma_store_2d(part ? &tmOut2 : &tmOut, stg, col, y);
+              tma_store_2d(part ? &tmOut2 : &tmOut, stg, part ? grp * 128 + q * 32 : col, y);
               bulk_commit();
             }
           }
@@ -323,6 +336,19 @@ int gemm_pair_slices(int N, int K, int num_sms) {
   return s;
 }
 
+size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms) {
+  GemmPairPlan p;
+  p.N = N; p.K = K; p.cap = cap; p.pairs = num_sms / 2;
+  p.n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N;
+  p.slices = gemm_pair_slices(N, K, num_sms);
+  int most = 1;
+  for (int R = 256; R < cap + 256; R += 256) {
+    const PairShape q = pair_shape(p, R, false);
+    if (q.units - q.whole > most) most = q.units - q.whole;
+  }
+  return (size_t)most * 256 * GEMM_TILE_N;
+}
+
 int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms) {
   if (N <= 0 || N % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out || num_sms < 2) return CORUN_EINVAL;
   p->N = N; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = false; p->out = out; p->part = part;
@@ -332,7 +358,7 @@ int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const 
   if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
   if ((rc = tma_encode_store_2d(&p->tmOut, out, 1, cap, N)) != 0) return rc;
   if (p->slices > 1) {
-    if ((rc = tma_encode_store_2d(&p->tmOut2, part, 1, (unsigned long long)p->slices * cap, N)) != 0) return rc;
+    if ((rc = tma_encode_store_2d(&p->tmOut2, part, 1, gemm_pair_part_floats(N, K, cap, num_sms) / GEMM_TILE_N, GEMM_TILE_N)) != 0) return rc;
   } else {
     p->tmOut2 = p->tmOut;
   }
@@ -346,6 +372,11 @@ GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles) {
   g.whole = q.whole;
   g.slices = p.slices;
   return g;
+}
+
+int gemm_pair_has_parts(const GemmPairPlan &p, int R) {
+  const PairShape q = pair_shape(p, R, false);
+  return q.whole < q.row_tiles * p.n_tiles ? 1 : 0;
 }
 
 cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st) {
@@ -382,7 +413,7 @@ cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int 
   const int pairs = q.units < p.pairs ? q.units : p.pairs;
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, q.half == 96 ? *tmW96 : tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2,
-                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, q.half, p.cap, d_status);
+                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, q.half, d_status, p.row_blocks);
   };
   return p.swiglu ? go(gemm_pair_kernel<true>) : go(gemm_pair_kernel<false>);
 }
