@@ -1,0 +1,363 @@
+// Causal attention of a prefill chunk of a decoder with multi-head latent attention: the chunk's rows are consecutive
+// tokens, so the heads' keys and values are decompressed once per cached token (one GEMM over the latents) and a tile of
+// 128 query tokens shares every key / value tile.  The decode form (absorbed, one query token at a time over the latents)
+// does 2176 multiply-adds per query, key and head and streams a request's whole latent cache once per token: 118 us per
+// 256 tokens of a chunk; here it is 960, and the cache is read once per chunk.
+//
+// The cached latents are fp16 and enter the GEMM exactly (bf16 hi + lo); its fp32 results are kept as fp16 hi + lo pairs,
+// queries and weights are hi + lo pairs too, and of the products only lo * lo is left out.
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <math_constants.h>
+
+#include "launch.cuh"
+#include "mla.cuh"
+#include "ptx.cuh"
+
+namespace corun {
+
+namespace {
+
+constexpr int ML_THREADS = 320;                     // warp 0 TMA, warp 1 MMA, warps 2-5 softmax, warps 6-9 output
+constexpr int ML_KEYS = 64;                         // keys per block
+constexpr uint32_t ML_BOX = ML_KEYS * 128;          // [64 tokens x 64 dims] fp16
+constexpr uint32_t ML_Q_BYTES = 3 * 128 * 128;      // hi or lo: [3 blocks of 64 dims][128 rows x 128 B]
+constexpr uint32_t ML_K_BYTES = 5 * ML_BOX;         // hi, lo of the 128 no-rope dims, the rotary key
+constexpr uint32_t ML_V_BYTES = 4 * ML_BOX;         // hi, lo
+constexpr uint32_t ML_P_BYTES = 128 * 128;          // hi or lo of a weight tile [128 rows x 64 keys]
+constexpr size_t ML_SMEM = 1024 + 2 * ML_Q_BYTES + ML_K_BYTES + ML_V_BYTES + 2 * ML_P_BYTES;
+
+__device__ __forceinline__ uint32_t ml_swz(int row, int chunk) { return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4)); }
+__device__ __forceinline__ float ml_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// eight fp32 -> fp16 hi and lo parts, 16 bytes each
+__device__ __forceinline__ void ml_split8(const float *x, uint4 &hi, uint4 &lo) {
+  __half2 h[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    h[i] = __floats2half2_rn(x[2 * i], x[2 * i + 1]);
+    const float2 f = __half22float2(h[i]);
+    l[i] = __floats2half2_rn(x[2 * i] - f.x, x[2 * i + 1] - f.y);
+  }
+  hi = *reinterpret_cast<const uint4 *>(h);
+  lo = *reinterpret_cast<const uint4 *>(l);
+}
+
+// The latents of the segments' cached tokens as a bf16 hi / lo pair (exact) and their rotary keys (fp16), one warp per token.
+__global__ void __launch_bounds__(256)
+mla_gather_kernel(const __grid_constant__ MlaSegs g, MlaCache cache, int rank, int rope, int total, __nv_bfloat16 *__restrict__ c_hi,
+                  __nv_bfloat16 *__restrict__ c_lo, __half *__restrict__ kr) {
+  griddep_launch_dependents();
+  griddep_wait();
+  const int t = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (t >= total) return;
+  int s = 0;
+  while (s + 1 < g.n && t >= g.off[s + 1]) ++s;
+  const int pos = t - g.off[s];
+  if (pos >= g.len[s]) return;                      // the rest of a segment's last block: never weighted
+  const int blk = cache.block_table[(size_t)g.slot[s] * cache.max_blocks + pos / KV_BLOCK];
+  for (int c = lane; c < (rank + rope) / 8; c += 32) {
+    const uint4 raw = *reinterpret_cast<const uint4 *>(mla_cache_at(cache, rank + rope, blk, pos % KV_BLOCK, 8 * c));
+    if (8 * c >= rank) {
+      *reinterpret_cast<uint4 *>(kr + (size_t)t * 64 + 8 * c - rank) = raw;
+      continue;
+    }
+    const __half *x = reinterpret_cast<const __half *>(&raw);
+    __nv_bfloat16 a[8], b[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float v = __half2float(x[i]);
+      a[i] = __float2bfloat16_rn(v);
+      b[i] = __float2bfloat16_rn(v - __bfloat162float(a[i]));
+    }
+    *reinterpret_cast<uint4 *>(c_hi + (size_t)t * rank + 8 * c) = *reinterpret_cast<const uint4 *>(a);
+    *reinterpret_cast<uint4 *>(c_lo + (size_t)t * rank + 8 * c) = *reinterpret_cast<const uint4 *>(b);
+  }
+}
+
+// One CTA per (head, tile of 128 chunk rows = consecutive tokens of one request).  Per block of 64 keys:
+//   S[128 x 64] = Qhi Khi + Qlo Khi + Qhi Klo (12 k-slices) into one of two TMEM buffers;
+//   softmax warps, a thread per row: running maximum, P = exp2(S - max) as an fp16 hi / lo tile, the factor by which the
+//     earlier sums shrink;
+//   O'[128 x 128] = Phi Vhi + Plo Vhi + Phi Vlo (4 k-slices) into one of two TMEM buffers;
+//   output warps, a thread per row: O = O * factor + O', in registers.
+// The scores of block j + 1 are issued ahead of the values of block j, so the tensor cores work while the rows do.  What
+// bounds a CTA is the number of MMA instructions (44 per block) and, with one key buffer, the 40 KB of keys per block that
+// can only be requested once the scores before them are done.  Every reduction runs in one fixed order that depends on the
+// row's own position only.  All waits are bounded.
+__global__ void __launch_bounds__(ML_THREADS, 1)
+mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmR, const __nv_bfloat16 *__restrict__ qn_hi,
+                   const __nv_bfloat16 *__restrict__ qn_lo, const float *__restrict__ q_rope, Rows rows, int rows_per_head, int nh, int rope,
+                   int cap, const int *__restrict__ tile_base, float scale_log2e, __nv_bfloat16 *__restrict__ ao_hi,
+                   __nv_bfloat16 *__restrict__ ao_lo, int *status) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t kfull, kempty, vfull, vempty, s_full[2], s_free[2], p_ready, p_free, o_full[2], o_free[2], c_ready[4], l_ready;
+  __shared__ uint32_t tmem_base_s;
+  __shared__ int abort_flag;
+  __shared__ float corr_s[4][128], l_s[128];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int h = blockIdx.x, tile = (int)gridDim.y - 1 - (int)blockIdx.y;   // the last tiles (the most keys) first
+  const int row0 = tile * 128;
+  // the tile's rows with a token are the first ones
+  const int n_rows = __syncthreads_count(tid < 128 && row0 + tid < rows.R && rows.active[row0 + tid] != 0);
+  if (n_rows == 0) return;
+  const int n_blocks = rows.pos[row0 + n_rows - 1] / ML_KEYS + 1, base_tok = tile_base[tile];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
+  const uint32_t q_hi = base, q_lo = base + ML_Q_BYTES, k_buf = q_lo + ML_Q_BYTES, v_buf = k_buf + ML_K_BYTES, p_hi = v_buf + ML_V_BYTES,
+                 p_lo = p_hi + ML_P_BYTES;
+  if (tid == 0) {
+    abort_flag = 0;
+    mbar_init(smem_u32(&kfull), 1); mbar_init(smem_u32(&kempty), 1);
+    mbar_init(smem_u32(&vfull), 1); mbar_init(smem_u32(&vempty), 1);
+    mbar_init(smem_u32(&p_ready), 128); mbar_init(smem_u32(&p_free), 1);
+    mbar_init(smem_u32(&l_ready), 128);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&s_full[i]), 1); mbar_init(smem_u32(&s_free[i]), 128);
+      mbar_init(smem_u32(&o_full[i]), 1); mbar_init(smem_u32(&o_free[i]), 128);
+    }
+    for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&c_ready[i]), 128);
+    fence_mbar_init();
+    fence_proxy_async();
+    prefetch_tensormap(&tmKV);
+    prefetch_tensormap(&tmR);
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&tmem_base_s), 512);        // scores 2 x 64 columns, outputs 2 x 128
+    tmem_relinquish();
+  }
+  if (warp >= 2) {
+    // the query tile: row m = token m, 24 chunks of 8 dims (128 no-rope, then the rotary ones, zeros beyond them)
+    const int m = (tid - 64) & 127, r = row0 + m;
+    const bool on = r < rows.R;
+    for (int c = (tid - 64) >> 7; c < 24; c += 2) {
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = 0.f;
+      if (on && c < 16) {
+        const size_t o = ((size_t)h * rows_per_head + r) * 128 + 8 * c;
+        const uint4 a = *reinterpret_cast<const uint4 *>(qn_hi + o), b = *reinterpret_cast<const uint4 *>(qn_lo + o);
+        const __nv_bfloat16 *pa = reinterpret_cast<const __nv_bfloat16 *>(&a), *pb = reinterpret_cast<const __nv_bfloat16 *>(&b);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = __bfloat162float(pa[i]) + __bfloat162float(pb[i]);
+      } else if (on && 8 * (c - 16) < rope) {
+        const float *q = q_rope + ((size_t)r * nh + h) * rope + 8 * (c - 16);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = q[i];
+      }
+      uint4 hi, lo;
+      ml_split8(x, hi, lo);
+      const uint32_t off = (uint32_t)(c >> 3) * (128 * 128) + ml_swz(m, c & 7);
+      *reinterpret_cast<uint4 *>(base_ptr + off) = hi;
+      *reinterpret_cast<uint4 *>(base_ptr + ML_Q_BYTES + off) = lo;
+    }
+    fence_proxy_async();                            // the MMAs read these tiles through the async proxy
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base_s;
+  bool failed = false;
+  // warps 2-5 and 6-9: this thread's row
+  const int quad = warp & 3, tl = quad * 32 + lane;
+  const bool real = tl < n_rows;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------- TMA producer ----------------
+      const uint64_t pol = l2_policy_evict_last();  // the tiles of the same head read the same keys and values
+      for (int j = 0; j < n_blocks && !failed; ++j) {
+        const int tok = base_tok + j * ML_KEYS;
+        auto y = [&](int part) { return (part * nh + h) * cap + tok; };   // part: key hi, key lo, value hi, value lo
+        if (j > 0 && !mbar_wait(smem_u32(&kempty), (uint32_t)(j - 1) & 1u, &abort_flag)) { failed = true; break; }
+        mbar_arrive_expect_tx(smem_u32(&kfull), ML_K_BYTES);
+        for (int i = 0; i < 4; ++i)
+          tma_load_2d(k_buf + (uint32_t)i * ML_BOX, &tmKV, (i & 1) * 64, y(i >> 1), smem_u32(&kfull), pol);
+        tma_load_2d(k_buf + 4 * ML_BOX, &tmR, 0, tok, smem_u32(&kfull), pol);
+        if (j > 0 && !mbar_wait(smem_u32(&vempty), (uint32_t)(j - 1) & 1u, &abort_flag)) { failed = true; break; }
+        mbar_arrive_expect_tx(smem_u32(&vfull), ML_V_BYTES);
+        for (int i = 0; i < 4; ++i)
+          tma_load_2d(v_buf + (uint32_t)i * ML_BOX, &tmKV, (i & 1) * 64, y(2 + (i >> 1)), smem_u32(&vfull), pol);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---------------- MMA issuer ----------------
+      const uint32_t idesc_s = (1u << 4) | ((uint32_t)(ML_KEYS >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+      const uint32_t idesc_o = (1u << 4) | (1u << 16) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);   // values MN-major
+      for (int j = 0; j <= n_blocks && !failed; ++j) {
+        if (j < n_blocks) {
+          const int sb = j & 1;
+          if (j >= 2 && !mbar_wait(smem_u32(&s_free[sb]), (uint32_t)((j >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
+          if (!mbar_wait(smem_u32(&kfull), (uint32_t)j & 1u, &abort_flag)) { failed = true; break; }
+          tc_fence_after();
+          const uint32_t d = tmem + (uint32_t)sb * 64;
+#pragma unroll
+          for (int ks = 0; ks < 12; ++ks) {
+            const uint64_t adv = (uint64_t)((ks & 3) * 2);
+            const uint32_t b = (uint32_t)(ks >> 2);
+            const uint64_t qh = umma_desc_sw128(q_hi + b * (128 * 128)) + adv, ql = umma_desc_sw128(q_lo + b * (128 * 128)) + adv;
+            const uint64_t kh = umma_desc_sw128(k_buf + (ks < 8 ? b : 4u) * ML_BOX) + adv;
+            umma_bf16(d, qh, kh, idesc_s, ks > 0 ? 1u : 0u);   // operand format (fp16) is in idesc
+            umma_bf16(d, ql, kh, idesc_s, 1u);
+            if (ks < 8) umma_bf16(d, qh, umma_desc_sw128(k_buf + (2 + b) * ML_BOX) + adv, idesc_s, 1u);   // (the rotary key is fp16 as cached)
+          }
+          umma_commit(smem_u32(&kempty));
+          umma_commit(smem_u32(&s_full[sb]));
+        }
+        if (j >= 1) {
+          const int i = j - 1, ob = i & 1;
+          if (!mbar_wait(smem_u32(&p_ready), (uint32_t)i & 1u, &abort_flag)) { failed = true; break; }
+          if (!mbar_wait(smem_u32(&vfull), (uint32_t)i & 1u, &abort_flag)) { failed = true; break; }
+          if (i >= 2 && !mbar_wait(smem_u32(&o_free[ob]), (uint32_t)((i >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
+          tc_fence_after();
+          const uint32_t d = tmem + 128 + (uint32_t)ob * 128;
+#pragma unroll
+          for (int ks = 0; ks < ML_KEYS / 16; ++ks) {
+            const uint64_t ph = umma_desc_sw128(p_hi) + (uint64_t)(ks * 2), pl = umma_desc_sw128(p_lo) + (uint64_t)(ks * 2);
+            // values [128 dims x 16 tokens], MN-major: blocks of 64 dims a box apart, groups of 8 tokens 1 KiB apart
+            const uint64_t vh = umma_desc_sw128_mn(v_buf + (uint32_t)ks * 2048, ML_BOX, 1024u);
+            const uint64_t vl = umma_desc_sw128_mn(v_buf + 2 * ML_BOX + (uint32_t)ks * 2048, ML_BOX, 1024u);
+            umma_bf16(d, ph, vh, idesc_o, ks > 0 ? 1u : 0u);
+            umma_bf16(d, pl, vh, idesc_o, 1u);
+            umma_bf16(d, ph, vl, idesc_o, 1u);
+          }
+          umma_commit(smem_u32(&vempty));
+          umma_commit(smem_u32(&p_free));
+          umma_commit(smem_u32(&o_full[ob]));
+        }
+      }
+    }
+  } else if (warp < 6) {
+    // ---------------- softmax: one thread per row ----------------
+    const int pos = real ? rows.pos[row0 + tl] : -1;
+    float mx = -CUDART_INF_F, l = 0.f;
+    for (int j = 0; j < n_blocks; ++j) {
+      const int sb = j & 1;
+      bool ok = mbar_wait(smem_u32(&s_full[sb]), (uint32_t)(j >> 1) & 1u, &abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) { failed = true; break; }
+      tc_fence_after();
+      uint32_t sv[4][16];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(sb * 64 + 16 * x), sv[x]);
+      tmem_ld_wait();
+      tc_fence_before();
+      mbar_arrive(smem_u32(&s_free[sb]));
+      const int lim = pos - j * ML_KEYS;            // keys 0 .. lim of the block are visible
+      float bm = -CUDART_INF_F;
+      if (lim >= ML_KEYS - 1) {
+#pragma unroll
+        for (int i = 0; i < ML_KEYS; ++i) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale_log2e);
+      } else {
+#pragma unroll
+        for (int i = 0; i < ML_KEYS; ++i)
+          if (i <= lim) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale_log2e);
+      }
+      const float m_new = fmaxf(mx, bm), m_use = m_new == -CUDART_INF_F ? 0.f : m_new;   // (rows without a token: nothing visible)
+      const float corr = ml_ex2(mx - m_use);
+      mx = m_new;
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      float p[ML_KEYS];
+#pragma unroll
+      for (int i = 0; i < ML_KEYS; ++i) {
+        p[i] = i <= lim ? ml_ex2(fmaf(__uint_as_float(sv[i >> 4][i & 15]), scale_log2e, -m_use)) : 0.f;
+        acc[i & 3] += p[i];
+      }
+      l = l * corr + ((acc[0] + acc[1]) + (acc[2] + acc[3]));
+      corr_s[j & 3][tl] = corr;
+      if (j > 0) {
+        bool okp = mbar_wait(smem_u32(&p_free), (uint32_t)(j - 1) & 1u, &abort_flag);
+        okp = __all_sync(0xffffffffu, okp);
+        if (!okp) { failed = true; break; }
+      }
+      uint8_t *ph = base_ptr + (p_hi - base), *pl = base_ptr + (p_lo - base);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        uint4 hi, lo;
+        ml_split8(&p[8 * c], hi, lo);
+        *reinterpret_cast<uint4 *>(ph + ml_swz(tl, c)) = hi;
+        *reinterpret_cast<uint4 *>(pl + ml_swz(tl, c)) = lo;
+      }
+      fence_proxy_async();
+      mbar_arrive(smem_u32(&p_ready));
+      mbar_arrive(smem_u32(&c_ready[j & 3]));
+    }
+    l_s[tl] = l;
+    mbar_arrive(smem_u32(&l_ready));
+  } else {
+    // ---------------- output: one thread per row, 128 dims in registers ----------------
+    float o[128];
+#pragma unroll
+    for (int i = 0; i < 128; ++i) o[i] = 0.f;
+    for (int j = 0; j < n_blocks; ++j) {
+      const int ob = j & 1;
+      bool ok = mbar_wait(smem_u32(&c_ready[j & 3]), (uint32_t)(j >> 2) & 1u, &abort_flag);
+      ok = ok && mbar_wait(smem_u32(&o_full[ob]), (uint32_t)(j >> 1) & 1u, &abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) { failed = true; break; }
+      const float corr = corr_s[j & 3][tl];
+      tc_fence_after();
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        uint32_t v[8];
+        tmem_ld8(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(128 + ob * 128 + 8 * q), v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[8 * q + i] = fmaf(o[8 * q + i], corr, __uint_as_float(v[i]));
+      }
+      tc_fence_before();
+      mbar_arrive(smem_u32(&o_free[ob]));
+    }
+    bool ok = !failed && mbar_wait(smem_u32(&l_ready), 0u, &abort_flag);
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok && real) {
+      const float inv = 1.f / l_s[tl];
+      const size_t at = ((size_t)(row0 + tl) * nh + h) * 128;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        __nv_bfloat16 a[8], b[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float y = o[8 * q + i] * inv;
+          a[i] = __float2bfloat16_rn(y);
+          b[i] = __float2bfloat16_rn(y - __bfloat162float(a[i]));
+        }
+        *reinterpret_cast<uint4 *>(ao_hi + at + 8 * q) = *reinterpret_cast<const uint4 *>(a);
+        *reinterpret_cast<uint4 *>(ao_lo + at + 8 * q) = *reinterpret_cast<const uint4 *>(b);
+      }
+    }
+  }
+  __syncwarp();
+  if (failed || abort_flag) {
+    if (lane == 0) atomicCAS(status, 0, DEV_TIMEOUT_EPILOGUE);
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let copies in flight land before the CTA retires
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc(tmem, 512);
+}
+
+}  // namespace
+
+cudaError_t launch_mla_gather(const MlaSegs &g, const MlaCache &cache, int rank, int rope, int total, __nv_bfloat16 *c_hi,
+                              __nv_bfloat16 *c_lo, __half *kr, cudaStream_t st) {
+  return launch_k(mla_gather_kernel, dim3((total + 7) / 8), dim3(256), 0, st, true, g, cache, rank, rope, total, c_hi, c_lo, kr);
+}
+
+cudaError_t mla_prefill_prepare() {
+  return cudaFuncSetAttribute(mla_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ML_SMEM);
+}
+
+cudaError_t launch_mla_prefill(const CUtensorMap &tmKV, const CUtensorMap &tmR, const __nv_bfloat16 *qn_hi, const __nv_bfloat16 *qn_lo,
+                               const float *q_rope, const Rows &rows, int rows_per_head, const MlaDims &d, int cap, const int *tile_base,
+                               float scale, __nv_bfloat16 *ao_hi, __nv_bfloat16 *ao_lo, int *d_status, cudaStream_t st) {
+  return launch_k(mla_prefill_kernel, dim3(d.nh, (rows.R + 127) / 128), dim3(ML_THREADS), ML_SMEM, st, false, tmKV, tmR, qn_hi, qn_lo, q_rope,
+                  rows, rows_per_head, d.nh, d.rope, cap, tile_base, scale * 1.4426950408889634f, ao_hi, ao_lo, d_status);
+}
+
+}  // namespace corun

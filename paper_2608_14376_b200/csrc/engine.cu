@@ -108,6 +108,16 @@ struct Program {
   std::vector<GemmPlan> s_qkv, s_o, s_gu, s_down;
   GemmPairPlan b_qkv, b_o, b_gu, b_down, b_router;
   float *router_out = nullptr, *pair_part = nullptr;
+  // Latent attention of long prompts over decompressed keys and values (attention_prefill_mla.cu): the gathered latents of
+  // the chunk's requests, up to kv_cap tokens, their keys and values, and the chunk's segments
+  bool mla_tiles = false;
+  int kv_cap = 0, kv_tokens = 0;
+  GemmPairPlan b_kv;
+  bf16 *c_hi = nullptr, *c_lo = nullptr;
+  __half *kr = nullptr, *kvd = nullptr;
+  int *tile_base = nullptr;
+  CUtensorMap tm_kvd, tm_kr;
+  MlaSegs segs{};
   uint32_t *moe_mask = nullptr;
   DevMem allocs;
 };
@@ -136,7 +146,7 @@ struct corun_engine {
   const bf16 *embed = nullptr, *lm_head = nullptr, *final_norm = nullptr;
   std::vector<const bf16 *> attn_norm, mlp_norm;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
-  std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down, tb_router, tb_gu96;   // boxes of 128 rows (96): the GEMMs on pairs of SMs
+  std::vector<CUtensorMap> tb_qkv, tb_o, tb_gu, tb_down, tb_router, tb_gu96, tb_uv;   // boxes of 128 rows (96): the GEMMs on pairs of SMs
   CUtensorMap tb_lm;
   std::vector<CUtensorMap> tb_gu_half;     // dense layers of a decoder with expert layers: the box of the GEMM with SwiGLU
   std::vector<CUtensorMap> tm_gu_half;     // dense gate / up matrices with the box of the GEMM with SwiGLU in its epilogue
@@ -150,6 +160,7 @@ struct corun_engine {
   bool mla = false;
   MlaDims md{};
   int first_dense = 0, dense_ffn = 0, mla_splits = 0;
+  bool big_mla_tiles = false;            // Program::mla_tiles of the prefill program
   std::vector<const bf16 *> kv_norm;
   bf16 *w_ukT = nullptr;                 // [L][nh * rank][nope]: the key up-projections transposed
   std::vector<CUtensorMap> tm_uk, tm_uv, tm_c, tm_cv, tm_gu_d, tm_down_d;
@@ -531,6 +542,21 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
                                 64, P.q_lat, P.tab_uk, e->num_sms));
     RC(gemm_plan_create_grouped(&P.p_uv, e->w0_uv, (long long)md.nh * (md.nope + md.vh), md.rank, md.nope + md.vh, md.rank, P.ol_hi,
                                 P.ol_lo, n_groups, 64, P.uv_out, P.tab_uv, e->num_sms));
+    if (e->big_mla_tiles) {
+      P.mla_tiles = true;
+      // at most one request of a chunk began in an earlier one: the others' tokens are rows of the chunk
+      P.kv_cap = (e->max_ctx + cap + 64 * MLA_MAX_SEGS + 255) / 256 * 256;
+      const size_t kc = (size_t)P.kv_cap;
+      RC(dmalloc(A, &P.c_hi, kc * md.rank));
+      RC(dmalloc(A, &P.c_lo, kc * md.rank));
+      RC(dmalloc(A, &P.kr, kc * 64));               // zeros beyond rope, and finite everywhere: masked keys have weight zero
+      RC(dmalloc(A, &P.kvd, 4 * kc * md.nh * 128));
+      RC(dmalloc(A, &P.tile_base, (size_t)cap / 128));
+      RC(gemm_pair_plan_create_kv(&P.b_kv, md.nh, md.rank, P.c_hi, P.c_lo, P.kv_cap, P.kvd, e->num_sms));
+      RC(tma_encode_2d(&P.tm_kvd, P.kvd, 1, 4 * kc * md.nh, 128, 64, 64));
+      RC(tma_encode_2d(&P.tm_kr, P.kr, 1, kc, 64, 64, 64));
+      if (mla_prefill_prepare() != cudaSuccess) return CORUN_ECUDA;
+    }
     P.p_uk.keep_div = P.p_uv.keep_div = -1;         // the tables are copied ahead of a chunk's kernels (set_mla_rows)
   }
   if (e->moe_E) {
@@ -647,6 +673,12 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
           STAGE(launch_mla_post(P.s_qkv[b].out(), block_rows(b), e->d_rope, md, e->kv_norm[l], s.rms_eps, cache, P.RPH, P.qn_hi + r0 * md.nope,
                                 P.qn_lo + r0 * md.nope, P.q_rope + r0 * md.nh * md.rope, e->d_status, e->st));
         }
+        if (P.mla_tiles && !P.shorts) {
+          STAGE(launch_mla_gather(P.segs, cache, md.rank, md.rope, P.kv_tokens, P.c_hi, P.c_lo, P.kr, e->st));
+          STAGE(gemm_pair_launch(P.b_kv, e->tb_uv[l], P.kv_tokens, e->d_status, e->st));
+          STAGE(launch_mla_prefill(P.tm_kvd, P.tm_kr, P.qn_hi, P.qn_lo, P.q_rope, rows, P.RPH, md, P.kv_cap, P.tile_base,
+                                   1.0f / sqrtf((float)(md.nope + md.rope)), P.ao_hi, P.ao_lo, e->d_status, e->st));
+        } else {
         STAGE(gemm_launch(P.p_uk, &e->tm_uk[l], e->d_status, e->st, nullptr, true));
         for (int r0 = 0; r0 < P.R; r0 += MLA_ROWS) {
           const int nr = P.R - r0 < MLA_ROWS ? P.R - r0 : MLA_ROWS;
@@ -659,6 +691,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         }
         STAGE(gemm_launch(P.p_uv, &e->tm_uv[l], e->d_status, e->st, nullptr, true));
         STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
+        }
       } else {
         if (!P.shorts) STAGE(launch_qkv_post(gemm_pair_out(P.b_qkv, P.R, P.plain_tiles), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
         for (int b = 0; b < n_blk; ++b) {
@@ -1085,12 +1118,16 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     if ((rc = dmalloc(e->allocs, &e->w_ukT, per_layer * s.n_layers, false))) return fail(rc);
     e->tm_uk.resize(s.n_layers);
     e->tm_uv.resize(s.n_layers);
+    // (contexts beyond 16384 would need more than half a GB of decompressed keys and values: the decode form serves them)
+    e->big_mla_tiles = big_cap > 0 && md.nope == 128 && md.vh == 128 && max_context <= 16384;
+    if (e->big_mla_tiles) e->tb_uv.resize(s.n_layers);
     for (int l = 0; l < s.n_layers; ++l) {
       e->kv_norm.push_back((const bf16 *)mla->kv_norm[l]);
       bf16 *dst = e->w_ukT + (size_t)l * per_layer;
       if (launch_mla_transpose_uk((const bf16 *)mla->wkv_b[l], md, dst, 0) != cudaSuccess) return fail(CORUN_ECUDA);
       if ((rc = gemm_encode_map(&e->tm_uk[l], dst, md.nh * md.rank, md.nope, GEMM_TILE_N))) return fail(rc);
       if ((rc = gemm_encode_map(&e->tm_uv[l], mla->wkv_b[l], md.nh * (md.nope + md.vh), md.rank, GEMM_TILE_N))) return fail(rc);
+      if (e->big_mla_tiles && (rc = gemm_encode_map(&e->tb_uv[l], mla->wkv_b[l], md.nh * 256, md.rank, 128))) return fail(rc);
     }
   }
   if (moe) {
@@ -1355,8 +1392,11 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
   const corun_shape &s = e->sh;
   const int CH = P.pair ? P.cap : e->chunk;
   int unit = 128 / (s.n_q_heads / s.n_kv_heads);    // tokens per attention tile
-  if (e->mla) unit = 16;                            // no query tiles there: every row is on its own
+  const bool tiles = P.mla_tiles && !P.shorts;
+  if (e->mla) unit = tiles ? 128 : 16;              // (16: no query tiles, every row is on its own)
   if (unit > CH || CH % unit) unit = CH;
+  struct Piece { int slot, row0, rows, end; };      // a request's piece of the chunk; end: its tokens cached after it
+  std::vector<Piece> pieces;
   std::vector<int> tok((size_t)CH), pos((size_t)CH), act((size_t)CH), slt((size_t)CH);
   std::vector<std::pair<int, int>> fins;           // (request, chunk row of its last prompt token)
   int fill = 0, pad_slot = reqs[0]->slot;
@@ -1377,6 +1417,20 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
       P.row_slot = P.row_active + fill;
       CK(cudaMemcpyAsync(P.row_token, h, 4 * bytes, cudaMemcpyHostToDevice, e->st));
       if (e->mla) RC(set_mla_rows(e, P, fill, tabs));
+      if (tiles) {                                  // whose tokens are gathered where
+        int *tb = blocks + 32, at = 0;
+        P.segs.n = (int)pieces.size();
+        for (size_t k = 0; k < pieces.size(); ++k) {
+          const Piece &pc = pieces[k];
+          P.segs.slot[k] = pc.slot;
+          P.segs.off[k] = at;
+          P.segs.len[k] = pc.end;
+          for (int t = pc.row0 / 128; t <= (pc.row0 + pc.rows - 1) / 128; ++t) tb[t] = at;
+          at += (pc.end + 63) / 64 * 64;
+        }
+        P.kv_tokens = at;
+        CK(cudaMemcpyAsync(P.tile_base, tb, (size_t)((fill + 127) / 128) * sizeof(int), cudaMemcpyHostToDevice, e->st));
+      }
       if (P.shorts) {                               // which blocks of 64 rows exist
         const int nb = (fill + SHORT_ROWS - 1) / SHORT_ROWS;
         for (int b = 0; b < nb; ++b) blocks[b] = 1 | (fill > b * SHORT_ROWS + 64 ? 2 : 0);
@@ -1398,6 +1452,7 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
       RC(prefill_finish(e, P, &fins[i], (int)(fins.size() - i < FINISH_ROWS ? fins.size() - i : FINISH_ROWS), reqs));
     CK(cudaStreamSynchronize(e->st));   // the staging arrays are reused by the next chunk
     fins.clear();
+    pieces.clear();
     fill = 0;
     return CORUN_OK;
   };
@@ -1413,6 +1468,7 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
         act[fill + i] = 1;
         slt[fill + i] = q.slot;
       }
+      if (take > 0) pieces.push_back(Piece{q.slot, fill, take, done + take});
       fill += take;
       done += take;
       pad_slot = q.slot;                            // padding up to the tile's end belongs to this request's tile

@@ -219,6 +219,7 @@ struct GemmPairPlan {
   int N = 0, K = 0, cap = 0, pairs = 0, n_tiles = 0;   // weight rows, reduction length, rows the buffers hold
   int slices = 1;                    // cuts of K (gemm_pair_slices)
   bool swiglu = false;
+  int kv_heads = 0;                  // gemm_pair_plan_create_kv
   float *out = nullptr, *part = nullptr;   // not owned
   const int *row_blocks = nullptr;   // device, not owned (cap 256): bit 1 = rows 128 .. hold a request; null = they do
 };
@@ -236,6 +237,9 @@ cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st
 // W is [2F, K] (F gate rows, then F up rows; F % 8 == 0): out_hi / out_lo [cap, F] = silu(gate) * up as a bf16 hi/lo pair.
 int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,
                                  __nv_bfloat16 *out_lo, int num_sms);
+// Decompression of latents into keys and values: W is [nh * 256, K] (per head 128 key rows, 128 value rows); the fp16 hi / lo
+// pairs of the products go to kv [key hi | key lo | value hi | value lo][nh][cap][128] (cap % 32 == 0).
+int gemm_pair_plan_create_kv(GemmPairPlan *p, int nh, int K, const void *Xhi, const void *Xlo, int cap, void *kv, int num_sms);
 int gemm_pair_prepare();             // opts the kernels into their shared-memory size (idempotent)
 // Rows 0 .. R-1 (R <= cap).  tmW: the weight matrix with a box of 128 rows (gemm_encode_map(.., 128)); tmW96 (swiglu): the
 // same with 96 rows, taken where it shortens the waves.

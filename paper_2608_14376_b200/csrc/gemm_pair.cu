@@ -1,5 +1,6 @@
 // tcgen05 GEMM for many activation rows (long prompts, decode steps above 128 rows): two SMs work as a pair on one tile.
 #include <cudaTypedefs.h>
+#include <cuda_fp16.h>
 
 #include "../../include/corun.h"
 #include "gemm.cuh"
@@ -13,6 +14,7 @@ namespace {
 constexpr int PG_THREADS = 320;                     // warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue
 constexpr int PG_EPI = 8;                           // epilogue warps: two per TMEM lane quarter, half of the columns each
 constexpr int PG_STAGES = 4;
+enum : int { PG_PLAIN = 0, PG_SWIGLU = 1, PG_KV = 2 };
 constexpr uint32_t PG_X_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: a CTA's 128 activation rows, hi or lo
 constexpr uint32_t PG_W_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: a CTA's half of the 256 weight rows
 constexpr uint32_t PG_STAGE_BYTES = 2 * PG_X_BYTES + PG_W_BYTES;
@@ -43,12 +45,15 @@ constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + PG_EPI * 
 //
 // SWIGLU: W is a gate / up matrix ([2F, K]); a tile is `half` gate rows (first CTA) and the up rows of the same outputs
 // (second CTA), whole K, and the epilogue writes silu(gate) * up as the bf16 hi/lo pair the down GEMM reads.
-template <bool SWIGLU>
+// KV (gemm_pair_plan_create_kv): a tile's 256 columns are one head's 128 key and 128 value columns, stored as fp16 hi / lo
+// pairs, keys by the first half of the epilogue warps, values by the second; cap: rows of one of the four matrices per head.
+template <int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                  const __grid_constant__ CUtensorMap tmLo, const __grid_constant__ CUtensorMap tmOut,
                  const __grid_constant__ CUtensorMap tmOut2, int R, int N, int KB, int row_tiles, int whole, int units, int slices,
-                 int half, int *status, const int *row_blocks) {
+                 int half, int *status, const int *row_blocks, int cap) {
+  constexpr bool SWIGLU = MODE == PG_SWIGLU, KV = MODE == PG_KV;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[PG_STAGES];      // used in the first CTA: both CTAs' loads of a stage
   __shared__ __align__(8) uint64_t empty_bar[PG_STAGES];     // in each CTA: the MMAs have read the stage
@@ -189,7 +194,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       const Unit un = unit(u);
       const int nt = un.tile / row_tiles;
       const int row0 = (un.tile % row_tiles) * 256 + rank * 128 + lane_base;   // this warp's 32 rows
-      float sum[128];                               // (not SWIGLU) this thread's row, 128 columns
+      float sum[128];                               // (PLAIN) this thread's row, 128 columns
       for (int sl = un.s0; sl < un.s1; ++sl, ++seg) {
         const int acc = seg & 1;
         ok = mbar_wait(smem_u32(&tmem_full_bar[acc]), (uint32_t)(seg >> 1) & 1u, abort_p);
@@ -230,6 +235,36 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 bulk_commit();
               }
             }
+          } else if (KV) {
+            const int nh = N / GEMM_TILE_N;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              uint32_t v[32];
+              tmem_ld32(ta + (uint32_t)(grp * 128 + q * 32), v);
+              if (lane == 0) bulk_wait_read<0>();
+              __syncwarp();
+              tmem_ld_wait();
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                __half a[8], b[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const float x = __uint_as_float(v[8 * c + j]);
+                  a[j] = __float2half_rn(x);
+                  b[j] = __float2half_rn(x - __half2float(a[j]));
+                }
+                const uint32_t off = (uint32_t)lane * 64 + (((uint32_t)c ^ (((uint32_t)lane >> 1) & 3u)) << 4);
+                *reinterpret_cast<uint4 *>(stg_p + off) = *reinterpret_cast<const uint4 *>(a);
+                *reinterpret_cast<uint4 *>(stg_p + PG_OUT_BYTES / 2 + off) = *reinterpret_cast<const uint4 *>(b);
+              }
+              fence_proxy_async();
+              __syncwarp();
+              if (lane == 0) {
+                tma_store_2d(&tmOut, stg, q * 32, ((2 * grp) * nh + nt) * cap + row0);
+                tma_store_2d(&tmOut, stg + PG_OUT_BYTES / 2, q * 32, ((2 * grp + 1) * nh + nt) * cap + row0);
+                bulk_commit();
+              }
+            }
           } else {
 #pragma unroll
             for (int q = 0; q < 16; ++q) {          // (8 columns at a time: 128 running sums leave few registers)
@@ -244,7 +279,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         tc_fence_before();
         mbar_arrive_cluster(cluster_map(smem_u32(&tmem_empty_bar[acc]), 0));
       }
-      if (!SWIGLU && ok && row0 < R) {
+      if (MODE == PG_PLAIN && ok && row0 < R) {
         // a whole tile goes to the output, a slice to its partial matrix
         const bool part = u >= whole;
         const int y = part ? ((un.tile - whole) * slices + un.s0) * 256 + rank * 128 + lane_base : row0;
@@ -400,9 +435,23 @@ int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi,
   return gemm_pair_prepare();
 }
 
+int gemm_pair_plan_create_kv(GemmPairPlan *p, int nh, int K, const void *Xhi, const void *Xlo, int cap, void *kv, int num_sms) {
+  if (nh < 1 || K <= 0 || K % GEMM_BLOCK_K || cap < 32 || cap % 32 || !kv || num_sms < 2) return CORUN_EINVAL;
+  p->N = nh * GEMM_TILE_N; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = false; p->out = nullptr;
+  p->n_tiles = nh;
+  p->slices = 1;
+  p->kv_heads = nh;
+  int rc;
+  if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
+  if ((rc = tma_encode_store_2d(&p->tmOut, kv, 0, (unsigned long long)4 * nh * cap, 128)) != 0) return rc;
+  p->tmOut2 = p->tmOut;
+  return gemm_pair_prepare();
+}
+
 int gemm_pair_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
+  cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<PG_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair_kernel<PG_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair_kernel<PG_KV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
   if (e != cudaSuccess) { g_last_cuda_error = (int)e; return CORUN_ECUDA; }
   return CORUN_OK;
 }
@@ -413,9 +462,9 @@ cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int 
   const int pairs = q.units < p.pairs ? q.units : p.pairs;
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, q.half == 96 ? *tmW96 : tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2,
-                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, q.half, d_status, p.row_blocks);
+                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, q.half, d_status, p.row_blocks, p.cap);
   };
-  return p.swiglu ? go(gemm_pair_kernel<true>) : go(gemm_pair_kernel<false>);
+  return p.kv_heads ? go(gemm_pair_kernel<PG_KV>) : p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU>) : go(gemm_pair_kernel<PG_PLAIN>);
 }
 
 }  // namespace corun

@@ -72,6 +72,21 @@ cudaError_t launch_mla_attention(const CUtensorMap &tmC, const CUtensorMap &tmV,
                                  float2 *part_ml, float *part_o, float *o_lat, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo,
                                  int rows_per_head, int num_sms, int *d_status, bool pdl, cudaStream_t st, int page_run);
 
+// ---- prefill of long prompts (attention_prefill_mla.cu; no-rope and value widths of 128) ----
+// The requests of a chunk: `len` cached tokens of a slot, gathered from token `off` (a multiple of 64, ascending) on.
+constexpr int MLA_MAX_SEGS = 17;
+struct MlaSegs { int n, slot[MLA_MAX_SEGS], off[MLA_MAX_SEGS], len[MLA_MAX_SEGS]; };
+// -> latents as a bf16 hi / lo pair [total][rank], rotary keys fp16 [total][64] (columns beyond rope are left alone).
+cudaError_t launch_mla_gather(const MlaSegs &g, const MlaCache &cache, int rank, int rope, int total, __nv_bfloat16 *c_hi,
+                              __nv_bfloat16 *c_lo, __half *kr, cudaStream_t st);
+cudaError_t mla_prefill_prepare();   // opts the kernel into its shared-memory size (idempotent)
+// Causal attention of the chunk's rows (tiles of 128 rows, each of one request, whose gathered tokens start at
+// tile_base[tile]) -> bf16 hi / lo [R][nh * 128].  tmKV: boxes of 64 x 64 over the decompressed [key hi | key lo | value hi |
+// value lo][nh][cap][128] fp16; tmR: the same over the rotary keys [cap][64].
+cudaError_t launch_mla_prefill(const CUtensorMap &tmKV, const CUtensorMap &tmR, const __nv_bfloat16 *qn_hi, const __nv_bfloat16 *qn_lo,
+                               const float *q_rope, const Rows &rows, int rows_per_head, const MlaDims &d, int cap, const int *tile_base,
+                               float scale, __nv_bfloat16 *ao_hi, __nv_bfloat16 *ao_lo, int *d_status, cudaStream_t st);
+
 // The value part of the grouped up-projection result uv [nh * rows_per_head][nope + vh] (columns nope.. of every
 // row) -> bf16 hi/lo [R][nh * vh], the o-projection's activations.
 cudaError_t launch_mla_ao_split(const float *uv, int R, int rows_per_head, const MlaDims &d, __nv_bfloat16 *ao_hi,
