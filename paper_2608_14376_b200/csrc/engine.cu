@@ -102,6 +102,11 @@ struct Program {
   // Decode above 128 rows (wide): the dense projections and the LM head on pairs of SMs too.  Per Qwen3-8B layer at 256 rows
   // 248 us of GEMMs (hi and lo of two row blocks per weight tile on one SM each, two stages of shared memory) and 17 us of
   // SwiGLU, against 179 us.
+  // A pair multiplies both halves of its 256 rows whether requests fill them or not, so with up to 128 requests in the step
+  // a decoder that is bound by streaming large dense matrices pays for it: 140 slots, 25 / 125 / 139 requests, 12 Qwen3-8B
+  // layers 2.45 / 2.77 / 3.58 ms before and 2.74 / 3.06 / 3.21 with pairs, 230 slots, 60 / 120 / 150: 2.83 / 3.00 / 4.05 and
+  // 2.87 / 3.13 / 3.56.  Those take pairs from WIDE_ROWS rows on; the hidden-1024 decoder and the decoders with expert layers
+  // gain at every count (1.04 / 1.22 / 1.86 -> 1.02 / 1.20 / 1.48 ms; 3.71 / 4.43 / 5.26 -> 3.59 / 4.31 / 4.87).
   bool wide = false;
   GemmPairPlan b_lm;
   bool shorts = false;
@@ -130,6 +135,7 @@ constexpr int PREFILL_SMALL = 128, PREFILL_BIG = 2048;
 // Rows of a long prompt's chunk that the latent attention takes at a time (its partial results are kept per row).
 constexpr int MLA_ROWS = 256;
 constexpr int SHORT_ROWS = 128;
+constexpr int WIDE_ROWS = 192;               // see Program::wide
 static_assert(PREFILL_BIG <= MOE_MANY_ROWS, "a chunk of a long prompt is grouped in one go");
 
 }  // namespace
@@ -160,6 +166,7 @@ struct corun_engine {
   bool mla = false;
   MlaDims md{};
   int first_dense = 0, dense_ffn = 0, mla_splits = 0;
+  bool wide = false;                     // Program::wide of the decode program
   bool big_mla_tiles = false;            // Program::mla_tiles of the prefill program
   std::vector<const bf16 *> kv_norm;
   bf16 *w_ukT = nullptr;                 // [L][nh * rank][nope]: the key up-projections transposed
@@ -276,7 +283,7 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
   P.BN = pad16(R);
   P.has_layers = layers;
   P.has_lm = lm;
-  P.wide = layers && lm && P.BN > 128 && V % 8 == 0;
+  P.wide = layers && lm && e->wide;
   const int RB = P.wide ? 256 : P.BN, RR = P.wide ? 256 : R;   // rows of the projections' inputs and outputs
   auto &A = P.allocs;
   RC(dmalloc(A, &P.xn_hi, (size_t)RB * H));
@@ -1070,7 +1077,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG
   const long long big_rows = (long long)B * ((max_context + 127) / 128 * 128);
   const int big_cap = !big_ok ? 0 : big_rows < PREFILL_BIG ? (int)((big_rows + 255) / 256 * 256) : PREFILL_BIG;
-  const bool wide = pad16(B) > 128;                 // decode on pairs of SMs (Program::wide)
+  const bool large_dense = !moe && (long long)2 * F * H > (16ll << 20);
+  const bool wide = e->wide = pad16(B) > 128 && s.vocab % 8 == 0 && (!large_dense || pad16(B) >= WIDE_ROWS);   // (Program::wide)
   if (wide && gemm_encode_map(&e->tb_lm, w->lm_head, s.vocab, H, 128)) return fail(CORUN_EINVAL);
   e->tm_qkv.resize(s.n_layers);
   e->tm_o.resize(s.n_layers);
