@@ -691,7 +691,7 @@ cudaError_t launch_attention(const CUtensorMap &tmK, const CUtensorMap &tmV, con
   const int group = nq / kv.n_kv;
   if (group * kv.n_kv != nq || max_splits > 256) return cudaErrorInvalidValue;
   if (reuse == 1)   // a prefill chunk: consecutive tokens of one request
-    return launch_attention_prefill(tmK, tmV, q, rows, nq, kv, out_hi, out_lo, d_status, st);
+    return launch_attention_prefill(tmK, q, rows, nq, kv, out_hi, out_lo, d_status, st);
   const int whole_pairs = reuse == 2;   // the ablation: the item list carries the pair table
   const long long most = (long long)rows.R * max_splits * kv.n_kv;
   const int grid = (int)(most < grid_ctas ? most : grid_ctas);

@@ -156,8 +156,7 @@ struct corun_engine {
   CUtensorMap tb_lm;
   std::vector<CUtensorMap> tb_gu_half;     // dense layers of a decoder with expert layers: the box of the GEMM with SwiGLU
   std::vector<CUtensorMap> tm_gu_half;     // dense gate / up matrices with the box of the GEMM with SwiGLU in its epilogue
-  std::vector<CUtensorMap> tm_k, tm_v;   // per layer: the pages as rows of head_dim halfs (keys and values alike)
-  std::vector<CUtensorMap> tm_k4;        // the same memory as [8-token group][64-dim half][8 tokens][64 dims]: one box per (page, head) tile
+  std::vector<CUtensorMap> tm_k4;        // per layer: the pages (keys and values alike) as [8-token group][64-dim half][8 tokens][64 dims]: one box per (page, head) tile
   // Mixture-of-Experts feed-forward layers (E = 0: dense).  sh.ffn is then (E + S) * F.
   int moe_E = 0, moe_K = 0, moe_F = 0, moe_S = 0, moe_renorm = 0;
   std::vector<const bf16 *> router;      // per layer: [E, H], borrowed
@@ -706,7 +705,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
           STAGE(launch_qkv_post(P.s_qkv[b].out(), block_rows(b), e->d_rope, s.n_q_heads, kv, l, P.q + (size_t)b * SHORT_ROWS * QD, e->d_status,
                                 e->st));
         }
-        STAGE(launch_attention_prefill(e->tm_k[l], e->tm_v[l], P.q, rows, s.n_q_heads, kv, P.ao_hi, P.ao_lo, e->d_status, e->st));
+        STAGE(launch_attention_prefill(e->tm_k4[l], P.q, rows, s.n_q_heads, kv, P.ao_hi, P.ao_lo, e->d_status, e->st));
       }
       if (!P.shorts) {
         STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
@@ -767,8 +766,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       n += 3 + (&P == &e->dec ? 0 : 1);               // beyond the count below: two grouped GEMMs, the split, and in prefill too a second attention kernel
     } else {
     STAGE(launch_qkv_post(qkv, rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
-    // (the decode kernel takes the one-box-per-tile view of the pages, the prefill kernel the row view)
-    STAGE(launch_attention(&P == &e->dec ? e->tm_k4[l] : e->tm_k[l], &P == &e->dec ? e->tm_k4[l] : e->tm_v[l], P.q, rows, s.n_q_heads, kv, l, e->max_splits, P.att_work, P.att_n_work,
+    STAGE(launch_attention(e->tm_k4[l], e->tm_k4[l], P.q, rows, s.n_q_heads, kv, l, e->max_splits, P.att_work, P.att_n_work,
                            e->num_sms, P.part_acc, P.part_ml, P.att_pool + l, P.ao_hi, P.ao_lo, &P == &e->dec ? (e->whole_pairs ? 2 : 0) : 1,
                            e->d_status, e->st));
     }
@@ -1164,13 +1162,9 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     // one layer's pages seen as rows of hd halfs (16 rows per page and head, keys first, then values)
     const unsigned long long halfs = (unsigned long long)e->layer_stride;
     if (halfs / KV_BLOCK >= (1ull << 31)) return fail(CORUN_EINVAL);
-    e->tm_k.resize(s.n_layers);
-    e->tm_v.resize(s.n_layers);
     for (int l = 0; l < s.n_layers; ++l) {
       const __half *base = e->kv_pool + (size_t)l * e->layer_stride;
-      if ((rc = tma_encode_2d(&e->tm_k[l], base, 1, halfs / s.head_dim, s.head_dim, KV_BLOCK, 64))) return fail(rc);
-      e->tm_v[l] = e->tm_k[l];   // keys and values are cached alike: the same view serves both
-      // decode attention: a tile's 16 tokens x head_dim in ONE box, [2 groups of 8 tokens][halves of 64 dims][8][64]
+      // keys and values are cached alike, one view serves both: a tile's 16 tokens x head_dim in ONE box, [2 groups of 8 tokens][halves of 64 dims][8][64]
       const unsigned long long row_b = (unsigned long long)s.head_dim * 2;
       const unsigned long long d4[4] = {64, 8, (unsigned long long)(s.head_dim / 64), halfs / s.head_dim / 8};
       const unsigned long long s4[3] = {row_b, 128, 8 * row_b};

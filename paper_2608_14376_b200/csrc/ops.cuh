@@ -83,9 +83,9 @@ cudaError_t launch_attn_worklist(const Rows &rows, int n_kv, int *work, int *n_w
                                  int n_pool_counts, int whole_pairs, cudaStream_t st);
 // Causal attention of a prefill chunk (rows = consecutive tokens of one request, all of one slot): query
 // tiles share the key / value tiles they read; writes the bf16 hi/lo output directly (attention_prefill.cu).
-cudaError_t launch_attention_prefill(const CUtensorMap &tmK, const CUtensorMap &tmV, const float *q, const Rows &rows,
-                                     int nq, const KvLayout &kv, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo,
-                                     int *d_status, cudaStream_t st);
+// tmKV: the pages with one box per (page, head) tile (the decode kernel's view).
+cudaError_t launch_attention_prefill(const CUtensorMap &tmKV, const float *q, const Rows &rows, int nq, const KvLayout &kv,
+                                     __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int *d_status, cudaStream_t st);
 cudaError_t attention_prepare();   // opts the kernels into their shared-memory size (idempotent)
 // y = silu(gate) * up from the gate-up GEMM result -> bf16 hi/lo [R, F].
 cudaError_t launch_swiglu(const GemmOut &gu, int R, int F, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, cudaStream_t st);
