@@ -348,11 +348,11 @@ PairShape pair_shape(const GemmPairPlan &p, int R, bool narrow) {
   if (p.slices > 1) {
     const int full = tiles / p.pairs * p.pairs, tail = tiles - full;
     // worth it where the time of the last wave that is saved (0.8 us per k-block) exceeds what writing and reading the
-    // partials costs (0.5 MB per slice of a tile at 5 TB/s): 16 of 16 tiles of the Qwen3-8B O projection at 256 rows 51 -> 21
+    // partials costs (0.06 us per slice of a tile): 16 of 16 tiles of the Qwen3-8B O projection at 256 rows 51 -> 21
     // us, not 54 of 128 at 2048 rows
     const int parts = (tail * p.slices + p.pairs - 1) / p.pairs;
     const float saved = 0.8f * (float)(p.K / GEMM_BLOCK_K) * (float)(p.slices - parts) / (float)p.slices;
-    if (tail && saved > 0.1f * (float)(tail * p.slices)) {
+    if (tail && saved > 0.06f * (float)(tail * p.slices)) {
       q.whole = full;
       q.units = full + tail * p.slices;
     }

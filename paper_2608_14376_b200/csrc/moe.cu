@@ -306,15 +306,16 @@ __global__ void __launch_bounds__(256) moe_mask_kernel(const float *__restrict__
   griddep_launch_dependents();
   griddep_wait();
   w = after_wait(w); active = after_wait(active);
-  const int r0 = (int)blockIdx.x * 32;
+  const int r0 = (int)blockIdx.x * 32, lane = (int)threadIdx.x & 31;
+  const uint32_t on = __ballot_sync(0xffffffffu, r0 + lane < R && active[r0 + lane] != 0);   // the rows with a token
   for (int e = (int)threadIdx.x; e < NB; e += 256) {
+    float v[32];                                     // all of the expert's loads in flight
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = r0 + i < R ? w[(size_t)(r0 + i) * NB + e] : 0.f;
     uint32_t m = 0u;
-#pragma unroll 8
-    for (int i = 0; i < 32; ++i) {
-      const int r = r0 + i;
-      if (r < R && active[r] != 0 && w[(size_t)r * NB + e] != 0.f) m |= 1u << i;
-    }
-    mask[e * MOE_MASK_WORDS + (int)blockIdx.x] = m;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) m |= v[i] != 0.f ? 1u << i : 0u;
+    mask[e * MOE_MASK_WORDS + (int)blockIdx.x] = m & on;
   }
 }
 
