@@ -69,6 +69,7 @@ struct Program {
   // Mixture-of-Experts feed-forward layers: p_gu / p_down are then the GEMMs over all experts' gate / up rows
   // and over the concatenated hidden activations; moe_w the rows' routing weights
   float *moe_w = nullptr;
+  RouterScratch router_rs{};
   // selected-experts form (decode up to 64 rows): only the experts that a row selected are streamed; p_gug / p_dng are its
   // GEMMs, hg / yg hold [expert][BN] rows, moe_sel every row's experts.  Measured per step, 12 layers of the Qwen3-30B-A3B
   // shape, against every row through every expert: 1 row of 1 3.15 -> 1.24 ms, 16 of 32 3.54 -> 2.72, 40 of 64
@@ -385,6 +386,8 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
     if (P.select) {
       const int nb = e->moe_E + e->moe_S, per_row = e->moe_K + e->moe_S, Fm = e->moe_F;
       RC(dmalloc(A, &P.moe_w, (size_t)R * nb));
+      RC(dmalloc(A, &P.router_rs.logit, (size_t)R * e->moe_E));
+      RC(dmalloc(A, &P.router_rs.count, (size_t)R));
       RC(dmalloc(A, &P.moe_sel, (size_t)R * per_row));
       RC(dmalloc(A, &P.hg_hi, (size_t)nb * P.BN * Fm));
       RC(dmalloc(A, &P.hg_lo, (size_t)nb * P.BN * Fm));
@@ -404,6 +407,8 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
     if (e->moe_E && !P.select) {
       const int NB = e->moe_E + e->moe_S;
       RC(dmalloc(A, &P.moe_w, (size_t)R * NB));
+      RC(dmalloc(A, &P.router_rs.logit, (size_t)R * e->moe_E));
+      RC(dmalloc(A, &P.router_rs.count, (size_t)R));
       if (groups) {
       } else if (moe_fused)
         RC(gemm_plan_create_swiglu_blocks(&P.p_gu, e->w0_gu, NB, e->moe_F, H, P.xn_hi, P.xn_lo, R, P.BN, P.ff_hi, P.ff_lo, P.moe_w,
@@ -791,7 +796,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       // experts summed in ascending expert id
       const int NB = e->moe_E + e->moe_S;
       STAGE(launch_moe_router(P.xn_hi, P.xn_lo, s.hidden, e->router[l], P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, nullptr,
-                              nullptr, e->st));
+                              nullptr, P.router_rs, e->st, P.row_active));
       STAGE(launch_moe_group(P.moe_w, P.row_active, P.R, e->moe_E, e->moe_S, e->moe_F, P.grp, e->st));
       STAGE(launch_moe_gather(P.xn_hi, P.xn_lo, s.hidden, P.grp, P.xg_hi, P.xg_lo, e->st));
       if (P.p_gug.sw_hi) {                            // routing weight and SwiGLU in the GEMM's epilogue
@@ -809,7 +814,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       // router -> top-k weights and the rows' experts -> gate / up with routing weight and SwiGLU, then down, per selected
       // expert for all rows -> the row's experts summed in ascending expert id
       STAGE(launch_moe_router(P.xn_hi, P.xn_lo, s.hidden, e->router[l], P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, nullptr,
-                              nullptr, e->st, P.row_active, P.moe_sel));
+                              nullptr, P.router_rs, e->st, P.row_active, P.moe_sel));
       STAGE(gemm_launch(P.p_gug, &e->tm_gu_half[l], e->d_status, e->st, nullptr, true));
       STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
       STAGE(launch_moe_combine_select(P.yg_out, P.moe_sel, e->moe_K + e->moe_S, P.BN, P.R, s.hidden, P.down_out, e->st));
@@ -819,7 +824,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       // router -> top-k weights -> all experts' gate / up (rows that did not select a tile's expert are not
       // stored) -> masked, weighted SwiGLU; the down GEMM then sums over the row's experts in its accumulator
       STAGE(launch_moe_router(P.xn_hi, P.xn_lo, s.hidden, e->router[l], P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, nullptr,
-                              nullptr, e->st));
+                              nullptr, P.router_rs, e->st));
       if (P.p_gu.sw_hi) {                             // routing weight and SwiGLU in the GEMM's epilogue
         STAGE(gemm_launch(P.p_gu, &e->tm_gu_half[l], e->d_status, e->st, tr(4 * l + 2), true));
       } else {                                        // (the router is the one kernel beyond the count below)
@@ -1854,7 +1859,7 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
                  if (ce == cudaSuccess) ce = launch_moe_gather(P.xn_hi, P.xn_lo, s.hidden, P.grp, P.xg_hi, P.xg_lo, e->st);
                  break;
         case 12: ce = launch_moe_router(P.xn_hi, P.xn_lo, s.hidden, e->router[l], P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm,
-                                        P.moe_w, nullptr, nullptr, e->st, P.row_active, P.moe_sel);
+                                        P.moe_w, nullptr, nullptr, P.router_rs, e->st, P.row_active, P.moe_sel);
                  break;
       }
     }

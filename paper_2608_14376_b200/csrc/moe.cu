@@ -21,6 +21,7 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 constexpr int MOE_MAX_TOPK = 16;
+constexpr int ROUTER_WARPS = 8;
 constexpr int MOE_MAX_EXPERTS = 256;
 
 #define MCK(call)                               \
@@ -69,99 +70,132 @@ __device__ __forceinline__ void moe_route_row(LoadLogit load, int r, int lane, i
   for (int e = lane; e < E; e += 32) wr[e] = 0.f;
   for (int s = lane; s < S; s += 32) wr[E + s] = 1.f;
   __syncwarp();
-  int ids[MOE_MAX_TOPK];
-  float ps[MOE_MAX_TOPK];
-  float picked = 0.f;                                // sum of the selected probabilities, in selection order
+  int id = 0;                                        // lane k: the k-th selected expert and its probability
+  float prob = 0.f, picked = 0.f;                    // picked: sum of the selected probabilities, in selection order
   for (int k = 0; k < top_k; ++k) {
     float bz = -1.f;                                 // this lane's best: largest value, lowest id on ties
     int be = 0x7fffffff;
 #pragma unroll
     for (int j = 0; j < PER; ++j)
       if (z[j] > bz) { bz = z[j]; be = lane + 32 * j; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float oz = __shfl_xor_sync(0xffffffffu, bz, o);
-      const int oe = __shfl_xor_sync(0xffffffffu, be, o);
-      if (oz > bz || (oz == bz && oe < be)) { bz = oz; be = oe; }
-    }
+    // the warp's: values are -1 or not below 0, and those order as their bits do
+    const int top = __reduce_max_sync(0xffffffffu, __float_as_int(bz));
+    be = __reduce_min_sync(0xffffffffu, __float_as_int(bz) == top ? be : 0x7fffffff);
     if (be >= E) be = k;                             // a row of NaNs: any valid id
-    const float p = __fdiv_rn(bz, sum);
+    const float p = __fdiv_rn(__int_as_float(top), sum);
 #pragma unroll
     for (int j = 0; j < PER; ++j)
       if (lane + 32 * j == be) z[j] = -2.f;          // taken
-    ids[k] = be;
-    ps[k] = p;
+    if (lane == k) { id = be; prob = p; }
     picked += p;
   }
-  if (lane == 0)
-    for (int k = 0; k < top_k; ++k) {
-      const float p = renormalize ? __fdiv_rn(ps[k], picked) : ps[k];
-      wr[ids[k]] = p;
-      if (experts) experts[(size_t)r * top_k + k] = ids[k];
-      if (probs) probs[(size_t)r * top_k + k] = p;
-    }
-  if (sel) {                                         // every lane knows all ids: lane k places the k-th
+  if (lane < top_k) {
+    const float p = renormalize ? __fdiv_rn(prob, picked) : prob;
+    wr[id] = p;
+    if (experts) experts[(size_t)r * top_k + lane] = id;
+    if (probs) probs[(size_t)r * top_k + lane] = p;
+  }
+  if (sel) {                                         // ascending ids, the shared experts last
     int *out = sel + (size_t)r * (top_k + S);
-    for (int k = 0; k < top_k; ++k) {
-      int place = 0;
-      for (int j = 0; j < top_k; ++j) place += ids[j] < ids[k] ? 1 : 0;
-      if (lane == k) out[place] = on ? ids[k] : -1;
-    }
+    int place = 0;
+    for (int j = 0; j < top_k; ++j) place += __shfl_sync(0xffffffffu, id, j) < id ? 1 : 0;
+    if (lane < top_k) out[place] = on ? id : -1;
     for (int s = lane; s < S; s += 32) out[top_k + s] = on ? E + s : -1;
   }
 }
 
-// Router of one row per CTA: logits = Wr x on the CUDA cores (E dot products of H terms: far too little for a
-// tensor-core launch of its own), then the routing above.  x is the row's bf16 hi + lo pair (exactly what the
-// GEMMs of the block see); every warp takes experts warp, warp + 32, ...: a lane adds its terms in ascending
-// order (8 consecutive terms per step, the weights of four steps requested together), then a fixed butterfly
-// over the lanes.  A row's routing depends on the row alone.
-constexpr int ROUTER_THREADS = 1024;
-__global__ void __launch_bounds__(ROUTER_THREADS) moe_router_kernel(const bf16 *__restrict__ x_hi, const bf16 *__restrict__ x_lo, int H,
-                                                                    const bf16 *__restrict__ Wr, int E, int S, int top_k,
-                                                                    int renormalize, float *__restrict__ w,
-                                                                    int *__restrict__ experts, float *__restrict__ probs,
-                                                                    const int *active, int *__restrict__ sel) {
+// Router: logits = Wr x on the CUDA cores (E dot products of H terms a row: far too little for a tensor-core launch of its
+// own), then the routing above.  blockIdx.y: NR rows, as their bf16 hi + lo pairs (exactly what the GEMMs of the block
+// see); blockIdx.x: ROUTER_WARPS experts, one per warp.  A lane adds its terms in ascending order (8 consecutive terms per
+// step, the weights of eight steps requested together, the first ones ahead of the wait for the predecessor), then a fixed
+// butterfly over the lanes: a row's routing depends on the row alone.  The CTA that finishes its rows last routes them.
+template <int NR>
+__global__ void __launch_bounds__(32 * ROUTER_WARPS) moe_router_kernel(const bf16 *__restrict__ x_hi, const bf16 *__restrict__ x_lo, int H,
+                                                                       const bf16 *__restrict__ Wr, int R, int E, int S, int top_k,
+                                                                       int renormalize, float *__restrict__ w,
+                                                                       int *__restrict__ experts, float *__restrict__ probs,
+                                                                       const int *active, int *__restrict__ sel, RouterScratch rs) {
   griddep_launch_dependents();
-  extern __shared__ float xs[];                      // the row as fp32 [H]
-  __shared__ float logit[MOE_MAX_EXPERTS];
-  const int r = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  griddep_wait();
-  for (int i = 4 * tid; i < H; i += 4 * ROUTER_THREADS) {
-    const uint2 rh = *reinterpret_cast<const uint2 *>(x_hi + (size_t)r * H + i), rl = *reinterpret_cast<const uint2 *>(x_lo + (size_t)r * H + i);
-    const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&rh), *l2 = reinterpret_cast<const __nv_bfloat162 *>(&rl);
-    const float2 h0 = __bfloat1622float2(h2[0]), h1 = __bfloat1622float2(h2[1]), l0 = __bfloat1622float2(l2[0]), l1 = __bfloat1622float2(l2[1]);
-    *reinterpret_cast<float4 *>(xs + i) = make_float4(h0.x + l0.x, h0.y + l0.y, h1.x + l1.x, h1.y + l1.y);
-  }
-  __syncthreads();
-  for (int e = warp; e < E; e += ROUTER_THREADS / 32) {
-    const bf16 *wrow = Wr + (size_t)e * H;
-    float acc = 0.f;
-    for (int i0 = 8 * lane; i0 < H; i0 += 4 * 8 * 32) {
-      uint4 raw[4];
+  extern __shared__ float xs[];                      // the rows as fp32 [NR][H]
+  __shared__ int last;
+  constexpr int U = 8;
+  const int r0 = (int)blockIdx.y * NR, nr = R - r0 < NR ? R - r0 : NR, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int e = (int)blockIdx.x * ROUTER_WARPS + warp;
+  uint4 raw[U];
+  auto request = [&](int i0) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * 8 * 32;
-        raw[u] = i < H ? __ldg(reinterpret_cast<const uint4 *>(wrow + i)) : make_uint4(0u, 0u, 0u, 0u);
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * 8 * 32;
+      raw[u] = i < H ? __ldg(reinterpret_cast<const uint4 *>(Wr + (size_t)e * H + i)) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if (e < E) request(8 * lane);
+  griddep_wait();
+  x_hi = after_wait(x_hi);
+  x_lo = after_wait(x_lo);
+  bool any = !active;
+  if (active)
+    for (int q = 0; q < nr; ++q) any |= after_wait(active)[r0 + q] != 0;
+  if (!any && blockIdx.x) return;                    // rows without a request need no logits; the first CTA writes their -1s
+  if (any) {
+    for (int i = 4 * tid; i < H; i += 4 * 32 * ROUTER_WARPS) {
+      uint2 rh[NR], rl[NR];
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+        const size_t o = (size_t)(r0 + (q < nr ? q : 0)) * H + i;
+        rh[q] = *reinterpret_cast<const uint2 *>(x_hi + o);
+        rl[q] = *reinterpret_cast<const uint2 *>(x_lo + o);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * 8 * 32;
-        if (i >= H) break;
-        const __nv_bfloat162 *w2 = reinterpret_cast<const __nv_bfloat162 *>(&raw[u]);
-        const float4 xa = *reinterpret_cast<const float4 *>(xs + i), xb = *reinterpret_cast<const float4 *>(xs + i + 4);
-        const float2 w0 = __bfloat1622float2(w2[0]), w1 = __bfloat1622float2(w2[1]), w2f = __bfloat1622float2(w2[2]), w3 = __bfloat1622float2(w2[3]);
-        acc = fmaf(w0.x, xa.x, acc); acc = fmaf(w0.y, xa.y, acc); acc = fmaf(w1.x, xa.z, acc); acc = fmaf(w1.y, xa.w, acc);
-        acc = fmaf(w2f.x, xb.x, acc); acc = fmaf(w2f.y, xb.y, acc); acc = fmaf(w3.x, xb.z, acc); acc = fmaf(w3.y, xb.w, acc);
+      for (int q = 0; q < NR; ++q) {
+        const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&rh[q]), *l2 = reinterpret_cast<const __nv_bfloat162 *>(&rl[q]);
+        const float2 h0 = __bfloat1622float2(h2[0]), h1 = __bfloat1622float2(h2[1]), l0 = __bfloat1622float2(l2[0]), l1 = __bfloat1622float2(l2[1]);
+        *reinterpret_cast<float4 *>(xs + (size_t)q * H + i) = make_float4(h0.x + l0.x, h0.y + l0.y, h1.x + l1.x, h1.y + l1.y);
       }
     }
+    __syncthreads();
+    if (e < E) {
+      float acc[NR] = {};
+      for (int i0 = 8 * lane; i0 < H; i0 += U * 8 * 32) {
+        if (i0 >= U * 8 * 32) request(i0);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) logit[e] = acc;
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u * 8 * 32;
+          if (i >= H) break;
+          const __nv_bfloat162 *w2 = reinterpret_cast<const __nv_bfloat162 *>(&raw[u]);
+          const float2 w0 = __bfloat1622float2(w2[0]), w1 = __bfloat1622float2(w2[1]), w2f = __bfloat1622float2(w2[2]), w3 = __bfloat1622float2(w2[3]);
+#pragma unroll
+          for (int q = 0; q < NR; ++q) {
+            const float4 xa = *reinterpret_cast<const float4 *>(xs + (size_t)q * H + i), xb = *reinterpret_cast<const float4 *>(xs + (size_t)q * H + i + 4);
+            float a = acc[q];
+            a = fmaf(w0.x, xa.x, a); a = fmaf(w0.y, xa.y, a); a = fmaf(w1.x, xa.z, a); a = fmaf(w1.y, xa.w, a);
+            a = fmaf(w2f.x, xb.x, a); a = fmaf(w2f.y, xb.y, a); a = fmaf(w3.x, xb.z, a); a = fmaf(w3.y, xb.w, a);
+            acc[q] = a;
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+        if (lane == 0 && q < nr) rs.logit[(size_t)(r0 + q) * E + e] = acc[q];
+      }
+      if (lane == 0) __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) {
+      last = gridDim.x == 1 || atomicAdd(rs.count + blockIdx.y, 1) == (int)gridDim.x - 1;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    if (tid == 0) rs.count[blockIdx.y] = 0;          // for the next launch
   }
-  __syncthreads();
-  if (warp == 0) moe_route_row([&](int e) { return logit[e]; }, r, lane, E, S, top_k, renormalize, w, experts, probs, sel,
-                               !sel || active[r] != 0);
+  if (warp < nr) {
+    const int r = r0 + warp;
+    moe_route_row([&](int e) { return any ? __ldcg(rs.logit + (size_t)r * E + e) : 0.f; }, r, lane, E, S, top_k, renormalize, w, experts,
+                  probs, sel, !active || after_wait(active)[r] != 0);
+  }
 }
 
 // h[r, e*F + f] = w[r, e] * silu(gate) * up as a bf16 hi/lo pair; zeros where w[r, e] == 0 (nothing is read
@@ -554,9 +588,18 @@ cudaError_t launch_moe_combine(const float *yg, const int *active, int R, int n_
 }
 
 cudaError_t launch_moe_router(const bf16 *x_hi, const bf16 *x_lo, int H, const bf16 *Wr, int R, int E, int S, int top_k,
-                              int renormalize, float *w, int *experts, float *probs, cudaStream_t st, const int *active, int *sel) {
-  return launch_k(moe_router_kernel, dim3(R), dim3(ROUTER_THREADS), (size_t)H * sizeof(float), st, true, x_hi, x_lo, H, Wr, E, S, top_k,
-                  renormalize, w, experts, probs, active, sel);
+                              int renormalize, float *w, int *experts, float *probs, const RouterScratch &rs, cudaStream_t st, const int *active,
+                              int *sel) {
+  const int shares = (E + ROUTER_WARPS - 1) / ROUTER_WARPS;
+  auto go = [&](auto kernel, int n) {
+    return launch_k(kernel, dim3(shares, (R + n - 1) / n), dim3(32 * ROUTER_WARPS), (size_t)n * H * sizeof(float), st, true, x_hi, x_lo, H, Wr,
+                    R, E, S, top_k, renormalize, w, experts, probs, active, sel, rs);
+  };
+  // Few rows: the latency of one expert's weights bounds it, so a CTA per row and 8 experts (one CTA per row did all experts:
+  // steps of 12 layers with 128 experts 1234 -> 1095 us at 1 row, 3890 -> 3770 at 40 of 64 rows; 4 rows a CTA 1139 / 3816).
+  // Many rows: the weights from L2 once per row bound it (100 of 128 rows 4670 us, 4 rows a CTA 4609; 200 of 256 rows 5120
+  // with one CTA per row, 5065 with 4 rows).  The rows of a CTA have to fit into 48 KB of shared memory.
+  return R > 96 && 4 * (size_t)H * sizeof(float) <= 46 * 1024 ? go(moe_router_kernel<4>, 4) : go(moe_router_kernel<1>, 1);
 }
 
 cudaError_t launch_moe_combine_select(const float *yg, const int *sel, int n_per_row, int BN, int R, int H, float *y, cudaStream_t st) {
@@ -582,6 +625,7 @@ struct corun_moe {
   int *d_status = nullptr;
   GemmPlan p_gu, p_d;
   // grouped form (more than 64 padded rows): an expert's rows gathered into blocks of 64
+  RouterScratch rs{};
   bool grouped = false;
   MoeGroups grp{};
   bf16 *xg_hi = nullptr, *xg_lo = nullptr, *hg_hi = nullptr, *hg_lo = nullptr;
@@ -634,6 +678,7 @@ int corun_moe_create(const corun_moe_shape *shape, const void *router, const voi
       (rc = moe_alloc(m, &m->h_lo, (size_t)m->BN * K2)) ||
       (rc = moe_alloc(m, &m->out_gu, (size_t)m->BN * N1)) || (rc = moe_alloc(m, &m->out_d, (size_t)m->BN * H)) ||
       (rc = moe_alloc(m, &m->ws, gemm_ws_floats(m->num_sms, m->BN))) || (rc = moe_alloc(m, &m->w, (size_t)B * NB)) ||
+      (rc = moe_alloc(m, &m->rs.logit, (size_t)B * E)) || (rc = moe_alloc(m, &m->rs.count, (size_t)B)) ||
       (rc = moe_alloc(m, &m->d_status, 1)))
     return fail(rc);
   m->router = (const bf16 *)router;
@@ -699,7 +744,7 @@ int corun_moe_forward(corun_moe *m, const float *x, float *y, int32_t *experts, 
   const corun_moe_shape &s = m->sh;
   const int H = s.hidden, E = s.n_experts, F = s.expert_ffn, NB = E + s.n_shared;
   MCK(launch_split(x, m->B, H, m->x_hi, m->x_lo, m->st));
-  MCK(launch_moe_router(m->x_hi, m->x_lo, H, m->router, m->B, E, s.n_shared, s.top_k, s.renormalize, m->w, experts, probs, m->st));
+  MCK(launch_moe_router(m->x_hi, m->x_lo, H, m->router, m->B, E, s.n_shared, s.top_k, s.renormalize, m->w, experts, probs, m->rs, m->st));
   if (m->grouped) {
     // rows grouped by expert -> gate / up with routing weight and SwiGLU, and down, per group -> the row's experts
     // summed in ascending expert id

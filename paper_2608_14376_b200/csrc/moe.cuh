@@ -10,11 +10,15 @@ namespace corun {
 // Router of every row: logits = Wr x (Wr bf16 [E, H]; x the row's bf16 hi + lo pair, [R or more, H]) on the CUDA
 // cores, softmax over all E experts, top_k by repeated arg-max with ties to the lower id, optional
 // renormalisation; writes the row of SwiGLU weights w[r, 0 .. E + S) (p_e for the selected experts, 0 for the
-// others, 1 for the shared ones) and, when not null, the routing.  One CTA per row; H * 4 bytes of shared memory
-// (H <= 12288).
+// others, 1 for the shared ones) and, when not null, the routing.  Several CTAs per row meet in `rs`; H * 4 bytes of shared
+// memory (H <= 12288).
+struct RouterScratch {
+  float *logit;   // [R, E]
+  int *count;     // [R], zero between launches
+};
 cudaError_t launch_moe_router(const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_lo, int H, const __nv_bfloat16 *Wr, int R, int E,
-                              int S, int top_k, int renormalize, float *w, int *experts, float *probs, cudaStream_t st,
-                              const int *active = nullptr, int *sel = nullptr);
+                              int S, int top_k, int renormalize, float *w, int *experts, float *probs, const RouterScratch &rs,
+                              cudaStream_t st, const int *active = nullptr, int *sel = nullptr);
 // (active, sel: when sel is not null, sel[r * (top_k + S) ..] receives the row's experts in ascending id, the shared ones
 // last, or -1 for a row with active[r] == 0)
 // y[r, :] = sum over the row's experts (sel, ascending) of yg[e * BN + r, :]; rows without experts are left alone.
