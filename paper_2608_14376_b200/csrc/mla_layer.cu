@@ -16,7 +16,7 @@ __device__ __forceinline__ void mla_split_bf16(float x, __nv_bfloat16 &hi, __nv_
   lo = __float2bfloat16_rn(x - __bfloat162float(hi));
 }
 
-constexpr int MLA_POST_THREADS = 256;
+constexpr int MLA_POST_THREADS = 128;   // four columns each: a latent of up to 512
 
 __device__ __forceinline__ void mla_store_split4(float4 y, __nv_bfloat16 *hi, __nv_bfloat16 *lo) {
   __nv_bfloat16 a[4], b[4];
@@ -34,7 +34,9 @@ __device__ __forceinline__ void mla_rotate4(const float4 a, const float4 b, cons
   rb = make_float4(a.x * t01.y + b.x * t01.x, a.y * t01.w + b.y * t01.z, a.z * t23.y + b.z * t23.x, a.w * t23.w + b.w * t23.z);
 }
 
-// One CTA per row; four consecutive columns per thread and pass (nope, rope / 2 and rank are multiples of 4).
+// blockIdx.y: the row; blockIdx.x: 0 its cache row, else a share of its query.  Four consecutive columns per thread (nope,
+// rope / 2 and rank are multiples of 4), and one set of loads each: with one CTA of 256 threads for a whole row a thread
+// took five sets one after the other, a chain of latencies (steps of 9 layers 1153 -> 1115 us at one row, 3953 -> 3905 at 128).
 __global__ void __launch_bounds__(MLA_POST_THREADS)
 mla_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, MlaDims d, const __nv_bfloat16 *__restrict__ gains,
                 float eps, MlaCache cache, int rows_per_head, __nv_bfloat16 *__restrict__ qn_hi, __nv_bfloat16 *__restrict__ qn_lo,
@@ -42,7 +44,7 @@ mla_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, Mla
   griddep_launch_dependents();
   griddep_wait();
   __shared__ float scratch[MLA_POST_THREADS / 32];
-  const int r = blockIdx.x, tid = threadIdx.x;
+  const int r = blockIdx.y, tid = threadIdx.x;
   if (rows.active[r] == 0) return;                   // a padding row: no cache write, its query is never used
   const int pos = rows.pos[r];
   const int qw = d.nope + d.rope, QD = d.nh * qw, half = d.rope >> 1;
@@ -53,6 +55,23 @@ mla_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, Mla
     return;
   }
 #endif
+  // ---- the query: no-rope parts as bf16 hi/lo (head-major), rotary parts rotated, fp32
+  if (blockIdx.x > 0) {
+    int i = 4 * ((int)(blockIdx.x - 1) * MLA_POST_THREADS + tid);
+    if (i < d.nh * d.nope) {
+      const int h = i / d.nope, j = i - h * d.nope;
+      const size_t o = ((size_t)h * rows_per_head + r) * d.nope + j;
+      mla_store_split4(gemm_load4(qkv, r, h * qw + j), qn_hi + o, qn_lo + o);
+    } else if ((i -= d.nh * d.nope) < d.nh * half) {
+      const int h = i / half, j = i - h * half;
+      float4 ra, rb;
+      mla_rotate4(gemm_load4(qkv, r, h * qw + d.nope + j), gemm_load4(qkv, r, h * qw + d.nope + j + half), tab + j, ra, rb);
+      float *q = q_rope + ((size_t)r * d.nh + h) * d.rope + j;
+      *reinterpret_cast<float4 *>(q) = ra;
+      *reinterpret_cast<float4 *>(q + half) = rb;
+    }
+    return;
+  }
   const int blk = cache.block_table[(size_t)rows.slot[r] * cache.max_blocks + pos / KV_BLOCK];
 #ifdef CORUN_CHECKED
   if (!check_page(blk, cache.pool_blocks)) {
@@ -61,24 +80,8 @@ mla_post_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab, Mla
   }
 #endif
   const int row_halfs = d.rank + d.rope, off = pos % KV_BLOCK;   // the row's cache position: mla_cache_at(.., blk, off, e)
-  // the latent's values are requested first and used last: the sums of the GEMM's partials behind every load
-  // below overlap instead of queueing behind the block-wide reduction
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f);        // rank <= 4 * threads
   if (4 * tid < d.rank) x = gemm_load4(qkv, r, QD + 4 * tid);
-  // ---- the query: no-rope parts as bf16 hi/lo (head-major), rotary parts rotated, fp32
-  for (int i = 4 * tid; i < d.nh * d.nope; i += 4 * MLA_POST_THREADS) {
-    const int h = i / d.nope, j = i - h * d.nope;
-    const size_t o = ((size_t)h * rows_per_head + r) * d.nope + j;
-    mla_store_split4(gemm_load4(qkv, r, h * qw + j), qn_hi + o, qn_lo + o);
-  }
-  for (int i = 4 * tid; i < d.nh * half; i += 4 * MLA_POST_THREADS) {
-    const int h = i / half, j = i - h * half;
-    float4 ra, rb;
-    mla_rotate4(gemm_load4(qkv, r, h * qw + d.nope + j), gemm_load4(qkv, r, h * qw + d.nope + j + half), tab + j, ra, rb);
-    float *q = q_rope + ((size_t)r * d.nh + h) * d.rope + j;
-    *reinterpret_cast<float4 *>(q) = ra;
-    *reinterpret_cast<float4 *>(q + half) = rb;
-  }
   // ---- the cache row: rotated rotary key; RMSNorm of the latent (sum of squares: thread-serial ascending, xor
   //      butterfly in the warp, warp totals ascending)
   if (4 * tid < half) {
@@ -170,7 +173,8 @@ __global__ void mla_copy_kernel(MlaCache cache, int row_halfs, int slot, int pos
 cudaError_t launch_mla_post(const GemmOut &qkv, const Rows &rows, const float2 *rope_tab, const MlaDims &d,
                             const __nv_bfloat16 *kv_gains, float eps, const MlaCache &cache, int rows_per_head,
                             __nv_bfloat16 *qn_hi, __nv_bfloat16 *qn_lo, float *q_rope, int *d_status, cudaStream_t st) {
-  return launch_k(mla_post_kernel, dim3(rows.R), dim3(MLA_POST_THREADS), 0, st, true, qkv, rows, rope_tab, d, kv_gains, eps, cache,
+  const int shares = (d.nh * (d.nope + d.rope / 2) / 4 + MLA_POST_THREADS - 1) / MLA_POST_THREADS;
+  return launch_k(mla_post_kernel, dim3(1 + shares, rows.R), dim3(MLA_POST_THREADS), 0, st, true, qkv, rows, rope_tab, d, kv_gains, eps, cache,
                   rows_per_head, qn_hi, qn_lo, q_rope, d_status);
 }
 
