@@ -38,6 +38,7 @@ WORKLOADS = {
     # Mixture-of-Experts decoder (Qwen3-30B-A3B shape); no CPU baseline (the weights do not fit the host leg)
     "qwen3_30b_a3b_b64": (synth.QWEN3_30B_A3B, 64, 40, 512, 4096, 0.7, 0.95, 1.28),
 }
+PREFILL_ROWS = 2048   # rows of a long prompt's chunk (the layers' weights are streamed once per chunk)
 MOE = {"qwen3_30b_a3b_b64": (synth.QWEN3_30B_A3B_MOE, synth.QWEN3_30B_A3B_EFF)}
 # Decoder with multi-head latent attention and expert layers (DeepSeek-V2-Lite shape): 128 slots, all active
 MLA = {"deepseek_v2_lite_b128": (synth.DEEPSEEK_V2_LITE, synth.DEEPSEEK_V2_LITE_MLA, synth.DEEPSEEK_V2_LITE_MOE, 128, 128, 512, 4096, 0.7, 0.95, 0.5)}
@@ -290,21 +291,26 @@ def run_corun(args, rank, world):
     gemm_ms = L * (kt["gemm_qkv"] + kt["gemm_o"] + kt["gemm_gate_up"] + kt["gemm_down"]) + kt["gemm_lm_head"]
     n_gemm = 4 * L + 1                                 # (the small router GEMMs of an MoE model are left out)
     w_bytes = sh.weight_bytes_per_step()
+    # expert layers up to 64 slots: the step streams the experts that one of its rows selected (expected share of them)
+    met = 1.0
+    if moe_cfg and B <= 64:
+        met = 1.0 - (1.0 - moe_cfg[0]["top_k"] / moe_cfg[0]["n_experts"]) ** n_active
+    w_step = int(w_bytes - (1.0 - met) * 2 * 3 * sh.ffn * sh.hidden * L)
     cur_ctx = [eng.context_len(int(s)) for s in slots]
     kv_bytes = sum(c * sh.kv_bytes_per_token(2) for c in cur_ctx)
     kv_bytes_mid = sum((int(c) + W + K // 2) * sh.kv_bytes_per_token(2) for c in ctx)
     hbm, tf, which = measured_peaks()
-    flops = 2 * B * (w_bytes // 2) + 4 * sh.n_q_heads * sh.head_dim * sh.n_layers * sum(int(c) for c in ctx)
-    t_roof_ms = max((w_bytes + kv_bytes_mid) / (hbm * 1e9), flops / (tf * 1e12)) * 1e3
+    flops = 2 * B * (w_step / 2) + 4 * sh.n_q_heads * sh.head_dim * sh.n_layers * sum(int(c) for c in ctx)
+    t_roof_ms = max((w_step + kv_bytes_mid) / (hbm * 1e9), flops / (tf * 1e12)) * 1e3
     traffic = None
     tp = os.path.join(ROOT, "profiles", "gemm_dram_traffic.json")
     if os.path.exists(tp) and args.workload == "qwen3_8b_b64":
         traffic = json.load(open(tp)).get("dram_bytes_per_launch_avg")
     roofline = {
         "kernel": "gemm_streamk_kernel (all %d launches of a step)" % n_gemm, "bound": "hbm",
-        "achieved": (w_bytes / n_gemm) / (gemm_ms / n_gemm * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
+        "achieved": (w_step / n_gemm) / (gemm_ms / n_gemm * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
         "peak_source": which + " (MEASURED_PEAKS.json hbm_gbs)" if which == "measured" else "fallback 6650",
-        "traffic": traffic, "bytes_per_launch_avg": w_bytes / n_gemm, "ms_per_launch_avg": gemm_ms / n_gemm,
+        "traffic": traffic, "bytes_per_launch_avg": w_step / n_gemm, "ms_per_launch_avg": gemm_ms / n_gemm,
         "scope": "the dominant kernel only; the whole step against its roofline is in step_roofline",
         "timing": "CUDA events over back-to-back launches under programmatic stream serialization (a launch's first "
                   "weight stages overlap its predecessor's tail); launched one by one under a profiler the same kernels "
@@ -312,20 +318,20 @@ def run_corun(args, rank, world):
     }
     roofline["frac"] = roofline["achieved"] / hbm
     att_bytes = kv_bytes / L
-    step_roof = {"bytes": w_bytes + kv_bytes_mid, "flops": flops, "t_roofline_ms": t_roof_ms,
+    step_roof = {"bytes": w_step + kv_bytes_mid, "flops": flops, "t_roofline_ms": t_roof_ms,
                  "frac_of_" + which: t_roof_ms / ms_per_step,
-                 "frac_of_nominal_8TBs": max((w_bytes + kv_bytes_mid) / 8e12, flops / 2.25e15) * 1e3 / ms_per_step}
+                 "frac_of_nominal_8TBs": max((w_step + kv_bytes_mid) / 8e12, flops / 2.25e15) * 1e3 / ms_per_step}
     kernels = {k: ({"ms_per_launch": v} if v > 5e-4 else {"ms_per_launch": 0.0, "note": "no such launch: fused into a neighbour"})
                for k, v in kt.items()}
     for k, n in (("gemm_qkv", sh.qkv_dim * sh.hidden), ("gemm_o", sh.hidden * sh.q_dim),
-                 ("gemm_gate_up", 2 * sh.ffn * sh.hidden), ("gemm_down", sh.hidden * sh.ffn),
+                 ("gemm_gate_up", met * 2 * sh.ffn * sh.hidden), ("gemm_down", met * sh.hidden * sh.ffn),
                  ("gemm_lm_head", sh.vocab * sh.hidden)):
         kernels[k]["GBs"] = 2 * n / (kt[k] * 1e-3) / 1e9
     kernels["attention"]["GBs"] = att_bytes / (kt["attention"] * 1e-3) / 1e9
     launches = eng.decode_launches()
 
     # ---- isolated prefill of one request into a free slot (the other half of the hot path): wall time of
-    # corun_prefill with the prompt in host memory; roofline per 256-token chunk = max(executed MMA work at the
+    # corun_prefill with the prompt in host memory; roofline per chunk = max(executed MMA work at the
     # measured dense bf16 rate, the layers' weights streamed once), plus the LM head for the last position
     prefill = None
     free = [s for s in range(B) if not active[s]]
@@ -358,7 +364,7 @@ def run_corun(args, rank, world):
             w_mma = w_layers - (mc["n_experts"] - mc["top_k"]) * w_exp
         t_mma = t_hbm = 0.0
         while left > 0:
-            rows = min(256, left)
+            rows = min(PREFILL_ROWS, left)
             t_mma += 2 * 2 * (w_mma // 2) * rows / (tf_s * 1e12)
             t_hbm += w_layers / (hbm * 1e9)
             t_roof += max(2 * 2 * (w_mma // 2) * rows / (tf_s * 1e12), w_layers / (hbm * 1e9))
@@ -368,15 +374,15 @@ def run_corun(args, rank, world):
         t_alg = w_lm / (hbm * 1e9)
         left = n_pf
         while left > 0:
-            rows = min(256, left)
+            rows = min(PREFILL_ROWS, left)
             t_alg += max(2 * (w_mma // 2) * rows / (tf_s * 1e12), w_layers / (hbm * 1e9))
             left -= rows
         prefill = {"tokens": n_pf, "ms": dt * 1e3, "tok_per_s": n_pf / dt, "roofline_ms": t_alg * 1e3,
                    "frac": t_alg / dt, "executed_work_roofline_ms": t_roof * 1e3, "frac_of_executed_work": t_roof / dt,
                    "bound": "tensor" if t_mma >= t_hbm else "hbm",
-                   "note": "frac: per 256-token chunk the larger of the algorithmic MMA work (2 FLOPs per weight and token at "
+                   "note": "frac: per chunk of up to %d tokens the larger of the algorithmic MMA work (2 FLOPs per weight and token at "
                            "%.0f TFLOP/s sustained) and the layers' weights streamed once; frac_of_executed_work counts the "
-                           "two MMAs per weight tile that the bf16 hi/lo pair of the activations costs; attention not counted" % tf_s}
+                           "two MMAs per weight tile that the bf16 hi/lo pair of the activations costs; attention not counted" % (PREFILL_ROWS, tf_s)}
 
     # ---- the Mixture-of-Experts feed-forward block (DeepSeek-V2-Lite block shape, B = 128 padded rows): time per
     # call with CUDA events against the bytes of expert weights a call streams (rank 0, full-size workload only)
@@ -620,10 +626,11 @@ def run_corun_mla(args, rank, world):
         torch.cuda.synchronize()
         dt = time.perf_counter() - t0
         eng.release(s_pf)
-    chunks = -(-n_pf // 256)
+    chunks = -(-n_pf // PREFILL_ROWS)
     prefill = {"tokens": n_pf, "ms": dt * 1e3, "tok_per_s": n_pf / dt,
                "weights_streamed_once_per_chunk_ms": chunks * (w_bytes - 2 * sh.vocab * sh.hidden) / (hbm * 1e9) * 1e3,
-               "note": "chunks of 256 rows; expert layers in their grouped form; attention by the decode kernel row by row"}
+               "note": "chunks of up to %d rows; expert layers in their grouped form; keys and values decompressed once per "
+                       "chunk, attention in tiles of 128 query tokens" % PREFILL_ROWS}
     eng.close()
     del eng, w_t, m_t, e_t
     torch.cuda.empty_cache()
