@@ -132,8 +132,9 @@ int corun_init_moe(const corun_shape *shape, const corun_weights *weights, const
  * be NULL when first_dense == n_layers.
  *   kv_norm  L device pointers, bf16 [rank]          wkv_b  L device pointers, bf16 [n_q_heads * (qk_nope + v_head), rank]
  * kv_lora_rank 256 or 512; qk_nope a multiple of 64; qk_rope even, a multiple of 8, at most 64;
- * qk_nope + v_head a multiple of 256; n_q_heads * v_head a multiple of 64.  A decode step of B slots and a
- * prefill chunk run the same kernels; a prefill row attends to its request's cache up to its own position.
+ * qk_nope + v_head a multiple of 256; n_q_heads * v_head a multiple of 64.  A prefill row attends to its request's
+ * cache up to its own position: row by row as in a decode step for prompts of up to 128 tokens (and where qk_nope or
+ * v_head is not 128, or max_context is above 16384), else in tiles of 128 rows over keys and values decompressed per chunk.
  * kv_block may be 16 or 64 here: with 64 a slot's cache grows in blocks of 64 tokens (four pages of 16 tokens that
  * are neighbours in the pool, which the attention kernel fetches with one TMA box instead of four); kv_pool_blocks,
  * corun_free_blocks and corun_engine_info then count blocks of 64 tokens.  No value depends on the choice.
@@ -241,8 +242,9 @@ int64_t corun_free_blocks(corun_engine *e);
 /* The engine's fixed dimensions: slots, largest context, tokens per page, pages in the pool
  * (any of the out pointers may be NULL). */
 int corun_engine_info(corun_engine *e, int32_t *B, int32_t *max_context, int32_t *kv_block, int64_t *pool_blocks);
-/* How corun_prefill_batch packs prompts: rows per prefill chunk, and the row granularity on which every
- * piece of a request starts (the query tile of the prefill attention kernel).  Either pointer may be NULL. */
+/* How a scheduler should pack prompts for corun_prefill_batch: the rows it should count as one chunk, and the row
+ * granularity on which every piece of a request starts (the query tile of the prefill attention kernel).  Either pointer
+ * may be NULL. */
 int corun_prefill_geometry(corun_engine *e, int32_t *chunk_rows, int32_t *tile_rows);
 /* Number of kernel launches in one decode iteration. */
 int corun_decode_launches(corun_engine *e);
