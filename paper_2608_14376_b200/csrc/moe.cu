@@ -98,8 +98,12 @@ __device__ __forceinline__ void moe_route_row(LoadLogit load, int r, int lane, i
   if (sel) {                                         // ascending ids, the shared experts last
     int *out = sel + (size_t)r * (top_k + S);
     int place = 0;
-    for (int j = 0; j < top_k; ++j) place += __shfl_sync(0xffffffffu, id, j) < id ? 1 : 0;
-    if (lane < top_k) out[place] = on ? id : -1;
+    for (int j = 0; j < top_k; ++j) {
+      const int other = __shfl_sync(0xffffffffu, id, j);
+      place += other < id || (other == id && j < lane) ? 1 : 0;   // (a row of NaNs may pick an id twice)
+    }
+    // a probability that has vanished is no selection: the GEMMs neither compute nor store the row for that expert
+    if (lane < top_k) out[place] = on && wr[id] != 0.f ? id : -1;
     for (int s = lane; s < S; s += 32) out[top_k + s] = on ? E + s : -1;
   }
 }
@@ -489,7 +493,8 @@ __global__ void __launch_bounds__(256) moe_swiglu_grouped_kernel(const float *__
   }
 }
 
-// Selected-experts form: y[r, :] = the sum of the row's experts in ascending id; their rows sit at e * BN + r.
+// Selected-experts form: y[r, :] = the sum of the row's experts in ascending id; their rows sit at e * BN + r.  Negative
+// entries (a vanished weight, a row without a request) have no such row: what is there belongs to other rows and steps.
 __global__ void __launch_bounds__(256) moe_combine_select_kernel(const float *__restrict__ yg, const int *__restrict__ sel, int n_per_row,
                                                                  int BN, int H, float *__restrict__ y) {
   griddep_launch_dependents();
@@ -497,18 +502,22 @@ __global__ void __launch_bounds__(256) moe_combine_select_kernel(const float *__
   yg = after_wait(yg); sel = after_wait(sel);
   const int r = blockIdx.y, i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   const int *mine = sel + (size_t)r * n_per_row;
-  if (i >= H || mine[0] < 0) return;
+  if (i >= H) return;
+  bool any = false;                                  // a row without a request has no entry
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int k0 = 0; k0 < n_per_row; k0 += 8) {        // eight loads in flight; the additions stay in ascending order
+    int e[8];
     float4 v[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k0 + k < n_per_row) v[k] = *reinterpret_cast<const float4 *>(yg + ((size_t)mine[k0 + k] * BN + r) * H + i);
+    for (int k = 0; k < 8; ++k) {
+      e[k] = k0 + k < n_per_row ? mine[k0 + k] : -1;
+      if (e[k] >= 0) v[k] = *reinterpret_cast<const float4 *>(yg + ((size_t)e[k] * BN + r) * H + i);
+    }
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (k0 + k < n_per_row) { acc.x += v[k].x; acc.y += v[k].y; acc.z += v[k].z; acc.w += v[k].w; }
+      if (e[k] >= 0) { acc.x += v[k].x; acc.y += v[k].y; acc.z += v[k].z; acc.w += v[k].w; any = true; }
   }
-  *reinterpret_cast<float4 *>(y + (size_t)r * H + i) = acc;
+  if (any) *reinterpret_cast<float4 *>(y + (size_t)r * H + i) = acc;
 }
 
 __global__ void __launch_bounds__(256) moe_combine_kernel(const float *__restrict__ yg, const int *__restrict__ active, int NB,

@@ -20,8 +20,9 @@ cudaError_t launch_moe_router(const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_
                               int S, int top_k, int renormalize, float *w, int *experts, float *probs, const RouterScratch &rs,
                               cudaStream_t st, const int *active = nullptr, int *sel = nullptr);
 // (active, sel: when sel is not null, sel[r * (top_k + S) ..] receives the row's experts in ascending id, the shared ones
-// last, or -1 for a row with active[r] == 0)
-// y[r, :] = sum over the row's experts (sel, ascending) of yg[e * BN + r, :]; rows without experts are left alone.
+// last; -1 in the place of an expert whose weight is 0, and everywhere for a row with active[r] == 0)
+// y[r, :] = sum over the row's experts (sel, ascending; negative: none) of yg[e * BN + r, :]; rows without experts are left
+// alone.
 cudaError_t launch_moe_combine_select(const float *yg, const int *sel, int n_per_row, int BN, int R, int H, float *y, cudaStream_t st);
 // h[r, e*F + f] = w[r, e] * silu(gate) * up as a bf16 hi/lo pair (zeros where w[r, e] == 0); gate / up are
 // columns e*2F + f and e*2F + F + f of `gu`; n_blocks = E + S.
