@@ -64,6 +64,19 @@ int corun_debug_set_eager(corun_engine *e, int32_t eager);
  * (CORUN_EINVAL otherwise, before anything is launched).  Uses the engine-independent
  * kernel path (split activations, tcgen05 MMA, fixed K order). */
 int corun_debug_gemm(const void *W, int32_t N, int32_t K, const float *X, int32_t R, float *out, void *cuda_stream);
+/* Stand-alone run of the GEMM on pairs of SMs (long prompts, decode above 128 slots), X and W as above:
+ *   form 0  out [R, N] = X W^T, N % 8 == 0
+ *   form 1  N = 2F (F gate rows, then F up rows of W; F % 64 == 0): out [R, F] = silu(X Wg^T) * (X Wu^T)
+ *   form 2  N = 256 heads (per head 128 key rows, then 128 value rows): out [R, N] = X W^T by way of the fp16 hi / lo pairs
+ *           that the latent prefill attention reads
+ * (forms 1 and 2: the sum of the stored pair).  1 <= R <= 2048, K % 64 == 0; pointers as above. */
+int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, const float *X, int32_t R, float *out,
+                          void *cuda_stream);
+/* The attention kernel of long prompts for n query rows at positions pos0 .. pos0 + n - 1 of an occupied slot, over the layer's
+ * cached positions 0 .. pos0 + n - 1 (host arrays): q fp32 [n][n_q_heads][head_dim], latent attention [n][n_q_heads][qk_nope +
+ * qk_rope], both rotated; out fp32 [n][n_q_heads][head_dim (v_head)], the sum of the stored bf16 pair.  EINVAL where the engine
+ * takes no such kernel, or for more rows than a chunk has. */
+int corun_debug_prefill_attention(corun_engine *e, int32_t slot, int32_t layer, int32_t pos0, int32_t n, const float *q, float *out);
 /* R(seed, t) as the engine computes it (top 24 bits of the first Philox word), on the device. */
 int corun_debug_variate(uint64_t seed, uint64_t t, uint32_t *out_u24 /* host */);
 /* Runs the engine's sampler on host logits rows [n_rows, vocab] (copied to the device). */

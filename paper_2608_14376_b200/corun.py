@@ -20,7 +20,7 @@ EXPORTS = [
     "corun_init", "corun_init_moe", "corun_init_mla", "corun_prefill", "corun_prefill_batch", "corun_decode_step", "corun_decode_enqueue", "corun_decode_wait",
     "corun_release", "corun_destroy", "corun_get_logits", "corun_force_token", "corun_context_len",
     "corun_free_blocks", "corun_debug_kv_read", "corun_debug_kv_write", "corun_debug_adopt",
-    "corun_debug_set_eager", "corun_debug_read", "corun_debug_kv_fill", "corun_debug_time_kernel", "corun_decode_launches", "corun_debug_gemm", "corun_debug_variate",
+    "corun_debug_set_eager", "corun_debug_read", "corun_debug_kv_fill", "corun_debug_time_kernel", "corun_decode_launches", "corun_debug_gemm", "corun_debug_gemm_pair", "corun_debug_prefill_attention", "corun_debug_variate",
     "corun_debug_sample", "corun_debug_wait_probe", "corun_debug_microbench", "corun_debug_check_index", "corun_gemm_static", "corun_strerror", "corun_last_cuda_error", "corun_engine_info",
     "corun_sched_create", "corun_sched_create_for_engine", "corun_sched_destroy", "corun_sched_submit",
     "corun_sched_step", "corun_sched_poll", "corun_sched_slot_of", "corun_sched_counts",
@@ -141,6 +141,8 @@ def lib():
         L.corun_debug_time_kernel.argtypes = [vp, i32, i32, C.POINTER(C.c_float)]
         L.corun_decode_launches.argtypes = [vp]
         L.corun_debug_gemm.argtypes = [vp, i32, i32, vp, i32, vp, vp]
+        L.corun_debug_gemm_pair.argtypes = [i32, vp, i32, i32, vp, i32, vp, vp]
+        L.corun_debug_prefill_attention.argtypes = [vp, i32, i32, i32, i32, vp, vp]
         L.corun_debug_variate.argtypes = [u64, u64, C.POINTER(C.c_uint32)]
         L.corun_debug_sample.argtypes = [vp, i32, i32, C.POINTER(Sampling), vp, vp]
         L.corun_gemm_static.argtypes = [vp, i32, i32, vp, i32, vp, vp]
@@ -399,6 +401,14 @@ class Engine:
         _check(lib().corun_debug_read(self._h, which, out.ctypes.data, n), "corun_debug_read")
         return out
 
+    def prefill_attention(self, slot: int, layer: int, pos0: int, q) -> np.ndarray:
+        """The long prompts' attention kernel for query rows q [n, heads, dims] at positions pos0 .."""
+        q = np.ascontiguousarray(q, dtype=np.float32)
+        out = np.empty(q.shape[:2] + (self._mla["v_head"] if getattr(self, "_mla", None) else q.shape[2],), np.float32)
+        _check(lib().corun_debug_prefill_attention(self._h, slot, layer, pos0, q.shape[0], q.ctypes.data, out.ctypes.data),
+               "corun_debug_prefill_attention")
+        return out
+
     def set_eager(self, eager: bool):
         _check(lib().corun_debug_set_eager(self._h, int(eager)), "set_eager")
 
@@ -476,6 +486,18 @@ def debug_gemm(W, X):
     out = torch.empty((R, N), dtype=torch.float32, device=X.device)
     torch.cuda.synchronize()
     _check(lib().corun_debug_gemm(W.data_ptr(), N, K, X.data_ptr(), R, out.data_ptr(), None), "corun_debug_gemm")
+    return out
+
+
+def debug_gemm_pair(form, W, X):
+    """The GEMM on pairs of SMs (``corun_debug_gemm_pair``): form 0 plain, 1 with SwiGLU (result [R, N / 2]), 2 keys and values."""
+    import torch
+
+    N, K = W.shape
+    R = X.shape[0]
+    out = torch.empty((R, N // 2 if form == 1 else N), dtype=torch.float32, device=X.device)
+    torch.cuda.synchronize()
+    _check(lib().corun_debug_gemm_pair(form, W.data_ptr(), N, K, X.data_ptr(), R, out.data_ptr(), None), "corun_debug_gemm_pair")
     return out
 
 

@@ -639,6 +639,18 @@ GemmOut ffn_out(const corun_engine *e, const Program &P, int layer) {
   return P.p_down.out();
 }
 
+// Latent attention of a chunk of long prompts: the segments' keys and values, then their tiles of 128 query tokens.
+cudaError_t run_mla_tiles(corun_engine *e, Program &P, int l, const Rows &rows) {
+  const MlaDims &md = e->md;
+  const MlaCache cache{e->kv_pool + (size_t)l * e->layer_stride, e->d_block_table, e->max_blocks, e->B, (long long)e->pool_blocks, e->kv_run};
+  cudaError_t ce = launch_mla_gather(P.segs, cache, md.rank, md.rope, P.kv_tokens, P.c_hi, P.c_lo, P.kr, e->st);
+  if (ce == cudaSuccess) ce = gemm_pair_launch(P.b_kv, e->tb_uv[l], P.kv_tokens, e->d_status, e->st);
+  if (ce == cudaSuccess)
+    ce = launch_mla_prefill(P.tm_kvd, P.tm_kr, P.qn_hi, P.qn_lo, P.q_rope, rows, P.RPH, md, P.kv_cap, P.tile_base,
+                            1.0f / sqrtf((float)(md.nope + md.rope)), P.ao_hi, P.ao_lo, e->d_status, e->st);
+  return ce;
+}
+
 // Enqueues embed -> all layers (ends with the last down GEMM; prefill: with the final norm of every row).  Counts launches.
 int run_layers(corun_engine *e, Program &P, int *launches) {
   const corun_shape &s = e->sh;
@@ -691,23 +703,20 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
                                 P.qn_lo + r0 * md.nope, P.q_rope + r0 * md.nh * md.rope, e->d_status, e->st));
         }
         if (P.mla_tiles && !P.shorts) {
-          STAGE(launch_mla_gather(P.segs, cache, md.rank, md.rope, P.kv_tokens, P.c_hi, P.c_lo, P.kr, e->st));
-          STAGE(gemm_pair_launch(P.b_kv, e->tb_uv[l], P.kv_tokens, e->d_status, e->st));
-          STAGE(launch_mla_prefill(P.tm_kvd, P.tm_kr, P.qn_hi, P.qn_lo, P.q_rope, rows, P.RPH, md, P.kv_cap, P.tile_base,
-                                   1.0f / sqrtf((float)(md.nope + md.rope)), P.ao_hi, P.ao_lo, e->d_status, e->st));
+          STAGE(run_mla_tiles(e, P, l, rows));
         } else {
-        STAGE(gemm_launch(P.p_uk, &e->tm_uk[l], e->d_status, e->st, nullptr, true));
-        for (int r0 = 0; r0 < P.R; r0 += MLA_ROWS) {
-          const int nr = P.R - r0 < MLA_ROWS ? P.R - r0 : MLA_ROWS;
-          const Rows part{P.row_token + r0, P.row_pos + r0, P.row_active + r0, P.row_slot + r0, nr};
-          STAGE(launch_mla_attention(e->tm_c[l], e->tm_cv[l], P.q_lat + (size_t)r0 * md.rank, md.rank, (long long)P.RPH * md.rank,
-                                     P.q_rope + (size_t)r0 * md.nh * md.rope, e->d_block_table, e->max_blocks, nullptr, &part, nr, md,
-                                     1.0f / sqrtf((float)(md.nope + md.rope)), e->mla_splits, P.mla_ml, P.mla_po, nullptr,
-                                     P.ol_hi + (size_t)r0 * md.rank, P.ol_lo + (size_t)r0 * md.rank, P.RPH, e->num_sms, e->d_status, true,
-                                     e->st, e->kv_run));
-        }
-        STAGE(gemm_launch(P.p_uv, &e->tm_uv[l], e->d_status, e->st, nullptr, true));
-        STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
+          STAGE(gemm_launch(P.p_uk, &e->tm_uk[l], e->d_status, e->st, nullptr, true));
+          for (int r0 = 0; r0 < P.R; r0 += MLA_ROWS) {
+            const int nr = P.R - r0 < MLA_ROWS ? P.R - r0 : MLA_ROWS;
+            const Rows part{P.row_token + r0, P.row_pos + r0, P.row_active + r0, P.row_slot + r0, nr};
+            STAGE(launch_mla_attention(e->tm_c[l], e->tm_cv[l], P.q_lat + (size_t)r0 * md.rank, md.rank, (long long)P.RPH * md.rank,
+                                       P.q_rope + (size_t)r0 * md.nh * md.rope, e->d_block_table, e->max_blocks, nullptr, &part, nr, md,
+                                       1.0f / sqrtf((float)(md.nope + md.rope)), e->mla_splits, P.mla_ml, P.mla_po, nullptr,
+                                       P.ol_hi + (size_t)r0 * md.rank, P.ol_lo + (size_t)r0 * md.rank, P.RPH, e->num_sms, e->d_status, true,
+                                       e->st, e->kv_run));
+          }
+          STAGE(gemm_launch(P.p_uv, &e->tm_uv[l], e->d_status, e->st, nullptr, true));
+          STAGE(launch_mla_ao_split(P.uv_out, P.R, P.RPH, md, P.ao_hi, P.ao_lo, e->st));
         }
       } else {
         if (!P.shorts) STAGE(launch_qkv_post(gemm_pair_out(P.b_qkv, P.R, P.plain_tiles), rows, e->d_rope, s.n_q_heads, kv, l, P.q, e->d_status, e->st));
@@ -2002,6 +2011,110 @@ int corun_debug_gemm(const void *W, int32_t N, int32_t K, const float *X, int32_
   gemm_plan_destroy(&p);
   for (void *q : keep) cudaFree(q);
   return rc;
+}
+
+int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, const float *X, int32_t R, float *out,
+                          void *cuda_stream) {
+  if (form < 0 || form > 2 || !W || !X || !out || N < 8 || K < 64 || K % 64 || R < 1 || R > PREFILL_BIG) return CORUN_EINVAL;
+  if (form == 0 ? N % 8 : form == 1 ? N % 128 : N % GEMM_TILE_N) return CORUN_EINVAL;
+  if (((uintptr_t)out & 15u) || ((uintptr_t)W & 15u) || ((uintptr_t)X & 3u)) return CORUN_EINVAL;
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  int dev = 0, sms = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int cap = (R + 255) / 256 * 256, F = N / 2, nh = N / GEMM_TILE_N;
+  const size_t c = (size_t)cap;
+  std::vector<void *> keep;
+  bf16 *hi = nullptr, *lo = nullptr, *ohi = nullptr, *olo = nullptr;
+  __half *kv = nullptr;
+  float *part = nullptr, *full = nullptr;
+  int *status = nullptr, rc = CORUN_OK;
+  GemmPairPlan p;
+  CUtensorMap tw, tw96;
+  auto ok = [&](int r) { return (rc = r) == CORUN_OK; };
+  if (ok(dmalloc(keep, &hi, c * K)) && ok(dmalloc(keep, &lo, c * K)) && ok(dmalloc(keep, &status, 1)) &&
+      ok(gemm_encode_map(&tw, W, N, K, 128)) && ok(gemm_encode_map(&tw96, W, N, K, 96))) {
+    if (form == 0)
+      ok(dmalloc(keep, &part, gemm_pair_part_floats(N, K, cap, sms))) && ok(dmalloc(keep, &full, c * N)) &&
+          ok(gemm_pair_plan_create(&p, N, K, hi, lo, cap, full, part, sms));
+    else if (form == 1)
+      ok(dmalloc(keep, &ohi, c * F)) && ok(dmalloc(keep, &olo, c * F)) && ok(gemm_pair_plan_create_swiglu(&p, F, K, hi, lo, cap, ohi, olo, sms));
+    else
+      ok(dmalloc(keep, &kv, 4 * c * nh * 128)) && ok(gemm_pair_plan_create_kv(&p, nh, K, hi, lo, cap, kv, sms));
+  }
+  if (rc == CORUN_OK) {
+    cudaError_t ce = cudaDeviceSynchronize();       // allocations were cleared through the legacy stream
+    if (ce == cudaSuccess) ce = launch_split(X, R, K, hi, lo, st);
+    if (ce == cudaSuccess) ce = gemm_pair_launch(p, tw, R, status, st, form == 1 ? &tw96 : nullptr);
+    if (ce == cudaSuccess && form == 0) ce = gemm_pair_fixup_launch(p, R, st);
+    if (ce == cudaSuccess && form == 0) ce = cudaMemcpyAsync(out, full, (size_t)R * N * sizeof(float), cudaMemcpyDeviceToDevice, st);
+    if (ce == cudaSuccess && form == 1) ce = launch_join(ohi, olo, false, R, F, out, F, st);
+    for (int i = 0; form == 2 && i < 2 * nh && ce == cudaSuccess; ++i) {   // head i / 2: its keys, its values
+      const __half *a = kv + ((size_t)(2 * (i & 1)) * nh + i / 2) * c * 128;
+      ce = launch_join(a, a + c * nh * 128, true, R, 128, out + i * 128, N, st);
+    }
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+    int hs = 0;
+    if (ce == cudaSuccess) ce = cudaMemcpy(&hs, status, sizeof(int), cudaMemcpyDeviceToHost);
+    if (ce != cudaSuccess) { g_last_cuda_error = (int)ce; rc = CORUN_ECUDA; }
+    else if (hs != 0) rc = CORUN_ETIMEOUT;
+  }
+  for (void *q : keep) cudaFree(q);
+  return rc;
+}
+
+int corun_debug_prefill_attention(corun_engine *e, int32_t slot, int32_t layer, int32_t pos0, int32_t n, const float *q, float *out) {
+  if (!e || !q || !out || pos0 < 0 || n < 1 || layer < 0 || layer >= e->sh.n_layers) return CORUN_EINVAL;
+  if (!slot_ok(e, slot) || !e->in_use[slot]) return CORUN_ESLOT;
+  Program &P = e->big;
+  if (!P.pair || n > P.cap || pos0 + n > e->ctx[slot] || (e->mla && !P.mla_tiles)) return CORUN_EINVAL;
+  RC(sync_stream(e));
+  const corun_shape &s = e->sh;
+  const MlaDims &md = e->md;
+  std::vector<int> rows((size_t)4 * n, 0);           // token | position | active | slot
+  for (int i = 0; i < n; ++i) { rows[(size_t)n + i] = pos0 + i; rows[(size_t)2 * n + i] = 1; rows[(size_t)3 * n + i] = slot; }
+  P.R = n;
+  P.row_pos = P.row_token + n;
+  P.row_active = P.row_pos + n;
+  P.row_slot = P.row_active + n;
+  const Rows r{P.row_token, P.row_pos, P.row_active, P.row_slot, n};
+  cudaError_t ce = cudaMemcpyAsync(P.row_token, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice, e->st);
+  const int width = e->mla ? md.nh * md.vh : s.n_q_heads * s.head_dim;
+  float *tmp = nullptr;
+  if (cudaMalloc(&tmp, (size_t)n * (e->mla ? md.nh * (md.nope + md.rope) : width) * sizeof(float)) != cudaSuccess) return CORUN_ENOMEM;
+  std::vector<float> part;
+  if (!e->mla) {
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(P.q, q, (size_t)n * width * sizeof(float), cudaMemcpyHostToDevice, e->st);
+    if (ce == cudaSuccess) ce = launch_attention_prefill(e->tm_k4[layer], P.q, r, s.n_q_heads, kv_layout(e), P.ao_hi, P.ao_lo, e->d_status, e->st);
+  } else {
+    const int qw = md.nope + md.rope, rph = (n + 63) / 64 * 64;
+    P.RPH = rph;
+    part.resize((size_t)n * qw);
+    for (int h = 0; h < md.nh && ce == cudaSuccess; ++h) {           // a head's no-rope parts, head-major
+      for (int i = 0; i < n; ++i) memcpy(&part[(size_t)i * md.nope], q + ((size_t)i * md.nh + h) * qw, md.nope * sizeof(float));
+      const size_t at = (size_t)h * rph * md.nope;
+      ce = cudaMemcpyAsync(tmp, part.data(), (size_t)n * md.nope * sizeof(float), cudaMemcpyHostToDevice, e->st);
+      if (ce == cudaSuccess) ce = launch_split(tmp, n, md.nope, P.qn_hi + at, P.qn_lo + at, e->st);
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(e->st);
+    }
+    part.resize((size_t)n * md.nh * md.rope);
+    for (int i = 0; i < n * md.nh; ++i) memcpy(&part[(size_t)i * md.rope], q + (size_t)i * qw + md.nope, md.rope * sizeof(float));
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(P.q_rope, part.data(), part.size() * sizeof(float), cudaMemcpyHostToDevice, e->st);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(P.tile_base, 0, (size_t)(P.cap / 128) * sizeof(int), e->st);
+    P.segs.n = 1;
+    P.segs.slot[0] = slot;
+    P.segs.off[0] = 0;
+    P.segs.len[0] = pos0 + n;
+    P.kv_tokens = (pos0 + n + 63) / 64 * 64;
+    if (ce == cudaSuccess) ce = run_mla_tiles(e, P, layer, r);
+  }
+  if (ce == cudaSuccess) ce = launch_join(P.ao_hi, P.ao_lo, false, n, width, tmp, width, e->st);
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, tmp, (size_t)n * width * sizeof(float), cudaMemcpyDeviceToHost, e->st);
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(e->h_status, e->d_status, sizeof(int), cudaMemcpyDeviceToHost, e->st);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(e->st);
+  cudaFree(tmp);
+  if (ce != cudaSuccess) { g_last_cuda_error = (int)ce; return CORUN_ECUDA; }
+  return check_status(e);
 }
 
 int corun_debug_variate(uint64_t seed, uint64_t t, uint32_t *out_u24) {

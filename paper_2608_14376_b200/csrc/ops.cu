@@ -900,6 +900,12 @@ __global__ void set_slot_kernel(SlotArrays a, int slot, int in_use, int ctx, int
   a.top_p[slot] = top_p;
 }
 
+template <typename T>
+__global__ void join_kernel(const T *hi, const T *lo, size_t n, int cols, float *out, int pitch) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i / cols * pitch + i % cols] = (float)hi[i] + (float)lo[i];
+}
+
 __global__ void kv_copy_kernel(KvLayout kv, int layer, int slot, int pos0, int n, float *k, float *v, int write) {
   const int KD = kv.n_kv * kv.hd;
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -978,6 +984,14 @@ cudaError_t launch_swiglu(const GemmOut &gu, int R, int F, __nv_bfloat16 *out_hi
 cudaError_t launch_split(const float *x, int R, int K, __nv_bfloat16 *hi, __nv_bfloat16 *lo, cudaStream_t st) {
   const size_t n = (size_t)R * K;
   split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, n, hi, lo);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_join(const void *hi, const void *lo, bool is_fp16, int rows, int cols, float *out, int pitch, cudaStream_t st) {
+  const size_t n = (size_t)rows * cols;
+  const unsigned blocks = (unsigned)((n + 255) / 256);
+  if (is_fp16) join_kernel<<<blocks, 256, 0, st>>>((const __half *)hi, (const __half *)lo, n, cols, out, pitch);
+  else join_kernel<<<blocks, 256, 0, st>>>((const __nv_bfloat16 *)hi, (const __nv_bfloat16 *)lo, n, cols, out, pitch);
   return cudaGetLastError();
 }
 

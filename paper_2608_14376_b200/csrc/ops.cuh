@@ -91,6 +91,8 @@ cudaError_t attention_prepare();   // opts the kernels into their shared-memory 
 cudaError_t launch_swiglu(const GemmOut &gu, int R, int F, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, cudaStream_t st);
 // x fp32 [R, K] -> bf16 hi/lo.
 cudaError_t launch_split(const float *x, int R, int K, __nv_bfloat16 *hi, __nv_bfloat16 *lo, cudaStream_t st);
+// out[r * pitch + c] = (hi + lo)[r * cols + c]; the pair is bf16 or fp16 (is_fp16).
+cudaError_t launch_join(const void *hi, const void *lo, bool is_fp16, int rows, int cols, float *out, int pitch, cudaStream_t st);
 cudaError_t launch_sampler(const SampleArgs &a, int R, cudaStream_t st, bool pdl = false);
 // decode bookkeeping
 // The step's inputs (active mask, seeds) and results (tokens, status word) live in pinned host memory and are

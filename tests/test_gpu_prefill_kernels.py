@@ -1,0 +1,88 @@
+"""The kernels of long prompts run by themselves against 64-bit arithmetic: the attention of a chunk's rows over the slot's
+cached positions."""
+import numpy as np
+import pytest
+
+from paper_2608_14376_b200 import synth
+from tests.helpers import have_gpu
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not have_gpu(), reason="needs a GPU")]
+
+HALF_ULP = 2.0 ** -11       # a weight in fp16 (11 significant bits) is off by at most this share of itself
+
+
+def _dense(nq, nkv, hd, T):
+    from paper_2608_14376_b200 import corun
+
+    sh = synth.ModelShape(1, 256, nq, nkv, hd, 256, 512, 1e-6, 10000.0)
+    return corun.Engine(sh, synth.weights_numpy_to_torch(synth.make_weights_numpy(sh, seed=1), "cuda"), 2, T)
+
+
+def _fill(eng, slot, k, v):
+    eng.adopt(slot, 0, k.shape[0], 0)
+    eng.kv_write(slot, 0, 0, k, v)
+    return eng.kv_read(slot, 0, 0, k.shape[0])
+
+
+def _attend(q, k, v, pos0, scale):
+    """q [n, nq, d], k [T, nkv, d], v [T, nkv, dv] -> (output, sqrt(sum p^2 v^2)) in fp64; row i sees positions 0 .. pos0 + i."""
+    q, k, v = (np.asarray(x, np.float64) for x in (q, k, v))
+    G = q.shape[1] // k.shape[1]
+    out, spread = np.empty(q.shape[:2] + v.shape[2:]), np.empty(q.shape[:2] + v.shape[2:])
+    for i in range(q.shape[0]):
+        T = pos0 + i + 1
+        for h in range(q.shape[1]):
+            s = k[:T, h // G] @ q[i, h] * scale
+            p = np.exp(s - s.max())
+            p /= p.sum()
+            out[i, h] = p @ v[:T, h // G]
+            spread[i, h] = np.sqrt((p * p) @ (v[:T, h // G] ** 2))
+    return out, spread
+
+
+# group sizes 8, 4, 2, 1 and both head widths; one row, ragged tiles, several blocks of 128 keys, keys of an earlier chunk
+@pytest.mark.parametrize("nq,nkv,hd,pos0,n", [(8, 1, 128, 0, 1), (8, 2, 128, 0, 77), (8, 2, 128, 500, 33), (4, 2, 64, 0, 130),
+                                              (4, 4, 64, 700, 5), (16, 2, 64, 127, 18), (2, 2, 128, 255, 129)])
+def test_prefill_attention_matches_fp64(nq, nkv, hd, pos0, n):
+    rng = np.random.default_rng(nq + hd + n)
+    T = pos0 + n
+    eng = _dense(nq, nkv, hd, T)
+    try:
+        k, v = _fill(eng, 1, *(rng.standard_normal((T, nkv * hd)).astype(np.float32) for _ in range(2)))
+        q = (8 * rng.standard_normal((n, nq, hd))).astype(np.float32)          # scores of +-8
+        got = eng.prefill_attention(1, 0, pos0, q)
+    finally:
+        eng.close()
+    k, v = k.reshape(T, nkv, hd), v.reshape(T, nkv, hd)
+    want, spread = _attend(q, k, v, pos0, hd ** -0.5)
+    rms = lambda x: np.sqrt(np.mean(np.square(x)))
+    # rounding of the weights to fp16: an error uniform in +-half an ulp is 0.73 / sqrt(3) of HALF_ULP in the mean over the
+    # binade; beside it 2^-17 of the result (stored as a bf16 pair) and scores of up to 40 in fp32
+    bound = 1.25 * 0.73 / np.sqrt(3) * HALF_ULP * rms(spread) + 1e-5 * rms(want)
+    assert rms(got - want) <= bound, (rms(got - want), bound)
+    # queries in half the precision (their fp16 part alone) would not pass
+    if T > 100:
+        assert rms(_attend(q.astype(np.float16), k, v, pos0, hd ** -0.5)[0] - want) > bound
+
+
+@pytest.mark.parametrize("hd", [64, 128])
+def test_a_blocks_largest_weight_is_exact(hd):
+    """One key per block of 128 carries the block's weight: fp16 weights are 1 for it, whatever the other blocks hold, so
+    the result has the accuracy of its fp32 sums (a weight rounded to fp16 would be off by up to 5e-4 of itself)."""
+    rng = np.random.default_rng(hd)
+    T, A = 128 * 5 + 40, 32.0
+    k = np.zeros((T, hd), np.float32)
+    k[:, 0] = -40 * hd ** 0.5 / A
+    top = [5, 130, 300, 511, 512, T - 3]
+    k[top, 0] = np.array([-0.31, -1.27, 0.13, -0.74, -2.09, -0.55]) * hd ** 0.5 / A
+    v = rng.standard_normal((T, hd)).astype(np.float32)
+    q = np.zeros((1, 1, hd), np.float32)
+    q[0, 0, 0] = A
+    eng = _dense(1, 1, hd, T)
+    try:
+        k, v = _fill(eng, 1, k, v)
+        got = eng.prefill_attention(1, 0, T - 1, q)
+    finally:
+        eng.close()
+    want, _ = _attend(q, k.reshape(T, 1, hd), v.reshape(T, 1, hd), T - 1, hd ** -0.5)
+    assert np.abs(got - want).max() <= 2e-5 * np.abs(want).max() + 2 ** -17 * np.abs(want).max()
