@@ -213,23 +213,22 @@ int tma_encode_fp16_4d(CUtensorMap *m, const void *base, const unsigned long lon
 // The same with 2 to 5 dimensions (dims / box: nd values, strides: nd - 1 byte strides of dimensions 1 ..).
 int tma_encode_fp16_nd(CUtensorMap *m, const void *base, int nd, const unsigned long long *dims, const unsigned long long *strides,
                        const unsigned *box);
-// ---- many rows (gemm_pair.cu): tiles of 256 rows x 256 weight rows, one per pair of SMs, whole K, no partials ----
+// ---- many rows (gemm_pair.cu): tiles of 256 rows x 256 weight rows, one per pair of SMs; K in up to 8 slices, and the tiles of
+// an unfilled wave are left as partial matrices, a slice each: `out` alone is not the result (gemm_pair_out) ----
 struct GemmPairPlan {
   CUtensorMap tmHi, tmLo, tmOut, tmOut2;
   int N = 0, K = 0, cap = 0, pairs = 0, n_tiles = 0;   // weight rows, reduction length, rows the buffers hold
-  int slices = 1;                    // cuts of K (gemm_pair_slices)
+  int slices = 1, per_unit = 1;      // cuts of K, a function of the matrix and the GPU, never of the rows; slices per unit of work
   bool swiglu = false;
   int kv_heads = 0;                  // gemm_pair_plan_create_kv
   float *out = nullptr, *part = nullptr;   // not owned
   const int *row_blocks = nullptr;   // device, not owned (cap 256): bit 1 = rows 128 .. hold a request; null = they do
 };
-// Into how many slices K is cut: a function of the matrix and the GPU, never of the rows.
-int gemm_pair_slices(int N, int K, int num_sms);
 // Floats of partial tiles that launches over up to cap rows leave (the next kernel of the stream consumes them, so one
 // buffer serves all plans of a program).
 size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms);
 // X W^T for activations Xhi / Xlo [cap, K] (N % 8 == 0) -> out [cap, N] fp32 and, for the tiles of an unfilled wave, part
-// (gemm_pair_part_floats; null: one slice).  Read through gemm_pair_out(p, R, zeros).
+// (gemm_pair_part_floats).  Read through gemm_pair_out(p, R, zeros).
 int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms);
 GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles);
 int gemm_pair_has_parts(const GemmPairPlan &p, int R);   // 1 if some of the result of R rows is left in partial matrices

@@ -14,6 +14,7 @@ namespace {
 constexpr int PG_THREADS = 320;                     // warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue
 constexpr int PG_EPI = 8;                           // epilogue warps: two per TMEM lane quarter, half of the columns each
 constexpr int PG_STAGES = 4;
+constexpr int PG_CHAIN = 16;                        // k-blocks that are summed in one accumulator (see below)
 enum : int { PG_PLAIN = 0, PG_SWIGLU = 1, PG_KV = 2 };
 constexpr uint32_t PG_X_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: a CTA's 128 activation rows, hi or lo
 constexpr uint32_t PG_W_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: a CTA's half of the 256 weight rows
@@ -32,10 +33,15 @@ constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + PG_EPI * 
 //
 // K is cut into `slices` (a function of N, K and the number of SMs): a slice is summed in one accumulator, the slices in
 // ascending order in fp32.  A pair that has a whole tile does both itself (the running sum in the epilogue's registers);
-// the tiles that do not fill a wave of the pairs are dealt out slice by slice, each leaving a partial matrix, and the
-// consumer adds them in the same order (gemm_load_pair4).  So a row's result depends on its own activations only, not on
-// its place among the rows nor on their number: 256 rows of the Qwen3-8B QKV projection are 24 tiles, 72 units of a third
-// of K each for 74 pairs (43 us as 24 whole tiles).
+// the tiles that do not fill a wave of the pairs are dealt out in units of `per_unit` slices, every slice leaving a partial
+// matrix, and the consumer adds them in the same order (gemm_load_pair4).  So a row's result depends on its own activations
+// only, not on its place among the rows nor on their number: 256 rows of the Qwen3-8B QKV projection are 24 tiles, 72 units
+// of a third of K each for 74 pairs (43 us as 24 whole tiles).
+//
+// A slice is short because the tensor core's accumulator cuts every sum off: a product is off by 1.7e-8 (2-norm, relative) per
+// MMA of a slice, K = 4096 in one accumulator (512 MMAs, hi and lo) by 9e-6, slices of 16 k-blocks by 2.2e-6 beside the 2.5e-6
+// of the activations' 16 bits.  Prompts of 300 / 1003 tokens, 12 Qwen3-8B layers, against 64 bits: 1.1e-4 / 6.7e-5 with the
+// gate / up matrix in one slice and 3 or 4 of the others, 9.6e-5 / 5.3e-5 so (8 k-blocks: no nearer, and 3 % slower).
 //
 // Launched in plain stream order (no programmatic launch): a pair's two SMs are taken and left together, never while a
 // CTA of a neighbouring kernel of the stream is on one of them.
@@ -44,7 +50,7 @@ constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + PG_EPI * 
 // time share weight tiles in L2 and the weights are read from HBM once.
 //
 // SWIGLU: W is a gate / up matrix ([2F, K]); a tile is `half` gate rows (first CTA) and the up rows of the same outputs
-// (second CTA), whole K, and the epilogue writes silu(gate) * up as the bf16 hi/lo pair the down GEMM reads.
+// (second CTA), always whole (the slices meet in registers), and the epilogue writes silu(gate) * up as the bf16 hi/lo pair the down GEMM reads.
 // KV (gemm_pair_plan_create_kv): a tile's 256 columns are one head's 128 key and 128 value columns, stored as fp16 hi / lo
 // pairs, keys by the first half of the epilogue warps, values by the second; cap: rows of one of the four matrices per head.
 template <int MODE>
@@ -52,7 +58,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                  const __grid_constant__ CUtensorMap tmLo, const __grid_constant__ CUtensorMap tmOut,
                  const __grid_constant__ CUtensorMap tmOut2, int R, int N, int KB, int row_tiles, int whole, int units, int slices,
-                 int half, int *status, const int *row_blocks, int cap) {
+                 int per_unit, int half, int *status, const int *row_blocks, int cap) {
   constexpr bool SWIGLU = MODE == PG_SWIGLU, KV = MODE == PG_KV;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[PG_STAGES];      // used in the first CTA: both CTAs' loads of a stage
@@ -105,12 +111,12 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   volatile int *abort_p = &abort_flag;
   int fail = 0;
 
-  // Work unit u: a whole tile (all slices in turn), or one slice of a tile beyond the `whole` first ones.
+  // Work unit u: a whole tile (all slices in turn), or per_unit slices of a tile beyond the `whole` first ones.
   struct Unit { int tile, s0, s1; };
   auto unit = [&](int u) {
     if (u < whole) return Unit{u, 0, slices};
-    const int v = u - whole, t = v / slices, sl = v - t * slices;
-    return Unit{whole + t, sl, sl + 1};
+    const int v = u - whole, n = slices / per_unit, t = v / n, sl = (v - t * n) * per_unit;
+    return Unit{whole + t, sl, sl + per_unit};
   };
   auto cut = [&](int sl) { return sl * KB / slices; };       // first k-block of a slice
 
@@ -194,7 +200,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       const Unit un = unit(u);
       const int nt = un.tile / row_tiles;
       const int row0 = (un.tile % row_tiles) * 256 + rank * 128 + lane_base;   // this warp's 32 rows
-      float sum[128];                               // (PLAIN) this thread's row, 128 columns
+      const bool part = u >= whole;                 // its slices go to partial matrices, a whole tile to the output
+      float sum[128];                               // this thread's row: 128 columns (SWIGLU: up to 64 gate and 64 up columns)
+      // first accumulator column of the sums 8 q ..; SWIGLU: blocks of 32 outputs, gate then up columns of each
+      auto acc_col = [&](int q) { return SWIGLU ? grp * 32 + (q >> 3) * 64 + ((q >> 2) & 1) * half + (q & 3) * 8 : grp * 128 + q * 8; };
       for (int sl = un.s0; sl < un.s1; ++sl, ++seg) {
         const int acc = seg & 1;
         ok = mbar_wait(smem_u32(&tmem_full_bar[acc]), (uint32_t)(seg >> 1) & 1u, abort_p);
@@ -203,39 +212,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         tc_fence_after();
         const uint32_t ta = tmem_base + (uint32_t)acc * GEMM_TILE_N + lane_off;
         if (row0 < R) {                             // warp-uniform
-          if (SWIGLU) {
-            for (int c0 = grp * 32; c0 < half; c0 += 64) {
-              const int col = nt * half + c0;
-              if (col >= (N >> 1)) break;
-              uint32_t g[32], up[32];
-              tmem_ld32(ta + (uint32_t)c0, g);
-              tmem_ld32(ta + (uint32_t)(half + c0), up);
-              if (lane == 0) bulk_wait_read<0>();   // the staging tile has been read
-              __syncwarp();
-              tmem_ld_wait();
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {         // 16 bytes = 8 outputs; 64-byte rows, 64-byte swizzle
-                __nv_bfloat16 a[8], b[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const float gt = __uint_as_float(g[8 * q + j]);
-                  const float y = gt / (1.f + expf(-gt)) * __uint_as_float(up[8 * q + j]);
-                  a[j] = __float2bfloat16_rn(y);
-                  b[j] = __float2bfloat16_rn(y - __bfloat162float(a[j]));
-                }
-                const uint32_t off = (uint32_t)lane * 64 + (((uint32_t)q ^ (((uint32_t)lane >> 1) & 3u)) << 4);
-                *reinterpret_cast<uint4 *>(stg_p + off) = *reinterpret_cast<const uint4 *>(a);
-                *reinterpret_cast<uint4 *>(stg_p + PG_OUT_BYTES / 2 + off) = *reinterpret_cast<const uint4 *>(b);
-              }
-              fence_proxy_async();
-              __syncwarp();
-              if (lane == 0) {
-                tma_store_2d(&tmOut, stg, col, row0);
-                tma_store_2d(&tmOut2, stg + PG_OUT_BYTES / 2, col, row0);
-                bulk_commit();
-              }
-            }
-          } else if (KV) {
+          if (KV) {
             const int nh = N / GEMM_TILE_N;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -266,23 +243,22 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
               }
             }
           } else {
+            const bool first = sl == un.s0 || part;
 #pragma unroll
             for (int q = 0; q < 16; ++q) {          // (8 columns at a time: 128 running sums leave few registers)
+              if (SWIGLU && grp * 32 + (q >> 3) * 64 >= half) break;
               uint32_t v[8];
-              tmem_ld8(ta + (uint32_t)(grp * 128 + q * 8), v);
+              tmem_ld8(ta + (uint32_t)acc_col(q), v);
               tmem_ld_wait();
 #pragma unroll
-              for (int j = 0; j < 8; ++j) sum[8 * q + j] = (sl == un.s0 ? 0.f : sum[8 * q + j]) + __uint_as_float(v[j]);
+              for (int j = 0; j < 8; ++j) sum[8 * q + j] = (first ? 0.f : sum[8 * q + j]) + __uint_as_float(v[j]);
             }
           }
         }
         tc_fence_before();
         mbar_arrive_cluster(cluster_map(smem_u32(&tmem_empty_bar[acc]), 0));
-      }
-      if (MODE == PG_PLAIN && ok && row0 < R) {
-        // a whole tile goes to the output, a slice to its partial matrix
-        const bool part = u >= whole;
-        const int y = part ? ((un.tile - whole) * slices + un.s0) * 256 + rank * 128 + lane_base : row0;
+        if (MODE != PG_PLAIN || row0 >= R || !(part || sl + 1 == un.s1)) continue;
+        const int y = part ? ((un.tile - whole) * slices + sl) * 256 + rank * 128 + lane_base : row0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int col = nt * GEMM_TILE_N + grp * 128 + q * 32;
@@ -299,6 +275,36 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
               tma_store_2d(part ? &tmOut2 : &tmOut, stg, part ? grp * 128 + q * 32 : col, y);
               bulk_commit();
             }
+          }
+        }
+      }
+      if (SWIGLU && ok && row0 < R) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {               // blocks of 32 outputs
+          const int c0 = grp * 32 + 64 * i, col = nt * half + c0;
+          if (c0 >= half || col >= (N >> 1)) break;
+          if (lane == 0) bulk_wait_read<0>();       // the staging tile has been read
+          __syncwarp();
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {             // 16 bytes = 8 outputs; 64-byte rows, 64-byte swizzle
+            __nv_bfloat16 a[8], b[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float gt = sum[64 * i + 8 * q + j];
+              const float y = gt / (1.f + expf(-gt)) * sum[64 * i + 32 + 8 * q + j];
+              a[j] = __float2bfloat16_rn(y);
+              b[j] = __float2bfloat16_rn(y - __bfloat162float(a[j]));
+            }
+            const uint32_t off = (uint32_t)lane * 64 + (((uint32_t)q ^ (((uint32_t)lane >> 1) & 3u)) << 4);
+            *reinterpret_cast<uint4 *>(stg_p + off) = *reinterpret_cast<const uint4 *>(a);
+            *reinterpret_cast<uint4 *>(stg_p + PG_OUT_BYTES / 2 + off) = *reinterpret_cast<const uint4 *>(b);
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_2d(&tmOut, stg, col, row0);
+            tma_store_2d(&tmOut2, stg + PG_OUT_BYTES / 2, col, row0);
+            bulk_commit();
           }
         }
       }
@@ -328,8 +334,8 @@ __global__ void __launch_bounds__(256) gemm_pair_fixup_kernel(GemmOut g, float *
   if (n < g.N && r < g.BN) direct[(size_t)r * g.N + n] = gemm_load_pair(g, r, n);
 }
 
-// How a launch over R rows divides its tiles: the first `whole` as whole tiles, the others slice by slice where that
-// shortens the last wave.
+// How a launch over R rows divides its tiles: the first `whole` as whole tiles, the others in units of per_unit slices where
+// that shortens the last wave.
 struct PairShape { int row_tiles, whole, units, half; };
 PairShape pair_shape(const GemmPairPlan &p, int R, bool narrow) {
   PairShape q{};
@@ -345,50 +351,59 @@ PairShape pair_shape(const GemmPairPlan &p, int R, bool narrow) {
   const int tiles = q.row_tiles * n_tiles;
   q.whole = tiles;
   q.units = tiles;
-  if (p.slices > 1) {
+  const int n = p.slices / p.per_unit;              // units of a tile
+  if (n > 1 && !p.swiglu) {
     const int full = tiles / p.pairs * p.pairs, tail = tiles - full;
     // worth it where the time of the last wave that is saved (0.8 us per k-block) exceeds what writing and reading the
     // partials costs (0.06 us per slice of a tile): 16 of 16 tiles of the Qwen3-8B O projection at 256 rows 51 -> 21
     // us, not 54 of 128 at 2048 rows
-    const int parts = (tail * p.slices + p.pairs - 1) / p.pairs;
-    const float saved = 0.8f * (float)(p.K / GEMM_BLOCK_K) * (float)(p.slices - parts) / (float)p.slices;
+    const int parts = (tail * n + p.pairs - 1) / p.pairs;
+    const float saved = 0.8f * (float)(p.K / GEMM_BLOCK_K) * (float)(n - parts) / (float)n;
     if (tail && saved > 0.06f * (float)(tail * p.slices)) {
       q.whole = full;
-      q.units = full + tail * p.slices;
+      q.units = full + tail * n;
     }
   }
   return q;
 }
 
-}  // namespace
-
-int gemm_pair_slices(int N, int K, int num_sms) {
-  const int n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N, kb = K / GEMM_BLOCK_K, pairs = num_sms / 2;
-  int s = pairs / n_tiles;                          // one row tile in one wave
-  if (s < 1) s = 4;                                 // more tiles than pairs: the slices serve the last wave only
-  if (s > 8) s = 8;
-  while (s > 1 && kb / s < 8) --s;                  // a slice of fewer than 8 k-blocks costs more than it shortens
-  return s;
+// The cuts of K: units of a tile whose one row tile fills a wave, each of one or more slices of at most PG_CHAIN k-blocks as
+// far as eight slices allow (each is a matrix for the consumer to read).
+void pair_slices(GemmPairPlan &p) {
+  const int kb = p.K / GEMM_BLOCK_K;
+  if (p.swiglu) {                                   // no units: the slices meet in the epilogue's registers
+    p.slices = p.per_unit = (kb + PG_CHAIN - 1) / PG_CHAIN;
+    return;
+  }
+  int n = p.pairs / p.n_tiles;
+  if (n < 1) n = 4;                                 // more tiles than pairs: the units serve the last wave only
+  if (n > 8) n = 8;
+  while (n > 1 && kb / n < 8) --n;                  // a unit of fewer than 8 k-blocks costs more than it shortens
+  p.per_unit = 1;
+  while (kb > PG_CHAIN * n * p.per_unit && n * (p.per_unit + 1) <= 8) ++p.per_unit;
+  p.slices = n * p.per_unit;
 }
+
+}  // namespace
 
 size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms) {
   GemmPairPlan p;
   p.N = N; p.K = K; p.cap = cap; p.pairs = num_sms / 2;
   p.n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N;
-  p.slices = gemm_pair_slices(N, K, num_sms);
+  pair_slices(p);
   int most = 1;
   for (int R = 256; R < cap + 256; R += 256) {
     const PairShape q = pair_shape(p, R, false);
-    if (q.units - q.whole > most) most = q.units - q.whole;
+    if ((q.units - q.whole) * p.per_unit > most) most = (q.units - q.whole) * p.per_unit;
   }
   return (size_t)most * 256 * GEMM_TILE_N;
 }
 
 int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms) {
-  if (N <= 0 || N % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out || num_sms < 2) return CORUN_EINVAL;
+  if (N <= 0 || N % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out || !part || num_sms < 2) return CORUN_EINVAL;
   p->N = N; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = false; p->out = out; p->part = part;
   p->n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N;
-  p->slices = part ? gemm_pair_slices(N, K, num_sms) : 1;
+  pair_slices(*p);
   int rc;
   if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
   if ((rc = tma_encode_store_2d(&p->tmOut, out, 1, cap, N)) != 0) return rc;
@@ -427,7 +442,7 @@ int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi,
   if (F <= 0 || F % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out_hi || !out_lo || num_sms < 2) return CORUN_EINVAL;
   p->N = 2 * F; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = true; p->out = nullptr;
   p->n_tiles = (F + 127) / 128;
-  p->slices = 1;
+  pair_slices(*p);
   int rc;
   if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
   if ((rc = tma_encode_store_2d(&p->tmOut, out_hi, 0, cap, F)) != 0 || (rc = tma_encode_store_2d(&p->tmOut2, out_lo, 0, cap, F)) != 0)
@@ -439,7 +454,7 @@ int gemm_pair_plan_create_kv(GemmPairPlan *p, int nh, int K, const void *Xhi, co
   if (nh < 1 || K <= 0 || K % GEMM_BLOCK_K || cap < 32 || cap % 32 || !kv || num_sms < 2) return CORUN_EINVAL;
   p->N = nh * GEMM_TILE_N; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = false; p->out = nullptr;
   p->n_tiles = nh;
-  p->slices = 1;
+  p->slices = p->per_unit = 1;                      // (a latent of at most 512 values)
   p->kv_heads = nh;
   int rc;
   if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
@@ -462,7 +477,7 @@ cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int 
   const int pairs = q.units < p.pairs ? q.units : p.pairs;
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, q.half == 96 ? *tmW96 : tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2,
-                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, q.half, d_status, p.row_blocks, p.cap);
+                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, p.per_unit, q.half, d_status, p.row_blocks, p.cap);
   };
   return p.kv_heads ? go(gemm_pair_kernel<PG_KV>) : p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU>) : go(gemm_pair_kernel<PG_PLAIN>);
 }

@@ -1,5 +1,5 @@
 """The kernels of long prompts run by themselves against 64-bit arithmetic: the attention of a chunk's rows over the slot's
-cached positions."""
+cached positions, and the GEMM on pairs of SMs."""
 import numpy as np
 import pytest
 
@@ -86,3 +86,39 @@ def test_a_blocks_largest_weight_is_exact(hd):
         eng.close()
     want, _ = _attend(q, k.reshape(T, 1, hd), v.reshape(T, 1, hd), T - 1, hd ** -0.5)
     assert np.abs(got - want).max() <= 2e-5 * np.abs(want).max() + 2 ** -17 * np.abs(want).max()
+
+
+def _product(form, N, K, R, seed):
+    """The GEMM on pairs of SMs -> (result, 64-bit result, 64-bit result of the activations as bf16 pairs, that of their bf16 part
+    alone).  Forms: 0 plain, 1 with SwiGLU, 2 keys and values."""
+    import torch
+
+    from paper_2608_14376_b200 import corun
+
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    W = (torch.randn((N, K), generator=g, device="cuda") * 0.02).bfloat16()
+    X = torch.randn((R, K), generator=g, device="cuda")
+    hi = X.bfloat16()
+    lo = (X - hi.float()).bfloat16()
+
+    def f(x):
+        y = x @ W.double().T
+        return torch.nn.functional.silu(y[:, :N // 2]) * y[:, N // 2:] if form == 1 else y
+
+    return corun.debug_gemm_pair(form, W, X).double(), f(X.double()), f(hi.double() + lo.double()), f(hi.double())
+
+
+# edges of the tiles (256 rows, 128 per SM, 32 per store; 256 columns, 96 or 128 outputs with SwiGLU), whole tiles and tiles dealt
+# out slice by slice, one slice and eight
+@pytest.mark.parametrize("form,N,K,R", [(0, 8, 64, 1), (0, 200, 192, 257), (0, 1536, 1024, 300), (0, 4096, 4096, 256), (0, 6144, 4096, 129),
+                                        (0, 1024, 3072, 1000), (0, 4096, 12288, 515), (1, 128, 64, 31), (1, 1408, 1024, 255),
+                                        (1, 2 * 12288, 4096, 256), (1, 2 * 3072, 1024, 777), (2, 256, 256, 65), (2, 1024, 512, 513)])
+def test_pair_gemm_matches_fp64(form, N, K, R):
+    got, want, pairs, bf16 = _product(form, N, K, R, seed=N + K + R)
+    off = lambda a, b: float((a - b).norm() / b.norm())
+    # 16 significand bits of the activations (2.5e-6), a slice's sum cut off at every MMA (1.7e-8 each, at most 24 k-blocks of 8:
+    # 3.3e-6); a SwiGLU's result is a product of two such sums and stored as a bf16 pair (2e-6)
+    bound = 4.5e-6 if form != 1 else 8e-6
+    assert off(got, want) <= bound, off(got, want)
+    assert off(got, pairs) <= off(got, want) + 1e-6
+    assert off(bf16, want) > 10 * bound                # without the lo part it would not pass
