@@ -69,7 +69,8 @@ int corun_debug_gemm(const void *W, int32_t N, int32_t K, const float *X, int32_
  *   form 1  N = 2F (F gate rows, then F up rows of W; F % 64 == 0): out [R, F] = silu(X Wg^T) * (X Wu^T)
  *   form 2  N = 256 heads (per head 128 key rows, then 128 value rows): out [R, N] = X W^T by way of the fp16 hi / lo pairs
  *           that the latent prefill attention reads
- * (forms 1 and 2: the sum of the stored pair).  1 <= R <= 2048, K % 64 == 0; pointers as above. */
+ *   form 3, 4  as 0, 1 in the form of a decode step (R <= 256; up to 128 rows: that of a step without requests beyond them)
+ * (forms 1, 2 and 4: the sum of the stored pair).  1 <= R <= 2048, K % 64 == 0; pointers as above. */
 int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, const float *X, int32_t R, float *out,
                           void *cuda_stream);
 /* The attention kernel of long prompts for n query rows at positions pos0 .. pos0 + n - 1 of an occupied slot, over the layer's

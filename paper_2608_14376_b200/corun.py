@@ -490,12 +490,13 @@ def debug_gemm(W, X):
 
 
 def debug_gemm_pair(form, W, X):
-    """The GEMM on pairs of SMs (``corun_debug_gemm_pair``): form 0 plain, 1 with SwiGLU (result [R, N / 2]), 2 keys and values."""
+    """The GEMM on pairs of SMs (``corun_debug_gemm_pair``): form 0 plain, 1 with SwiGLU (result [R, N / 2]), 2 keys and
+    values; 3, 4: 0, 1 as a decode step runs them."""
     import torch
 
     N, K = W.shape
     R = X.shape[0]
-    out = torch.empty((R, N // 2 if form == 1 else N), dtype=torch.float32, device=X.device)
+    out = torch.empty((R, N // 2 if form in (1, 4) else N), dtype=torch.float32, device=X.device)
     torch.cuda.synchronize()
     _check(lib().corun_debug_gemm_pair(form, W.data_ptr(), N, K, X.data_ptr(), R, out.data_ptr(), None), "corun_debug_gemm_pair")
     return out

@@ -100,14 +100,13 @@ struct Program {
   // rows as for long ones.
   bool pair = false;
   int cap = 0;
-  // Decode above 128 rows (wide): the dense projections and the LM head on pairs of SMs too.  Per Qwen3-8B layer at 256 rows
-  // 248 us of GEMMs (hi and lo of two row blocks per weight tile on one SM each, two stages of shared memory) and 17 us of
-  // SwiGLU, against 179 us.
-  // A pair multiplies both halves of its 256 rows whether requests fill them or not, so with up to 128 requests in the step
-  // a decoder that is bound by streaming large dense matrices pays for it: 140 slots, 25 / 125 / 139 requests, 12 Qwen3-8B
-  // layers 2.45 / 2.77 / 3.58 ms before and 2.74 / 3.06 / 3.21 with pairs, 230 slots, 60 / 120 / 150: 2.83 / 3.00 / 4.05 and
-  // 2.87 / 3.13 / 3.56.  Those take pairs from WIDE_ROWS rows on; the hidden-1024 decoder and the decoders with expert layers
-  // gain at every count (1.04 / 1.22 / 1.86 -> 1.02 / 1.20 / 1.48 ms; 3.71 / 4.43 / 5.26 -> 3.59 / 4.31 / 4.87).
+  // Decode above 128 rows (wide): the dense projections and the LM head on pairs of SMs too, with expert layers from 129 rows
+  // on, else from WIDE_ROWS rows on: below, the fixed cost of a pair GEMM (clusters, no programmatic launch; 15 us for the
+  // matrices of the hidden-1024 decoder) outweighs what the steps of more than 128 requests save.
+  // ms per step of 12 layers, one-SM GEMMs / pairs, at three counts of requests: Qwen3-8B 140 slots (25, 125, 139 requests)
+  // 2.44 2.91 3.79 / 2.61 3.03 3.61, 200 slots (30, 128, 200) 2.69 3.36 4.75 / 2.65 3.26 4.39, 256 slots (40, 128, 256) 2.87 3.38
+  // 5.33 / 2.73 3.17 4.82; hidden 1024 140 slots .99 1.28 1.53 / 1.09 1.39 1.55, 200 slots 1.03 1.33 1.84 / 1.10 1.41 1.76, 256
+  // slots (25, 128, 256) 1.06 1.36 2.17 / 1.10 1.41 1.87; Qwen3-30B-A3B 140 slots (25, 128, 139) 3.51 4.50 4.88 / 3.46 4.44 4.71.
   bool wide = false;
   GemmPairPlan b_lm;
   bool shorts = false;
@@ -362,17 +361,17 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
     // the plans carry layer 0's weights; the per-layer tensor maps override them at launch
     if (P.wide) {
       const bool ffn = !e->moe_E;
-      size_t part = gemm_pair_part_floats(QKVN, H, 256, e->num_sms);
-      for (size_t x : {gemm_pair_part_floats(H, QD, 256, e->num_sms), ffn ? gemm_pair_part_floats(H, F, 256, e->num_sms) : 0,
-                       gemm_pair_part_floats(V, H, 256, e->num_sms)})
+      size_t part = gemm_pair_part_floats(QKVN, H, 256, e->num_sms, true);
+      for (size_t x : {gemm_pair_part_floats(H, QD, 256, e->num_sms, true), ffn ? gemm_pair_part_floats(H, F, 256, e->num_sms, true) : 0,
+                       gemm_pair_part_floats(V, H, 256, e->num_sms, true)})
         part = x > part ? x : part;
       RC(dmalloc(A, &P.pair_part, part, false));
       if (!P.plain_tiles) RC(dmalloc(A, &P.plain_tiles, (size_t)((QKVN > V ? QKVN : V) / GEMM_TILE_N + 1)));
-      RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, 256, P.qkv_out, P.pair_part, e->num_sms));
-      RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, 256, P.o_out, P.pair_part, e->num_sms));
+      RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, 256, P.qkv_out, P.pair_part, e->num_sms, true));
+      RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, 256, P.o_out, P.pair_part, e->num_sms, true));
       if (ffn) {
-        RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, 256, P.ff_hi, P.ff_lo, e->num_sms));
-        RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, 256, P.down_out, P.pair_part, e->num_sms));
+        RC(gemm_pair_plan_create_swiglu(&P.b_gu, F, H, P.xn_hi, P.xn_lo, 256, P.ff_hi, P.ff_lo, e->num_sms, true));
+        RC(gemm_pair_plan_create(&P.b_down, H, F, P.ff_hi, P.ff_lo, 256, P.down_out, P.pair_part, e->num_sms, true));
       }
     } else {
       RC(gemm_plan_create(&P.p_qkv, e->w0_qkv, QKVN, H, P.xn_hi, P.xn_lo, R, P.BN, P.qkv_out, P.ws, e->num_sms));
@@ -428,7 +427,7 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
   }
   if (lm) {
     RC(dmalloc(A, &P.logits, (size_t)RR * V));
-    if (P.wide) return gemm_pair_plan_create(&P.b_lm, V, H, P.xn_hi, P.xn_lo, 256, P.logits, P.pair_part, e->num_sms);
+    if (P.wide) return gemm_pair_plan_create(&P.b_lm, V, H, P.xn_hi, P.xn_lo, 256, P.logits, P.pair_part, e->num_sms, true);
     RC(gemm_plan_create(&P.p_lm, e->lm_head, V, H, P.xn_hi, P.xn_lo, R, P.BN, P.logits, P.ws, e->num_sms));
   }
   return CORUN_OK;
@@ -1095,8 +1094,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG
   const long long big_rows = (long long)B * ((max_context + 127) / 128 * 128);
   const int big_cap = !big_ok ? 0 : big_rows < PREFILL_BIG ? (int)((big_rows + 255) / 256 * 256) : PREFILL_BIG;
-  const bool large_dense = !moe && (long long)2 * F * H > (16ll << 20);
-  const bool wide = e->wide = pad16(B) > 128 && s.vocab % 8 == 0 && (!large_dense || pad16(B) >= WIDE_ROWS);   // (Program::wide)
+  const bool wide = e->wide = pad16(B) >= (moe ? 129 : WIDE_ROWS) && s.vocab % 8 == 0;   // (Program::wide)
   if (wide && gemm_encode_map(&e->tb_lm, w->lm_head, s.vocab, H, 128)) return fail(CORUN_EINVAL);
   e->tm_qkv.resize(s.n_layers);
   e->tm_o.resize(s.n_layers);
@@ -2015,7 +2013,10 @@ int corun_debug_gemm(const void *W, int32_t N, int32_t K, const float *X, int32_
 
 int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, const float *X, int32_t R, float *out,
                           void *cuda_stream) {
-  if (form < 0 || form > 2 || !W || !X || !out || N < 8 || K < 64 || K % 64 || R < 1 || R > PREFILL_BIG) return CORUN_EINVAL;
+  const bool decode = form >= 3;
+  if (decode) form -= 3;
+  if (form < 0 || form > 2 || (decode && form > 1) || !W || !X || !out || N < 8 || K < 64 || K % 64 || R < 1 || R > (decode ? 256 : PREFILL_BIG))
+    return CORUN_EINVAL;
   if (form == 0 ? N % 8 : form == 1 ? N % 128 : N % GEMM_TILE_N) return CORUN_EINVAL;
   if (((uintptr_t)out & 15u) || ((uintptr_t)W & 15u) || ((uintptr_t)X & 3u)) return CORUN_EINVAL;
   cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -2028,25 +2029,28 @@ int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, con
   bf16 *hi = nullptr, *lo = nullptr, *ohi = nullptr, *olo = nullptr;
   __half *kv = nullptr;
   float *part = nullptr, *full = nullptr;
-  int *status = nullptr, rc = CORUN_OK;
+  int *status = nullptr, rc = CORUN_OK;              // status word | row_blocks
   GemmPairPlan p;
   CUtensorMap tw, tw96;
   auto ok = [&](int r) { return (rc = r) == CORUN_OK; };
-  if (ok(dmalloc(keep, &hi, c * K)) && ok(dmalloc(keep, &lo, c * K)) && ok(dmalloc(keep, &status, 1)) &&
+  if (ok(dmalloc(keep, &hi, c * K)) && ok(dmalloc(keep, &lo, c * K)) && ok(dmalloc(keep, &status, 2)) &&
       ok(gemm_encode_map(&tw, W, N, K, 128)) && ok(gemm_encode_map(&tw96, W, N, K, 96))) {
     if (form == 0)
-      ok(dmalloc(keep, &part, gemm_pair_part_floats(N, K, cap, sms))) && ok(dmalloc(keep, &full, c * N)) &&
-          ok(gemm_pair_plan_create(&p, N, K, hi, lo, cap, full, part, sms));
+      ok(dmalloc(keep, &part, gemm_pair_part_floats(N, K, cap, sms, decode))) && ok(dmalloc(keep, &full, c * N)) &&
+          ok(gemm_pair_plan_create(&p, N, K, hi, lo, cap, full, part, sms, decode));
     else if (form == 1)
-      ok(dmalloc(keep, &ohi, c * F)) && ok(dmalloc(keep, &olo, c * F)) && ok(gemm_pair_plan_create_swiglu(&p, F, K, hi, lo, cap, ohi, olo, sms));
+      ok(dmalloc(keep, &ohi, c * F)) && ok(dmalloc(keep, &olo, c * F)) && ok(gemm_pair_plan_create_swiglu(&p, F, K, hi, lo, cap, ohi, olo, sms, decode));
     else
       ok(dmalloc(keep, &kv, 4 * c * nh * 128)) && ok(gemm_pair_plan_create_kv(&p, nh, K, hi, lo, cap, kv, sms));
   }
   if (rc == CORUN_OK) {
     cudaError_t ce = cudaDeviceSynchronize();       // allocations were cleared through the legacy stream
+    const int blocks = R > 128 ? 3 : 1;
+    if (ce == cudaSuccess && decode) ce = cudaMemcpy(status + 1, &blocks, sizeof(int), cudaMemcpyHostToDevice);
+    if (decode) p.row_blocks = status + 1;
     if (ce == cudaSuccess) ce = launch_split(X, R, K, hi, lo, st);
-    if (ce == cudaSuccess) ce = gemm_pair_launch(p, tw, R, status, st, form == 1 ? &tw96 : nullptr);
-    if (ce == cudaSuccess && form == 0) ce = gemm_pair_fixup_launch(p, R, st);
+    if (ce == cudaSuccess) ce = gemm_pair_launch(p, tw, decode ? 256 : R, status, st, form == 1 ? &tw96 : nullptr);
+    if (ce == cudaSuccess && form == 0) ce = gemm_pair_fixup_launch(p, decode ? 256 : R, st);
     if (ce == cudaSuccess && form == 0) ce = cudaMemcpyAsync(out, full, (size_t)R * N * sizeof(float), cudaMemcpyDeviceToDevice, st);
     if (ce == cudaSuccess && form == 1) ce = launch_join(ohi, olo, false, R, F, out, F, st);
     for (int i = 0; form == 2 && i < 2 * nh && ce == cudaSuccess; ++i) {   // head i / 2: its keys, its values

@@ -222,20 +222,22 @@ struct GemmPairPlan {
   bool swiglu = false;
   int kv_heads = 0;                  // gemm_pair_plan_create_kv
   float *out = nullptr, *part = nullptr;   // not owned
-  const int *row_blocks = nullptr;   // device, not owned (cap 256): bit 1 = rows 128 .. hold a request; null = they do
+  bool decode = false;               // rows of a decode step (cap 256), in two halves that may be without a request
+  const int *row_blocks = nullptr;   // (decode) device, not owned: bit 1 = rows 128 .. hold a request
 };
 // Floats of partial tiles that launches over up to cap rows leave (the next kernel of the stream consumes them, so one
 // buffer serves all plans of a program).
-size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms);
+size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms, bool decode = false);
 // X W^T for activations Xhi / Xlo [cap, K] (N % 8 == 0) -> out [cap, N] fp32 and, for the tiles of an unfilled wave, part
 // (gemm_pair_part_floats).  Read through gemm_pair_out(p, R, zeros).
-int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms);
+int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms,
+                          bool decode = false);
 GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles);
 int gemm_pair_has_parts(const GemmPairPlan &p, int R);   // 1 if some of the result of R rows is left in partial matrices
 cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st);   // makes `out` a plain matrix
 // W is [2F, K] (F gate rows, then F up rows; F % 8 == 0): out_hi / out_lo [cap, F] = silu(gate) * up as a bf16 hi/lo pair.
 int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,
-                                 __nv_bfloat16 *out_lo, int num_sms);
+                                 __nv_bfloat16 *out_lo, int num_sms, bool decode = false);
 // Decompression of latents into keys and values: W is [nh * 256, K] (per head 128 key rows, 128 value rows); the fp16 hi / lo
 // pairs of the products go to kv [key hi | key lo | value hi | value lo][nh][cap][128] (cap % 32 == 0).
 int gemm_pair_plan_create_kv(GemmPairPlan *p, int nh, int K, const void *Xhi, const void *Xlo, int cap, void *kv, int num_sms);

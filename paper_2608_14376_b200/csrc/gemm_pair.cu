@@ -53,7 +53,15 @@ constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + PG_EPI * 
 // (second CTA), always whole (the slices meet in registers), and the epilogue writes silu(gate) * up as the bf16 hi/lo pair the down GEMM reads.
 // KV (gemm_pair_plan_create_kv): a tile's 256 columns are one head's 128 key and 128 value columns, stored as fp16 hi / lo
 // pairs, keys by the first half of the epilogue warps, values by the second; cap: rows of one of the four matrices per head.
-template <int MODE>
+//
+// DECODE (up to 256 rows, one row tile; row_blocks says which halves of them hold requests this step): hi and lo have an
+// accumulator each, a slice's value is their sum.  With requests in rows 128 .. each CTA keeps both accumulators (512 columns:
+// one buffer).  Without, a CTA's 128 operand rows are the hi and the lo parts of 64 rows, so that one MMA does what takes two
+// above, and the halves of the accumulator meet through shared memory (the stages' unused lo parts): the tensor work is that
+// of 128 rows, and a row has the same value either way.  (With both halves multiplied in every step, 200 slots with 30 / 60 /
+// 128 requests took 2.83 / 3.06 / 3.54 ms per step of 12 Qwen3-8B layers, now 2.65 / 2.78 / 3.26; with 200 requests 4.27, now
+// 4.40: the end of a slice is not hidden behind the next one.  Others: Program::wide.)
+template <int MODE, bool DECODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                  const __grid_constant__ CUtensorMap tmLo, const __grid_constant__ CUtensorMap tmOut,
@@ -65,6 +73,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   __shared__ __align__(8) uint64_t empty_bar[PG_STAGES];     // in each CTA: the MMAs have read the stage
   __shared__ __align__(8) uint64_t tmem_full_bar[2];         // in each CTA: an accumulator is complete
   __shared__ __align__(8) uint64_t tmem_empty_bar[2];        // in the first CTA: both CTAs' epilogues have read it
+  __shared__ __align__(8) uint64_t x_full_bar[4], x_free_bar[4];   // (stacked) lo sums of 32 rows x 128 columns handed over / read
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
 
@@ -73,17 +82,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
-  // (decode) the step's requests are in the first rows: without one in rows 128 .. the second CTA's activations are zeros,
-  // neither loaded nor stored (200 against 100 requests in 256 rows: what is saved is L2 traffic and power)
-  const bool upper = !row_blocks || (*reinterpret_cast<const volatile int *>(row_blocks) & 2);
-  if (!upper && R > 128) R = 128;
-  if (!upper && rank == 1) {
-    for (int s = 0; s < PG_STAGES; ++s) {
-      uint4 *z = reinterpret_cast<uint4 *>(smem_raw + (base - smem_u32(smem_raw)) + s * PG_STAGE_BYTES);
-      for (uint32_t i = threadIdx.x; i < 2 * PG_X_BYTES / 16; i += PG_THREADS) z[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    fence_proxy_async();
-  }
+  // (DECODE) the step's requests are in the first rows; stacked: none in rows 128 ..
+  const bool stacked = DECODE && !(*reinterpret_cast<const volatile int *>(row_blocks) & 2);
+  const bool one_buffer = DECODE && !stacked;
+  if (stacked && R > 128) R = 128;
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < PG_STAGES; ++s) {
@@ -93,6 +95,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&tmem_full_bar[a]), 1);
       mbar_init(smem_u32(&tmem_empty_bar[a]), 2 * 32 * PG_EPI);
+    }
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(smem_u32(&x_full_bar[i]), 32);
+      mbar_init(smem_u32(&x_free_bar[i]), 32);
     }
     fence_mbar_init();
     fence_proxy_async();
@@ -125,7 +131,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       // ---------------- TMA producer (both CTAs; the bytes count on the first CTA's barrier) ----------------
       const uint64_t pol_w = l2_policy_evict_first();        // a weight tile is used by the row tiles that run now
       const uint64_t pol_x = l2_policy_evict_last();
-      const uint32_t stage_tx = 2u * (uint32_t)half * 128u + (upper ? 2u : 1u) * 2u * PG_X_BYTES;
+      const uint32_t stage_tx = 2u * (uint32_t)half * 128u + (stacked ? 2u : 4u) * PG_X_BYTES;   // of both CTAs
       int it = 0;
       for (int u = pair; u < units && !fail; u += n_pairs) {
         const Unit un = unit(u);
@@ -142,7 +148,15 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           if (rank == 0) mbar_arrive_expect_tx(fb, stage_tx);
           const uint32_t fb0 = cluster_map(fb, 0);
           tma_load_2d_pair(dst + 2 * PG_X_BYTES, &tmW, kb * GEMM_BLOCK_K, yw, fb0, pol_w);
-          if (rank == 0 || upper) {
+          if (stacked) {
+            tma_load_2d_pair(dst, &tmHi, kb * GEMM_BLOCK_K, 64 * rank, fb0, pol_x);
+            tma_load_2d_pair(dst + PG_X_BYTES / 2, &tmLo, kb * GEMM_BLOCK_K, 64 * rank, fb0, pol_x);
+          } else if (DECODE) {                      // (boxes of 64 rows)
+            for (int b = 0; b < 2; ++b) {
+              tma_load_2d_pair(dst + b * (PG_X_BYTES / 2), &tmHi, kb * GEMM_BLOCK_K, yx + 64 * b, fb0, pol_x);
+              tma_load_2d_pair(dst + PG_X_BYTES + b * (PG_X_BYTES / 2), &tmLo, kb * GEMM_BLOCK_K, yx + 64 * b, fb0, pol_x);
+            }
+          } else {
             tma_load_2d_pair(dst, &tmHi, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
             tma_load_2d_pair(dst + PG_X_BYTES, &tmLo, kb * GEMM_BLOCK_K, yx, fb0, pol_x);
           }
@@ -165,10 +179,12 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       for (int u = pair; u < units && !fail; u += n_pairs) {
         const Unit un = unit(u);
         for (int sl = un.s0; sl < un.s1 && !fail; ++sl, ++seg) {
-          const int acc = seg & 1;
-          if (!mbar_wait(smem_u32(&tmem_empty_bar[acc]), ((uint32_t)(seg >> 1) & 1u) ^ 1u, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
+          const int acc = one_buffer ? 0 : seg & 1;
+          const uint32_t turn = (uint32_t)(one_buffer ? seg : seg >> 1) & 1u;
+          if (!mbar_wait(smem_u32(&tmem_empty_bar[acc]), turn ^ 1u, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
           tc_fence_after();
           const uint32_t d = tmem_base + (uint32_t)acc * GEMM_TILE_N;
+          const uint32_t d_lo = one_buffer ? d + GEMM_TILE_N : d;
           const int kb0 = cut(sl), kb1 = cut(sl + 1);
           for (int kb = kb0; kb < kb1; ++kb, ++it) {
             const int s = it % PG_STAGES;
@@ -180,7 +196,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
               const uint64_t adv = (uint64_t)(k * 2);
               umma_bf16_pair(d, hi + adv, w + adv, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-              umma_bf16_pair(d, lo + adv, w + adv, idesc, 1u);
+              if (!stacked) umma_bf16_pair(d_lo, lo + adv, w + adv, idesc, (!DECODE || kb > kb0 || k > 0) ? 1u : 0u);
             }
             umma_commit_pair(smem_u32(&empty_bar[s]));
           }
@@ -194,23 +210,44 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     const uint32_t stg = base + PG_STAGES * PG_STAGE_BYTES + (uint32_t)(warp - 2) * PG_OUT_BYTES;
     uint8_t *stg_p = smem_raw + (stg - smem_u32(smem_raw));
     const uint32_t lane_off = (uint32_t)lane_base << 16;
+    // stacked: lanes 64 .. of the accumulator are the lo sums of the rows in lanes 0 .. 63
+    const bool lo_warp = stacked && lane_base >= 64;
+    const int in_tile = stacked ? rank * 64 + (lane_base & 32) : rank * 128 + lane_base;   // this warp's 32 rows of a tile
+    const uint32_t x_full = smem_u32(&x_full_bar[grp * 2 + (warp & 1)]), x_free = smem_u32(&x_free_bar[grp * 2 + (warp & 1)]);
+    // (stacked) where this thread's row is handed over: 64 columns of 64 rows per stage, two stages per half of the columns
+    uint8_t *const handed_p = smem_raw + (base - smem_u32(smem_raw)) + 2 * grp * PG_STAGE_BYTES + PG_X_BYTES + ((lane_base & 32) + lane) * 4;
+    auto handed = [&](int i) -> float & { return *reinterpret_cast<float *>(handed_p + (i >> 6) * PG_STAGE_BYTES + (i & 63) * 256); };
     int seg = 0;
     bool ok = true;
     for (int u = pair; u < units && ok; u += n_pairs) {
       const Unit un = unit(u);
       const int nt = un.tile / row_tiles;
-      const int row0 = (un.tile % row_tiles) * 256 + rank * 128 + lane_base;   // this warp's 32 rows
+      const int row0 = (un.tile % row_tiles) * 256 + in_tile;   // this warp's 32 rows
       const bool part = u >= whole;                 // its slices go to partial matrices, a whole tile to the output
-      float sum[128];                               // this thread's row: 128 columns (SWIGLU: up to 64 gate and 64 up columns)
+      auto add = [](uint32_t a, uint32_t b) { return __float_as_uint(__uint_as_float(a) + __uint_as_float(b)); };
       // first accumulator column of the sums 8 q ..; SWIGLU: blocks of 32 outputs, gate then up columns of each
       auto acc_col = [&](int q) { return SWIGLU ? grp * 32 + (q >> 3) * 64 + ((q >> 2) & 1) * half + (q & 3) * 8 : grp * 128 + q * 8; };
-      for (int sl = un.s0; sl < un.s1; ++sl, ++seg) {
-        const int acc = seg & 1;
-        ok = mbar_wait(smem_u32(&tmem_full_bar[acc]), (uint32_t)(seg >> 1) & 1u, abort_p);
+      auto accumulator = [&]() { return tmem_base + (uint32_t)(one_buffer ? 0 : seg & 1) * GEMM_TILE_N + lane_off; };
+      auto wait_full = [&]() {                      // the segment's accumulator is complete
+        ok = mbar_wait(smem_u32(&tmem_full_bar[one_buffer ? 0 : seg & 1]), (uint32_t)(one_buffer ? seg : seg >> 1) & 1u, abort_p);
+        // (one row tile: every segment, or none, has rows for this warp)
+        if (lo_warp && row0 < R && seg > 0) ok = ok && mbar_wait(x_free, (uint32_t)(seg - 1) & 1u, abort_p);
         ok = __all_sync(0xffffffffu, ok);
-        if (!ok) { fail = DEV_TIMEOUT_EPILOGUE; break; }
         tc_fence_after();
-        const uint32_t ta = tmem_base + (uint32_t)acc * GEMM_TILE_N + lane_off;
+      };
+      auto lo_ready = [&]() {                       // (stacked) the lo sums of this thread's row have been handed over
+        ok = mbar_wait(x_full, (uint32_t)seg & 1u, abort_p);
+        ok = __all_sync(0xffffffffu, ok);
+      };
+      auto read_out = [&]() {
+        tc_fence_before();
+        mbar_arrive_cluster(cluster_map(smem_u32(&tmem_empty_bar[one_buffer ? 0 : seg & 1]), 0));
+      };
+      uint32_t sum[128];                            // this thread's row: 128 columns (SWIGLU: up to 64 gate and 64 up columns), fp32
+      for (int sl = un.s0; sl < un.s1; ++sl, ++seg) {
+        wait_full();
+        if (!ok) { fail = DEV_TIMEOUT_EPILOGUE; break; }
+        const uint32_t ta = accumulator();
         if (row0 < R) {                             // warp-uniform
           if (KV) {
             const int nh = N / GEMM_TILE_N;
@@ -243,32 +280,78 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
               }
             }
           } else {
-            const bool first = sl == un.s0 || part;
+            auto there = [&](int q) { return !SWIGLU || grp * 32 + (q >> 3) * 64 < half; };
+            if (lo_warp || sl == un.s0 || part) {   // no sum yet: straight into the registers, all loads in flight together
+              // (the first half is always there; a branch must not end between a load and its wait)
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {          // (8 columns at a time: 128 running sums leave few registers)
-              if (SWIGLU && grp * 32 + (q >> 3) * 64 >= half) break;
-              uint32_t v[8];
-              tmem_ld8(ta + (uint32_t)acc_col(q), v);
+              for (int g = 0; g < (SWIGLU ? 4 : 8); ++g) tmem_ld16(ta + (uint32_t)acc_col(2 * g), *reinterpret_cast<uint32_t(*)[16]>(&sum[16 * g]));
               tmem_ld_wait();
+              if (SWIGLU && there(8)) {
 #pragma unroll
-              for (int j = 0; j < 8; ++j) sum[8 * q + j] = (first ? 0.f : sum[8 * q + j]) + __uint_as_float(v[j]);
+                for (int g = 4; g < 8; ++g) tmem_ld16(ta + (uint32_t)acc_col(2 * g), *reinterpret_cast<uint32_t(*)[16]>(&sum[16 * g]));
+                tmem_ld_wait();
+              }
+              if (lo_warp) {
+#pragma unroll
+                for (int i = 0; i < 128; ++i)
+                  if (there(i / 8)) handed(i) = __uint_as_float(sum[i]);
+                mbar_arrive(x_full);
+              } else if (stacked) {
+                lo_ready();
+#pragma unroll
+                for (int i = 0; i < 128; ++i)
+                  if (there(i / 8)) sum[i] = add(sum[i], __float_as_uint(handed(i)));
+                mbar_arrive(x_free);
+              } else if (DECODE) {
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                  if (!there(2 * g)) break;
+                  uint32_t lo[16];
+                  tmem_ld16(ta + (uint32_t)(GEMM_TILE_N + acc_col(2 * g)), lo);
+                  tmem_ld_wait();
+#pragma unroll
+                  for (int j = 0; j < 16; ++j) sum[16 * g + j] = add(sum[16 * g + j], lo[j]);
+                }
+              }
+            } else {
+              if (stacked) lo_ready();
+#pragma unroll
+              for (int q = 0; q < 16; ++q) {        // (8 columns at a time: 128 running sums leave few registers)
+                if (!there(q)) break;
+                uint32_t v[8], lo[8];
+                tmem_ld8(ta + (uint32_t)acc_col(q), v);
+                if (DECODE && !stacked) {
+                  tmem_ld8(ta + (uint32_t)(GEMM_TILE_N + acc_col(q)), lo);
+                  tmem_ld_wait();
+                } else {
+                  tmem_ld_wait();
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  if (stacked) lo[j] = __float_as_uint(handed(8 * q + j));
+                  if (DECODE) v[j] = add(v[j], lo[j]);
+                  sum[8 * q + j] = add(sum[8 * q + j], v[j]);
+                }
+              }
+              if (stacked) mbar_arrive(x_free);
             }
           }
         }
-        tc_fence_before();
-        mbar_arrive_cluster(cluster_map(smem_u32(&tmem_empty_bar[acc]), 0));
-        if (MODE != PG_PLAIN || row0 >= R || !(part || sl + 1 == un.s1)) continue;
-        const int y = part ? ((un.tile - whole) * slices + sl) * 256 + rank * 128 + lane_base : row0;
+        if (!ok) { fail = DEV_TIMEOUT_EPILOGUE; break; }
+        read_out();
+        if (MODE != PG_PLAIN || row0 >= R || lo_warp || !(part || sl + 1 == un.s1)) continue;
+        // a whole tile goes to the output, a slice to its partial matrix
+        const int y = part ? ((un.tile - whole) * slices + sl) * 256 + in_tile : row0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int col = nt * GEMM_TILE_N + grp * 128 + q * 32;
           if (col < N) {
-            if (lane == 0) bulk_wait_read<0>();
+            if (lane == 0) bulk_wait_read<0>();     // the staging tile has been read
             __syncwarp();
 #pragma unroll
             for (int c = 0; c < 8; ++c)
-              *reinterpret_cast<float4 *>(stg_p + lane * 128 + (((uint32_t)c ^ ((uint32_t)lane & 7u)) << 4)) =
-                  make_float4(sum[32 * q + 4 * c], sum[32 * q + 4 * c + 1], sum[32 * q + 4 * c + 2], sum[32 * q + 4 * c + 3]);
+              *reinterpret_cast<uint4 *>(stg_p + lane * 128 + (((uint32_t)c ^ ((uint32_t)lane & 7u)) << 4)) =
+                  make_uint4(sum[32 * q + 4 * c], sum[32 * q + 4 * c + 1], sum[32 * q + 4 * c + 2], sum[32 * q + 4 * c + 3]);
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) {
@@ -278,7 +361,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           }
         }
       }
-      if (SWIGLU && ok && row0 < R) {
+      if (SWIGLU && ok && row0 < R && !lo_warp) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {               // blocks of 32 outputs
           const int c0 = grp * 32 + 64 * i, col = nt * half + c0;
@@ -290,8 +373,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             __nv_bfloat16 a[8], b[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const float gt = sum[64 * i + 8 * q + j];
-              const float y = gt / (1.f + expf(-gt)) * sum[64 * i + 32 + 8 * q + j];
+              const float gt = __uint_as_float(sum[64 * i + 8 * q + j]);
+              const float y = gt / (1.f + expf(-gt)) * __uint_as_float(sum[64 * i + 32 + 8 * q + j]);
               a[j] = __float2bfloat16_rn(y);
               b[j] = __float2bfloat16_rn(y - __bfloat162float(a[j]));
             }
@@ -371,23 +454,26 @@ PairShape pair_shape(const GemmPairPlan &p, int R, bool narrow) {
 // far as eight slices allow (each is a matrix for the consumer to read).
 void pair_slices(GemmPairPlan &p) {
   const int kb = p.K / GEMM_BLOCK_K;
+  // (decode: hi on its own makes half the MMAs, and the end of a slice is not hidden behind the next one)
+  const int chain = !p.decode ? PG_CHAIN : p.swiglu ? 2 * PG_CHAIN : 3 * PG_CHAIN;
   if (p.swiglu) {                                   // no units: the slices meet in the epilogue's registers
-    p.slices = p.per_unit = (kb + PG_CHAIN - 1) / PG_CHAIN;
+    p.slices = p.per_unit = (kb + chain - 1) / chain;
     return;
   }
   int n = p.pairs / p.n_tiles;
-  if (n < 1) n = 4;                                 // more tiles than pairs: the units serve the last wave only
+  if (n < 1) n = p.decode ? 2 : 4;                  // more tiles than pairs: the units serve the last wave only
   if (n > 8) n = 8;
   while (n > 1 && kb / n < 8) --n;                  // a unit of fewer than 8 k-blocks costs more than it shortens
   p.per_unit = 1;
-  while (kb > PG_CHAIN * n * p.per_unit && n * (p.per_unit + 1) <= 8) ++p.per_unit;
+  while (kb > chain * n * p.per_unit && n * (p.per_unit + 1) <= 8) ++p.per_unit;
   p.slices = n * p.per_unit;
 }
 
 }  // namespace
 
-size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms) {
+size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms, bool decode) {
   GemmPairPlan p;
+  p.decode = decode;
   p.N = N; p.K = K; p.cap = cap; p.pairs = num_sms / 2;
   p.n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N;
   pair_slices(p);
@@ -399,16 +485,19 @@ size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms) {
   return (size_t)most * 256 * GEMM_TILE_N;
 }
 
-int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms) {
+int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms,
+                          bool decode) {
   if (N <= 0 || N % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out || !part || num_sms < 2) return CORUN_EINVAL;
   p->N = N; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = false; p->out = out; p->part = part;
+  p->decode = decode;
   p->n_tiles = (N + GEMM_TILE_N - 1) / GEMM_TILE_N;
   pair_slices(*p);
   int rc;
-  if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
+  const int box = decode ? 64 : 128;
+  if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, box)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, box)) != 0) return rc;
   if ((rc = tma_encode_store_2d(&p->tmOut, out, 1, cap, N)) != 0) return rc;
   if (p->slices > 1) {
-    if ((rc = tma_encode_store_2d(&p->tmOut2, part, 1, gemm_pair_part_floats(N, K, cap, num_sms) / GEMM_TILE_N, GEMM_TILE_N)) != 0) return rc;
+    if ((rc = tma_encode_store_2d(&p->tmOut2, part, 1, gemm_pair_part_floats(N, K, cap, num_sms, decode) / GEMM_TILE_N, GEMM_TILE_N)) != 0) return rc;
   } else {
     p->tmOut2 = p->tmOut;
   }
@@ -438,13 +527,15 @@ cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st
 }
 
 int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,
-                                 __nv_bfloat16 *out_lo, int num_sms) {
+                                 __nv_bfloat16 *out_lo, int num_sms, bool decode) {
   if (F <= 0 || F % 8 || K <= 0 || K % GEMM_BLOCK_K || cap < 1 || !out_hi || !out_lo || num_sms < 2) return CORUN_EINVAL;
   p->N = 2 * F; p->K = K; p->cap = cap; p->pairs = num_sms / 2; p->swiglu = true; p->out = nullptr;
+  p->decode = decode;
   p->n_tiles = (F + 127) / 128;
   pair_slices(*p);
   int rc;
-  if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, 128)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, 128)) != 0) return rc;
+  const int box = decode ? 64 : 128;
+  if ((rc = gemm_encode_map(&p->tmHi, Xhi, cap, K, box)) != 0 || (rc = gemm_encode_map(&p->tmLo, Xlo, cap, K, box)) != 0) return rc;
   if ((rc = tma_encode_store_2d(&p->tmOut, out_hi, 0, cap, F)) != 0 || (rc = tma_encode_store_2d(&p->tmOut2, out_lo, 0, cap, F)) != 0)
     return rc;
   return gemm_pair_prepare();
@@ -464,22 +555,24 @@ int gemm_pair_plan_create_kv(GemmPairPlan *p, int nh, int K, const void *Xhi, co
 }
 
 int gemm_pair_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<PG_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair_kernel<PG_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_pair_kernel<PG_KV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
-  if (e != cudaSuccess) { g_last_cuda_error = (int)e; return CORUN_ECUDA; }
+  for (auto kernel : {gemm_pair_kernel<PG_PLAIN, false>, gemm_pair_kernel<PG_SWIGLU, false>, gemm_pair_kernel<PG_KV, false>,
+                      gemm_pair_kernel<PG_PLAIN, true>, gemm_pair_kernel<PG_SWIGLU, true>}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
+    if (e != cudaSuccess) { g_last_cuda_error = (int)e; return CORUN_ECUDA; }
+  }
   return CORUN_OK;
 }
 
 cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st, const CUtensorMap *tmW96) {
-  if (R < 1 || R > p.cap) return cudaErrorInvalidValue;
+  if (R < 1 || R > p.cap || (p.decode && (p.cap != 256 || !p.row_blocks))) return cudaErrorInvalidValue;
   const PairShape q = pair_shape(p, R, tmW96 != nullptr);
   const int pairs = q.units < p.pairs ? q.units : p.pairs;
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, q.half == 96 ? *tmW96 : tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2,
                     R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, p.per_unit, q.half, d_status, p.row_blocks, p.cap);
   };
-  return p.kv_heads ? go(gemm_pair_kernel<PG_KV>) : p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU>) : go(gemm_pair_kernel<PG_PLAIN>);
+  if (p.decode) return p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU, true>) : go(gemm_pair_kernel<PG_PLAIN, true>);
+  return p.kv_heads ? go(gemm_pair_kernel<PG_KV, false>) : p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU, false>) : go(gemm_pair_kernel<PG_PLAIN, false>);
 }
 
 }  // namespace corun

@@ -38,7 +38,7 @@ def test_router_shares(H, E, K, B):
             np.testing.assert_allclose(pr[b], p_all[ex[b]], atol=2e-6, rtol=1e-5)
 
 
-@pytest.mark.parametrize("arch,B", [("moe", 1), ("moe", 16), ("moe", 17), ("moe", 64), ("moe", 130), ("dense", 130)])
+@pytest.mark.parametrize("arch,B", [("moe", 1), ("moe", 16), ("moe", 17), ("moe", 64), ("moe", 130), ("dense", 130), ("dense", 200)])
 def test_one_request_and_all_slots(orc, arch, B):
     from paper_2608_14376_b200 import corun
 

@@ -90,7 +90,7 @@ def test_a_blocks_largest_weight_is_exact(hd):
 
 def _product(form, N, K, R, seed):
     """The GEMM on pairs of SMs -> (result, 64-bit result, 64-bit result of the activations as bf16 pairs, that of their bf16 part
-    alone).  Forms: 0 plain, 1 with SwiGLU, 2 keys and values."""
+    alone).  Forms: 0 plain, 1 with SwiGLU, 2 keys and values; 3, 4: 0, 1 of a decode step."""
     import torch
 
     from paper_2608_14376_b200 import corun
@@ -103,7 +103,7 @@ def _product(form, N, K, R, seed):
 
     def f(x):
         y = x @ W.double().T
-        return torch.nn.functional.silu(y[:, :N // 2]) * y[:, N // 2:] if form == 1 else y
+        return torch.nn.functional.silu(y[:, :N // 2]) * y[:, N // 2:] if form in (1, 4) else y
 
     return corun.debug_gemm_pair(form, W, X).double(), f(X.double()), f(hi.double() + lo.double()), f(hi.double())
 
@@ -112,13 +112,31 @@ def _product(form, N, K, R, seed):
 # out slice by slice, one slice and eight
 @pytest.mark.parametrize("form,N,K,R", [(0, 8, 64, 1), (0, 200, 192, 257), (0, 1536, 1024, 300), (0, 4096, 4096, 256), (0, 6144, 4096, 129),
                                         (0, 1024, 3072, 1000), (0, 4096, 12288, 515), (1, 128, 64, 31), (1, 1408, 1024, 255),
-                                        (1, 2 * 12288, 4096, 256), (1, 2 * 3072, 1024, 777), (2, 256, 256, 65), (2, 1024, 512, 513)])
+                                        (1, 2 * 12288, 4096, 256), (1, 2 * 3072, 1024, 777), (2, 256, 256, 65), (2, 1024, 512, 513),
+                                        (3, 200, 192, 1), (3, 4096, 12288, 33), (3, 6144, 4096, 128), (3, 1536, 1024, 129), (3, 4096, 4096, 256),
+                                        (4, 1408, 1024, 65), (4, 2 * 12288, 4096, 128), (4, 2 * 12288, 4096, 200), (4, 2 * 3072, 1024, 97)])
 def test_pair_gemm_matches_fp64(form, N, K, R):
     got, want, pairs, bf16 = _product(form, N, K, R, seed=N + K + R)
     off = lambda a, b: float((a - b).norm() / b.norm())
     # 16 significand bits of the activations (2.5e-6), a slice's sum cut off at every MMA (1.7e-8 each, at most 24 k-blocks of 8:
     # 3.3e-6); a SwiGLU's result is a product of two such sums and stored as a bf16 pair (2e-6)
-    bound = 4.5e-6 if form != 1 else 8e-6
+    bound = 8e-6 if form in (1, 4) else 4.5e-6
     assert off(got, want) <= bound, off(got, want)
     assert off(got, pairs) <= off(got, want) + 1e-6
     assert off(bf16, want) > 10 * bound                # without the lo part it would not pass
+
+
+@pytest.mark.parametrize("form,N,K", [(3, 200, 192), (3, 6144, 4096), (3, 4096, 12288), (4, 1408, 1024), (4, 2 * 12288, 4096)])
+def test_decode_pair_gemm_gives_a_row_the_same_bytes_in_both_forms(form, N, K):
+    """Up to 128 rows the hi and lo parts are stacked in one operand, above they have an accumulator each."""
+    import torch
+
+    from paper_2608_14376_b200 import corun
+
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    W = (torch.randn((N, K), generator=g, device="cuda") * 0.02).bfloat16()
+    X = torch.randn((256, K), generator=g, device="cuda")
+    full = corun.debug_gemm_pair(form, W, X)
+    for R in (1, 31, 64, 65, 97, 128, 129, 200):
+        assert torch.equal(corun.debug_gemm_pair(form, W, X[:R].contiguous()), full[:R]), R
+    assert torch.equal(corun.debug_gemm_pair(form, W, X[100:200].contiguous()), full[100:200])
