@@ -5,7 +5,10 @@
 // 256 tokens of a chunk; here it is 960, and the cache is read once per chunk.
 //
 // The cached latents are fp16 and enter the GEMM exactly (bf16 hi + lo); its fp32 results are kept as fp16 hi + lo pairs,
-// queries and weights are hi + lo pairs too, and of the products only lo * lo is left out.
+// queries and weights are hi + lo pairs too, and of the products only lo * lo is left out.  Such a pair holds 22 bits of values
+// between 2^-13 and 2^15 only, so what goes into one is scaled by powers of two: keys and values per layer and head by what
+// the weights allow at most (mla_kv_scale_kernel), a row's query by its own largest value.  The scales leave with the scores
+// and with the division by the weights' sum, exactly.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math_constants.h>
@@ -33,6 +36,14 @@ __device__ __forceinline__ float ml_ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// 2^e with x * 2^e <= 2^top, as large as that (1 for zero and for what is not finite; within 2^-60 .. 2^60)
+__device__ __forceinline__ float ml_pow2_below(float x, int top) {
+  if (!(x > 0.f) || x > 3.0e38f) return 1.f;
+  int e;
+  frexpf(x, &e);                                    // x < 2^e
+  e = top - e;
+  return __int_as_float(((e < -60 ? -60 : e > 60 ? 60 : e) + 127) << 23);
+}
 // eight fp32 -> fp16 hi and lo parts, 16 bytes each
 __device__ __forceinline__ void ml_split8(const float *x, uint4 &hi, uint4 &lo) {
   __half2 h[4], l[4];
@@ -44,6 +55,30 @@ __device__ __forceinline__ void ml_split8(const float *x, uint4 &hi, uint4 &lo) 
   }
   hi = *reinterpret_cast<const uint4 *>(h);
   lo = *reinterpret_cast<const uint4 *>(l);
+}
+
+// The largest power of two that keeps a head's keys (blockIdx.y 0) or values (1) at 2^10 or below: |sum_c w_c g_c x_c| <=
+// rank * max |w_c g_c| for a normalised latent x (the sum of its squares is rank); what is met in practice lies some 2^6 below.
+__global__ void __launch_bounds__(256)
+mla_kv_scale_kernel(const __nv_bfloat16 *__restrict__ wkv_b, const __nv_bfloat16 *__restrict__ gains, MlaDims d, float *__restrict__ scale) {
+  __shared__ float most[8];
+  const int h = blockIdx.x, part = blockIdx.y, width = part ? d.vh : d.nope;
+  const __nv_bfloat16 *w = wkv_b + ((size_t)h * (d.nope + d.vh) + (part ? d.nope : 0)) * d.rank;
+  float m = 0.f;
+  for (int i = 8 * threadIdx.x; i < width * d.rank; i += 8 * 256) {
+    const uint4 a = *reinterpret_cast<const uint4 *>(w + i);
+    const __nv_bfloat16 *x = reinterpret_cast<const __nv_bfloat16 *>(&a), *g = gains + i % d.rank;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(__bfloat162float(x[j]) * __bfloat162float(g[j])));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) most[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) m = fmaxf(m, most[i]);
+    scale[2 * h + part] = ml_pow2_below(m * (float)d.rank, 10);
+  }
 }
 
 // The latents of the segments' cached tokens as a bf16 hi / lo pair (exact) and their rotary keys (fp16), one warp per token.
@@ -91,16 +126,17 @@ mla_gather_kernel(const __grid_constant__ MlaSegs g, MlaCache cache, int rank, i
 __global__ void __launch_bounds__(ML_THREADS, 1)
 mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmR, const __nv_bfloat16 *__restrict__ qn_hi,
                    const __nv_bfloat16 *__restrict__ qn_lo, const float *__restrict__ q_rope, Rows rows, int rows_per_head, int nh, int rope,
-                   int cap, const int *__restrict__ tile_base, float scale_log2e, __nv_bfloat16 *__restrict__ ao_hi,
+                   int cap, const int *__restrict__ tile_base, float scale_log2e, const float2 *__restrict__ kv_scale, __nv_bfloat16 *__restrict__ ao_hi,
                    __nv_bfloat16 *__restrict__ ao_lo, int *status) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t kfull, kempty, vfull, vempty, s_full[2], s_free[2], p_ready, p_free, o_full[2], o_free[2], c_ready[4], l_ready;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
-  __shared__ float corr_s[4][128], l_s[128];
+  __shared__ float corr_s[4][128], l_s[128], row_scale_s[128], q_most[2][128];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int h = blockIdx.x, tile = (int)gridDim.y - 1 - (int)blockIdx.y;   // the last tiles (the most keys) first
   const int row0 = tile * 128;
+  const float2 kvs = __ldg(kv_scale + h);           // the head's keys and values are stored times these
   // the tile's rows with a token are the first ones
   const int n_rows = __syncthreads_count(tid < 128 && row0 + tid < rows.R && rows.active[row0 + tid] != 0);
   if (n_rows == 0) return;
@@ -131,10 +167,13 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
   }
   if (warp >= 2) {
     // the query tile: row m = token m, 24 chunks of 8 dims (128 no-rope, then the rotary ones, zeros beyond them)
-    const int m = (tid - 64) & 127, r = row0 + m;
+    const int m = (tid - 64) & 127, r = row0 + m, part = (tid - 64) >> 7;
     const bool on = r < rows.R;
-    for (int c = (tid - 64) >> 7; c < 24; c += 2) {
-      float x[8];
+    float all[12][8], most = 0.f;                   // every other chunk; the rotary ones at the scale of the keys beside theirs
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const int c = part + 2 * k;
+      float *x = all[k];
 #pragma unroll
       for (int i = 0; i < 8; ++i) x[i] = 0.f;
       if (on && c < 16) {
@@ -146,8 +185,21 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
       } else if (on && 8 * (c - 16) < rope) {
         const float *q = q_rope + ((size_t)r * nh + h) * rope + 8 * (c - 16);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = q[i];
+        for (int i = 0; i < 8; ++i) x[i] = q[i] * kvs.x;
       }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) most = fmaxf(most, fabsf(x[i]));
+    }
+    q_most[part][m] = most;
+    asm volatile("bar.sync 1, 256;" ::: "memory");   // warps 2-9
+    const float q_scale = ml_pow2_below(fmaxf(q_most[0][m], q_most[1][m]), 14);
+    if (part == 0) row_scale_s[m] = scale_log2e / q_scale / kvs.x;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const int c = part + 2 * k;
+      float *x = all[k];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] *= q_scale;
       uint4 hi, lo;
       ml_split8(x, hi, lo);
       const uint32_t off = (uint32_t)(c >> 3) * (128 * 128) + ml_swz(m, c & 7);
@@ -234,6 +286,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
   } else if (warp < 6) {
     // ---------------- softmax: one thread per row ----------------
     const int pos = real ? rows.pos[row0 + tl] : -1;
+    const float scale = row_scale_s[tl];            // scores to the base-2 domain, without the operands' scales
     float mx = -CUDART_INF_F, l = 0.f;
     for (int j = 0; j < n_blocks; ++j) {
       const int sb = j & 1;
@@ -251,11 +304,11 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
       float bm = -CUDART_INF_F;
       if (lim >= ML_KEYS - 1) {
 #pragma unroll
-        for (int i = 0; i < ML_KEYS; ++i) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale_log2e);
+        for (int i = 0; i < ML_KEYS; ++i) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale);
       } else {
 #pragma unroll
         for (int i = 0; i < ML_KEYS; ++i)
-          if (i <= lim) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale_log2e);
+          if (i <= lim) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale);
       }
       const float m_new = fmaxf(mx, bm), m_use = m_new == -CUDART_INF_F ? 0.f : m_new;   // (rows without a token: nothing visible)
       const float corr = ml_ex2(mx - m_use);
@@ -264,7 +317,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
       float p[ML_KEYS];
 #pragma unroll
       for (int i = 0; i < ML_KEYS; ++i) {
-        p[i] = i <= lim ? ml_ex2(fmaf(__uint_as_float(sv[i >> 4][i & 15]), scale_log2e, -m_use)) : 0.f;
+        p[i] = i <= lim ? ml_ex2(fmaf(__uint_as_float(sv[i >> 4][i & 15]), scale, -m_use)) : 0.f;
         acc[i & 3] += p[i];
       }
       l = l * corr + ((acc[0] + acc[1]) + (acc[2] + acc[3]));
@@ -315,7 +368,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
     bool ok = !failed && mbar_wait(smem_u32(&l_ready), 0u, &abort_flag);
     ok = __all_sync(0xffffffffu, ok);
     if (ok && real) {
-      const float inv = 1.f / l_s[tl];
+      const float inv = 1.f / l_s[tl] / kvs.y;
       const size_t at = ((size_t)(row0 + tl) * nh + h) * 128;
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
@@ -349,15 +402,20 @@ cudaError_t launch_mla_gather(const MlaSegs &g, const MlaCache &cache, int rank,
   return launch_k(mla_gather_kernel, dim3((total + 7) / 8), dim3(256), 0, st, true, g, cache, rank, rope, total, c_hi, c_lo, kr);
 }
 
+cudaError_t launch_mla_kv_scale(const __nv_bfloat16 *wkv_b, const __nv_bfloat16 *gains, const MlaDims &d, float2 *scale, cudaStream_t st) {
+  mla_kv_scale_kernel<<<dim3(d.nh, 2), 256, 0, st>>>(wkv_b, gains, d, reinterpret_cast<float *>(scale));
+  return cudaGetLastError();
+}
+
 cudaError_t mla_prefill_prepare() {
   return cudaFuncSetAttribute(mla_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ML_SMEM);
 }
 
 cudaError_t launch_mla_prefill(const CUtensorMap &tmKV, const CUtensorMap &tmR, const __nv_bfloat16 *qn_hi, const __nv_bfloat16 *qn_lo,
                                const float *q_rope, const Rows &rows, int rows_per_head, const MlaDims &d, int cap, const int *tile_base,
-                               float scale, __nv_bfloat16 *ao_hi, __nv_bfloat16 *ao_lo, int *d_status, cudaStream_t st) {
+                               float scale, const float2 *kv_scale, __nv_bfloat16 *ao_hi, __nv_bfloat16 *ao_lo, int *d_status, cudaStream_t st) {
   return launch_k(mla_prefill_kernel, dim3(d.nh, (rows.R + 127) / 128), dim3(ML_THREADS), ML_SMEM, st, false, tmKV, tmR, qn_hi, qn_lo, q_rope,
-                  rows, rows_per_head, d.nh, d.rope, cap, tile_base, scale * 1.4426950408889634f, ao_hi, ao_lo, d_status);
+                  rows, rows_per_head, d.nh, d.rope, cap, tile_base, scale * 1.4426950408889634f, kv_scale, ao_hi, ao_lo, d_status);
 }
 
 }  // namespace corun

@@ -173,6 +173,7 @@ struct corun_engine {
   bool big_mla_tiles = false;            // Program::mla_tiles of the prefill program
   std::vector<const bf16 *> kv_norm;
   bf16 *w_ukT = nullptr;                 // [L][nh * rank][nope]: the key up-projections transposed
+  float2 *kv_scale = nullptr;            // [L][nh]: scales of decompressed keys and values (launch_mla_kv_scale)
   std::vector<CUtensorMap> tm_uk, tm_uv, tm_c, tm_cv, tm_gu_d, tm_down_d;
   const void *w0_uv = nullptr, *w0_gu_d = nullptr, *w0_down_d = nullptr;
   // KV
@@ -643,10 +644,11 @@ cudaError_t run_mla_tiles(corun_engine *e, Program &P, int l, const Rows &rows) 
   const MlaDims &md = e->md;
   const MlaCache cache{e->kv_pool + (size_t)l * e->layer_stride, e->d_block_table, e->max_blocks, e->B, (long long)e->pool_blocks, e->kv_run};
   cudaError_t ce = launch_mla_gather(P.segs, cache, md.rank, md.rope, P.kv_tokens, P.c_hi, P.c_lo, P.kr, e->st);
-  if (ce == cudaSuccess) ce = gemm_pair_launch(P.b_kv, e->tb_uv[l], P.kv_tokens, e->d_status, e->st);
+  const float2 *scale = e->kv_scale + (size_t)l * md.nh;
+  if (ce == cudaSuccess) ce = gemm_pair_launch(P.b_kv, e->tb_uv[l], P.kv_tokens, e->d_status, e->st, nullptr, reinterpret_cast<const float *>(scale));
   if (ce == cudaSuccess)
     ce = launch_mla_prefill(P.tm_kvd, P.tm_kr, P.qn_hi, P.qn_lo, P.q_rope, rows, P.RPH, md, P.kv_cap, P.tile_base,
-                            1.0f / sqrtf((float)(md.nope + md.rope)), P.ao_hi, P.ao_lo, e->d_status, e->st);
+                            1.0f / sqrtf((float)(md.nope + md.rope)), scale, P.ao_hi, P.ao_lo, e->d_status, e->st);
   return ce;
 }
 
@@ -1144,14 +1146,21 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     e->tm_uv.resize(s.n_layers);
     // (contexts beyond 16384 would need more than half a GB of decompressed keys and values: the decode form serves them)
     e->big_mla_tiles = big_cap > 0 && md.nope == 128 && md.vh == 128 && max_context <= 16384;
-    if (e->big_mla_tiles) e->tb_uv.resize(s.n_layers);
+    if (e->big_mla_tiles) {
+      e->tb_uv.resize(s.n_layers);
+      if ((rc = dmalloc(e->allocs, &e->kv_scale, (size_t)s.n_layers * md.nh, false))) return fail(rc);
+    }
     for (int l = 0; l < s.n_layers; ++l) {
       e->kv_norm.push_back((const bf16 *)mla->kv_norm[l]);
       bf16 *dst = e->w_ukT + (size_t)l * per_layer;
       if (launch_mla_transpose_uk((const bf16 *)mla->wkv_b[l], md, dst, 0) != cudaSuccess) return fail(CORUN_ECUDA);
       if ((rc = gemm_encode_map(&e->tm_uk[l], dst, md.nh * md.rank, md.nope, GEMM_TILE_N))) return fail(rc);
       if ((rc = gemm_encode_map(&e->tm_uv[l], mla->wkv_b[l], md.nh * (md.nope + md.vh), md.rank, GEMM_TILE_N))) return fail(rc);
-      if (e->big_mla_tiles && (rc = gemm_encode_map(&e->tb_uv[l], mla->wkv_b[l], md.nh * 256, md.rank, 128))) return fail(rc);
+      if (e->big_mla_tiles) {
+        if ((rc = gemm_encode_map(&e->tb_uv[l], mla->wkv_b[l], md.nh * 256, md.rank, 128))) return fail(rc);
+        if (launch_mla_kv_scale((const bf16 *)mla->wkv_b[l], e->kv_norm[l], md, e->kv_scale + (size_t)l * md.nh, 0) != cudaSuccess)
+          return fail(CORUN_ECUDA);
+      }
     }
   }
   if (moe) {
@@ -2028,7 +2037,7 @@ int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, con
   std::vector<void *> keep;
   bf16 *hi = nullptr, *lo = nullptr, *ohi = nullptr, *olo = nullptr;
   __half *kv = nullptr;
-  float *part = nullptr, *full = nullptr;
+  float *part = nullptr, *full = nullptr, *ones = nullptr;   // ones: form 2's scales
   int *status = nullptr, rc = CORUN_OK;              // status word | row_blocks
   GemmPairPlan p;
   CUtensorMap tw, tw96;
@@ -2041,15 +2050,16 @@ int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, con
     else if (form == 1)
       ok(dmalloc(keep, &ohi, c * F)) && ok(dmalloc(keep, &olo, c * F)) && ok(gemm_pair_plan_create_swiglu(&p, F, K, hi, lo, cap, ohi, olo, sms, decode));
     else
-      ok(dmalloc(keep, &kv, 4 * c * nh * 128)) && ok(gemm_pair_plan_create_kv(&p, nh, K, hi, lo, cap, kv, sms));
+      ok(dmalloc(keep, &kv, 4 * c * nh * 128)) && ok(dmalloc(keep, &ones, (size_t)2 * nh)) && ok(gemm_pair_plan_create_kv(&p, nh, K, hi, lo, cap, kv, sms));
   }
   if (rc == CORUN_OK) {
     cudaError_t ce = cudaDeviceSynchronize();       // allocations were cleared through the legacy stream
     const int blocks = R > 128 ? 3 : 1;
     if (ce == cudaSuccess && decode) ce = cudaMemcpy(status + 1, &blocks, sizeof(int), cudaMemcpyHostToDevice);
     if (decode) p.row_blocks = status + 1;
+    if (ce == cudaSuccess && form == 2) ce = cudaMemcpy(ones, std::vector<float>((size_t)2 * nh, 1.f).data(), (size_t)2 * nh * sizeof(float), cudaMemcpyHostToDevice);
     if (ce == cudaSuccess) ce = launch_split(X, R, K, hi, lo, st);
-    if (ce == cudaSuccess) ce = gemm_pair_launch(p, tw, decode ? 256 : R, status, st, form == 1 ? &tw96 : nullptr);
+    if (ce == cudaSuccess) ce = gemm_pair_launch(p, tw, decode ? 256 : R, status, st, form == 1 ? &tw96 : nullptr, ones);
     if (ce == cudaSuccess && form == 0) ce = gemm_pair_fixup_launch(p, decode ? 256 : R, st);
     if (ce == cudaSuccess && form == 0) ce = cudaMemcpyAsync(out, full, (size_t)R * N * sizeof(float), cudaMemcpyDeviceToDevice, st);
     if (ce == cudaSuccess && form == 1) ce = launch_join(ohi, olo, false, R, F, out, F, st);

@@ -239,13 +239,14 @@ cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st
 int gemm_pair_plan_create_swiglu(GemmPairPlan *p, int F, int K, const void *Xhi, const void *Xlo, int cap, __nv_bfloat16 *out_hi,
                                  __nv_bfloat16 *out_lo, int num_sms, bool decode = false);
 // Decompression of latents into keys and values: W is [nh * 256, K] (per head 128 key rows, 128 value rows); the fp16 hi / lo
-// pairs of the products go to kv [key hi | key lo | value hi | value lo][nh][cap][128] (cap % 32 == 0).
+// pairs of the products, times the launch's kv_scale [nh][2] (keys, values; device), go to kv [key hi | key lo | value hi | value
+// lo][nh][cap][128] (cap % 32 == 0).
 int gemm_pair_plan_create_kv(GemmPairPlan *p, int nh, int K, const void *Xhi, const void *Xlo, int cap, void *kv, int num_sms);
 int gemm_pair_prepare();             // opts the kernels into their shared-memory size (idempotent)
 // Rows 0 .. R-1 (R <= cap).  tmW: the weight matrix with a box of 128 rows (gemm_encode_map(.., 128)); tmW96 (swiglu): the
 // same with 96 rows, taken where it shortens the waves.
 cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st,
-                             const CUtensorMap *tmW96 = nullptr);
+                             const CUtensorMap *tmW96 = nullptr, const float *kv_scale = nullptr);
 // Tensor map for TMA stores of tiles of 32 rows x 32 columns into a [rows, cols] row-major matrix (fp32: 128-byte swizzle; bf16: 64).
 int tma_encode_store_2d(CUtensorMap *m, const void *base, int is_fp32, unsigned long long rows, int cols);
 // direct[r, n] = gemm_load(r, n) for every tile that has partials (makes `direct` a plain matrix).

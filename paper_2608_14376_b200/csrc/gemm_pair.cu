@@ -52,7 +52,8 @@ constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + PG_EPI * 
 // SWIGLU: W is a gate / up matrix ([2F, K]); a tile is `half` gate rows (first CTA) and the up rows of the same outputs
 // (second CTA), always whole (the slices meet in registers), and the epilogue writes silu(gate) * up as the bf16 hi/lo pair the down GEMM reads.
 // KV (gemm_pair_plan_create_kv): a tile's 256 columns are one head's 128 key and 128 value columns, stored as fp16 hi / lo
-// pairs, keys by the first half of the epilogue warps, values by the second; cap: rows of one of the four matrices per head.
+// pairs, keys by the first half of the epilogue warps, values by the second; cap: rows of one of the four matrices per head;
+// kv_scale: [head][2] powers of two that keep a head's keys and values within the range of such a pair.
 //
 // DECODE (up to 256 rows, one row tile; row_blocks says which halves of them hold requests this step): hi and lo have an
 // accumulator each, a slice's value is their sum.  With requests in rows 128 .. each CTA keeps both accumulators (512 columns:
@@ -66,7 +67,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                  const __grid_constant__ CUtensorMap tmLo, const __grid_constant__ CUtensorMap tmOut,
                  const __grid_constant__ CUtensorMap tmOut2, int R, int N, int KB, int row_tiles, int whole, int units, int slices,
-                 int per_unit, int half, int *status, const int *row_blocks, int cap) {
+                 int per_unit, int half, int *status, const int *row_blocks, int cap, const float *kv_scale) {
   constexpr bool SWIGLU = MODE == PG_SWIGLU, KV = MODE == PG_KV;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[PG_STAGES];      // used in the first CTA: both CTAs' loads of a stage
@@ -251,6 +252,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         if (row0 < R) {                             // warp-uniform
           if (KV) {
             const int nh = N / GEMM_TILE_N;
+            const float scale = __ldg(kv_scale + 2 * nt + grp);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               uint32_t v[32];
@@ -263,7 +265,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 __half a[8], b[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                  const float x = __uint_as_float(v[8 * c + j]);
+                  const float x = __uint_as_float(v[8 * c + j]) * scale;
                   a[j] = __float2half_rn(x);
                   b[j] = __float2half_rn(x - __half2float(a[j]));
                 }
@@ -563,13 +565,14 @@ int gemm_pair_prepare() {
   return CORUN_OK;
 }
 
-cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st, const CUtensorMap *tmW96) {
-  if (R < 1 || R > p.cap || (p.decode && (p.cap != 256 || !p.row_blocks))) return cudaErrorInvalidValue;
+cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st, const CUtensorMap *tmW96,
+                             const float *kv_scale) {
+  if (R < 1 || R > p.cap || (p.decode && (p.cap != 256 || !p.row_blocks)) || (p.kv_heads && !kv_scale)) return cudaErrorInvalidValue;
   const PairShape q = pair_shape(p, R, tmW96 != nullptr);
   const int pairs = q.units < p.pairs ? q.units : p.pairs;
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, q.half == 96 ? *tmW96 : tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2,
-                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, p.per_unit, q.half, d_status, p.row_blocks, p.cap);
+                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, p.per_unit, q.half, d_status, p.row_blocks, p.cap, kv_scale);
   };
   if (p.decode) return p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU, true>) : go(gemm_pair_kernel<PG_PLAIN, true>);
   return p.kv_heads ? go(gemm_pair_kernel<PG_KV, false>) : p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU, false>) : go(gemm_pair_kernel<PG_PLAIN, false>);

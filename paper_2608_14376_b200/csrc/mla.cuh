@@ -80,12 +80,14 @@ struct MlaSegs { int n, slot[MLA_MAX_SEGS], off[MLA_MAX_SEGS], len[MLA_MAX_SEGS]
 cudaError_t launch_mla_gather(const MlaSegs &g, const MlaCache &cache, int rank, int rope, int total, __nv_bfloat16 *c_hi,
                               __nv_bfloat16 *c_lo, __half *kr, cudaStream_t st);
 cudaError_t mla_prefill_prepare();   // opts the kernel into its shared-memory size (idempotent)
+// Powers of two that bring a layer's decompressed keys and values into the range of an fp16 hi / lo pair: scale[h] = (keys, values).
+cudaError_t launch_mla_kv_scale(const __nv_bfloat16 *wkv_b, const __nv_bfloat16 *gains, const MlaDims &d, float2 *scale, cudaStream_t st);
 // Causal attention of the chunk's rows (tiles of 128 rows, each of one request, whose gathered tokens start at
 // tile_base[tile]) -> bf16 hi / lo [R][nh * 128].  tmKV: boxes of 64 x 64 over the decompressed [key hi | key lo | value hi |
-// value lo][nh][cap][128] fp16; tmR: the same over the rotary keys [cap][64].
+// value lo][nh][cap][128] fp16, scaled by kv_scale; tmR: the same over the rotary keys [cap][64].
 cudaError_t launch_mla_prefill(const CUtensorMap &tmKV, const CUtensorMap &tmR, const __nv_bfloat16 *qn_hi, const __nv_bfloat16 *qn_lo,
                                const float *q_rope, const Rows &rows, int rows_per_head, const MlaDims &d, int cap, const int *tile_base,
-                               float scale, __nv_bfloat16 *ao_hi, __nv_bfloat16 *ao_lo, int *d_status, cudaStream_t st);
+                               float scale, const float2 *kv_scale, __nv_bfloat16 *ao_hi, __nv_bfloat16 *ao_lo, int *d_status, cudaStream_t st);
 
 // The value part of the grouped up-projection result uv [nh * rows_per_head][nope + vh] (columns nope.. of every
 // row) -> bf16 hi/lo [R][nh * vh], the o-projection's activations.

@@ -140,3 +140,79 @@ def test_decode_pair_gemm_gives_a_row_the_same_bytes_in_both_forms(form, N, K):
     for R in (1, 31, 64, 65, 97, 128, 129, 200):
         assert torch.equal(corun.debug_gemm_pair(form, W, X[:R].contiguous()), full[:R]), R
     assert torch.equal(corun.debug_gemm_pair(form, W, X[100:200].contiguous()), full[100:200])
+
+
+MLA = dict(kv_lora_rank=256, qk_nope=128, qk_rope=32, v_head=128, first_dense=2)
+
+
+def _latent(scale_k=None, scale_v=None, B=2, T=700, seed=2, kv_block=64, mla=MLA):
+    """A dense decoder with latent attention; scale_k, scale_v: per head, powers of two that its keys (queries: their inverse)
+    and its values (output projection: their inverse) are multiplied by, which changes nothing in exact arithmetic."""
+    from paper_2608_14376_b200 import corun
+
+    nh, nope, rope, vh = 4, mla["qk_nope"], mla["qk_rope"], mla["v_head"]
+    sh = synth.ModelShape(2, 256, nh, nh, 128, 384, 1024, 1e-6, 10000.0)
+    w, m = synth.make_mla_weights_numpy(sh, mla, seed=seed, std=0.05)
+
+    def times(bits, where, f):
+        x = synth.bf16_bits_to_f32(bits)
+        x[where] *= np.float32(f)
+        bits[:] = synth.f32_to_bf16_bits(x)
+
+    for l in range(sh.n_layers):
+        for h in range(nh) if scale_k is not None else ():
+            times(m["wkv_b"][l], slice(h * (nope + vh), h * (nope + vh) + nope), scale_k[h])
+            times(w["wqkv"][l], slice(h * (nope + rope), h * (nope + rope) + nope), 1 / scale_k[h])
+            times(m["wkv_b"][l], slice(h * (nope + vh) + nope, (h + 1) * (nope + vh)), scale_v[h])
+            times(w["wo"][l], (slice(None), slice(h * vh, (h + 1) * vh)), 1 / scale_v[h])
+    wt, mt = synth.mla_numpy_to_torch(w, m, "cuda")
+    return sh, m, corun.Engine(sh, wt, B, T, mla=mt, kv_block=kv_block)
+
+
+@pytest.mark.parametrize("pos0,n", [(0, 1), (0, 129), (63, 2), (500, 77), (64, 300)])
+def test_latent_prefill_attention_matches_fp64(pos0, n):
+    rng = np.random.default_rng(n)
+    T = pos0 + n
+    sh, m, eng = _latent(T=T)
+    nh, rank, nope, rope = 4, MLA["kv_lora_rank"], MLA["qk_nope"], MLA["qk_rope"]
+    try:
+        eng.adopt(1, 0, T, 0)
+        eng.kv_write(1, 0, 0, rng.standard_normal((T, rank + rope)).astype(np.float32), None)
+        c = eng.kv_read(1, 0, 0, T)[0].astype(np.float64)
+        pair = lambda x: (lambda hi: hi + synth.bf16_bits_to_f32(synth.f32_to_bf16_bits(x - hi)))(synth.bf16_bits_to_f32(synth.f32_to_bf16_bits(x)))
+        q = pair(2 * rng.standard_normal((n, nh, nope + rope)).astype(np.float32))   # what a bf16 pair holds exactly
+        got = eng.prefill_attention(1, 0, pos0, q)
+    finally:
+        eng.close()
+    W = synth.bf16_bits_to_f32(m["wkv_b"][0]).astype(np.float64).reshape(nh, nope + 128, rank)
+    k = np.concatenate([np.einsum("tc,hdc->thd", c[:, :rank], W[:, :nope]), np.repeat(c[:, None, rank:], nh, 1)], -1)
+    v = np.einsum("tc,hdc->thd", c[:, :rank], W[:, nope:])
+    scale = (nope + rope) ** -0.5
+    want, _ = _attend(q, k, v, pos0, scale)
+    rms = lambda x: np.sqrt(np.mean(np.square(x)))
+    # the result is stored as a bf16 pair (3e-6 in the mean); sums cut off by the tensor core (1.7e-8 for each of 64 MMAs over a
+    # latent, 44 over a block) move scores of up to 20 by some 1e-6 and values by as much of themselves
+    bound = 1e-5 * rms(want)
+    assert rms(got - want) <= bound, rms(got - want) / rms(want)
+    if T > 100:                                       # keys or values without their lo part would not pass
+        assert rms(_attend(q, k.astype(np.float16), v, pos0, scale)[0] - want) > 3 * bound
+        assert rms(_attend(q, k, v.astype(np.float16), pos0, scale)[0] - want) > 3 * bound
+
+
+def test_latent_prefill_does_not_depend_on_the_scale_of_keys_and_values():
+    """Keys, values and queries a million times larger or smaller, per head, are the same bytes in the end (as fp16 pairs they
+    would overflow above 65504 and lose their low bits below 1e-4)."""
+    prompt = synth.make_prompts(1024, [300], seed=5)[0]
+    out = []
+    for ks, vs in ((None, None), ([2.0 ** -20, 2.0 ** 20, 2.0 ** 9, 2.0 ** -20], [2.0 ** -20, 2.0 ** 20, 2.0 ** -9, 2.0 ** 22])):
+        _, _, eng = _latent(ks, vs, T=310)
+        try:
+            eng.prefill(1, prompt, 310)
+            out.append(eng.logits(1))
+            eng.force_token(1, 7)
+            eng.decode_step(np.array([0, 1], np.uint8), np.zeros(2, np.uint64))
+            out.append(eng.logits(1))
+        finally:
+            eng.close()
+    assert np.isfinite(out[2]).all()
+    assert out[0].tobytes() == out[2].tobytes() and out[1].tobytes() == out[3].tobytes()
