@@ -672,6 +672,7 @@ cudaError_t attention_prepare() {
   if (e == cudaSuccess) e = prepare_one<64, 2>();
   if (e == cudaSuccess) e = prepare_one<64, 4>();
   if (e == cudaSuccess) e = prepare_one<64, 8>();
+  if (e == cudaSuccess) e = attention_prefill_prepare();
   return e;
 }
 

@@ -337,20 +337,19 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
 }
 
 template <int HD, int GROUP>
-cudaError_t pf_launch(dim3 grid, cudaStream_t st, const CUtensorMap &tmKV, const float *q, const Rows &rows, int nq, const KvLayout &kv,
-                      __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int *d_status) {
-  static bool prepared = false;
-  if (!prepared) {
-    cudaError_t e = cudaFuncSetAttribute(attn_prefill_kernel<HD, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)PfLayout<HD>::SMEM);
-    if (e != cudaSuccess) return e;
-    prepared = true;
-  }
-  return launch_k(attn_prefill_kernel<HD, GROUP>, grid, dim3(PF_THREADS), PfLayout<HD>::SMEM, st, true, tmKV, q, rows, nq, kv, out_hi,
-                  out_lo, d_status);
+cudaError_t pf_prepare() {
+  return cudaFuncSetAttribute(attn_prefill_kernel<HD, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PfLayout<HD>::SMEM);
 }
 
 }  // namespace
+
+cudaError_t attention_prefill_prepare() {
+  cudaError_t e = cudaSuccess;
+  for (auto prepare : {pf_prepare<128, 1>, pf_prepare<128, 2>, pf_prepare<128, 4>, pf_prepare<128, 8>, pf_prepare<64, 1>, pf_prepare<64, 2>,
+                       pf_prepare<64, 4>, pf_prepare<64, 8>})
+    if (e == cudaSuccess) e = prepare();
+  return e;
+}
 
 cudaError_t launch_attention_prefill(const CUtensorMap &tmKV, const float *q, const Rows &rows, int nq, const KvLayout &kv,
                                      __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int *d_status, cudaStream_t st) {
@@ -360,7 +359,8 @@ cudaError_t launch_attention_prefill(const CUtensorMap &tmKV, const float *q, co
   const int tpt = 128 / group;
   const dim3 grid(kv.n_kv, (rows.R + tpt - 1) / tpt);
 #define CORUN_PF_CASE(HD_, G_) \
-  if (kv.hd == HD_ && group == G_) return pf_launch<HD_, G_>(grid, st, tmKV, q, rows, nq, kv, out_hi, out_lo, d_status);
+  if (kv.hd == HD_ && group == G_)   \
+    return launch_k(attn_prefill_kernel<HD_, G_>, grid, dim3(PF_THREADS), PfLayout<HD_>::SMEM, st, true, tmKV, q, rows, nq, kv, out_hi, out_lo, d_status);
   CORUN_PF_CASE(128, 1) CORUN_PF_CASE(128, 2) CORUN_PF_CASE(128, 4) CORUN_PF_CASE(128, 8)
   CORUN_PF_CASE(64, 1) CORUN_PF_CASE(64, 2) CORUN_PF_CASE(64, 4) CORUN_PF_CASE(64, 8)
 #undef CORUN_PF_CASE

@@ -1178,6 +1178,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   // zero-filled: masked positions of a page are multiplied by zero weights, so they must be finite
   if ((rc = dmalloc(A, &e->kv_pool, e->layer_stride * s.n_layers, true))) return fail(rc);
   if (mla) {
+    if (mla_attention_prepare() != cudaSuccess) return fail(CORUN_ECUDA);
     // one layer's pages: rows of rank + rope halfs, 16 per page
     e->tm_c.resize(s.n_layers);
     e->tm_cv.resize(s.n_layers);

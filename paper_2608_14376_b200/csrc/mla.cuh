@@ -61,6 +61,7 @@ long long mla_part_ml_floats(int R, int nh, int max_context);
 long long mla_part_o_floats(int R, int nh, int rank, int max_context);
 int mla_max_splits(int max_context);
 
+cudaError_t mla_attention_prepare();   // opts the kernel into its shared-memory size on the current device (idempotent)
 // Absorbed attention of every row over its cached tokens.  q_lat element (r, h, d) sits at
 // q_lat[r * q_row_stride + h * q_head_stride + d]; q_rope is [R][nh][rope].  A row's cached-token count is
 // ctx[r] (rows == nullptr; its block-table row is r) or rows->active[r] ? rows->pos[r] + 1 : 0 (its block-table

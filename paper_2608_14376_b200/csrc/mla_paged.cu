@@ -620,17 +620,13 @@ int mla_encode_maps(CUtensorMap *tmC, CUtensorMap *tmV, const void *pool, long l
   return tma_encode_fp16_4d(tmV, pool, dims, strides, box);
 }
 
+cudaError_t mla_attention_prepare() { return cudaFuncSetAttribute(mla_paged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MP_SMEM); }
+
 cudaError_t launch_mla_attention(const CUtensorMap &tmC, const CUtensorMap &tmV, const float *q_lat, long long q_row_stride,
                                  long long q_head_stride, const float *q_rope, const int *block_table, int max_blocks,
                                  const int *ctx, const Rows *rows, int R, const MlaDims &d, float scale, int max_splits,
                                  float2 *part_ml, float *part_o, float *o_lat, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo,
                                  int rows_per_head, int num_sms, int *d_status, bool pdl, cudaStream_t st, int page_run) {
-  static bool prepared = false;                     // idempotent; a race only repeats it
-  if (!prepared) {
-    cudaError_t e = cudaFuncSetAttribute(mla_paged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MP_SMEM);
-    if (e != cudaSuccess) return e;
-    prepared = true;
-  }
   const int *row_slot = rows ? rows->slot : nullptr, *row_pos = rows ? rows->pos : nullptr, *row_active = rows ? rows->active : nullptr;
   cudaError_t ce = launch_k(mla_paged_kernel, dim3(num_sms), dim3(MP_THREADS), MP_SMEM, st, pdl, tmC, tmV, q_lat, q_row_stride,
                             q_head_stride, q_rope, block_table, max_blocks, ctx, row_slot, row_pos, row_active, R, d.nh, d.rank, d.rope,
@@ -674,7 +670,8 @@ int corun_mla_attend(const float *q_lat, const float *q_rope, const void *pool, 
   float2 *part_ml = reinterpret_cast<float2 *>(ws + 64);
   float *part_o = ws + 64 + mla_part_ml_floats(B, n_heads, max_blocks * MP_PAGE);
   const MlaDims dims{n_heads, d_latent, 0, d_rope, 0};
-  ce = cudaMemsetAsync(status, 0, sizeof(int), st);
+  ce = mla_attention_prepare();
+  if (ce == cudaSuccess) ce = cudaMemsetAsync(status, 0, sizeof(int), st);
   if (ce == cudaSuccess)
     ce = launch_mla_attention(tm, tv, q_lat, (long long)n_heads * d_latent, d_latent, q_rope, block_table, max_blocks, ctx, nullptr, B, dims,
                               scale, max_splits, part_ml, part_o, o_lat, nullptr, nullptr, 0, sms, status, false, st, 1);

@@ -86,7 +86,10 @@ cudaError_t launch_attn_worklist(const Rows &rows, int n_kv, int *work, int *n_w
 // tmKV: the pages with one box per (page, head) tile (the decode kernel's view).
 cudaError_t launch_attention_prefill(const CUtensorMap &tmKV, const float *q, const Rows &rows, int nq, const KvLayout &kv,
                                      __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int *d_status, cudaStream_t st);
-cudaError_t attention_prepare();   // opts the kernels into their shared-memory size (idempotent)
+// Opt the kernels into their shared-memory size on the current device (idempotent; an engine's creation calls the first, which
+// calls the second).
+cudaError_t attention_prepare();
+cudaError_t attention_prefill_prepare();
 // y = silu(gate) * up from the gate-up GEMM result -> bf16 hi/lo [R, F].
 cudaError_t launch_swiglu(const GemmOut &gu, int R, int F, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, cudaStream_t st);
 // x fp32 [R, K] -> bf16 hi/lo.

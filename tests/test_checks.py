@@ -1,7 +1,12 @@
 """The index checks a -DCORUN_CHECKED build applies inside its kernels (csrc/checks.cuh), exercised on the host
 through the C ABI: good indices pass, every kind of bad index is caught.  No GPU is involved: a bad index is
 never handed to a kernel."""
+import os
+import re
+
 import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_14376_b200", "csrc")
 
 
 @pytest.fixture(scope="module")
@@ -50,3 +55,11 @@ def test_unknown_kind(chk):
     from paper_2608_14376_b200 import corun
 
     assert chk(9, 0) == corun.EINVAL
+
+
+def test_no_flag_of_the_process_stands_for_a_device():
+    """A kernel's shared-memory size is opted into per device: a flag that remembers it for the process leaves it out on a
+    second GPU (where the launch is then refused)."""
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh")):
+            assert not re.search(r"^\s+static bool\b", open(os.path.join(CSRC, f)).read(), re.M), f
