@@ -61,7 +61,7 @@ extern "C" {
 typedef struct corun_moe corun_moe;
 
 typedef struct {
-  int32_t hidden;      /* H, multiple of 64 */
+  int32_t hidden;      /* H, multiple of 64, at most 12288 */
   int32_t n_experts;   /* E routed experts, 1..256 */
   int32_t top_k;       /* 1..min(E, 16) */
   int32_t expert_ffn;  /* F, multiple of 64; 2F a multiple of 4 */

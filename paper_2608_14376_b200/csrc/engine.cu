@@ -1164,7 +1164,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     }
   }
   if (moe) {
-    if (H > 12288) return fail(CORUN_EINVAL);       // the router kernel keeps a row in shared memory
+    if (H > MOE_MAX_HIDDEN) return fail(CORUN_EINVAL);   // the router kernel keeps a row in shared memory
+    if (moe_router_prepare() != cudaSuccess) return fail(CORUN_ECUDA);
     for (int l = 0; l < s.n_layers; ++l) {
       if (l >= first_dense && ((uintptr_t)moe->router[l] & 15u)) return fail(CORUN_EINVAL);
       e->router.push_back(l >= first_dense ? (const bf16 *)moe->router[l] : nullptr);

@@ -596,6 +596,10 @@ cudaError_t launch_moe_combine(const float *yg, const int *active, int R, int n_
   return launch_k(moe_combine_kernel, dim3((H / 4 + 255) / 256, R), dim3(256), 0, st, true, yg, active, n_blocks, H, g, y);
 }
 
+cudaError_t moe_router_prepare() {
+  return cudaFuncSetAttribute(moe_router_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOE_MAX_HIDDEN * (int)sizeof(float));
+}
+
 cudaError_t launch_moe_router(const bf16 *x_hi, const bf16 *x_lo, int H, const bf16 *Wr, int R, int E, int S, int top_k,
                               int renormalize, float *w, int *experts, float *probs, const RouterScratch &rs, cudaStream_t st, const int *active,
                               int *sel) {
@@ -664,7 +668,7 @@ int corun_moe_create(const corun_moe_shape *shape, const void *router, const voi
                      int32_t B, void *cuda_stream, corun_moe **out) {
   if (!shape || !router || !gate_up || !down || !out || B < 1 || B > 256) return CORUN_EINVAL;
   const corun_moe_shape &s = *shape;
-  if (s.hidden < 64 || s.hidden % 64 || s.n_experts < 1 || s.n_experts > MOE_MAX_EXPERTS || s.top_k < 1 ||
+  if (s.hidden < 64 || s.hidden % 64 || s.hidden > MOE_MAX_HIDDEN || s.n_experts < 1 || s.n_experts > MOE_MAX_EXPERTS || s.top_k < 1 ||
       s.top_k > MOE_MAX_TOPK || s.top_k > s.n_experts || s.expert_ffn < 64 || s.expert_ffn % 64 || s.n_shared < 0)
     return CORUN_EINVAL;
   corun_moe *m = new (std::nothrow) corun_moe();
@@ -676,7 +680,7 @@ int corun_moe_create(const corun_moe_shape *shape, const void *router, const voi
   m->st = (cudaStream_t)cuda_stream;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || moe_router_prepare() != cudaSuccess)
     return fail(CORUN_ECUDA);
   const int H = s.hidden, E = s.n_experts, F = s.expert_ffn, NB = E + s.n_shared;
   const size_t N1 = (size_t)NB * 2 * F, K2 = (size_t)NB * F;

@@ -11,7 +11,9 @@ namespace corun {
 // cores, softmax over all E experts, top_k by repeated arg-max with ties to the lower id, optional
 // renormalisation; writes the row of SwiGLU weights w[r, 0 .. E + S) (p_e for the selected experts, 0 for the
 // others, 1 for the shared ones) and, when not null, the routing.  Several CTAs per row meet in `rs`; H * 4 bytes of shared
-// memory (H <= 12288).
+// memory (H <= MOE_MAX_HIDDEN, which is all there is without moe_router_prepare and not quite enough).
+constexpr int MOE_MAX_HIDDEN = 12288;
+cudaError_t moe_router_prepare();   // opts the kernel into its shared-memory size on the current device (idempotent)
 struct RouterScratch {
   float *logit;   // [R, E]
   int *count;     // [R], zero between launches

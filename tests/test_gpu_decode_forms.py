@@ -12,7 +12,7 @@ pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not have_gpu(), reason="needs 
 TOL = 3e-2          # as the other engine tests: logits of the tiny decoder against the oracle
 
 
-@pytest.mark.parametrize("H,E,K,B", [(2176, 13, 3, 1), (128, 8, 8, 96), (256, 13, 3, 97), (2176, 40, 4, 101), (256, 256, 16, 128)])
+@pytest.mark.parametrize("H,E,K,B", [(2176, 13, 3, 1), (12288, 9, 2, 3), (128, 8, 8, 96), (256, 13, 3, 97), (2176, 40, 4, 101), (256, 256, 16, 128)])
 def test_router_shares(H, E, K, B):
     """Logits from several CTAs per row (remainders of experts, of rows and of the row's length), twice, since the CTAs
     of a launch leave their meeting point as they found it."""
