@@ -54,7 +54,8 @@ int corun_debug_time_kernel(corun_engine *e, int32_t kind, int32_t reps, float *
  * the last decode step: which = 0 rotated queries [B, nq*hd]; 1 attention split partials
  * [B][nq][max_splits][hd]; 2 their (max, sum) pairs [B][nq][max_splits][2] (base-2 domain);
  * 3 the residual stream [B, hidden]; 4 / 5 the attention output's bf16 hi / lo halves [BN, nq*hd] as raw
- * memory (two bf16 per float); 6 the O-projection's direct output [B, hidden]; 7 the GEMM partial workspace. */
+ * memory (two bf16 per float); 6 the O-projection's direct output [B, hidden]; 7 the GEMMs' partial workspace (the
+ * projections' partial matrices where those run on pairs of SMs).  EINVAL for a buffer the engine does not have. */
 int corun_debug_read(corun_engine *e, int32_t which, float *out, int64_t n);
 /* eager != 0: launch the decode kernels one by one instead of replaying the graph. */
 int corun_debug_set_eager(corun_engine *e, int32_t eager);
@@ -117,7 +118,8 @@ int corun_debug_microbench(int32_t kind, int32_t variant, const float *x, int32_
 /* Runs GEMM `kind` (0 QKV, 1 O, 2 gate-up, 3 down, 4 LM head) of the decode program on one layer's
  * weights three times and returns the last launch's per-CTA timeline: stamps[cta*8 + i] (host, room for
  * 8 * 256 values) are globaltimer nanoseconds at: 0 kernel entry, 1 set-up done, 2 first TMA issued,
- * 3 last TMA issued, 4 first stage landed, 5 last MMA issued, 6 last accumulator complete, 7 epilogue done. */
+ * 3 last TMA issued, 4 first stage landed, 5 last MMA issued, 6 last accumulator complete, 7 epilogue done (GEMMs on
+ * pairs of SMs: 4 and 5 in the pair's first CTA only).  EINVAL for the experts in their grouped form. */
 int corun_debug_gemm_trace(corun_engine *e, int32_t kind, int32_t layer, uint64_t *stamps, int32_t *n_ctas);
 /* With CORUN_TRACE_STEP=1 in the environment at corun_init, every layer GEMM of the decode program records
  * its per-CTA timeline (the 8 stamps of corun_debug_gemm_trace) on every step; this copies the last step's

@@ -113,6 +113,7 @@ struct Program {
   std::vector<GemmPlan> s_qkv, s_o, s_gu, s_down;
   GemmPairPlan b_qkv, b_o, b_gu, b_down, b_router;
   float *router_out = nullptr, *pair_part = nullptr;
+  size_t pair_part_floats = 0;           // (decode) room of pair_part
   // Latent attention of long prompts over decompressed keys and values (attention_prefill_mla.cu): the gathered latents of
   // the chunk's requests, up to kv_cap tokens, their keys and values, and the chunk's segments
   bool mla_tiles = false;
@@ -367,6 +368,7 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
                        gemm_pair_part_floats(V, H, 256, e->num_sms, true)})
         part = x > part ? x : part;
       RC(dmalloc(A, &P.pair_part, part, false));
+      P.pair_part_floats = part;
       if (!P.plain_tiles) RC(dmalloc(A, &P.plain_tiles, (size_t)((QKVN > V ? QKVN : V) / GEMM_TILE_N + 1)));
       RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, 256, P.qkv_out, P.pair_part, e->num_sms, true));
       RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, 256, P.o_out, P.pair_part, e->num_sms, true));
@@ -768,7 +770,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       }
       continue;
     }
-    if (P.wide) STAGE(gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st));
+    if (P.wide) STAGE(gemm_pair_launch(P.b_qkv, e->tb_qkv[l], P.R, e->d_status, e->st, nullptr, nullptr, tr(4 * l + 0)));
     else STAGE(gemm_launch(P.p_qkv, &e->tm_qkv[l], e->d_status, e->st, tr(4 * l + 0), true));
     const GemmOut qkv = P.wide ? gemm_pair_out(P.b_qkv, P.R, P.plain_tiles) : P.p_qkv.out();
     if (e->mla) {
@@ -791,7 +793,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
                            e->num_sms, P.part_acc, P.part_ml, P.att_pool + l, P.ao_hi, P.ao_lo, &P == &e->dec ? (e->whole_pairs ? 2 : 0) : 1,
                            e->d_status, e->st));
     }
-    if (P.wide) STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
+    if (P.wide) STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st, nullptr, nullptr, tr(4 * l + 1)));
     else STAGE(gemm_launch(P.p_o, &e->tm_o[l], e->d_status, e->st, tr(4 * l + 1), true));
     GemmOut o = P.wide ? gemm_pair_out(P.b_o, P.R, P.plain_tiles) : P.p_o.out();
     STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
@@ -825,8 +827,8 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       // expert for all rows -> the row's experts summed in ascending expert id
       STAGE(launch_moe_router(P.xn_hi, P.xn_lo, s.hidden, e->router[l], P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, nullptr,
                               nullptr, P.router_rs, e->st, P.row_active, P.moe_sel));
-      STAGE(gemm_launch(P.p_gug, &e->tm_gu_half[l], e->d_status, e->st, nullptr, true));
-      STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
+      STAGE(gemm_launch(P.p_gug, &e->tm_gu_half[l], e->d_status, e->st, tr(4 * l + 2), true));
+      STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, tr(4 * l + 3), true));
       STAGE(launch_moe_combine_select(P.yg_out, P.moe_sel, e->moe_K + e->moe_S, P.BN, P.R, s.hidden, P.down_out, e->st));
       n += 10 + (&P == &e->dec ? 1 : 0);
       continue;
@@ -843,8 +845,8 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         n += 1;
       }
     } else if (P.wide) {
-      STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st, &e->tb_gu96[l]));
-      STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st));
+      STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st, &e->tb_gu96[l], nullptr, tr(4 * l + 2)));
+      STAGE(gemm_pair_launch(P.b_down, e->tb_down[l], P.R, e->d_status, e->st, nullptr, nullptr, tr(4 * l + 3)));
       n += 9;
       continue;
     } else {
@@ -1898,21 +1900,31 @@ int corun_debug_gemm_trace(corun_engine *e, int32_t kind, int32_t layer, uint64_
   if (!e || !stamps || !n_ctas || kind < 0 || kind > 4 || layer < 0 || layer >= e->sh.n_layers) return CORUN_EINVAL;
   RC(sync_stream(e));
   Program &P = e->dec;
-  const GemmPlan *pl[5] = {&P.p_qkv, &P.p_o, &P.p_gu, &P.p_down, &P.p_lm};
-  const CUtensorMap *tm[5] = {&e->tm_qkv[layer], &e->tm_o[layer], P.p_gu.sw_hi ? &e->tm_gu_half[layer] : &e->tm_gu[layer],
-                              &e->tm_down[layer], nullptr};
+  const bool ffn = kind == 2 || kind == 3, experts = e->moe_E && !dense_layer(e, layer);
+  const bool pairs = P.wide && !(ffn && e->moe_E), selected = ffn && experts && P.select;
+  const GemmPairPlan *pp[5] = {&P.b_qkv, &P.b_o, &P.b_gu, &P.b_down, &P.b_lm};
+  const GemmPlan *pl[5] = {&P.p_qkv, &P.p_o, selected ? &P.p_gug : &P.p_gu, selected ? &P.p_dng : &P.p_down, &P.p_lm};
   const GemmPlan &p = *pl[kind];
-  if (!p.grid) return CORUN_EINVAL;                 // expert layers in their grouped or selected form
+  // expert layers in their grouped form, and dense ones beside expert layers: no such GEMM
+  if (pairs ? false : !p.grid || (ffn && dense_layer(e, layer))) return CORUN_EINVAL;
+  const size_t n = (size_t)(pairs ? gemm_pair_ctas(*pp[kind], P.R, kind == 2) : p.grid) * 8;
   unsigned long long *d = nullptr;
-  if (cudaMalloc(&d, (size_t)p.grid * 8 * sizeof(unsigned long long)) != cudaSuccess) return CORUN_ENOMEM;
-  cudaError_t ce = cudaMemsetAsync(d, 0, (size_t)p.grid * 8 * sizeof(unsigned long long), e->st);
-  for (int i = 0; i < 3 && ce == cudaSuccess; ++i) ce = gemm_launch(p, tm[kind], e->d_status, e->st, d);   // last one counts
-  if (ce == cudaSuccess)
-    ce = cudaMemcpyAsync(stamps, d, (size_t)p.grid * 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, e->st);
+  if (cudaMalloc(&d, n * sizeof(unsigned long long)) != cudaSuccess) return CORUN_ENOMEM;
+  cudaError_t ce = cudaMemsetAsync(d, 0, n * sizeof(unsigned long long), e->st);
+  for (int i = 0; i < 3 && ce == cudaSuccess; ++i) {   // last one counts
+    if (pairs) {
+      const CUtensorMap *tb[5] = {&e->tb_qkv[layer], &e->tb_o[layer], &e->tb_gu[layer], &e->tb_down[layer], &e->tb_lm};
+      ce = gemm_pair_launch(*pp[kind], *tb[kind], P.R, e->d_status, e->st, kind == 2 ? &e->tb_gu96[layer] : nullptr, nullptr, d);
+    } else {
+      const CUtensorMap *tm[5] = {&e->tm_qkv[layer], &e->tm_o[layer], p.sw_hi ? &e->tm_gu_half[layer] : &e->tm_gu[layer], &e->tm_down[layer], nullptr};
+      ce = gemm_launch(p, tm[kind], e->d_status, e->st, d);
+    }
+  }
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(stamps, d, n * sizeof(unsigned long long), cudaMemcpyDeviceToHost, e->st);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(e->st);
   cudaFree(d);
   if (ce != cudaSuccess) { g_last_cuda_error = (int)ce; return CORUN_ECUDA; }
-  *n_ctas = p.grid;
+  *n_ctas = (int32_t)(n / 8);
   return CORUN_OK;
 }
 
@@ -1970,10 +1982,10 @@ int corun_debug_read(corun_engine *e, int32_t which, float *out, int64_t n) {
     case 4: src = (const float *)P.ao_hi; have = (size_t)P.BN * QD / 2; break;
     case 5: src = (const float *)P.ao_lo; have = (size_t)P.BN * QD / 2; break;
     case 6: src = P.o_out; have = (size_t)P.R * s.hidden; break;
-    case 7: src = P.ws; have = gemm_ws_floats(e->num_sms, P.BN); break;
+    case 7: src = P.ws ? P.ws : P.pair_part; have = P.ws ? gemm_ws_floats(e->num_sms, P.BN) : P.pair_part_floats; break;
     default: return CORUN_EINVAL;
   }
-  if ((size_t)n > have) return CORUN_EINVAL;
+  if (!src || (size_t)n > have) return CORUN_EINVAL;
   CK(cudaMemcpyAsync(out, src, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, e->st));
   CK(cudaStreamSynchronize(e->st));
   return CORUN_OK;

@@ -233,6 +233,7 @@ size_t gemm_pair_part_floats(int N, int K, int cap, int num_sms, bool decode = f
 int gemm_pair_plan_create(GemmPairPlan *p, int N, int K, const void *Xhi, const void *Xlo, int cap, float *out, float *part, int num_sms,
                           bool decode = false);
 GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles);
+int gemm_pair_ctas(const GemmPairPlan &p, int R, bool narrow);   // CTAs of a launch (narrow: with a map of 96 rows)
 int gemm_pair_has_parts(const GemmPairPlan &p, int R);   // 1 if some of the result of R rows is left in partial matrices
 cudaError_t gemm_pair_fixup_launch(const GemmPairPlan &p, int R, cudaStream_t st);   // makes `out` a plain matrix
 // W is [2F, K] (F gate rows, then F up rows; F % 8 == 0): out_hi / out_lo [cap, F] = silu(gate) * up as a bf16 hi/lo pair.
@@ -246,7 +247,8 @@ int gemm_pair_prepare();             // opts the kernels into their shared-memor
 // Rows 0 .. R-1 (R <= cap).  tmW: the weight matrix with a box of 128 rows (gemm_encode_map(.., 128)); tmW96 (swiglu): the
 // same with 96 rows, taken where it shortens the waves.
 cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st,
-                             const CUtensorMap *tmW96 = nullptr, const float *kv_scale = nullptr);
+                             const CUtensorMap *tmW96 = nullptr, const float *kv_scale = nullptr,
+                             unsigned long long *trace = nullptr);   // (debug) timeline, as gemm_launch's; 2 * pairs CTAs at most
 // Tensor map for TMA stores of tiles of 32 rows x 32 columns into a [rows, cols] row-major matrix (fp32: 128-byte swizzle; bf16: 64).
 int tma_encode_store_2d(CUtensorMap *m, const void *base, int is_fp32, unsigned long long rows, int cols);
 // direct[r, n] = gemm_load(r, n) for every tile that has partials (makes `direct` a plain matrix).

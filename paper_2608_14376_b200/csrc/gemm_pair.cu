@@ -67,7 +67,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                  const __grid_constant__ CUtensorMap tmLo, const __grid_constant__ CUtensorMap tmOut,
                  const __grid_constant__ CUtensorMap tmOut2, int R, int N, int KB, int row_tiles, int whole, int units, int slices,
-                 int per_unit, int half, int *status, const int *row_blocks, int cap, const float *kv_scale) {
+                 int per_unit, int half, int *status, const int *row_blocks, int cap, const float *kv_scale, unsigned long long *trace) {
+  // optional per-CTA timeline (debug): 8 globaltimer stamps, as the other GEMM's
+#define TRACE(i) do { if (trace) trace[(size_t)blockIdx.x * 8 + (i)] = globaltimer_ns(); } while (0)
+  if (threadIdx.x == 0) TRACE(0);
   constexpr bool SWIGLU = MODE == PG_SWIGLU, KV = MODE == PG_KV;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[PG_STAGES];      // used in the first CTA: both CTAs' loads of a stage
@@ -115,6 +118,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   cluster_sync_all();                               // the other CTA's barriers exist before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  if (threadIdx.x == 0) TRACE(1);
   volatile int *abort_p = &abort_flag;
   int fail = 0;
 
@@ -147,6 +151,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           }
           const uint32_t fb = smem_u32(&full_bar[s]), dst = base + (uint32_t)s * PG_STAGE_BYTES;
           if (rank == 0) mbar_arrive_expect_tx(fb, stage_tx);
+          if (it == 0) TRACE(2);
           const uint32_t fb0 = cluster_map(fb, 0);
           tma_load_2d_pair(dst + 2 * PG_X_BYTES, &tmW, kb * GEMM_BLOCK_K, yw, fb0, pol_w);
           if (stacked) {
@@ -163,6 +168,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           }
         }
       }
+      TRACE(3);
       // every stage's last release has arrived before this CTA may end: an arrival of the pair's MMAs must not find the
       // shared memory given to another CTA
       for (int i = 0; i < PG_STAGES && !fail; ++i) {
@@ -190,6 +196,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           for (int kb = kb0; kb < kb1; ++kb, ++it) {
             const int s = it % PG_STAGES;
             if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(it / PG_STAGES) & 1u, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
+            if (it == 0) TRACE(4);
             tc_fence_after();
             const uint32_t st = base + (uint32_t)s * PG_STAGE_BYTES;
             const uint64_t hi = umma_desc_sw128(st), lo = umma_desc_sw128(st + PG_X_BYTES), w = umma_desc_sw128(st + 2 * PG_X_BYTES);
@@ -204,6 +211,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           if (!fail) umma_commit_pair(smem_u32(&tmem_full_bar[acc]));
         }
       }
+      TRACE(5);
     }
   } else {
     // ---------------- epilogue: TMEM -> registers -> swizzled staging tile -> TMA store ----------------
@@ -247,6 +255,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       uint32_t sum[128];                            // this thread's row: 128 columns (SWIGLU: up to 64 gate and 64 up columns), fp32
       for (int sl = un.s0; sl < un.s1; ++sl, ++seg) {
         wait_full();
+        if (threadIdx.x == 64) TRACE(6);            // (the last one stays)
         if (!ok) { fail = DEV_TIMEOUT_EPILOGUE; break; }
         const uint32_t ta = accumulator();
         if (row0 < R) {                             // warp-uniform
@@ -395,6 +404,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       }
     }
     if (lane == 0) bulk_wait<0>();                  // the stores have been performed before the kernel ends
+    if (threadIdx.x == 64) TRACE(7);
   }
 
   if (fail) {
@@ -409,6 +419,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   cluster_sync_all();                               // neither CTA leaves while the other's MMAs or arrivals may still reach it
   tc_fence_after();
   if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
+#undef TRACE
 }
 
 // The tiles that were left as partial matrices, added up in place (for consumers that read a plain matrix).
@@ -515,6 +526,11 @@ GemmOut gemm_pair_out(const GemmPairPlan &p, int R, const int *zero_tiles) {
   return g;
 }
 
+int gemm_pair_ctas(const GemmPairPlan &p, int R, bool narrow) {
+  const PairShape q = pair_shape(p, R, narrow);
+  return 2 * (q.units < p.pairs ? q.units : p.pairs);
+}
+
 int gemm_pair_has_parts(const GemmPairPlan &p, int R) {
   const PairShape q = pair_shape(p, R, false);
   return q.whole < q.row_tiles * p.n_tiles ? 1 : 0;
@@ -566,13 +582,13 @@ int gemm_pair_prepare() {
 }
 
 cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st, const CUtensorMap *tmW96,
-                             const float *kv_scale) {
+                             const float *kv_scale, unsigned long long *trace) {
   if (R < 1 || R > p.cap || (p.decode && (p.cap != 256 || !p.row_blocks)) || (p.kv_heads && !kv_scale)) return cudaErrorInvalidValue;
   const PairShape q = pair_shape(p, R, tmW96 != nullptr);
   const int pairs = q.units < p.pairs ? q.units : p.pairs;
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(2 * pairs), dim3(PG_THREADS), PG_SMEM, st, false, q.half == 96 ? *tmW96 : tmW, p.tmHi, p.tmLo, p.tmOut, p.tmOut2,
-                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, p.per_unit, q.half, d_status, p.row_blocks, p.cap, kv_scale);
+                    R, p.N, p.K / GEMM_BLOCK_K, q.row_tiles, q.whole, q.units, p.slices, p.per_unit, q.half, d_status, p.row_blocks, p.cap, kv_scale, trace);
   };
   if (p.decode) return p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU, true>) : go(gemm_pair_kernel<PG_PLAIN, true>);
   return p.kv_heads ? go(gemm_pair_kernel<PG_KV, false>) : p.swiglu ? go(gemm_pair_kernel<PG_SWIGLU, false>) : go(gemm_pair_kernel<PG_PLAIN, false>);
