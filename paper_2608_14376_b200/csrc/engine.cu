@@ -231,6 +231,7 @@ int dmalloc(std::vector<void *> &keep, T **p, size_t n, bool zero = true) {
   if (n == 0) n = 1;
   cudaError_t e = cudaMalloc(&q, n * sizeof(T));
   if (e != cudaSuccess) {
+    cudaGetLastError();                             // (handled here: not the error of the next launch)
     g_last_cuda_error = (int)e;
     return CORUN_ENOMEM;
   }
@@ -251,6 +252,7 @@ int dmalloc(DevMem &m, T **p, size_t n, bool zero = true) {
     cudaError_t e = cudaMalloc(&q, want);
     if (e != cudaSuccess && want > bytes) { cudaGetLastError(); e = cudaMalloc(&q, want = bytes); }   // no room for a whole block
     if (e != cudaSuccess) {
+      cudaGetLastError();
       g_last_cuda_error = (int)e;
       return CORUN_ENOMEM;
     }
@@ -1068,18 +1070,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     e->moe_renorm = moe->renormalize ? 1 : 0;
   }
   e->pool_blocks = kv_pool_blocks ? kv_pool_blocks * e->kv_run : (int64_t)B * e->max_blocks;   // in pages of 16 tokens
-  if (!kv_pool_blocks) {
-    // default size: a full reservation for every slot, or as many pages as fit beside 6 GiB that are
-    // left for the programs' buffers, whichever is less (admission then refuses what does not fit)
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return fail(CORUN_ECUDA);
-    const size_t page_b = mla ? (size_t)s.n_layers * KV_BLOCK * (size_t)mla_token_halfs(mla->kv_lora_rank + mla->qk_rope, e->kv_run) * sizeof(__half)
-                              : (size_t)s.n_layers * 2 * s.n_kv_heads * KV_BLOCK * s.head_dim * sizeof(__half);
-    const size_t keep = (size_t)6 << 30;
-    const int64_t fit = free_b > keep ? (int64_t)((free_b - keep) / page_b) : 0;
-    if (fit < e->pool_blocks) e->pool_blocks = fit / e->kv_run * e->kv_run;
-    if (e->pool_blocks < e->kv_run) return fail(CORUN_ENOMEM);
-  }
+  size_t free_before = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_before, &total_b) != cudaSuccess) return fail(CORUN_ECUDA);
   e->chunk = 256;
   bool one_chunk_size = false;                      // the environment asks for chunks of its own size, for every prompt
   if (const char *c = getenv("CORUN_ATTN_WHOLE_PAIRS")) e->whole_pairs = atoi(c) != 0;   // ablation only
@@ -1097,7 +1089,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
                                 !getenv("CORUN_MOE_PREFILL_DENSE")));
   // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG
   const long long big_rows = (long long)B * ((max_context + 127) / 128 * 128);
-  const int big_cap = !big_ok ? 0 : big_rows < PREFILL_BIG ? (int)((big_rows + 255) / 256 * 256) : PREFILL_BIG;
+  int big_cap = !big_ok ? 0 : big_rows < PREFILL_BIG ? (int)((big_rows + 255) / 256 * 256) : PREFILL_BIG;
   const bool wide = e->wide = pad16(B) >= (moe ? 129 : WIDE_ROWS) && s.vocab % 8 == 0;   // (Program::wide)
   if (wide && gemm_encode_map(&e->tb_lm, w->lm_head, s.vocab, H, 128)) return fail(CORUN_EINVAL);
   e->tm_qkv.resize(s.n_layers);
@@ -1176,35 +1168,41 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
 
   auto &A = e->allocs;
   int rc;
-  e->layer_stride = mla ? (size_t)e->pool_blocks * KV_BLOCK * (size_t)mla_token_halfs(e->md.rank + e->md.rope, e->kv_run)
-                        : (size_t)e->pool_blocks * 2 * s.n_kv_heads * KV_BLOCK * s.head_dim;
-  // zero-filled: masked positions of a page are multiplied by zero weights, so they must be finite
-  if ((rc = dmalloc(A, &e->kv_pool, e->layer_stride * s.n_layers, true))) return fail(rc);
-  if (mla) {
-    if (mla_attention_prepare() != cudaSuccess) return fail(CORUN_ECUDA);
-    // one layer's pages: rows of rank + rope halfs, 16 per page
-    e->tm_c.resize(s.n_layers);
-    e->tm_cv.resize(s.n_layers);
-    for (int l = 0; l < s.n_layers; ++l)
-      if ((rc = mla_encode_maps(&e->tm_c[l], &e->tm_cv[l], e->kv_pool + (size_t)l * e->layer_stride, e->pool_blocks, e->md.rank, e->md.rope,
-                                e->kv_run)))
-        return fail(rc);
-  } else {
-    // one layer's pages seen as rows of hd halfs (16 rows per page and head, keys first, then values)
-    const unsigned long long halfs = (unsigned long long)e->layer_stride;
-    if (halfs / KV_BLOCK >= (1ull << 31)) return fail(CORUN_EINVAL);
-    for (int l = 0; l < s.n_layers; ++l) {
-      const __half *base = e->kv_pool + (size_t)l * e->layer_stride;
-      // keys and values are cached alike, one view serves both: a tile's 16 tokens x head_dim in ONE box, [2 groups of 8 tokens][halves of 64 dims][8][64]
-      const unsigned long long row_b = (unsigned long long)s.head_dim * 2;
-      const unsigned long long d4[4] = {64, 8, (unsigned long long)(s.head_dim / 64), halfs / s.head_dim / 8};
-      const unsigned long long s4[3] = {row_b, 128, 8 * row_b};
-      const unsigned b4[4] = {64, 8, (unsigned)(s.head_dim / 64), 2};
-      e->tm_k4.emplace_back();
-      if ((rc = tma_encode_fp16_4d(&e->tm_k4[l], base, d4, s4, b4))) return fail(rc);
+  // the pool, and the maps of its layers
+  auto make_pool = [&]() -> int {
+    int rc;
+    e->layer_stride = mla ? (size_t)e->pool_blocks * KV_BLOCK * (size_t)mla_token_halfs(e->md.rank + e->md.rope, e->kv_run)
+                          : (size_t)e->pool_blocks * 2 * s.n_kv_heads * KV_BLOCK * s.head_dim;
+    // zero-filled: masked positions of a page are multiplied by zero weights, so they must be finite
+    if ((rc = dmalloc(A, &e->kv_pool, e->layer_stride * s.n_layers, true))) return rc;
+    if (mla) {
+      if (mla_attention_prepare() != cudaSuccess) return (int)CORUN_ECUDA;
+      // one layer's pages: rows of rank + rope halfs, 16 per page
+      e->tm_c.resize(s.n_layers);
+      e->tm_cv.resize(s.n_layers);
+      for (int l = 0; l < s.n_layers; ++l)
+        if ((rc = mla_encode_maps(&e->tm_c[l], &e->tm_cv[l], e->kv_pool + (size_t)l * e->layer_stride, e->pool_blocks, e->md.rank, e->md.rope,
+                                  e->kv_run)))
+          return rc;
+    } else {
+      // one layer's pages seen as rows of hd halfs (16 rows per page and head, keys first, then values)
+      const unsigned long long halfs = (unsigned long long)e->layer_stride;
+      if (halfs / KV_BLOCK >= (1ull << 31)) return (int)CORUN_EINVAL;
+      for (int l = 0; l < s.n_layers; ++l) {
+        const __half *base = e->kv_pool + (size_t)l * e->layer_stride;
+        // keys and values are cached alike, one view serves both: a tile's 16 tokens x head_dim in ONE box, [2 groups of 8 tokens][halves of 64 dims][8][64]
+        const unsigned long long row_b = (unsigned long long)s.head_dim * 2;
+        const unsigned long long d4[4] = {64, 8, (unsigned long long)(s.head_dim / 64), halfs / s.head_dim / 8};
+        const unsigned long long s4[3] = {row_b, 128, 8 * row_b};
+        const unsigned b4[4] = {64, 8, (unsigned)(s.head_dim / 64), 2};
+        e->tm_k4.emplace_back();
+        if ((rc = tma_encode_fp16_4d(&e->tm_k4[l], base, d4, s4, b4))) return rc;
+      }
+      if (attention_prepare() != cudaSuccess) return (int)CORUN_ECUDA;
     }
-    if (attention_prepare() != cudaSuccess) return fail(CORUN_ECUDA);
-  }
+    return CORUN_OK;
+  };
+  if (kv_pool_blocks && (rc = make_pool())) return fail(rc);
   if ((rc = dmalloc(A, &e->d_block_table, (size_t)B * e->max_blocks))) return fail(rc);
   if ((rc = dmalloc(A, &e->d_in_use, B)) || (rc = dmalloc(A, &e->d_ctx, B)) || (rc = dmalloc(A, &e->d_step, B)) ||
       (rc = dmalloc(A, &e->d_pending, B)) || (rc = dmalloc(A, &e->d_temp, B)) || (rc = dmalloc(A, &e->d_top_p, B)) ||
@@ -1232,9 +1230,6 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     const std::vector<int> ones(FINISH_ROWS, 1);
     if (cudaMemcpy(e->d_pf_one, ones.data(), FINISH_ROWS * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return fail(CORUN_ECUDA);
   }
-  const int64_t n_runs = e->pool_blocks / e->kv_run;
-  e->free_blocks.resize((size_t)n_runs);
-  for (int64_t i = 0; i < n_runs; ++i) e->free_blocks[(size_t)i] = (int)(n_runs - 1 - i);
   e->slot_blocks.resize(B);
   e->in_use.assign(B, 0);
   e->ctx.assign(B, 0);
@@ -1280,12 +1275,45 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   for (GemmPairPlan *pl : {&e->dec.b_qkv, &e->dec.b_o, &e->dec.b_gu, &e->dec.b_down, &e->dec.b_lm}) pl->row_blocks = e->dec.row_blocks;
   for (GemmPlan *pl : {&e->dec.p_qkv, &e->dec.p_o, &e->dec.p_gu, &e->dec.p_down, &e->dec.p_lm, &e->dec.p_gu_d, &e->dec.p_down_d})
     pl->row_blocks = e->dec.row_blocks;
+  if ((rc = program_create(e, e->lm1, FINISH_ROWS, false, true))) return fail(rc);
+  // Prefill: chunks of as many rows as there is room for (a caller's pool may leave little: 128 MiB stay free for the step's
+  // graph); no value depends on that.  Where not even 256 rows fit, latent attention does without decompressed keys and values,
+  // and at last the chunk program serves: other forms, with other low bits.
+  while (big_cap) {
+    size_t free_b = 0;
+    rc = program_create_big(e, e->big, big_cap);
+    if (rc == CORUN_OK && big_cap > 256 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b < (size_t)128 << 20) rc = CORUN_ENOMEM;
+    if (rc != CORUN_ENOMEM) break;
+    program_destroy(e->big);
+    e->big = Program();
+    if (big_cap > 256) big_cap = (big_cap / 2 + 255) / 256 * 256;
+    else if (e->big_mla_tiles) e->big_mla_tiles = false;
+    else big_cap = 0;
+  }
+  if (big_cap && rc) return fail(rc);
   if (!big_cap && (rc = program_create(e, e->pre, e->chunk, true, false, e->moe_E > 0 && !getenv("CORUN_MOE_PREFILL_DENSE")))) return fail(rc);
   // a prefill chunk is filled from row 0: the host says which blocks of rows it reaches (prefill_run)
   for (GemmPlan *pl : {&e->pre.p_qkv, &e->pre.p_o, &e->pre.p_gu, &e->pre.p_down, &e->pre.p_gu_d, &e->pre.p_down_d})
     pl->row_blocks = e->pre.row_blocks;
-  if (big_cap && (rc = program_create_big(e, e->big, big_cap))) return fail(rc);
-  if ((rc = program_create(e, e->lm1, FINISH_ROWS, false, true))) return fail(rc);
+  if (!kv_pool_blocks) {
+    // default size: a full reservation for every slot, or as many pages as fit beside 6 GiB for the engine's other buffers --
+    // what is left of them, and 256 MiB, where these are larger --, whichever is less (admission then refuses what does not fit)
+    size_t free_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return fail(CORUN_ECUDA);
+    const size_t page_b = mla ? (size_t)s.n_layers * KV_BLOCK * (size_t)mla_token_halfs(mla->kv_lora_rank + mla->qk_rope, e->kv_run) * sizeof(__half)
+                              : (size_t)s.n_layers * 2 * s.n_kv_heads * KV_BLOCK * s.head_dim * sizeof(__half);
+    const size_t have = (size_t)6 << 30, used = free_before > free_b ? free_before - free_b : 0, least = (size_t)256 << 20;
+    const size_t keep = used + least < have ? have - used : least;
+    const int64_t fit = free_b > keep ? (int64_t)((free_b - keep) / page_b) : 0;
+    if (fit < e->pool_blocks) e->pool_blocks = fit / e->kv_run * e->kv_run;
+    if (e->pool_blocks < e->kv_run) return fail(CORUN_ENOMEM);
+    if ((rc = make_pool())) return fail(rc);
+  }
+  {
+    const int64_t n_runs = e->pool_blocks / e->kv_run;
+    e->free_blocks.resize((size_t)n_runs);
+    for (int64_t i = 0; i < n_runs; ++i) e->free_blocks[(size_t)i] = (int)(n_runs - 1 - i);
+  }
 
   // the allocations above were cleared and filled through the legacy stream, which the engine's
   // stream does not wait for: drain the device once before the first launch
@@ -1669,14 +1697,20 @@ int corun_engine_info(corun_engine *e, int32_t *B, int32_t *max_context, int32_t
   return CORUN_OK;
 }
 
-int corun_prefill_geometry(corun_engine *e, int32_t *chunk_rows, int32_t *tile_rows) {
-  if (!e) return CORUN_EINVAL;
+int corun_prefill_class(corun_engine *e, int32_t n_tokens, int32_t *prefill_class, int32_t *chunk_rows, int32_t *tile_rows) {
+  if (!e || n_tokens < 1) return CORUN_EINVAL;
+  const int cls = e->big.pair && n_tokens > PREFILL_SMALL ? 1 : 0;   // (as prefill_many divides them)
   int unit = 128 / (e->sh.n_q_heads / e->sh.n_kv_heads);
-  if (e->mla) unit = 16;
+  if (e->mla) unit = cls && e->big.mla_tiles ? 128 : 16;
   if (unit > e->chunk || e->chunk % unit) unit = e->chunk;
+  if (prefill_class) *prefill_class = cls;
   if (chunk_rows) *chunk_rows = e->chunk;
   if (tile_rows) *tile_rows = unit;
   return CORUN_OK;
+}
+
+int corun_prefill_geometry(corun_engine *e, int32_t *chunk_rows, int32_t *tile_rows) {
+  return corun_prefill_class(e, 1, nullptr, chunk_rows, tile_rows);
 }
 
 // MLA engines: k holds the cached rows ([n][rank + rope]), v is not used (may be NULL).
