@@ -79,10 +79,14 @@ void corun_sched_destroy(corun_sched *s);
  * ones taken before it, and (c) fits into the padding of the chunks the requests taken so far occupy
  * anyway: a request's rows start on a multiple of tile_rows, and the number of chunks of chunk_rows rows
  * must not grow.  It stops at the first request that fails one of the three (no request overtakes
- * another), so the head is never delayed by more than the others' LM heads, and short prompts ride in
- * chunks that would have been padding.  The tokens of every request are those of isolated prefill.
- * fn NULL: the engine's corun_prefill_batch and geometry (scheduler made by _create_for_engine; chunk_rows
- * and tile_rows are then ignored); else chunk_rows >= tile_rows >= 1, chunk_rows % tile_rows == 0.
+ * another).  Where a chunk is launched as a whole, the head is then never delayed by more than the others'
+ * LM heads, and short prompts ride in what would have been padding.  The tokens of every request are those of
+ * isolated prefill.
+ * fn NULL: the engine's corun_prefill_batch and the geometry of the head's class (corun_prefill_class), and (d) a
+ * request of another class stops the batch: it would be a second pass over the weights, behind which the head would
+ * wait.  An engine launches the rows there are: what rides along costs the head up to the difference to the chunk's
+ * end, for prompts of up to 128 tokens at most one more block of 128 rows.  (Scheduler made by _create_for_engine;
+ * chunk_rows and tile_rows are then ignored); else chunk_rows >= tile_rows >= 1, chunk_rows % tile_rows == 0.
  * corun_sched_step reports the number of requests prefilled in *n_active and the first one's id.
  */
 int corun_sched_enable_batched_prefill(corun_sched *s, corun_sched_prefill_batch_fn fn, int32_t chunk_rows,

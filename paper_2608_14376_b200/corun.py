@@ -24,7 +24,7 @@ EXPORTS = [
     "corun_debug_sample", "corun_debug_wait_probe", "corun_debug_microbench", "corun_debug_check_index", "corun_gemm_static", "corun_strerror", "corun_last_cuda_error", "corun_engine_info",
     "corun_sched_create", "corun_sched_create_for_engine", "corun_sched_destroy", "corun_sched_submit",
     "corun_sched_step", "corun_sched_poll", "corun_sched_slot_of", "corun_sched_counts",
-    "corun_sched_enable_batched_prefill", "corun_prefill_geometry",
+    "corun_sched_enable_batched_prefill", "corun_prefill_geometry", "corun_prefill_class",
     "corun_moe_create", "corun_moe_destroy", "corun_moe_forward", "corun_moe_sync", "corun_moe_weight_bytes",
     "corun_moe_launches", "corun_mla_attend", "corun_mla_workspace_floats", "corun_mla_sync",
 ]
@@ -141,6 +141,7 @@ def lib():
         L.corun_debug_time_kernel.argtypes = [vp, i32, i32, C.POINTER(C.c_float)]
         L.corun_decode_launches.argtypes = [vp]
         L.corun_debug_gemm.argtypes = [vp, i32, i32, vp, i32, vp, vp]
+        L.corun_prefill_class.argtypes = [vp, i32, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32)]
         L.corun_debug_gemm_pair.argtypes = [i32, vp, i32, i32, vp, i32, vp, vp]
         L.corun_debug_prefill_attention.argtypes = [vp, i32, i32, i32, i32, vp, vp]
         L.corun_debug_variate.argtypes = [u64, u64, C.POINTER(C.c_uint32)]
@@ -322,6 +323,12 @@ class Engine:
 
     def force_token(self, slot: int, token: int):
         _check(lib().corun_force_token(self._h, slot, int(token)), "corun_force_token")
+
+    def prefill_class(self, n_tokens: int):
+        """(class, rows to count as a chunk, tile rows) of prompts of that length (``corun_prefill_class``)."""
+        c, ch, t = C.c_int32(-1), C.c_int32(-1), C.c_int32(-1)
+        _check(lib().corun_prefill_class(self._h, n_tokens, C.byref(c), C.byref(ch), C.byref(t)), "corun_prefill_class")
+        return c.value, ch.value, t.value
 
     def context_len(self, slot: int) -> int:
         rc = lib().corun_context_len(self._h, slot)

@@ -38,6 +38,7 @@ struct corun_sched {
   corun_sched_prefill_batch_fn prefill_batch = nullptr;
   int32_t chunk_rows = 0, tile_rows = 0;
   bool for_engine = false;
+  bool classes = false;                  // batched prefill: the engine says which requests share a pass, and their geometry
 };
 
 namespace {
@@ -122,6 +123,7 @@ extern "C" int corun_sched_create_for_engine(corun_engine *e, corun_sched **out)
 extern "C" int corun_sched_enable_batched_prefill(corun_sched *s, corun_sched_prefill_batch_fn fn, int32_t chunk_rows,
                                                   int32_t tile_rows) {
   if (!s) return CORUN_EINVAL;
+  const bool classes = !fn;
   if (!fn) {
     if (!s->for_engine) return CORUN_EINVAL;
     const int rc = corun_prefill_geometry((corun_engine *)s->ctx, &chunk_rows, &tile_rows);
@@ -130,6 +132,7 @@ extern "C" int corun_sched_enable_batched_prefill(corun_sched *s, corun_sched_pr
   }
   if (tile_rows < 1 || chunk_rows < tile_rows || chunk_rows % tile_rows) return CORUN_EINVAL;
   s->prefill_batch = fn;
+  s->classes = classes;
   s->chunk_rows = chunk_rows;
   s->tile_rows = tile_rows;
   return CORUN_OK;
@@ -166,18 +169,26 @@ extern "C" int corun_sched_step(corun_sched *s, int32_t *action, int64_t *reques
     int status = CORUN_OK;
     if (can_fit_full_sequence(s, r, &status)) {
       if (s->prefill_batch) {
-        // ---- extension: the requests behind the head that fit into the padding of the head's chunks
+        // ---- extension: the requests behind the head that fit into the padding of the head's chunks and are of its class
+        int32_t chunk_rows = s->chunk_rows, tile_rows = s->tile_rows, cls = 0;
+        if (s->classes) {
+          const int rc = corun_prefill_class((corun_engine *)s->ctx, (int32_t)r.prompt.size(), &cls, &chunk_rows, &tile_rows);
+          if (rc != CORUN_OK) return rc;
+        }
         const int64_t free_pages = s->ops.free_blocks(s->ctx);
         if (free_pages < 0) return (int)free_pages;
         auto pages_of = [&](const Request &q) { return ((int64_t)q.prompt.size() + q.max_new + s->kv_block - 1) / s->kv_block; };
-        auto chunks_of = [&](int64_t rows) { return (rows + s->chunk_rows - 1) / s->chunk_rows; };
+        auto chunks_of = [&](int64_t rows) { return (rows + chunk_rows - 1) / chunk_rows; };
         std::vector<int64_t> ids{id};
         int64_t rows = (int64_t)r.prompt.size(), pages = pages_of(r);
         for (size_t w = 1; w < s->waiting.size(); ++w) {
           const Request &q = s->reqs[(size_t)s->waiting[w]];
           if ((int32_t)(s->running.size() + ids.size()) >= s->B) break;
           if (pages + pages_of(q) > free_pages) break;
-          const int64_t start = (rows + s->tile_rows - 1) / s->tile_rows * s->tile_rows;
+          int32_t its = 0;
+          if (s->classes && corun_prefill_class((corun_engine *)s->ctx, (int32_t)q.prompt.size(), &its, nullptr, nullptr) != CORUN_OK) break;
+          if (its != cls) break;
+          const int64_t start = (rows + tile_rows - 1) / tile_rows * tile_rows;
           if (chunks_of(start + (int64_t)q.prompt.size()) != chunks_of(rows)) break;
           ids.push_back(s->waiting[w]);
           rows = start + (int64_t)q.prompt.size();

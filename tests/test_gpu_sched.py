@@ -149,3 +149,33 @@ def test_batched_prefill_policy_serves_the_same_tokens_and_follows_its_oracle(ti
         assert i == len(log)
     finally:
         eng.close()
+
+
+def test_batched_prefill_takes_requests_of_the_heads_class_only(tiny):
+    """Prompts above 128 tokens run in another program than shorter ones: a short request behind a long head is not in the
+    padding of the head's chunk, it would be a second pass over the weights."""
+    from paper_2608_14376_b200 import corun
+    from tests.test_gpu_prefill_kernels import _latent
+
+    eng = corun.Engine(tiny.sh, tiny.w_t, B, 512)
+    try:
+        assert eng.prefill_class(1) == eng.prefill_class(128) == (0, 256, 64)
+        assert eng.prefill_class(129) == (1, 256, 64)
+        for lens, batches in (([150, 30, 30], [1, 2]), ([30, 150, 30], [1, 1, 1]), ([20, 40, 60], [3])):
+            sch = corun.Scheduler(engine=eng)
+            sch.enable_batched_prefill()
+            prompts = synth.make_prompts(tiny.sh.vocab, lens, seed=8)
+            for p in prompts:
+                sch.submit(p, 2, 0.0, 1.0, 5)
+            got = [sch.step() for _ in batches]
+            assert [(a, n) for a, _, n in got] == [(corun.SCHED_PREFILL, n) for n in batches]
+            while sch.step()[0] != 0:
+                pass
+            sch.close()
+    finally:
+        eng.close()
+    _, _, eng = _latent(T=512)                        # long prompts with latent attention: tiles of 128 rows, short ones of 16
+    try:
+        assert eng.prefill_class(30) == (0, 256, 16) and eng.prefill_class(300) == (1, 256, 128)
+    finally:
+        eng.close()
