@@ -9,7 +9,7 @@ from tests.helpers import have_gpu
 from tests.test_gpu_moe import GAP, _device_op, _weights
 
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not have_gpu(), reason="needs a GPU")]
-TOL = 3e-2          # as the other engine tests: logits of the tiny decoder against the oracle
+TOL = 3e-3          # logits of the tiny decoder (standard deviation 0.3) against the oracle; measured 5.6e-4 at most
 
 
 @pytest.mark.parametrize("H,E,K,B", [(2176, 13, 3, 1), (12288, 9, 2, 3), (128, 8, 8, 96), (256, 13, 3, 97), (2176, 40, 4, 101), (256, 256, 16, 128)])
@@ -106,7 +106,7 @@ def test_vanished_routing_weights_add_nothing(orc, E, K, S, renorm):
                     out.append(eng.logits(1))
                     # router logits, and what rounding moves them by, are 60 times those of the other tests (whose logits are
                     # off by some 3e-4): up to 60 * 3e-4; measured 9e-3, and 0.6 with what another layer left added
-                    assert np.abs(out[-1] - r.logits).max() <= TOL
+                    assert np.abs(out[-1] - r.logits).max() <= 10 * TOL
                 eng.release(1)
             runs.append([o.tobytes() for o in out])
         finally:

@@ -7,7 +7,9 @@ from paper_2608_14376_b200 import synth
 from tests.helpers import Tiny, have_gpu
 
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not have_gpu(), reason="needs a GPU")]
-TOL = 3e-2
+# against the fp64 oracle the largest of a row's logits (standard deviation 0.3 to 0.7) was off by at most 8.1e-4 in any of these
+# tests, most of it cached rows that round to the other fp16 neighbour
+TOL = 3e-3
 
 
 @pytest.fixture(scope="module")
@@ -146,3 +148,31 @@ def test_slices_of_the_projections_give_the_same_bytes_in_any_chunk(orc, lens):
     assert list(e.prefill_batch(slots, prompts, res, 0.7, 0.95, seeds)) == first
     assert after() == alone
     e.close()
+
+
+@pytest.mark.parametrize("nope,vh,max_context", [(64, 192, 512), (128, 128, 16400)])
+def test_long_latent_prompts_in_the_decode_form(orc, nope, vh, max_context):
+    """Widths other than 128, and contexts above 16384: the attention of a long prompt runs row by row, in pieces of 256
+    rows that share the buffers of their partial results."""
+    from paper_2608_14376_b200 import corun
+
+    sh = synth.ModelShape(2, 256, 4, 4, 128, 384, 1024, 1e-6, 10000.0)
+    w, m = synth.make_mla_weights_numpy(sh, dict(kv_lora_rank=256, qk_nope=nope, qk_rope=32, v_head=vh, first_dense=2), seed=9)
+    model = orc.Model(orc.Shape(**sh.dict()), w, mla=m)
+    wt, mt = synth.mla_numpy_to_torch(w, m, "cuda")
+    prompts = synth.make_prompts(sh.vocab, [290, 150], seed=10)
+    e = corun.Engine(sh, wt, 2, max_context, kv_pool_blocks=16, mla=mt, kv_block=64)
+    try:
+        alone = []
+        for s, p in enumerate(prompts):
+            e.prefill(s, p, len(p) + 2)
+            r = orc.Request(model, p, 1, max_T=len(p) + 2)
+            r.prefill()
+            assert np.abs(e.logits(s) - r.logits).max() <= TOL
+            alone.append(e.logits(s).tobytes())
+        for s in range(2):
+            e.release(s)
+        e.prefill_batch([0, 1], prompts, [len(p) + 2 for p in prompts])
+        assert [e.logits(s).tobytes() for s in range(2)] == alone
+    finally:
+        e.close()
