@@ -44,6 +44,7 @@ struct DevMem {
   std::vector<void *> blocks;
   char *cur = nullptr;
   size_t left = 0, next = (size_t)32 << 20;
+  bool tight = false;                                // there was no room for a whole block
   void release() {
     for (void *p : blocks) cudaFree(p);
     blocks.clear();
@@ -250,7 +251,7 @@ int dmalloc(DevMem &m, T **p, size_t n, bool zero = true) {
     else if (m.next < ((size_t)256 << 20)) m.next *= 2;
     void *q = nullptr;
     cudaError_t e = cudaMalloc(&q, want);
-    if (e != cudaSuccess && want > bytes) { cudaGetLastError(); e = cudaMalloc(&q, want = bytes); }   // no room for a whole block
+    if (e != cudaSuccess && want > bytes) { cudaGetLastError(); m.tight = true; e = cudaMalloc(&q, want = bytes); }
     if (e != cudaSuccess) {
       cudaGetLastError();
       g_last_cuda_error = (int)e;
@@ -1071,7 +1072,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   }
   e->pool_blocks = kv_pool_blocks ? kv_pool_blocks * e->kv_run : (int64_t)B * e->max_blocks;   // in pages of 16 tokens
   size_t free_before = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_before, &total_b) != cudaSuccess) return fail(CORUN_ECUDA);
+  if (!kv_pool_blocks && cudaMemGetInfo(&free_before, &total_b) != cudaSuccess) return fail(CORUN_ECUDA);
   e->chunk = 256;
   bool one_chunk_size = false;                      // the environment asks for chunks of its own size, for every prompt
   if (const char *c = getenv("CORUN_ATTN_WHOLE_PAIRS")) e->whole_pairs = atoi(c) != 0;   // ablation only
@@ -1267,7 +1268,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
 #endif
   // expert layers of the decode program: above 64 padded rows the grouped form (an expert's rows gathered into blocks of
   // 64: one MMA per k-slice covers the hi and lo halves of a block, where every row through every expert costs two on
-  // 128 rows and keeps the tensor pipe as busy as the weight stream); up to 64 rows every row through every expert
+  // 128 rows and keeps the tensor pipe as busy as the weight stream); up to 64 rows the experts that a row
+  // selected (Program::select), each for all rows of the step
   const bool dec_grouped = e->moe_E > 0 && pad16(B) > 64 && !getenv("CORUN_MOE_DECODE_DENSE");
   if ((rc = program_create(e, e->dec, B, true, true, dec_grouped, true))) return fail(rc);
   // the decode step's first kernel says which blocks of rows hold a request (64 rows each up to 128 padded rows, 128
@@ -1282,7 +1284,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   while (big_cap) {
     size_t free_b = 0;
     rc = program_create_big(e, e->big, big_cap);
-    if (rc == CORUN_OK && big_cap > 256 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b < (size_t)128 << 20) rc = CORUN_ENOMEM;
+    if (rc == CORUN_OK && big_cap > 256 && e->big.allocs.tight && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b < (size_t)128 << 20) rc = CORUN_ENOMEM;
     if (rc != CORUN_ENOMEM) break;
     program_destroy(e->big);
     e->big = Program();
