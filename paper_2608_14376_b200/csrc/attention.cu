@@ -421,7 +421,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
       if (stop_s[gi]) break;                         // the same decision in all 4 warps of the group
 
       // ---- 2. S^T = K * Q^T, issued by one thread once the item has landed
-      if (gtid == 0) {
+      if (gtid < 32 && elect_one()) {
         const bool ok = mbar_wait(smem_u32(&kfull_bar[slot]), (full_bits >> j) & 1u, &abort_flag);
         ATRACE(k, 1);
         if (ok) {
@@ -493,7 +493,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
       asm volatile("bar.sync %0, 128;" ::"r"(1 + gi) : "memory");
 
       // ---- 4. O^T = V^T * P^T, one MMA per loaded page (16 tokens)
-      if (gtid == 0) {
+      if (gtid < 32 && elect_one()) {
         ATRACE(k, 5);
         const bool ok = mbar_wait(smem_u32(&vfull_bar[slot]), (full_bits >> j) & 1u, &abort_flag);
         ATRACE(k, 6);

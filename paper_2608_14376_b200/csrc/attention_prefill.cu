@@ -166,7 +166,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: the scores of block j, then the values of block j - 1
-    if (lane == 0) {
+    if (elect_one()) {
       // fp16 x fp16 -> fp32; N at bit 17 (>> 3), M = 128 at bit 24 (>> 4); the values are an MN-major B operand
       const uint32_t idesc_s = (1u << 4) | ((uint32_t)(PF_KEYS >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t idesc_o = (1u << 4) | (1u << 16) | ((uint32_t)(HD >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);

@@ -218,7 +218,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
   const bool real = tl < n_rows;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- TMA producer ----------------
       const uint64_t pol = l2_policy_evict_last();  // the tiles of the same head read the same keys and values
       for (int j = 0; j < n_blocks && !failed; ++j) {
@@ -236,7 +236,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- MMA issuer ----------------
       const uint32_t idesc_s = (1u << 4) | ((uint32_t)(ML_KEYS >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t idesc_o = (1u << 4) | (1u << 16) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);   // values MN-major

@@ -214,7 +214,7 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   int fail = 0;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- TMA producer ----------------
       const uint64_t pol_w = l2_policy_evict_first();   // weights are streamed once per step
       const uint64_t pol_x = l2_policy_evict_last();    // activations are re-read by every CTA
@@ -290,7 +290,7 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       TRACE(3);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- MMA issuer ----------------
       read_blocks();
       int it = 0, seg = 0;

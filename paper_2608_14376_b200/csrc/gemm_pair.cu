@@ -132,7 +132,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   auto cut = [&](int sl) { return sl * KB / slices; };       // first k-block of a slice
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- TMA producer (both CTAs; the bytes count on the first CTA's barrier) ----------------
       const uint64_t pol_w = l2_policy_evict_first();        // a weight tile is used by the row tiles that run now
       const uint64_t pol_x = l2_policy_evict_last();
@@ -178,7 +178,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       // ---------------- MMA issuer (first CTA) ----------------
       // kind::f16: D fp32, A and B bf16, both K-major, N = 2 * half, M = 256 over the pair
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * half >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);

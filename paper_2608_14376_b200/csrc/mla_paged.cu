@@ -7,7 +7,7 @@
 //
 // An item is (row, split of 256 cached tokens = 16 pages); the items of a call are listed row by row and every
 // CTA (one per SM) takes one contiguous stretch of the list.  What bounds this op on the tensor cores is the
-// NUMBER of MMA instructions (each takes ~150 cycles whatever its shape), so the products are arranged to need
+// NUMBER of MMA instructions (an M = 64 or 128 MMA takes 39 cycles at least), so the products are arranged to need
 // few: the 16 heads (as fp16 hi + lo rows, 32 rows of a 64-row operand) are the M side, the tokens and the
 // latent dims the wide N side:
 //   scores   S[32 x 256 tokens] = Q[32 x 576] * [C | R]^T    4 MMAs (K = 16 each) per block of 64 dims: 36
@@ -260,7 +260,7 @@ mla_paged_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant_
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       // D fp32, A and B fp16 (format 0), M = 64; scores: N = 256, both K-major; output: N = NH, B MN-major
       const uint32_t idesc_s = (1u << 4) | ((uint32_t)(MP_T >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
       const uint32_t idesc_o = (1u << 4) | (1u << 16) | ((uint32_t)(NH >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
