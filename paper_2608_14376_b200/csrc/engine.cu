@@ -1104,8 +1104,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     e->mlp_norm.push_back((const bf16 *)w->mlp_norm[l]);
     int rc;
     const int qkv_rows = mla ? s.n_q_heads * (mla->qk_nope + mla->qk_rope) + mla->kv_lora_rank + mla->qk_rope : QD + 2 * KD;
-    if ((rc = gemm_encode_map(&e->tm_qkv[l], w->wqkv[l], qkv_rows, H, GEMM_TILE_N))) return fail(rc);
-    if ((rc = gemm_encode_map(&e->tm_o[l], w->wo[l], H, QD, GEMM_TILE_N))) return fail(rc);
+    if ((rc = gemm_encode_map(&e->tm_qkv[l], w->wqkv[l], qkv_rows, H, GEMM_W_BOX))) return fail(rc);
+    if ((rc = gemm_encode_map(&e->tm_o[l], w->wo[l], H, QD, GEMM_W_BOX))) return fail(rc);
     if (big_cap || wide) {                          // the programs of many rows
       if (e->tb_qkv.empty())
         for (auto *v : {&e->tb_qkv, &e->tb_o, &e->tb_gu, &e->tb_down, &e->tb_router, &e->tb_gu_half, &e->tb_gu96}) v->resize(s.n_layers);
@@ -1121,12 +1121,12 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
     }
     if (moe && l < first_dense) {                   // a dense feed-forward layer of a decoder with expert layers
       if (e->tm_gu_d.empty()) { e->tm_gu_d.resize(s.n_layers); e->tm_down_d.resize(s.n_layers); }
-      if ((rc = gemm_encode_map(&e->tm_gu_d[l], w->wgate_up[l], 2 * dense_ffn, H, GEMM_TILE_N))) return fail(rc);
-      if ((rc = gemm_encode_map(&e->tm_down_d[l], w->wdown[l], H, dense_ffn, GEMM_TILE_N))) return fail(rc);
+      if ((rc = gemm_encode_map(&e->tm_gu_d[l], w->wgate_up[l], 2 * dense_ffn, H, GEMM_W_BOX))) return fail(rc);
+      if ((rc = gemm_encode_map(&e->tm_down_d[l], w->wdown[l], H, dense_ffn, GEMM_W_BOX))) return fail(rc);
       continue;
     }
-    if ((rc = gemm_encode_map(&e->tm_gu[l], moe ? moe->gate_up[l] : w->wgate_up[l], 2 * F, H, GEMM_TILE_N))) return fail(rc);
-    if ((rc = gemm_encode_map(&e->tm_down[l], moe ? moe->down[l] : w->wdown[l], H, F, GEMM_TILE_N))) return fail(rc);
+    if ((rc = gemm_encode_map(&e->tm_gu[l], moe ? moe->gate_up[l] : w->wgate_up[l], 2 * F, H, GEMM_W_BOX))) return fail(rc);
+    if ((rc = gemm_encode_map(&e->tm_down[l], moe ? moe->down[l] : w->wdown[l], H, F, GEMM_W_BOX))) return fail(rc);
     if (!moe && (rc = gemm_encode_map(&e->tm_gu_half[l], w->wgate_up[l], 2 * F, H, gemm_swiglu_half(F, e->num_sms)))) return fail(rc);
     if (moe && moe_half && (rc = gemm_encode_map(&e->tm_gu_half[l], moe->gate_up[l], 2 * F, H, moe_half))) return fail(rc);
   }
@@ -1149,8 +1149,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
       e->kv_norm.push_back((const bf16 *)mla->kv_norm[l]);
       bf16 *dst = e->w_ukT + (size_t)l * per_layer;
       if (launch_mla_transpose_uk((const bf16 *)mla->wkv_b[l], md, dst, 0) != cudaSuccess) return fail(CORUN_ECUDA);
-      if ((rc = gemm_encode_map(&e->tm_uk[l], dst, md.nh * md.rank, md.nope, GEMM_TILE_N))) return fail(rc);
-      if ((rc = gemm_encode_map(&e->tm_uv[l], mla->wkv_b[l], md.nh * (md.nope + md.vh), md.rank, GEMM_TILE_N))) return fail(rc);
+      if ((rc = gemm_encode_map(&e->tm_uk[l], dst, md.nh * md.rank, md.nope, GEMM_W_BOX))) return fail(rc);
+      if ((rc = gemm_encode_map(&e->tm_uv[l], mla->wkv_b[l], md.nh * (md.nope + md.vh), md.rank, GEMM_W_BOX))) return fail(rc);
       if (e->big_mla_tiles) {
         if ((rc = gemm_encode_map(&e->tb_uv[l], mla->wkv_b[l], md.nh * 256, md.rank, 128))) return fail(rc);
         if (launch_mla_kv_scale((const bf16 *)mla->wkv_b[l], e->kv_norm[l], md, e->kv_scale + (size_t)l * md.nh, 0) != cudaSuccess)
@@ -1277,6 +1277,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   for (GemmPairPlan *pl : {&e->dec.b_qkv, &e->dec.b_o, &e->dec.b_gu, &e->dec.b_down, &e->dec.b_lm}) pl->row_blocks = e->dec.row_blocks;
   for (GemmPlan *pl : {&e->dec.p_qkv, &e->dec.p_o, &e->dec.p_gu, &e->dec.p_down, &e->dec.p_lm, &e->dec.p_gu_d, &e->dec.p_down_d})
     pl->row_blocks = e->dec.row_blocks;
+  if (e->dec.select) e->dec.p_gug.row_blocks = e->dec.p_dng.row_blocks = e->dec.row_blocks;
   if ((rc = program_create(e, e->lm1, FINISH_ROWS, false, true))) return fail(rc);
   // Prefill: chunks of as many rows as there is room for (a caller's pool may leave little: 128 MiB stay free for the step's
   // graph); no value depends on that.  Where not even 256 rows fit, latent attention does without decompressed keys and values,
@@ -1502,7 +1503,7 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
       }
       if (P.shorts) {                               // which blocks of 64 rows exist
         const int nb = (fill + SHORT_ROWS - 1) / SHORT_ROWS;
-        for (int b = 0; b < nb; ++b) blocks[b] = 1 | (fill > b * SHORT_ROWS + 64 ? 2 : 0);
+        for (int b = 0; b < nb; ++b) blocks[b] = gemm_row_blocks(fill - b * SHORT_ROWS < SHORT_ROWS ? fill - b * SHORT_ROWS : SHORT_ROWS, 64);
         CK(cudaMemcpyAsync(P.row_blocks, blocks, nb * sizeof(int), cudaMemcpyHostToDevice, e->st));
       }
     } else {
@@ -1513,7 +1514,7 @@ int prefill_run(corun_engine *e, Program &P, PfReq *const *reqs, int n_req) {
       // the chunk's rows are filled from row 0: the GEMMs leave out the blocks of rows behind the last one in use
       // (blocks of 64 rows up to 128 padded rows, of 128 rows above)
       const int blk = P.BN <= 128 ? 64 : 128;
-      blocks[0] = (fill > 0 ? 1 : 0) | (fill > blk ? 2 : 0);
+      blocks[0] = gemm_row_blocks(fill, blk);
       CK(cudaMemcpyAsync(P.row_blocks, blocks, sizeof(int), cudaMemcpyHostToDevice, e->st));
     }
     RC(run_layers(e, P, nullptr));

@@ -24,7 +24,11 @@ constexpr int GEMM_TILE_N = 256;   // weight rows per tile (the MMA's N)
 constexpr int GEMM_ROW_BLOCK = 128; // activation rows per MMA (the MMA's M)
 constexpr int GEMM_BLOCK_K = 64;   // bf16 elements per k-block (= one 128-byte swizzle row)
 constexpr int GEMM_MAX_SELECT = 288;  // experts of a selected-experts GEMM
-constexpr int GEMM_THREADS = 192;  // warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue
+constexpr int GEMM_W_BOX = 128;    // weight rows per TMA box
+constexpr int GEMM_MAX_ROWS = 128; // padded rows up to which gemm_rows.cu has the kernel
+constexpr int GEMM_NARROW_ROWS = 32;  // padded rows up to which a tile is 128 weight rows
+constexpr int GEMM_ROWS_MAX_SMEM = 224 * 1024;
+constexpr int GEMM_THREADS = 192;  // (above GEMM_MAX_ROWS) warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue
 
 // What a consumer kernel needs to read a GEMM result.
 struct GemmOut {
@@ -36,6 +40,7 @@ struct GemmOut {
   // Result of gemm_pair.cu (row_tiles > 0): tiles [256 rows x 256 columns], row tiles fastest; the first `whole` are in
   // `direct`, the others in `ws`, tile after tile as `slices` partial tiles [256][256].
   int row_tiles, whole, slices;
+  int tile_shift = 8;    // log2 of the tile's columns: partials are [(cta*2 + slot), BN, 1 << tile_shift]
 };
 
 // Values of a gemm_pair.cu result, the slices added in ascending order.
@@ -67,13 +72,13 @@ __device__ __forceinline__ float4 gemm_load_pair4(const GemmOut &g, int r, int n
 
 // Value (r, n) of a GEMM result, partials added in ascending CTA order.
 __device__ __forceinline__ float gemm_load(const GemmOut &g, int r, int n) {
-  const int t = n / GEMM_TILE_N, col = n % GEMM_TILE_N;
+  const int t = n >> g.tile_shift, col = n - (t << g.tile_shift);
   const int f = g.tile_first[t], c0 = f >> 1, c1 = g.tile_cend[t];
   if (c0 == c1) return g.direct[(size_t)r * g.N + n];
-  const float *p = g.ws + ((size_t)r) * GEMM_TILE_N + col;
-  const size_t cta_stride = (size_t)2 * g.BN * GEMM_TILE_N;
+  const float *p = g.ws + ((size_t)r << g.tile_shift) + col;
+  const size_t cta_stride = (size_t)2 * g.BN << g.tile_shift;
   float acc = 0.f;
-  acc += p[(size_t)f * g.BN * GEMM_TILE_N];
+  acc += p[(size_t)f * g.BN << g.tile_shift];
   for (int c = c0 + 1; c <= c1; ++c) acc += p[(size_t)c * cta_stride];
   return acc;
 }
@@ -82,12 +87,12 @@ __device__ __forceinline__ float gemm_load(const GemmOut &g, int r, int n) {
 // Loads are issued four partials at a time; an absent partial contributes +0.0f.
 __device__ __forceinline__ float4 gemm_load4(const GemmOut &g, int r, int n) {
   if (g.row_tiles) return gemm_load_pair4(g, r, n);
-  const int t = n / GEMM_TILE_N, col = n % GEMM_TILE_N;
+  const int t = n >> g.tile_shift, col = n - (t << g.tile_shift);
   const int f = g.tile_first[t], c0 = f >> 1, c1 = g.tile_cend[t];
   if (c0 == c1) return *reinterpret_cast<const float4 *>(g.direct + (size_t)r * g.N + n);
-  const float *p = g.ws + ((size_t)r) * GEMM_TILE_N + col;
-  const size_t cta_stride = (size_t)2 * g.BN * GEMM_TILE_N;
-  float4 acc = *reinterpret_cast<const float4 *>(p + (size_t)f * g.BN * GEMM_TILE_N);
+  const float *p = g.ws + ((size_t)r << g.tile_shift) + col;
+  const size_t cta_stride = (size_t)2 * g.BN << g.tile_shift;
+  float4 acc = *reinterpret_cast<const float4 *>(p + ((size_t)f * g.BN << g.tile_shift));
   acc.x += 0.f; acc.y += 0.f; acc.z += 0.f; acc.w += 0.f;   // same rounding path as 0 + first partial
   for (int c = c0 + 1; c <= c1; c += 4) {
     float4 v[4];
@@ -103,12 +108,19 @@ __device__ __forceinline__ float4 gemm_load4(const GemmOut &g, int r, int n) {
   return acc;
 }
 
+// Tensor maps of the split activations: boxes of 64, 32 and 16 rows (above GEMM_MAX_ROWS: of 128 rows, the first of each).
+struct GemmXMaps {
+  CUtensorMap hi[3], lo[3];
+};
+
 // Static launch description of one GEMM shape (built once at init).
 struct GemmPlan {
-  CUtensorMap tmW, tmHi, tmLo;
+  CUtensorMap tmW;
+  GemmXMaps tmX;
   int N = 0, K = 0, R = 0, BN = 0;   // weight rows, reduction length, real rows, padded rows
-  int n_tiles = 0, KB = 0, grid = 0, stages = 0, tmem_cols = 0;
-  uint32_t idesc = 0;
+  int tile_n = GEMM_TILE_N;          // weight rows per tile (without SwiGLU)
+  int n_tiles = 0, KB = 0, grid = 0, stages = 0;
+  uint32_t idesc = 0, stage_bytes = 0;
   size_t smem_bytes = 0;
   float *direct = nullptr;           // not owned
   float *ws = nullptr;               // not owned
@@ -128,12 +140,19 @@ struct GemmPlan {
   // Gate / up GEMM with SwiGLU in the epilogue (gemm_plan_create_swiglu): the bf16 hi/lo output [BN, N / 2].
   __nv_bfloat16 *sw_hi = nullptr, *sw_lo = nullptr;
   int sw_half = 0;                   // gate rows (= up rows) per tile
-  // Above 64 padded rows the rows form two blocks (65..128 rows: stacked blocks of 64 rows; above: row blocks of 128
-  // rows).  Device int, not owned, written by an earlier kernel of the step: bit b set = block b holds a request
-  // this step; null = both blocks.  An absent block is neither loaded nor multiplied nor stored.
+  // Device int, not owned, written by an earlier kernel of the step (null: all rows): how many rows hold a request this step
+  // (they are the first ones) at bits 8 .., and bit b set = block b of 128 rows (up to 128 padded rows: of 64) holds one.  Rows
+  // behind the padded count, or blocks without a request, are neither loaded nor multiplied nor stored.
   const int *row_blocks = nullptr;
-  GemmOut out() const { return GemmOut{direct, ws, d_tile_first, d_tile_cend, N, KB, BN}; }
+  GemmOut out() const {
+    GemmOut g{direct, ws, d_tile_first, d_tile_cend, N, KB, BN, 0, 0, 0};
+    g.tile_shift = tile_n == GEMM_TILE_N ? 8 : 7;
+    return g;
+  }
 };
+
+// The value of *row_blocks for n rows with a request, in blocks of `block` rows.
+__host__ __device__ inline int gemm_row_blocks(int n, int block) { return (n > 0 ? 1 : 0) | (n > block ? 2 : 0) | n << 8; }
 
 // Workspace floats needed by any plan with this grid and BN.
 inline size_t gemm_ws_floats(int grid, int BN) { return (size_t)grid * 2 * BN * GEMM_TILE_N; }
@@ -200,6 +219,11 @@ cudaError_t gemm_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int 
 int gemm_encode_map(CUtensorMap *m, const void *base, int rows, int K, int box_rows);
 // Opts the GEMM kernel into its dynamic shared-memory size (idempotent, allocates nothing).
 cudaError_t gemm_prepare_kernel();
+// gemm_rows.cu: sets a plan's ring; the activations' maps; the launch.
+int gemm_rows_stages(GemmPlan *p);
+int gemm_encode_x(GemmXMaps *m, const void *Xhi, const void *Xlo, unsigned long long rows, int K);
+cudaError_t gemm_rows_prepare();
+cudaError_t gemm_rows_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int *d_status, cudaStream_t st, unsigned long long *trace, bool pdl);
 // Tensor map for a 16-bit [rows, cols] row-major matrix with a [box_rows, box_cols] box: 64 columns
 // (128 bytes, 128-byte swizzle) or 16 columns (32 bytes, 32-byte swizzle).
 int tma_encode_2d(CUtensorMap *m, const void *base, int is_fp16, unsigned long long rows, int cols, int box_rows,

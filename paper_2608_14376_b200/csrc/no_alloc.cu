@@ -26,7 +26,7 @@ constexpr int NA_MAX_K = CORUN_STATIC_MAX_K;
 constexpr int NA_MAX_N = CORUN_STATIC_MAX_N;
 constexpr int NA_MAX_GRID = 192;                 // CTAs (= SMs) the partial-sum area is sized for
 constexpr int NA_BN = 16;                        // padded row count of the MMA's N operand
-constexpr int NA_MAX_TILES = NA_MAX_N / GEMM_TILE_N;
+constexpr int NA_MAX_TILES = (NA_MAX_N + GEMM_TILE_N / 2 - 1) / (GEMM_TILE_N / 2);   // (tiles of 128 weight rows)
 
 constexpr size_t NA_OFF_HI = 0;
 constexpr size_t NA_HILO_BYTES = (size_t)NA_BN * NA_MAX_K * sizeof(__nv_bfloat16);

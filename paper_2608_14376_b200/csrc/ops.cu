@@ -820,8 +820,7 @@ __global__ void __launch_bounds__(SMP_THREADS, 2) sampler_kernel(SampleArgs a) {
 // The rows of the step are the slots in a new order: the slots with a request this step first (ascending slot), the
 // others behind them.  Which row a request lands in depends on its co-tenants; no value of the step depends on the
 // row (that is the invariance the whole path is built for), and with the requests in the first rows the GEMMs can
-// leave out whole blocks of rows that hold none (row_blocks: bit b = block b holds a request; blocks of 64 rows up
-// to 128 padded rows, of 128 rows above).  Per-slot sampling state is copied to the row's place.  One CTA.
+// leave out what is behind them (row_blocks: GemmPlan::row_blocks).  Per-slot sampling state is copied to the row's place.  One CTA.
 __global__ void __launch_bounds__(256) prepare_rows_kernel(const uint8_t *active_mask, const uint64_t *seeds_in, uint64_t *seeds_out,
                                                            const int *in_use, const int *ctx_len, const int *pending,
                                                            const float *temp, const float *top_p, const int *step, int B,
@@ -843,7 +842,7 @@ __global__ void __launch_bounds__(256) prepare_rows_kernel(const uint8_t *active
   }
   if (s == 0 && row_blocks) {
     const int blk = B <= 128 ? 64 : 128;
-    *row_blocks = (n_act > 0 ? 1 : 0) | (n_act > blk ? 2 : 0);
+    *row_blocks = gemm_row_blocks(n_act, blk);
   }
   if (s >= B) return;
   const int r = act ? before : n_act + (s - before);   // requests first, in slot order; then the other slots
