@@ -679,6 +679,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
     CK(call);                                         \
     ++stage;                                          \
   } while (0)
+  const bool many = P.pair && !P.shorts;
   bool normed = false;                              // the layer's input has been normalised behind the layer before
   const int QD = s.n_q_heads * s.head_dim;
   // (short prompts) the blocks of the chunk: first row, and the rows of it as token-wise kernels take them
@@ -691,7 +692,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
     GemmOut prev = ffn_out(e, P, l > 0 ? l - 1 : 0);
     if (!normed)
       STAGE(launch_resid_norm(P.h, s.hidden, e->embed, rows, l == 0 ? nullptr : &prev, e->attn_norm[l], s.rms_eps,
-                              P.xn_hi, P.xn_lo, e->st));
+                              P.xn_hi, P.xn_lo, e->st, many));
     normed = false;
     if (P.pair) {
       // prefill; long prompts: projections on pairs of SMs, plain results
@@ -736,7 +737,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
       if (!P.shorts) {
         STAGE(gemm_pair_launch(P.b_o, e->tb_o[l], P.R, e->d_status, e->st));
         const GemmOut o = gemm_pair_out(P.b_o, P.R, P.plain_tiles);
-        STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st));
+        STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &o, e->mlp_norm[l], s.rms_eps, P.xn_hi, P.xn_lo, e->st, many));
       }
       const bool experts = e->moe_E && !dense_layer(e, l);
       const bf16 *next_norm = l + 1 < s.n_layers ? e->attn_norm[l + 1] : e->final_norm;
@@ -866,7 +867,7 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
   }
   if (&P != &e->dec && !normed) {                   // prefill: the final norm
     const GemmOut last = ffn_out(e, P, s.n_layers - 1);
-    STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &last, e->final_norm, s.rms_eps, P.xn_hi, P.xn_lo, e->st));
+    STAGE(launch_resid_norm(P.h, s.hidden, nullptr, rows, &last, e->final_norm, s.rms_eps, P.xn_hi, P.xn_lo, e->st, many));
   }
 #undef STAGE
   if (launches) *launches += n;

@@ -55,10 +55,10 @@ struct SampleArgs {
 };
 
 // h = E[token] (first = 1) or h += GEMM result (first = 0); then RMSNorm with
-// gains g -> bf16 hi/lo pair.
+// gains g -> bf16 hi/lo pair.  many: the rows are those of long prompts (prev: a plain matrix or a gemm_pair.cu result).
 cudaError_t launch_resid_norm(float *h, int H, const __nv_bfloat16 *embed, const Rows &rows, const GemmOut *prev,
                               const __nv_bfloat16 *gains, float eps, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo,
-                              cudaStream_t st);
+                              cudaStream_t st, bool many = false);
 // RoPE on q and k, q -> q_out fp32 [R, nq*hd], k/v -> pages (fp16) at the row's position.
 cudaError_t launch_qkv_post(const GemmOut &qkv, const Rows &rows, const float2 *rope_tab, int nq, const KvLayout &kv,
                             int layer, float *q_out, int *d_status, cudaStream_t st);
