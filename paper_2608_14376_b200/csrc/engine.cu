@@ -77,10 +77,11 @@ struct Program {
   // 3.94 -> 3.87, 64 of 64 (nearly all experts selected) 4.26 -> 4.28.
   bool select = false;
   int *moe_sel = nullptr;
-  // grouped form of the experts' GEMMs (prefill chunks: the rows of an expert gathered into blocks of 64)
+  // grouped form of the experts' GEMMs: the rows of an expert gathered into blocks of 64 (prompts: of 128, on pairs of SMs)
   bool grouped = false;
   MoeGroups grp{};
   GemmPlan p_gug, p_dng;
+  GemmExpertsPlan x_gu, x_down;          // (prompts: blocks of 128)
   bf16 *xg_hi = nullptr, *xg_lo = nullptr, *hg_hi = nullptr, *hg_lo = nullptr;
   float *gug_out = nullptr, *yg_out = nullptr;
   int *plain_tiles = nullptr;            // zeros: the table that makes a plain matrix readable as a GEMM result
@@ -276,7 +277,7 @@ int dmalloc(DevMem &m, T **p, size_t n, bool zero = true) {
 int pad16(int x) { return (x + 15) / 16 * 16; }
 
 void mla_group_table(std::vector<int> &t, int nh, int rows_per_head, int BG, int R, int w_rows, int count_at);
-int program_create_groups(corun_engine *e, Program &P, int R);
+int program_create_groups(corun_engine *e, Program &P, int R, int lg_rows);
 
 // fuse_swiglu: the gate / up GEMM writes silu(gate) * up itself (dense feed-forward, up to 128 padded rows: the
 // decode program while it is bound by the weight stream; whole tiles on fewer CTAs would cost a prefill chunk,
@@ -427,7 +428,7 @@ int program_create(corun_engine *e, Program &P, int R, bool layers, bool lm, boo
         // prefill chunks: every row through every expert would be (E + S) / top_k times the MMA work, which a
         // chunk of 256 rows does pay for; the rows of an expert are gathered into blocks of 64 instead
         if (!P.plain_tiles) RC(dmalloc(A, &P.plain_tiles, (size_t)(H / GEMM_TILE_N + 1)));
-        RC(program_create_groups(e, P, R));
+        RC(program_create_groups(e, P, R, 6));
       }
     }
   }
@@ -454,12 +455,13 @@ void mla_group_table(std::vector<int> &t, int nh, int rows_per_head, int BG, int
 }
 
 // Buffers and plans of the experts' grouped form for up to R rows.
-int program_create_groups(corun_engine *e, Program &P, int R) {
+int program_create_groups(corun_engine *e, Program &P, int R, int lg_rows) {
   const int Fm = e->moe_F, NB = e->moe_E + e->moe_S, H = e->sh.hidden;
   auto &A = P.allocs;
   MoeGroups &g = P.grp;
-  g.n_groups_max = moe_max_groups(R, e->moe_E, e->moe_S, e->moe_K);
-  const size_t slots = (size_t)g.n_groups_max * MOE_GROUP_ROWS;
+  g.lg_rows = lg_rows;
+  g.n_groups_max = moe_max_groups(R, e->moe_E, e->moe_S, e->moe_K, lg_rows);
+  const size_t slots = (size_t)g.n_groups_max << lg_rows;
   RC(dmalloc(A, &g.tab_up, (size_t)g.n_groups_max * 3 + 1));
   RC(dmalloc(A, &g.tab_down, (size_t)g.n_groups_max * 3 + 1));
   RC(dmalloc(A, &g.group_expert, (size_t)g.n_groups_max));
@@ -471,20 +473,24 @@ int program_create_groups(corun_engine *e, Program &P, int R) {
   RC(dmalloc(A, &P.hg_hi, slots * Fm));
   RC(dmalloc(A, &P.hg_lo, slots * Fm));
   RC(dmalloc(A, &P.yg_out, slots * H));
+  P.grouped = true;
+  if (P.pair) {                                     // prompts: on pairs of SMs
+    RC(gemm_experts_plan_create_swiglu(&P.x_gu, Fm, H, P.xg_hi, P.xg_lo, g.n_groups_max, P.hg_hi, P.hg_lo, g.slot_w, g.tab_up, e->num_sms));
+    return gemm_experts_plan_create(&P.x_down, H, Fm, P.hg_hi, P.hg_lo, g.n_groups_max, P.yg_out, g.tab_down, e->num_sms);
+  }
   // gate / up per group with the routing weight and the SwiGLU in the epilogue where a tile width divides the
   // experts' width, else fp32 sums and a kernel of its own
   const int half = gemm_swiglu_blocks_half(Fm, NB, e->num_sms);
   if (half) {
     RC(gemm_plan_create_grouped_swiglu(&P.p_gug, e->w0_gu, (long long)NB * 2 * Fm, Fm, H, half, P.xg_hi, P.xg_lo, g.n_groups_max,
-                                       MOE_GROUP_ROWS, P.hg_hi, P.hg_lo, g.slot_w, g.tab_up, e->num_sms));
+                                       g.rows(), P.hg_hi, P.hg_lo, g.slot_w, g.tab_up, e->num_sms));
   } else {
     RC(dmalloc(A, &P.gug_out, slots * 2 * Fm));
     RC(gemm_plan_create_grouped(&P.p_gug, e->w0_gu, (long long)NB * 2 * Fm, H, 2 * Fm, H, P.xg_hi, P.xg_lo, g.n_groups_max,
-                                MOE_GROUP_ROWS, P.gug_out, g.tab_up, e->num_sms));
+                                g.rows(), P.gug_out, g.tab_up, e->num_sms));
   }
-  RC(gemm_plan_create_grouped(&P.p_dng, e->w0_down, H, NB * Fm, H, Fm, P.hg_hi, P.hg_lo, g.n_groups_max, MOE_GROUP_ROWS,
+  RC(gemm_plan_create_grouped(&P.p_dng, e->w0_down, H, NB * Fm, H, Fm, P.hg_hi, P.hg_lo, g.n_groups_max, g.rows(),
                               P.yg_out, g.tab_down, e->num_sms));
-  P.grouped = true;
   return CORUN_OK;
 }
 
@@ -586,7 +592,7 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
     RC(dmalloc(A, &P.router_out, c * e->moe_E));
     RC(dmalloc(A, &P.moe_mask, (size_t)(e->moe_E + e->moe_S) * (MOE_MANY_ROWS / 32)));
     RC(gemm_pair_plan_create(&P.b_router, e->moe_E, H, P.xn_hi, P.xn_lo, cap, P.router_out, P.pair_part, e->num_sms));
-    RC(program_create_groups(e, P, cap));
+    RC(program_create_groups(e, P, cap, 7));
   }
   return CORUN_OK;
 }
@@ -760,13 +766,8 @@ int run_layers(corun_engine *e, Program &P, int *launches) {
         STAGE(launch_moe_route(gemm_pair_out(P.b_router, P.R, P.plain_tiles), P.R, e->moe_E, e->moe_S, e->moe_K, e->moe_renorm, P.moe_w, e->st));
         STAGE(launch_moe_group_many(P.moe_w, P.row_active, P.R, e->moe_E, e->moe_S, e->moe_F, P.moe_mask, P.grp, e->st));
         STAGE(launch_moe_gather(P.xn_hi, P.xn_lo, s.hidden, P.grp, P.xg_hi, P.xg_lo, e->st));
-        if (P.p_gug.sw_hi) {
-          STAGE(gemm_launch(P.p_gug, &e->tm_gu_half[l], e->d_status, e->st, nullptr, true));
-        } else {
-          STAGE(gemm_launch(P.p_gug, &e->tm_gu[l], e->d_status, e->st, nullptr, true));
-          STAGE(launch_moe_swiglu_grouped(P.gug_out, P.moe_w, NB, e->moe_F, P.grp, P.hg_hi, P.hg_lo, e->st));
-        }
-        STAGE(gemm_launch(P.p_dng, &e->tm_down[l], e->d_status, e->st, nullptr, true));
+        STAGE(gemm_experts_launch(P.x_gu, e->tm_gu[l], e->d_status, e->st));
+        STAGE(gemm_experts_launch(P.x_down, e->tm_down[l], e->d_status, e->st));
         STAGE(launch_moe_combine(P.yg_out, P.row_active, P.R, NB, s.hidden, P.grp, P.down_out, e->st));
       } else if (!P.shorts) {
         STAGE(gemm_pair_launch(P.b_gu, e->tb_gu[l], P.R, e->d_status, e->st, &e->tb_gu96[l]));

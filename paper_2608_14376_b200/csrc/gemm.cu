@@ -588,7 +588,7 @@ int gemm_plan_create_swiglu_blocks(GemmPlan *p, const void *W, int n_blocks, int
 
 int gemm_plan_create_grouped(GemmPlan *p, const void *W, long long w_rows, int w_cols, int N, int K, const void *Xhi,
                              const void *Xlo, int n_groups, int BN, float *direct, const int *group_tab, int num_sms) {
-  if (N <= 0 || N % GEMM_TILE_N || K <= 0 || K % GEMM_BLOCK_K || w_cols % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > 64 ||
+  if (N <= 0 || N % GEMM_TILE_N || K <= 0 || K % GEMM_BLOCK_K || w_cols % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > GEMM_MAX_ROWS ||
       n_groups < 1 || !group_tab || w_rows < N || num_sms < 1)
     return CORUN_EINVAL;
   p->N = N; p->K = K; p->R = BN; p->BN = BN;
@@ -622,7 +622,7 @@ int gemm_plan_create_grouped_swiglu(GemmPlan *p, const void *W, long long w_rows
                                     const void *Xlo, int n_groups, int BN, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo,
                                     const float *row_scale, const int *group_tab, int num_sms) {
   if (F <= 0 || half < 64 || half > GEMM_TILE_N / 2 || half % 8 || F % half || K <= 0 || K % GEMM_BLOCK_K || BN % 16 || BN < 16 ||
-      BN > 64 || n_groups < 1 || !group_tab || !out_hi || !out_lo || !row_scale || w_rows < 2 * F || num_sms < 1)
+      BN > GEMM_MAX_ROWS || n_groups < 1 || !group_tab || !out_hi || !out_lo || !row_scale || w_rows < 2 * F || num_sms < 1)
     return CORUN_EINVAL;
   p->sw_half = half;
   p->N = 2 * F; p->K = K; p->R = BN; p->BN = BN;

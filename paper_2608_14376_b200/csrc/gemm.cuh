@@ -163,7 +163,7 @@ inline size_t gemm_ws_floats(int grid, int BN) { return (size_t)grid * 2 * BN * 
 int gemm_plan_create(GemmPlan *p, const void *W, int N, int K, const void *Xhi, const void *Xlo, int R, int BN,
                      float *direct, float *ws, int num_sms);
 void gemm_plan_destroy(GemmPlan *p);
-// Grouped GEMM over at most n_groups groups of up to BN <= 64 rows each: group g multiplies rows g * BN .. of
+// Grouped GEMM over at most n_groups groups of up to BN <= 128 rows each: group g multiplies rows g * BN .. of
 // Xhi / Xlo ([n_groups * BN, K]) with N weight rows starting at the row, and K elements starting at the k-block,
 // that group_tab names for it, into rows g * BN .. of `direct` ([n_groups * BN, N]).  W is [w_rows, w_cols]
 // bf16.  group_tab has 3 * n_groups + 1 ints: the last one is the number of groups in use (groups 0 .. that - 1).
@@ -217,6 +217,10 @@ cudaError_t gemm_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int 
                         bool pdl = false);                     // programmatic dependent launch (row program)
 // Encodes a tensor map for a bf16 [rows, K] row-major matrix with a [box_rows, 64] box, 128-byte swizzle.
 int gemm_encode_map(CUtensorMap *m, const void *base, int rows, int K, int box_rows);
+// Padded rows of a launch (a group) with n <= 128 rows: boxes of 64, 32 and 16 rows, two at most.
+__host__ __device__ constexpr int gemm_rows_padded(int n) {
+  return n > 96 ? 128 : n > 80 ? 96 : n > 64 ? 80 : n > 48 ? 64 : n > 32 ? 48 : n > 16 ? 32 : 16;
+}
 // Opts the GEMM kernel into its dynamic shared-memory size (idempotent, allocates nothing).
 cudaError_t gemm_prepare_kernel();
 // gemm_rows.cu: sets a plan's ring; the activations' maps; the launch.
@@ -273,6 +277,21 @@ int gemm_pair_prepare();             // opts the kernels into their shared-memor
 cudaError_t gemm_pair_launch(const GemmPairPlan &p, const CUtensorMap &tmW, int R, int *d_status, cudaStream_t st,
                              const CUtensorMap *tmW96 = nullptr, const float *kv_scale = nullptr,
                              unsigned long long *trace = nullptr);   // (debug) timeline, as gemm_launch's; 2 * pairs CTAs at most
+// ---- the experts of a prompt (gemm_experts.cu): groups of up to 128 rows on pairs of SMs; groups and results as
+// gemm_plan_create_grouped / _swiglu with BN = 128.  tmW: the matrix with a box of GEMM_W_BOX rows ----
+struct GemmExpertsPlan {
+  GemmXMaps tmX;
+  int N = 0, K = 0, tiles_per_group = 0, n_groups_max = 0, pairs = 0;
+  const int *group_tab = nullptr;    // not owned, as are the others
+  const float *row_w = nullptr;
+  float *direct = nullptr;
+  __nv_bfloat16 *sw_hi = nullptr, *sw_lo = nullptr;
+};
+int gemm_experts_plan_create(GemmExpertsPlan *p, int N, int K, const void *Xhi, const void *Xlo, int n_groups, float *direct, const int *group_tab,
+                             int num_sms);
+int gemm_experts_plan_create_swiglu(GemmExpertsPlan *p, int F, int K, const void *Xhi, const void *Xlo, int n_groups, __nv_bfloat16 *out_hi,
+                                    __nv_bfloat16 *out_lo, const float *row_w, const int *group_tab, int num_sms);
+cudaError_t gemm_experts_launch(const GemmExpertsPlan &p, const CUtensorMap &tmW, int *d_status, cudaStream_t st);
 // Tensor map for TMA stores of tiles of 32 rows x 32 columns into a [rows, cols] row-major matrix (fp32: 128-byte swizzle; bf16: 64).
 int tma_encode_store_2d(CUtensorMap *m, const void *base, int is_fp32, unsigned long long rows, int cols);
 // direct[r, n] = gemm_load(r, n) for every tile that has partials (makes `direct` a plain matrix).

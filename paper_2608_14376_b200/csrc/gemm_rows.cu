@@ -15,11 +15,6 @@ constexpr int GR_THREADS = 320;                     // warp 0 TMA producer, warp
 constexpr int GR_MAX_STAGES = 11;
 constexpr uint32_t GR_W_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: what one MMA reads of the weights
 
-// Padded rows of a launch (a group) with n rows: boxes of 64, 32 and 16 rows, two at most.
-__host__ __device__ constexpr int gr_rows(int n) {
-  return n > 96 ? 128 : n > 80 ? 96 : n > 64 ? 80 : n > 48 ? 64 : n > 32 ? 48 : n > 16 ? 32 : 16;
-}
-
 struct GemmRowsArgs {
   float *direct, *ws;
   const int *cta_start;
@@ -87,7 +82,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t w_box = (uint32_t)a.w_rows * GEMM_BLOCK_K * 2, w_bytes = (uint32_t)MT * w_box;
   const int sw_fb = (SWIGLU && MASKED) ? N / (2 * a.keep_pitch) : N / 2;   // SWIGLU: gate rows of a matrix
-  int n_pad = gr_rows(BN);                          // padded rows (of the launch; GROUPED: of the segment)
+  int n_pad = gemm_rows_padded(BN);                          // padded rows (of the launch; GROUPED: of the segment)
 
   // the group of the CTA's i-th tile (read only after the wait for the table below)
   int g_tile = -1, g_id = 0, g_j = 0, g_wrow = 0, g_wk = 0, g_rows = 0;
@@ -107,7 +102,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       g_wrow = a.group_tab[3 * g_id];
       g_wk = a.group_tab[3 * g_id + 1];
       g_rows = a.group_tab[3 * g_id + 2];
-      n_pad = gr_rows(g_rows);
+      n_pad = gemm_rows_padded(g_rows);
     }
   };
   // behind the wait for the predecessor: the rows of this step
@@ -115,7 +110,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     if ((!GROUPED || SELECT) && a.row_blocks) {
       griddep_wait();
       const int v = *reinterpret_cast<const volatile int *>(a.row_blocks), n = v >> 8;
-      n_pad = gr_rows(min(BN, n > 0 ? n : (v & 2) ? BN : 64));
+      n_pad = gemm_rows_padded(min(BN, n > 0 ? n : (v & 2) ? BN : 64));
     }
   };
   // A segment's accumulators: block mt's columns start at mt * 128 of one half of tensor memory, or (more than 64 padded rows
@@ -450,7 +445,7 @@ cudaError_t each_kernel(F f) {
 int gemm_rows_stages(GemmPlan *p) {
   const int mt = p->sw_half ? 2 : p->tile_n / 128, box = p->sw_half ? p->sw_half : 128;
   const size_t w = (size_t)mt * box * GEMM_BLOCK_K * 2;
-  p->stage_bytes = (uint32_t)(w + (size_t)gr_rows(p->BN) * 256);
+  p->stage_bytes = (uint32_t)(w + (size_t)gemm_rows_padded(p->BN) * 256);
   // an MMA always reads 128 weight rows: what the last stage leaves behind the second block's rows must be readable
   const size_t over = GR_W_BYTES - (size_t)box * GEMM_BLOCK_K * 2, fixed = 1024 + over;
   int stages = (int)((GEMM_ROWS_MAX_SMEM - fixed) / p->stage_bytes);

@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(256) moe_readout_kernel(GemmOut d, int H, floa
 // ---------------------------------------------------------------- grouped form
 // One CTA per expert (routed experts, then the shared ones).  Every CTA counts the rows of ALL experts (the table
 // w[r, e] != 0 is small and comes from L2), so that it knows where its own expert's groups begin (experts ascending,
-// 64 rows per group) without a second kernel; it then writes its groups' table entries and hands its rows, in
+// g.rows() rows per group) without a second kernel; it then writes its groups' table entries and hands its rows, in
 // ascending row order, consecutive slots (slot_of is expert-major: [E + S][R]).  CTA 0 also clears the entries of
 // the groups nobody needs and publishes the number of groups in use.
 constexpr int MOE_GROUP_THREADS = 512;
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_kernel(const floa
     // groups before this expert, and in all: lanes take experts lane, lane + 32, ...
     int before = 0, all = 0;
     for (int ee = lane; ee < NB; ee += 32) {
-      const int n = (cnt[ee] + MOE_GROUP_ROWS - 1) / MOE_GROUP_ROWS;
+      const int n = (cnt[ee] + g.rows() - 1) >> g.lg_rows;
       all += n;
       if (ee < e) before += n;
     }
@@ -306,17 +306,17 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_kernel(const floa
     }
     if (tid == 0) g.tab_up[3 * g.n_groups_max] = g.tab_down[3 * g.n_groups_max] = used;   // what the GEMMs walk
   }
-  const int n_groups = (cnt[e] + MOE_GROUP_ROWS - 1) / MOE_GROUP_ROWS;
+  const int n_groups = (cnt[e] + g.rows() - 1) >> g.lg_rows;
   for (int k = tid; k < n_groups; k += MOE_GROUP_THREADS) {
     const int u = first + k;
     if (u >= g.n_groups_max) break;                 // cannot happen: n_groups_max bounds the sum
-    const int rows = min(MOE_GROUP_ROWS, cnt[e] - k * MOE_GROUP_ROWS);
+    const int rows = min(g.rows(), cnt[e] - (k << g.lg_rows));
     g.tab_up[3 * u] = e * 2 * F; g.tab_up[3 * u + 1] = 0; g.tab_up[3 * u + 2] = rows;
     g.tab_down[3 * u] = 0; g.tab_down[3 * u + 1] = e * F / GEMM_BLOCK_K; g.tab_down[3 * u + 2] = rows;
     g.group_expert[u] = e;
   }
   if (warp == 0) {
-    int base = first * MOE_GROUP_ROWS;               // slot of the expert's next row
+    int base = (first << g.lg_rows);               // slot of the expert's next row
     for (int r0 = 0; r0 < R; r0 += 32) {
       const int r = r0 + lane;
       const float wv = r < R ? wsel[r] : 0.f;
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_many_kernel(const
   if (warp == 0) {
     int before = 0, all = 0;
     for (int ee = lane; ee < NB; ee += 32) {
-      const int n = (cnt[ee] + MOE_GROUP_ROWS - 1) / MOE_GROUP_ROWS;
+      const int n = (cnt[ee] + g.rows() - 1) >> g.lg_rows;
       all += n;
       if (ee < e) before += n;
     }
@@ -408,11 +408,11 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_many_kernel(const
     }
     if (tid == 0) g.tab_up[3 * g.n_groups_max] = g.tab_down[3 * g.n_groups_max] = used;   // what the GEMMs walk
   }
-  const int n_groups = (cnt[e] + MOE_GROUP_ROWS - 1) / MOE_GROUP_ROWS;
+  const int n_groups = (cnt[e] + g.rows() - 1) >> g.lg_rows;
   for (int k = tid; k < n_groups; k += MOE_GROUP_THREADS) {
     const int u = first + k;
     if (u >= g.n_groups_max) break;                 // cannot happen: n_groups_max bounds the sum
-    const int rows = min(MOE_GROUP_ROWS, cnt[e] - k * MOE_GROUP_ROWS);
+    const int rows = min(g.rows(), cnt[e] - (k << g.lg_rows));
     g.tab_up[3 * u] = e * 2 * F; g.tab_up[3 * u + 1] = 0; g.tab_up[3 * u + 2] = rows;
     g.tab_down[3 * u] = 0; g.tab_down[3 * u + 1] = e * F / GEMM_BLOCK_K; g.tab_down[3 * u + 2] = rows;
     g.group_expert[u] = e;
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_many_kernel(const
     const uint32_t m = own[r >> 5], bit = 1u << (r & 31);
     int slot = -1;
     if (m & bit) {
-      slot = first * MOE_GROUP_ROWS + own_before[r >> 5] + __popc(m & (bit - 1u));
+      slot = (first << g.lg_rows) + own_before[r >> 5] + __popc(m & (bit - 1u));
       g.slot_row[slot] = r;
       g.slot_w[slot] = w[(size_t)r * NB + e];
     }
@@ -449,10 +449,10 @@ __global__ void __launch_bounds__(256) moe_gather_kernel(const bf16 *__restrict_
   griddep_wait();
   x_hi = after_wait(x_hi); x_lo = after_wait(x_lo);
   const int lane = threadIdx.x & 31;
-  const int n_slots = g.tab_up[3 * g.n_groups_max] * MOE_GROUP_ROWS;
+  const int n_slots = g.tab_up[3 * g.n_groups_max] << g.lg_rows;
   const int n_warps = (int)(gridDim.x * (blockDim.x >> 5));
   for (int slot = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); slot < n_slots; slot += n_warps) {
-    if (slot % MOE_GROUP_ROWS >= g.tab_up[3 * (slot / MOE_GROUP_ROWS) + 2]) continue;   // no row in this slot
+    if ((slot & (g.rows() - 1)) >= g.tab_up[3 * (slot >> g.lg_rows) + 2]) continue;   // no row in this slot
     const int r = g.slot_row[slot];
     const uint4 *sh = reinterpret_cast<const uint4 *>(x_hi + (size_t)r * H), *sl = reinterpret_cast<const uint4 *>(x_lo + (size_t)r * H);
     uint4 *dh = reinterpret_cast<uint4 *>(xg_hi + (size_t)slot * H), *dl = reinterpret_cast<uint4 *>(xg_lo + (size_t)slot * H);
@@ -474,9 +474,9 @@ __global__ void __launch_bounds__(256) moe_swiglu_grouped_kernel(const float *__
   griddep_launch_dependents();
   griddep_wait();
   const int slot = blockIdx.x;
-  if (slot % MOE_GROUP_ROWS >= g.tab_up[3 * (slot / MOE_GROUP_ROWS) + 2]) return;   // no row in this slot
+  if ((slot & (g.rows() - 1)) >= g.tab_up[3 * (slot >> g.lg_rows) + 2]) return;   // no row in this slot
   const int r = g.slot_row[slot];
-  const int e = g.group_expert[slot / MOE_GROUP_ROWS];
+  const int e = g.group_expert[slot >> g.lg_rows];
   const float we = w[(size_t)r * NB + e];
   const float *row = gu + (size_t)slot * 2 * F;
   for (int f = threadIdx.x * 4; f < F; f += blockDim.x * 4) {
@@ -581,13 +581,13 @@ cudaError_t launch_moe_route(const GemmOut &logits, int R, int E, int S, int top
 
 cudaError_t launch_moe_gather(const __nv_bfloat16 *x_hi, const __nv_bfloat16 *x_lo, int H, const MoeGroups &g,
                               __nv_bfloat16 *xg_hi, __nv_bfloat16 *xg_lo, cudaStream_t st) {
-  const int blocks = (g.n_groups_max * MOE_GROUP_ROWS + 7) / 8;   // a warp per slot, as far as 1184 CTAs go
+  const int blocks = ((g.n_groups_max << g.lg_rows) + 7) / 8;   // a warp per slot, as far as 1184 CTAs go
   return launch_k(moe_gather_kernel, dim3(blocks < 1184 ? blocks : 1184), dim3(256), 0, st, true, x_hi, x_lo, H, g, xg_hi, xg_lo);
 }
 
 cudaError_t launch_moe_swiglu_grouped(const float *gu, const float *w, int n_blocks, int F, const MoeGroups &g,
                                       __nv_bfloat16 *hg_hi, __nv_bfloat16 *hg_lo, cudaStream_t st) {
-  return launch_k(moe_swiglu_grouped_kernel, dim3(g.n_groups_max * MOE_GROUP_ROWS), dim3(192), 0, st, true, gu, w, n_blocks, F, g,
+  return launch_k(moe_swiglu_grouped_kernel, dim3(g.n_groups_max << g.lg_rows), dim3(192), 0, st, true, gu, w, n_blocks, F, g,
                   hg_hi, hg_lo);
 }
 
@@ -716,8 +716,9 @@ int corun_moe_create(const corun_moe_shape *shape, const void *router, const voi
   const int g_half = gemm_swiglu_blocks_half(F, NB, m->num_sms);
   if (m->BN > 64 && g_half > 0 && H % GEMM_TILE_N == 0 && !getenv("CORUN_MOE_DECODE_DENSE")) {
     MoeGroups &g = m->grp;
-    g.n_groups_max = moe_max_groups(B, E, s.n_shared, s.top_k);
-    const size_t slots = (size_t)g.n_groups_max * MOE_GROUP_ROWS;
+    g.lg_rows = 6;
+    g.n_groups_max = moe_max_groups(B, E, s.n_shared, s.top_k, g.lg_rows);
+    const size_t slots = (size_t)g.n_groups_max << g.lg_rows;
     if ((rc = moe_alloc(m, &g.tab_up, (size_t)g.n_groups_max * 3 + 1)) || (rc = moe_alloc(m, &g.tab_down, (size_t)g.n_groups_max * 3 + 1)) ||
         (rc = moe_alloc(m, &g.group_expert, (size_t)g.n_groups_max)) || (rc = moe_alloc(m, &g.slot_row, slots)) ||
         (rc = moe_alloc(m, &g.slot_of, (size_t)B * NB)) || (rc = moe_alloc(m, &g.slot_w, slots)) ||
@@ -728,8 +729,8 @@ int corun_moe_create(const corun_moe_shape *shape, const void *router, const voi
     std::vector<int> ones((size_t)B, 1);
     if (cudaMemcpy(m->d_active, ones.data(), (size_t)B * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return fail(CORUN_ECUDA);
     if ((rc = gemm_plan_create_grouped_swiglu(&m->p_gug, gate_up, (long long)NB * 2 * F, F, H, g_half, m->xg_hi, m->xg_lo, g.n_groups_max,
-                                              MOE_GROUP_ROWS, m->hg_hi, m->hg_lo, g.slot_w, g.tab_up, m->num_sms)) ||
-        (rc = gemm_plan_create_grouped(&m->p_dng, down, H, NB * F, H, F, m->hg_hi, m->hg_lo, g.n_groups_max, MOE_GROUP_ROWS, m->yg,
+                                              g.rows(), m->hg_hi, m->hg_lo, g.slot_w, g.tab_up, m->num_sms)) ||
+        (rc = gemm_plan_create_grouped(&m->p_dng, down, H, NB * F, H, F, m->hg_hi, m->hg_lo, g.n_groups_max, g.rows(), m->yg,
                                        g.tab_down, m->num_sms)))
       return fail(rc);
     m->grouped = true;

@@ -31,25 +31,26 @@ cudaError_t launch_moe_combine_select(const float *yg, const int *sel, int n_per
 cudaError_t launch_moe_swiglu(const GemmOut &gu, const float *w, int R, int F, int n_blocks, __nv_bfloat16 *out_hi,
                               __nv_bfloat16 *out_lo, cudaStream_t st);
 
-// ---- grouped form (prefill chunks): every expert's rows gathered into blocks of MOE_GROUP_ROWS rows ----
-constexpr int MOE_GROUP_ROWS = 64;
+// ---- grouped form: every expert's rows gathered into blocks of g.rows() rows ----
 constexpr int MOE_MANY_ROWS = 2048;   // most rows of the many-rows forms below
 // Most groups a chunk of R rows can need: one per expert plus one per full block of selected (row, expert) pairs.
-inline int moe_max_groups(int R, int E, int S, int top_k) { return E + S + R * (top_k + S) / MOE_GROUP_ROWS; }
+inline int moe_max_groups(int R, int E, int S, int top_k, int lg_rows) { return E + S + (R * (top_k + S) >> lg_rows); }
 
 // Buffers of the grouped form (device, owned by the caller).
 struct MoeGroups {
   int n_groups_max;      // moe_max_groups(...)
+  int lg_rows;           // log2 of the rows per group: 6, or 7 for the many rows of a prompt
   int *tab_up;           // [n_groups_max][3] + 1: first gate/up weight row (e * 2F), 0, rows   (gemm group table);
                          //   the last int: groups in use
   int *tab_down;         // [n_groups_max][3] + 1: 0, first down k-block (e * F / 64), rows; groups in use
   int *group_expert;     // [n_groups_max]
-  int *slot_row;         // [n_groups_max * 64]: the chunk row gathered into the slot (valid below the group's row count)
+  int *slot_row;         // [n_groups_max * rows]: the chunk row gathered into the slot (valid below the group's row count)
   int *slot_of;          // [E + S][R]: where the row sits in the expert's groups, -1 = not selected
-  float *slot_w;         // [n_groups_max * 64]: the slot's routing weight w[row, expert] (valid below the group's row count)
+  __host__ __device__ int rows() const { return 1 << lg_rows; }
+  float *slot_w;         // [n_groups_max * rows]: the slot's routing weight w[row, expert] (valid below the group's row count)
 };
 
-// Groups the chunk's (row, expert) pairs: experts ascending, an expert's rows ascending, 64 per group; rows with
+// Groups the chunk's (row, expert) pairs: experts ascending, an expert's rows ascending, g.rows() per group; rows with
 // active[r] == 0 are left out.  w: the routing weights [R][E + S] of launch_moe_route.  One CTA.
 cudaError_t launch_moe_group(const float *w, const int *active, int R, int E, int S, int F, const MoeGroups &g,
                              cudaStream_t st);
