@@ -38,7 +38,7 @@ WORKLOADS = {
     # Mixture-of-Experts decoder (Qwen3-30B-A3B shape); no CPU baseline (the weights do not fit the host leg)
     "qwen3_30b_a3b_b64": (synth.QWEN3_30B_A3B, 64, 40, 512, 4096, 0.7, 0.95, 1.28),
 }
-PREFILL_ROWS = 2048   # rows of a long prompt's chunk (the layers' weights are streamed once per chunk)
+PREFILL_ROWS = 4096   # rows of a long prompt's chunk (the layers' weights are streamed once per chunk)
 MOE = {"qwen3_30b_a3b_b64": (synth.QWEN3_30B_A3B_MOE, synth.QWEN3_30B_A3B_EFF)}
 # Decoder with multi-head latent attention and expert layers (DeepSeek-V2-Lite shape): 128 slots, all active
 MLA = {"deepseek_v2_lite_b128": (synth.DEEPSEEK_V2_LITE, synth.DEEPSEEK_V2_LITE_MLA, synth.DEEPSEEK_V2_LITE_MOE, 128, 128, 512, 4096, 0.7, 0.95, 0.5)}

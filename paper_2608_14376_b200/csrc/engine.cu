@@ -133,13 +133,18 @@ struct Program {
 // Prompts of up to PREFILL_SMALL tokens are short (Program::shorts), longer ones long.  Which one depends on the prompt's
 // own length only, so a prompt's values do not depend on what is prefilled with it.  Measured, GEMMs of the Qwen3-8B layer:
 // 64 rows 82 us and 128 rows 110 us in a block of SHORT_ROWS; 256 rows 179 us (two blocks: 220), 512 rows 299, 1024 rows
-// 543, 2048 rows 1049 on pairs of SMs (hence chunks as large as the buffers allow).
-constexpr int PREFILL_SMALL = 128, PREFILL_BIG = 2048;
+// 543, 2048 rows 1049 on pairs of SMs (hence chunks as large as the buffers allow; PREFILL_BIG 2048 -> 4096, that is one pass over
+// the experts and not two: 2505 tokens through 9 DeepSeek-V2-Lite layers 13.6 -> 10.9 ms; 6001 tokens through 12 Qwen3-8B layers
+// 54.3 -> 54.0, where the products are bound by the tensor cores).
+constexpr int PREFILL_SMALL = 128, PREFILL_BIG = 4096;
 // Rows of a long prompt's chunk that the latent attention takes at a time (its partial results are kept per row).
 constexpr int MLA_ROWS = 256;
 constexpr int SHORT_ROWS = 128;
 constexpr int WIDE_ROWS = 192;               // see Program::wide
 static_assert(PREFILL_BIG <= MOE_MANY_ROWS, "a chunk of a long prompt is grouped in one go");
+// (a request of a long prompt's chunk begins on a tile of 128 rows and has more than one, but for the first and the last)
+static_assert(PREFILL_BIG / 256 + 1 <= MLA_MAX_SEGS, "latent attention gathers all requests of a chunk");
+static_assert(PREFILL_BIG / SHORT_ROWS <= 32, "the staging buffer holds 32 blocks and 32 tiles");
 // corun_get_logits: a row goes to the host by way of pinned memory, from LOGITS_SPLIT values on in two pieces, the first copied
 // on to the caller while the second arrives.  A piece costs some 3 us of calls.  A call for 151936 / 102400 / 32000 values: 60 /
 // 48 / 30 us straight into the caller's pageable memory, 59 / 38 / 20 in one piece, 54 / 37 / 21 in two, 55 / 41 / 27 in four.

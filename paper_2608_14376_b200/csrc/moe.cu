@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_kernel(const floa
 }
 
 // ---- many rows (up to MOE_MANY_ROWS): the kernel above reads the whole table w[r, e] in every CTA, 1 MB at 2048 rows and
-// 128 experts.  Here a first kernel turns it into one bit per (expert, row), 32 KB in all, which every CTA of the second
+// 128 experts.  Here a first kernel turns it into one bit per (expert, row), 64 KB in all, which every CTA of the second
 // reads, and the second hands out the slots of all its rows at once.
 constexpr int MOE_MASK_WORDS = MOE_MANY_ROWS / 32;
 
@@ -369,20 +369,29 @@ __global__ void __launch_bounds__(MOE_GROUP_THREADS) moe_group_many_kernel(const
   griddep_wait();
   w = after_wait(w); mask = after_wait(mask);
   for (int ee = warp; ee < NB; ee += MOE_GROUP_THREADS / 32) {
-    const uint32_t a = lane < words ? mask[ee * MOE_MASK_WORDS + lane] : 0u, b = lane + 32 < words ? mask[ee * MOE_MASK_WORDS + lane + 32] : 0u;
-    const int na = __popc(a), nb = __popc(b);
-    int ia = na, ib = nb;                            // inclusive sums over the lanes
+    uint32_t m[MOE_MASK_WORDS / 32];                 // word lane + 32 k
+    int n[MOE_MASK_WORDS / 32], inc[MOE_MASK_WORDS / 32], all = 0;   // rows of a word, inclusive sums over the lanes
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int xa = __shfl_up_sync(0xffffffffu, ia, o), xb = __shfl_up_sync(0xffffffffu, ib, o);
-      if (lane >= o) { ia += xa; ib += xb; }
+    for (int k = 0; k < MOE_MASK_WORDS / 32; ++k) {
+      m[k] = lane + 32 * k < words ? mask[ee * MOE_MASK_WORDS + lane + 32 * k] : 0u;
+      n[k] = inc[k] = __popc(m[k]);
     }
-    const int all_a = __shfl_sync(0xffffffffu, ia, 31), all_b = __shfl_sync(0xffffffffu, ib, 31);
-    if (lane == 0) cnt[ee] = all_a + all_b;
-    if (ee == e) {
-      own[lane] = a; own[lane + 32] = b;
-      own_before[lane] = ia - na; own_before[lane + 32] = all_a + ib - nb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int k = 0; k < MOE_MASK_WORDS / 32; ++k) {
+        const int x = __shfl_up_sync(0xffffffffu, inc[k], o);
+        if (lane >= o) inc[k] += x;
+      }
+#pragma unroll
+    for (int k = 0; k < MOE_MASK_WORDS / 32; ++k) {
+      if (ee == e) {
+        own[lane + 32 * k] = m[k];
+        own_before[lane + 32 * k] = all + inc[k] - n[k];
+      }
+      all += __shfl_sync(0xffffffffu, inc[k], 31);
     }
+    if (lane == 0) cnt[ee] = all;
   }
   __syncthreads();
   if (warp == 0) {

@@ -32,7 +32,7 @@ cudaError_t launch_moe_swiglu(const GemmOut &gu, const float *w, int R, int F, i
                               __nv_bfloat16 *out_lo, cudaStream_t st);
 
 // ---- grouped form: every expert's rows gathered into blocks of g.rows() rows ----
-constexpr int MOE_MANY_ROWS = 2048;   // most rows of the many-rows forms below
+constexpr int MOE_MANY_ROWS = 4096;   // most rows of the many-rows forms below
 // Most groups a chunk of R rows can need: one per expert plus one per full block of selected (row, expert) pairs.
 inline int moe_max_groups(int R, int E, int S, int top_k, int lg_rows) { return E + S + (R * (top_k + S) >> lg_rows); }
 
