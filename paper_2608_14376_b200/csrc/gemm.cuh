@@ -70,6 +70,31 @@ __device__ __forceinline__ float4 gemm_load_pair4(const GemmOut &g, int r, int n
   return acc;
 }
 
+// Values (r, n) and (r, n2) of a GEMM result as gemm_load gives them, both sets of partials requested together.
+__device__ __forceinline__ float2 gemm_load_two(const GemmOut &g, int r, int n, int n2) {
+  const int t[2] = {n >> g.tile_shift, n2 >> g.tile_shift}, col[2] = {n - (t[0] << g.tile_shift), n2 - (t[1] << g.tile_shift)};
+  const int f[2] = {g.tile_first[t[0]], g.tile_first[t[1]]}, c1[2] = {g.tile_cend[t[0]], g.tile_cend[t[1]]};
+  const size_t cta_stride = (size_t)2 * g.BN << g.tile_shift;
+  float v[2][4], acc[2];
+  const float *p[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int c0 = f[i] >> 1;
+    p[i] = g.ws + ((size_t)r << g.tile_shift) + col[i];
+    acc[i] = c0 == c1[i] ? g.direct[(size_t)r * g.N + (i ? n2 : n)] : p[i][(size_t)f[i] * g.BN << g.tile_shift];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[i][j] = c0 + 1 + j <= c1[i] ? p[i][(size_t)(c0 + 1 + j) * cta_stride] : 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    acc[i] += 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i] += v[i][j];
+    for (int c = (f[i] >> 1) + 5; c <= c1[i]; ++c) acc[i] += p[i][(size_t)c * cta_stride];
+  }
+  return make_float2(acc[0], acc[1]);
+}
+
 // Value (r, n) of a GEMM result, partials added in ascending CTA order.
 __device__ __forceinline__ float gemm_load(const GemmOut &g, int r, int n) {
   const int t = n >> g.tile_shift, col = n - (t << g.tile_shift);

@@ -48,8 +48,8 @@ struct GemmRowsArgs {
 // MASKED: row r of tile column n is stored only where row_keep[r * keep_pitch + (n / 256) / keep_div] != 0 (rows that no
 //   consumer will read are skipped).
 // SWIGLU: W is a gate / up matrix ([2F, K]); a tile is w_rows gate rows and the up rows of the same outputs as the two blocks
-//   (fewer than 128 rows are loaded of each: the other lanes hold meaningless values that are never read back), every CTA owns
-//   whole tiles, and the epilogue writes silu(gate) * up as a bf16 hi / lo pair.
+//   (fewer than 128, or 64, rows are loaded of each: the other lanes hold meaningless values that are never read back; up to 64 rows the
+//   MMAs read 64, half the shared memory that bounds them at few activation rows), every CTA owns whole tiles, and the epilogue writes silu(gate) * up as a bf16 hi / lo pair.
 // SWIGLU with MASKED: a stack of keep_pitch such matrices (keep_div tiles each); times row_keep[r, block], exact zeros where it is zero.
 // GROUPED: a tile belongs to one group: group_tab holds, per group, the first weight row, the first weight k-block and the rows
 //   in use, and behind its keep_pitch entries the number of groups in use (the first ones); the CTAs take the tiles of those
@@ -81,6 +81,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   const int MT = SWIGLU ? 2 : a.tile_n >> 7;        // blocks of 128 weight rows per tile
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t w_box = (uint32_t)a.w_rows * GEMM_BLOCK_K * 2, w_bytes = (uint32_t)MT * w_box;
+  const bool m64 = SWIGLU && a.w_rows <= 64;        // MMAs of 64 weight rows: 16 of them in the first lanes of each quarter
   const int sw_fb = (SWIGLU && MASKED) ? N / (2 * a.keep_pitch) : N / 2;   // SWIGLU: gate rows of a matrix
   int n_pad = gemm_rows_padded(BN);                          // padded rows (of the launch; GROUPED: of the segment)
 
@@ -276,7 +277,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         if (!both) hv.next ^= 1;
         tc_fence_after();
         // kind::f16: D fp32 (bits 4-5 = 1), A and B bf16 (bits 7-9, 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_pad >> 2) << 17) | ((uint32_t)(128 >> 4) << 24);
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_pad >> 2) << 17) | ((uint32_t)((m64 ? 64 : 128) >> 4) << 24);
         const uint32_t d0 = tmem_base + mt_col(half, 0), d1 = tmem_base + mt_col(half, 1);
         uint32_t more = 0;
         for (int kb = kb_begin; kb < kb_end; ++kb) {
@@ -339,14 +340,14 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         return __ballot_sync(0xffffffffu, on) & 0xffu;
       };
       if (SWIGLU) {
-        // this thread's output f0 + lane_base + lane: gate sums in block 0, up sums in block 1, the same lane
+        // this thread's output: gate sums in block 0, up sums in block 1, the same lane
         const int blk = MASKED ? tile / a.keep_div : 0;
         const int f0 = (GROUPED ? g_j : MASKED ? tile - blk * a.keep_div : tile) * a.w_rows;
-        const int f = f0 + lane_base + lane, o_pitch = N / 2, col = blk * sw_fb + f;
-        const bool f_ok = lane_base + lane < a.w_rows && f < sw_fb;   // (F, the matrix and w_rows are multiples of 8: the same for both lanes of a pair)
+        const int w0 = m64 ? lane_base / 2 : lane_base, f = f0 + w0 + lane, o_pitch = N / 2, col = blk * sw_fb + f;   // w0: this warp's first weight row
+        const bool f_ok = w0 + lane < a.w_rows && f < sw_fb && (!m64 || lane < 16);   // (F, the matrix and w_rows are multiples of 8: the same for both lanes of a pair)
         const int row0 = GROUPED ? g_id * BN : 0;
         const uint32_t tg = t_lane + mt_col(half, 0), tu = t_lane + mt_col(half, 1);
-        if (lane_base < a.w_rows) {
+        if (w0 < a.w_rows) {
           for (int c = grp; c < chunks; c += 2) {
             uint32_t gh[8], gl[8], uh[8], ul[8];
             tmem_ld8(tg + (uint32_t)(8 * c), gh);

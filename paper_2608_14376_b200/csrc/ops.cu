@@ -173,13 +173,14 @@ qkv_post_few_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab,
   griddep_wait();
   const int head = blockIdx.x, r = blockIdx.y, i = threadIdx.x;
   const int hd = kv.hd, half = hd >> 1, nkv = kv.n_kv;
-  const int pos = rows.pos[r];
+  const int pos = rows.pos[r], slot = rows.slot[r];
   const bool active = rows.active[r] != 0;
-  if (head >= nq && !active) return;               // padding rows write no cache
   const int col = head * hd + i;                   // q, k and v heads are contiguous in the GEMM output
-  const float a = gemm_load(qkv, r, col), b = gemm_load(qkv, r, col + half);
+  const float2 ab = gemm_load_two(qkv, r, col, col + half);
+  const float2 t = rope_tab[(size_t)pos * half + i];     // (cos, sin); (a row without a request is at position 0)
+  if (head >= nq && !active) return;               // padding rows write no cache
+  const float a = ab.x, b = ab.y;
   if (head < nq) {
-    const float2 t = rope_tab[(size_t)pos * half + i];   // (cos, sin)
     float *q = q_out + (size_t)r * nq * hd + col;
     q[0] = a * t.x - b * t.y;
     q[half] = a * t.y + b * t.x;
@@ -191,7 +192,7 @@ qkv_post_few_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab,
     return;
   }
 #endif
-  const int blk = kv.block_table[(size_t)rows.slot[r] * kv.max_blocks + pos / KV_BLOCK];
+  const int blk = kv.block_table[(size_t)slot * kv.max_blocks + pos / KV_BLOCK];
 #ifdef CORUN_CHECKED
   if (!check_page(blk, kv.pool_blocks)) {
     atomicCAS(status, 0, DEV_BAD_INDEX);
@@ -201,7 +202,6 @@ qkv_post_few_kernel(GemmOut qkv, Rows rows, const float2 *__restrict__ rope_tab,
   __half *page = kv.pool + (size_t)layer * kv.layer_stride + (size_t)blk * 2 * nkv * KV_BLOCK * hd;
   const int tok = pos % KV_BLOCK;
   if (head < nq + nkv) {
-    const float2 t = rope_tab[(size_t)pos * half + i];
     const int g = head - nq;
     page[kv_k_off(hd, g, tok, i)] = __float2half_rn(a * t.x - b * t.y);
     page[kv_k_off(hd, g, tok, i + half)] = __float2half_rn(a * t.y + b * t.x);
