@@ -60,45 +60,32 @@ __device__ __forceinline__ void split_half(float x, __half &hi, __half &lo) {
   lo = __float2half_rn(x - __half2float(hi));
 }
 
-// Combines the splits of one (row, head) by one warp.  Lanes first hold one split each (max by
+// Combines the splits of 64 output dims (the d0-th and on) of one (row, head) by one warp.  Lanes first hold one split each (max by
 // butterfly, which is exact; the denominator by a fixed butterfly over at most 32 lanes, then
-// ascending chunks of 32), then every lane owns hd/32 output dims and adds the splits' weighted
-// partial outputs in ascending split order.  Output: bf16 hi/lo pair for the O projection.
+// ascending chunks of 32), then every lane owns two output dims and adds the splits' weighted
+// partial outputs in ascending split order, 32 of them in flight.  Output: bf16 hi/lo pair for the O projection.
 // The partials may come from other SMs: they are read past the L1 cache.
 template <int HD>
-__device__ __forceinline__ void attn_combine_pair(int r, int j, int nsplit, int nq, int max_splits,
+__device__ __forceinline__ void attn_combine_pair(int r, int j, int d0, int nsplit, int nq, int max_splits,
                                                   const float *__restrict__ part_acc, const float *__restrict__ part_ml,
                                                   __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo,
                                                   int lane) {
-  constexpr int DPL = HD / 32;                   // dims per lane (4 or 2)
-  float o[DPL];
-#pragma unroll
-  for (int i = 0; i < DPL; ++i) o[i] = 0.f;
+  constexpr int FLY = 32;                        // partial outputs in flight
+  float o[2] = {0.f, 0.f};
   const float2 *ml = reinterpret_cast<const float2 *>(part_ml) + ((size_t)r * nq + j) * max_splits;
-  const float *pa = part_acc + ((size_t)r * nq + j) * max_splits * HD + lane * DPL;
-  auto load_acc = [&](int s) -> float4 {
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (s < nsplit) {
-      const float *p = pa + (size_t)s * HD;
-      if (DPL == 4) a = __ldcg(reinterpret_cast<const float4 *>(p));
-      else { const float2 t = __ldcg(reinterpret_cast<const float2 *>(p)); a.x = t.x; a.y = t.y; }
-    }
-    return a;
-  };
-  auto add_acc = [&](const float4 &a, float ws) {
-    o[0] = fmaf(a.x, ws, o[0]); o[1] = fmaf(a.y, ws, o[1]);
-    if (DPL == 4) { o[DPL - 2] = fmaf(a.z, ws, o[DPL - 2]); o[DPL - 1] = fmaf(a.w, ws, o[DPL - 1]); }
-  };
+  const float *pa = part_acc + ((size_t)r * nq + j) * max_splits * HD + d0 + lane * 2;
+  auto load_acc = [&](int s) { return s < nsplit ? __ldcg(reinterpret_cast<const float2 *>(pa + (size_t)s * HD)) : make_float2(0.f, 0.f); };
+  auto add_acc = [&](const float2 &a, float ws) { o[0] = fmaf(a.x, ws, o[0]); o[1] = fmaf(a.y, ws, o[1]); };
   float den = 0.f;
   if (nsplit <= 64) {
     // usual case: the (max, sum) pairs of all splits sit in two registers per lane, and the first
-    // sixteen partial outputs are requested before anything depends on them
+    // partial outputs are requested before anything depends on them
     const float2 none = make_float2(-CUDART_INF_F, 0.f);
     const float2 v0 = lane < nsplit ? __ldcg(ml + lane) : none;
     const float2 v1 = 32 + lane < nsplit ? __ldcg(ml + 32 + lane) : none;
-    float4 a[16];
+    float2 a[FLY];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) a[u] = load_acc(u);
+    for (int u = 0; u < FLY; ++u) a[u] = load_acc(u);
     float M = fmaxf(v0.x, v1.x);
 #pragma unroll
     for (int k = 16; k > 0; k >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, k));
@@ -110,13 +97,13 @@ __device__ __forceinline__ void attn_combine_pair(int r, int j, int nsplit, int 
       d1 += __shfl_xor_sync(0xffffffffu, d1, k);
     }
     den = nsplit > 32 ? d0 + d1 : d0;
-    for (int sb = 0; sb < nsplit; sb += 16) {
+    for (int sb = 0; sb < nsplit; sb += FLY) {
       if (sb > 0) {
 #pragma unroll
-        for (int u = 0; u < 16; ++u) a[u] = load_acc(sb + u);
+        for (int u = 0; u < FLY; ++u) a[u] = load_acc(sb + u);
       }
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         const int sidx = sb + u;
         const float ws = __shfl_sync(0xffffffffu, sidx < 32 ? w0 : w1, sidx & 31);
         add_acc(a[u], ws);                         // beyond the last split: 0 * 0
@@ -139,23 +126,20 @@ __device__ __forceinline__ void attn_combine_pair(int r, int j, int nsplit, int 
       den += d;
       const int cnt = min(32, nsplit - s0);
       for (int sb = 0; sb < cnt; sb += 8) {          // eight splits' partial outputs are fetched together
-        float4 a[8];
+        float2 a[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] = sb + u < cnt ? load_acc(s0 + sb + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = 0; u < 8; ++u) a[u] = sb + u < cnt ? load_acc(s0 + sb + u) : make_float2(0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < 8; ++u) add_acc(a[u], __shfl_sync(0xffffffffu, w, (sb + u) & 31));
       }
     }
   }
-#pragma unroll
-  for (int i = 0; i < DPL; ++i) o[i] = o[i] / den;
-  const size_t idx = (size_t)r * nq * HD + (size_t)j * HD + lane * DPL;
-#pragma unroll
-  for (int i = 0; i < DPL; ++i) {
-    const __nv_bfloat16 a = __float2bfloat16_rn(o[i]);
-    out_hi[idx + i] = a;
-    out_lo[idx + i] = __float2bfloat16_rn(o[i] - __bfloat162float(a));
-  }
+  const float y0 = o[0] / den, y1 = o[1] / den;
+  const size_t idx = (size_t)r * nq * HD + (size_t)j * HD + d0 + lane * 2;
+  const __nv_bfloat16 h0 = __float2bfloat16_rn(y0), h1 = __float2bfloat16_rn(y1);
+  *reinterpret_cast<__nv_bfloat162 *>(out_hi + idx) = __halves2bfloat162(h0, h1);
+  *reinterpret_cast<__nv_bfloat162 *>(out_lo + idx) =
+      __halves2bfloat162(__float2bfloat16_rn(y0 - __bfloat162float(h0)), __float2bfloat16_rn(y1 - __bfloat162float(h1)));
 }
 
 template <int HD>
@@ -595,7 +579,7 @@ __global__ void __launch_bounds__(256) attn_worklist_kernel(Rows rows, int n_kv,
   }
 }
 
-// One warp per (row, query head): adds the row's split partials in ascending split order -> bf16 hi/lo.
+// One warp per (row, query head) and 64 dims: adds the row's split partials in ascending split order -> bf16 hi/lo.
 template <int HD>
 __global__ void __launch_bounds__(128) attn_combine_kernel(Rows rows, int nq, int max_splits,
                                                            const float *__restrict__ part_acc,
@@ -604,12 +588,13 @@ __global__ void __launch_bounds__(128) attn_combine_kernel(Rows rows, int nq, in
                                                            __nv_bfloat16 *__restrict__ out_lo) {
   griddep_launch_dependents();
   griddep_wait();
-  const int w = (int)blockIdx.x * 4 + ((int)threadIdx.x >> 5);
+  constexpr int PARTS = HD / 64;
+  const int u = (int)blockIdx.x * 4 + ((int)threadIdx.x >> 5), w = u / PARTS;
   if (w >= rows.R * nq) return;
   const int r = w / nq, j = w - r * nq;
   if (!rows.active[r]) return;                     // padding rows keep what they held
   const int ns = (rows.pos[r] + 1 + ATT_SPLIT - 1) / ATT_SPLIT;
-  attn_combine_pair<HD>(r, j, ns, nq, max_splits, part_acc, part_ml, out_hi, out_lo, (int)threadIdx.x & 31);
+  attn_combine_pair<HD>(r, j, (u % PARTS) * 64, ns, nq, max_splits, part_acc, part_ml, out_hi, out_lo, (int)threadIdx.x & 31);
 }
 
 }  // namespace
@@ -696,7 +681,7 @@ cudaError_t launch_attention(const CUtensorMap &tmK, const CUtensorMap &tmV, con
   const int whole_pairs = reuse == 2;   // the ablation: the item list carries the pair table
   const long long most = (long long)rows.R * max_splits * kv.n_kv;
   const int grid = (int)(most < grid_ctas ? most : grid_ctas);
-  const int cgrid = (rows.R * nq + 3) / 4;
+  const int cgrid = (rows.R * nq * (kv.hd / 64) + 3) / 4;
   cudaError_t ce = cudaErrorInvalidValue;
   if (kv.hd == 128) {
     ce = launch_attn_split<128>(group, grid, st, tmK, tmV, q, rows, nq, kv, max_splits, work, n_work, part_acc, part_ml,

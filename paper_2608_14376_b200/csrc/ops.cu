@@ -47,8 +47,10 @@ resid_norm_kernel(float *__restrict__ h, int H, const __nv_bfloat16 *__restrict_
   griddep_launch_dependents();
   uint2 gain0 = make_uint2(0u, 0u);
   if (4 * threadIdx.x < H) gain0 = __ldg(reinterpret_cast<const uint2 *>(gains + 4 * threadIdx.x));
+  __shared__ __align__(16) float scratch[NORM_MAX_THREADS / 32];   // (warps that there are not: zero)
+  if (threadIdx.x < NORM_MAX_THREADS / 32) scratch[threadIdx.x] = 0.f;
+  __syncthreads();
   griddep_wait();
-  __shared__ float scratch[NORM_MAX_THREADS / 32];
   const int r = blockIdx.x;
   float *hr = h + (size_t)r * H;
   float ss = 0.f;
@@ -76,11 +78,15 @@ resid_norm_kernel(float *__restrict__ h, int H, const __nv_bfloat16 *__restrict_
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) scratch[warp] = ss;
   __syncthreads();
   float tot = 0.f;
-  for (int w = 0; w < nwarps; ++w) tot += scratch[w];
+  float4 part[NORM_MAX_THREADS / 128];               // (all loads in flight: one by one the 32 totals took half a microsecond)
+#pragma unroll
+  for (int w = 0; w < NORM_MAX_THREADS / 128; ++w) part[w] = reinterpret_cast<const float4 *>(scratch)[w];
+#pragma unroll
+  for (int w = 0; w < NORM_MAX_THREADS / 128; ++w) { tot += part[w].x; tot += part[w].y; tot += part[w].z; tot += part[w].w; }
   const float inv = rsqrtf(tot / (float)H + eps);
   for (int i = threadIdx.x * 4; i < H; i += blockDim.x * 4) {
     float4 x = x0;
