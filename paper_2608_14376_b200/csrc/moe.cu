@@ -529,41 +529,46 @@ __global__ void __launch_bounds__(256) moe_combine_select_kernel(const float *__
   if (any) *reinterpret_cast<float4 *>(y + (size_t)r * H + i) = acc;
 }
 
-__global__ void __launch_bounds__(256) moe_combine_kernel(const float *__restrict__ yg, const int *__restrict__ active, int NB,
+// One CTA per row: every expert's slot of the row is looked up by a thread of its own, then a thread adds four columns, eight experts'
+// loads in flight.  Bound by the experts' rows (2505 rows of 2048 columns, 8 experts each: 164 MB).  With 256 threads (two CTAs a row,
+// one warp walking the experts) 49.6 us, so 42.0; 1003 rows 18.7 and 16.1.
+constexpr int COMBINE_THREADS = 512;
+__global__ void __launch_bounds__(COMBINE_THREADS) moe_combine_kernel(const float *__restrict__ yg, const int *__restrict__ active, int NB,
                                                           int H, MoeGroups g, float *__restrict__ y) {
   griddep_launch_dependents();
   griddep_wait();
   yg = after_wait(yg); active = after_wait(active);
-  const int r = blockIdx.y;
+  const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (!active[r]) return;
   __shared__ int slots[MOE_MAX_EXPERTS + 8];         // the row's slots, experts ascending (shared experts last), compacted
-  __shared__ int n_sel;
-  if (threadIdx.x < 32) {
-    int n = 0;
-    for (int e0 = 0; e0 < NB; e0 += 32) {
-      const int e = e0 + (int)threadIdx.x;
-      const int slot = e < NB ? g.slot_of[(size_t)e * gridDim.y + r] : -1;
-      const unsigned m = __ballot_sync(0xffffffffu, slot >= 0);
-      if (slot >= 0) slots[n + __popc(m & ((1u << threadIdx.x) - 1u))] = slot;
-      n += __popc(m);
-    }
-    if (threadIdx.x == 0) n_sel = n;
-  }
+  __shared__ int cnt[COMBINE_THREADS / 32];
+  static_assert(MOE_MAX_EXPERTS + 8 <= COMBINE_THREADS, "a thread per expert");
+  const int slot = tid < NB ? g.slot_of[(size_t)tid * gridDim.x + r] : -1;
+  const unsigned m = __ballot_sync(0xffffffffu, slot >= 0);
+  if (lane == 0) cnt[warp] = __popc(m);
   __syncthreads();
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (i >= H) return;
-  const int n = n_sel;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int k0 = 0; k0 < n; k0 += 8) {                // eight loads in flight; the additions stay in ascending order
-    float4 v[8];
+  int before = 0, n = 0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k0 + k < n) v[k] = *reinterpret_cast<const float4 *>(yg + (size_t)slots[k0 + k] * H + i);
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k0 + k < n) { acc.x += v[k].x; acc.y += v[k].y; acc.z += v[k].z; acc.w += v[k].w; }
+  for (int k = 0; k < COMBINE_THREADS / 32; ++k) {
+    const int c = cnt[k];
+    if (k < warp) before += c;
+    n += c;
   }
-  *reinterpret_cast<float4 *>(y + (size_t)r * H + i) = acc;
+  if (slot >= 0) slots[before + __popc(m & ((1u << lane) - 1u))] = slot;
+  __syncthreads();
+  for (int i = 4 * tid; i < H; i += 4 * COMBINE_THREADS) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = 0; k0 < n; k0 += 8) {              // eight loads in flight; the additions stay in ascending order
+      float4 v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k0 + k < n) v[k] = *reinterpret_cast<const float4 *>(yg + (size_t)slots[k0 + k] * H + i);
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k0 + k < n) { acc.x += v[k].x; acc.y += v[k].y; acc.z += v[k].z; acc.w += v[k].w; }
+    }
+    *reinterpret_cast<float4 *>(y + (size_t)r * H + i) = acc;
+  }
 }
 
 }  // namespace
@@ -602,7 +607,7 @@ cudaError_t launch_moe_swiglu_grouped(const float *gu, const float *w, int n_blo
 
 cudaError_t launch_moe_combine(const float *yg, const int *active, int R, int n_blocks, int H, const MoeGroups &g, float *y,
                                cudaStream_t st) {
-  return launch_k(moe_combine_kernel, dim3((H / 4 + 255) / 256, R), dim3(256), 0, st, true, yg, active, n_blocks, H, g, y);
+  return launch_k(moe_combine_kernel, dim3(R), dim3(COMBINE_THREADS), 0, st, true, yg, active, n_blocks, H, g, y);
 }
 
 cudaError_t moe_router_prepare() {
