@@ -21,14 +21,13 @@ namespace corun {
 
 namespace {
 
-constexpr int ML_THREADS = 320;                     // warp 0 TMA, warp 1 MMA, warps 2-5 softmax, warps 6-9 output
+constexpr int ML_THREADS = 352;                     // warp 0 TMA of the keys, warp 1 MMA, warps 2-5 softmax, warps 6-9 output, warp 10 TMA of the values
 constexpr int ML_KEYS = 64;                         // keys per block
 constexpr uint32_t ML_BOX = ML_KEYS * 128;          // [64 tokens x 64 dims] fp16
 constexpr uint32_t ML_Q_BYTES = 3 * 128 * 128;      // hi or lo: [3 blocks of 64 dims][128 rows x 128 B]
 constexpr uint32_t ML_K_BYTES = 5 * ML_BOX;         // hi, lo of the 128 no-rope dims, the rotary key
 constexpr uint32_t ML_V_BYTES = 4 * ML_BOX;         // hi, lo
-constexpr uint32_t ML_P_BYTES = 128 * 128;          // hi or lo of a weight tile [128 rows x 64 keys]
-constexpr size_t ML_SMEM = 1024 + 2 * ML_Q_BYTES + ML_K_BYTES + ML_V_BYTES + 2 * ML_P_BYTES;
+constexpr size_t ML_SMEM = 1024 + 2 * ML_Q_BYTES + 2 * ML_K_BYTES + ML_V_BYTES;
 
 __device__ __forceinline__ uint32_t ml_swz(int row, int chunk) { return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4)); }
 __device__ __forceinline__ float ml_ex2(float x) {
@@ -115,24 +114,25 @@ mla_gather_kernel(const __grid_constant__ MlaSegs g, MlaCache cache, int rank, i
 
 // One CTA per (head, tile of 128 chunk rows = consecutive tokens of one request).  Per block of 64 keys:
 //   S[128 x 64] = Qhi Khi + Qlo Khi + Qhi Klo (12 k-slices) into one of two TMEM buffers;
-//   softmax warps, a thread per row: running maximum, P = exp2(S - max) as an fp16 hi / lo tile, the factor by which the
-//     earlier sums shrink;
-//   O'[128 x 128] = Phi Vhi + Plo Vhi + Phi Vlo (4 k-slices) into one of two TMEM buffers;
+//   softmax warps, a thread per row: running maximum, P = exp2(S - max) as fp16 hi and lo in the scores' own columns, the factor by
+//     which the earlier sums shrink;
+//   O'[128 x 128] = Phi Vhi + Plo Vhi + Phi Vlo (4 k-slices), P from tensor memory, into one of two TMEM buffers;
 //   output warps, a thread per row: O = O * factor + O', in registers.
-// The scores of block j + 1 are issued ahead of the values of block j, so the tensor cores work while the rows do.  What
-// bounds a CTA is the number of MMA instructions (44 per block) and, with one key buffer, the 40 KB of keys per block that
-// can only be requested once the scores before them are done.  Every reduction runs in one fixed order that depends on the
-// row's own position only.  All waits are bounded.
+// The tensor pipe works in the order of issue: scores of block j + 2 after the values of block j, whose weights they overwrite; the
+// keys of two blocks are in shared memory.  (One key buffer, weights through shared memory and one producer for keys and values, so that
+// a block's keys were requested behind the values before them, and queries and results by a thread per row: 2505 tokens of 16 heads
+// 160 us per layer, now 125.)  What bounds a block are its 32 MMAs of 48 and 12 of 64 cycles.
+// Every reduction runs in one fixed order that depends on the row's own position only.  All waits are bounded.
 __global__ void __launch_bounds__(ML_THREADS, 1)
 mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmR, const __nv_bfloat16 *__restrict__ qn_hi,
                    const __nv_bfloat16 *__restrict__ qn_lo, const float *__restrict__ q_rope, Rows rows, int rows_per_head, int nh, int rope,
                    int cap, const int *__restrict__ tile_base, float scale_log2e, const float2 *__restrict__ kv_scale, __nv_bfloat16 *__restrict__ ao_hi,
                    __nv_bfloat16 *__restrict__ ao_lo, int *status) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t kfull, kempty, vfull, vempty, s_full[2], s_free[2], p_ready, p_free, o_full[2], o_free[2], c_ready[4], l_ready;
+  __shared__ __align__(8) uint64_t kfull[2], kempty[2], vfull, vempty, s_full[2], p_ready[2], o_full[2], o_free[2], c_ready[4], l_ready;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
-  __shared__ float corr_s[4][128], l_s[128], row_scale_s[128], q_most[2][128];
+  __shared__ float corr_s[4][128], l_s[128], row_scale_s[128];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int h = blockIdx.x, tile = (int)gridDim.y - 1 - (int)blockIdx.y;   // the last tiles (the most keys) first
   const int row0 = tile * 128;
@@ -143,16 +143,14 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
   const int n_blocks = rows.pos[row0 + n_rows - 1] / ML_KEYS + 1, base_tok = tile_base[tile];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t q_hi = base, q_lo = base + ML_Q_BYTES, k_buf = q_lo + ML_Q_BYTES, v_buf = k_buf + ML_K_BYTES, p_hi = v_buf + ML_V_BYTES,
-                 p_lo = p_hi + ML_P_BYTES;
+  const uint32_t q_hi = base, q_lo = base + ML_Q_BYTES, k_ring = q_lo + ML_Q_BYTES, v_buf = k_ring + 2 * ML_K_BYTES;
   if (tid == 0) {
     abort_flag = 0;
-    mbar_init(smem_u32(&kfull), 1); mbar_init(smem_u32(&kempty), 1);
     mbar_init(smem_u32(&vfull), 1); mbar_init(smem_u32(&vempty), 1);
-    mbar_init(smem_u32(&p_ready), 128); mbar_init(smem_u32(&p_free), 1);
     mbar_init(smem_u32(&l_ready), 128);
     for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(&s_full[i]), 1); mbar_init(smem_u32(&s_free[i]), 128);
+      mbar_init(smem_u32(&kfull[i]), 1); mbar_init(smem_u32(&kempty[i]), 1);
+      mbar_init(smem_u32(&s_full[i]), 1); mbar_init(smem_u32(&p_ready[i]), 128);
       mbar_init(smem_u32(&o_full[i]), 1); mbar_init(smem_u32(&o_free[i]), 128);
     }
     for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&c_ready[i]), 128);
@@ -165,46 +163,51 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
     tmem_alloc(smem_u32(&tmem_base_s), 512);        // scores 2 x 64 columns, outputs 2 x 128
     tmem_relinquish();
   }
-  if (warp >= 2) {
-    // the query tile: row m = token m, 24 chunks of 8 dims (128 no-rope, then the rotary ones, zeros beyond them)
-    const int m = (tid - 64) & 127, r = row0 + m, part = (tid - 64) >> 7;
-    const bool on = r < rows.R;
-    float all[12][8], most = 0.f;                   // every other chunk; the rotary ones at the scale of the keys beside theirs
+  if (warp >= 2 && warp < 10) {
+    // the query tile: row m = token m, 128 no-rope dims (four per lane), then the rotary ones (two per lane), zeros beyond them: a
+    // warp takes a row at a time, four in flight
+    for (int m0 = warp - 2; m0 < 128; m0 += 32) {
+      uint2 a[4], b[4];
+      float2 p[4];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const int c = part + 2 * k;
-      float *x = all[k];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = 0.f;
-      if (on && c < 16) {
-        const size_t o = ((size_t)h * rows_per_head + r) * 128 + 8 * c;
-        const uint4 a = *reinterpret_cast<const uint4 *>(qn_hi + o), b = *reinterpret_cast<const uint4 *>(qn_lo + o);
-        const __nv_bfloat16 *pa = reinterpret_cast<const __nv_bfloat16 *>(&a), *pb = reinterpret_cast<const __nv_bfloat16 *>(&b);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = __bfloat162float(pa[i]) + __bfloat162float(pb[i]);
-      } else if (on && 8 * (c - 16) < rope) {
-        const float *q = q_rope + ((size_t)r * nh + h) * rope + 8 * (c - 16);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = q[i] * kvs.x;
+      for (int k = 0; k < 4; ++k) {
+        const int r = row0 + m0 + 8 * k;
+        const bool on = r < rows.R;
+        const size_t o = ((size_t)h * rows_per_head + r) * 128 + 4 * lane;
+        a[k] = on ? *reinterpret_cast<const uint2 *>(qn_hi + o) : make_uint2(0u, 0u);
+        b[k] = on ? *reinterpret_cast<const uint2 *>(qn_lo + o) : make_uint2(0u, 0u);
+        p[k] = on && 2 * lane < rope ? *reinterpret_cast<const float2 *>(q_rope + ((size_t)r * nh + h) * rope + 2 * lane) : make_float2(0.f, 0.f);
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) most = fmaxf(most, fabsf(x[i]));
-    }
-    q_most[part][m] = most;
-    asm volatile("bar.sync 1, 256;" ::: "memory");   // warps 2-9
-    const float q_scale = ml_pow2_below(fmaxf(q_most[0][m], q_most[1][m]), 14);
-    if (part == 0) row_scale_s[m] = scale_log2e / q_scale / kvs.x;
+      for (int k = 0; k < 4; ++k) {
+        const int m = m0 + 8 * k;
+        const __nv_bfloat16 *pa = reinterpret_cast<const __nv_bfloat16 *>(&a[k]), *pb = reinterpret_cast<const __nv_bfloat16 *>(&b[k]);
+        float x[6], most = 0.f;                     // the rotary ones at the scale of the keys beside theirs
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const int c = part + 2 * k;
-      float *x = all[k];
+        for (int i = 0; i < 4; ++i) x[i] = __bfloat162float(pa[i]) + __bfloat162float(pb[i]);
+        x[4] = p[k].x * kvs.x;
+        x[5] = p[k].y * kvs.x;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] *= q_scale;
-      uint4 hi, lo;
-      ml_split8(x, hi, lo);
-      const uint32_t off = (uint32_t)(c >> 3) * (128 * 128) + ml_swz(m, c & 7);
-      *reinterpret_cast<uint4 *>(base_ptr + off) = hi;
-      *reinterpret_cast<uint4 *>(base_ptr + ML_Q_BYTES + off) = lo;
+        for (int i = 0; i < 6; ++i) most = fmaxf(most, fabsf(x[i]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
+        const float q_scale = ml_pow2_below(most, 14);
+        if (lane == 0) row_scale_s[m] = scale_log2e / q_scale / kvs.x;
+        __half hi[6], lo[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          const float y = x[i] * q_scale;
+          hi[i] = __float2half_rn(y);
+          lo[i] = __float2half_rn(y - __half2float(hi[i]));
+        }
+        const uint32_t on = (uint32_t)(lane >> 4) * (128 * 128) + ml_swz(m, (lane & 15) >> 1) + (uint32_t)(lane & 1) * 8;
+        const uint32_t orr = 2u * (128 * 128) + ml_swz(m, lane >> 2) + (uint32_t)(lane & 3) * 4;
+        const __half2 h01 = __halves2half2(hi[0], hi[1]), h23 = __halves2half2(hi[2], hi[3]), l01 = __halves2half2(lo[0], lo[1]), l23 = __halves2half2(lo[2], lo[3]);
+        *reinterpret_cast<uint2 *>(base_ptr + on) = make_uint2(*reinterpret_cast<const uint32_t *>(&h01), *reinterpret_cast<const uint32_t *>(&h23));
+        *reinterpret_cast<uint2 *>(base_ptr + ML_Q_BYTES + on) = make_uint2(*reinterpret_cast<const uint32_t *>(&l01), *reinterpret_cast<const uint32_t *>(&l23));
+        *reinterpret_cast<__half2 *>(base_ptr + orr) = __halves2half2(hi[4], hi[5]);
+        *reinterpret_cast<__half2 *>(base_ptr + ML_Q_BYTES + orr) = __halves2half2(lo[4], lo[5]);
+      }
     }
     fence_proxy_async();                            // the MMAs read these tiles through the async proxy
   }
@@ -217,22 +220,25 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
   const int quad = warp & 3, tl = quad * 32 + lane;
   const bool real = tl < n_rows;
 
-  if (warp == 0) {
+  if (warp == 0 || warp == 10) {
     if (elect_one()) {
-      // ---------------- TMA producer ----------------
+      // ---------------- TMA producers ----------------
       const uint64_t pol = l2_policy_evict_last();  // the tiles of the same head read the same keys and values
       for (int j = 0; j < n_blocks && !failed; ++j) {
-        const int tok = base_tok + j * ML_KEYS;
+        const int tok = base_tok + j * ML_KEYS, kb = j & 1;
         auto y = [&](int part) { return (part * nh + h) * cap + tok; };   // part: key hi, key lo, value hi, value lo
-        if (j > 0 && !mbar_wait(smem_u32(&kempty), (uint32_t)(j - 1) & 1u, &abort_flag)) { failed = true; break; }
-        mbar_arrive_expect_tx(smem_u32(&kfull), ML_K_BYTES);
-        for (int i = 0; i < 4; ++i)
-          tma_load_2d(k_buf + (uint32_t)i * ML_BOX, &tmKV, (i & 1) * 64, y(i >> 1), smem_u32(&kfull), pol);
-        tma_load_2d(k_buf + 4 * ML_BOX, &tmR, 0, tok, smem_u32(&kfull), pol);
-        if (j > 0 && !mbar_wait(smem_u32(&vempty), (uint32_t)(j - 1) & 1u, &abort_flag)) { failed = true; break; }
-        mbar_arrive_expect_tx(smem_u32(&vfull), ML_V_BYTES);
-        for (int i = 0; i < 4; ++i)
-          tma_load_2d(v_buf + (uint32_t)i * ML_BOX, &tmKV, (i & 1) * 64, y(2 + (i >> 1)), smem_u32(&vfull), pol);
+        if (warp == 0) {
+          const uint32_t fb = smem_u32(&kfull[kb]), dst = k_ring + (uint32_t)kb * ML_K_BYTES;
+          if (j > 1 && !mbar_wait(smem_u32(&kempty[kb]), (uint32_t)((j >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
+          mbar_arrive_expect_tx(fb, ML_K_BYTES);
+          for (int i = 0; i < 4; ++i) tma_load_2d(dst + (uint32_t)i * ML_BOX, &tmKV, (i & 1) * 64, y(i >> 1), fb, pol);
+          tma_load_2d(dst + 4 * ML_BOX, &tmR, 0, tok, fb, pol);
+        } else {
+          if (j > 0 && !mbar_wait(smem_u32(&vempty), (uint32_t)(j - 1) & 1u, &abort_flag)) { failed = true; break; }
+          mbar_arrive_expect_tx(smem_u32(&vfull), ML_V_BYTES);
+          for (int i = 0; i < 4; ++i)
+            tma_load_2d(v_buf + (uint32_t)i * ML_BOX, &tmKV, (i & 1) * 64, y(2 + (i >> 1)), smem_u32(&vfull), pol);
+        }
       }
     }
   } else if (warp == 1) {
@@ -240,47 +246,46 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
       // ---------------- MMA issuer ----------------
       const uint32_t idesc_s = (1u << 4) | ((uint32_t)(ML_KEYS >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t idesc_o = (1u << 4) | (1u << 16) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);   // values MN-major
-      for (int j = 0; j <= n_blocks && !failed; ++j) {
-        if (j < n_blocks) {
-          const int sb = j & 1;
-          if (j >= 2 && !mbar_wait(smem_u32(&s_free[sb]), (uint32_t)((j >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
-          if (!mbar_wait(smem_u32(&kfull), (uint32_t)j & 1u, &abort_flag)) { failed = true; break; }
-          tc_fence_after();
-          const uint32_t d = tmem + (uint32_t)sb * 64;
+      auto scores = [&](int j) {
+        const int sb = j & 1;
+        if (!mbar_wait(smem_u32(&kfull[sb]), (uint32_t)(j >> 1) & 1u, &abort_flag)) { failed = true; return; }
+        tc_fence_after();
+        const uint32_t d = tmem + (uint32_t)sb * 64, k_buf = k_ring + (uint32_t)sb * ML_K_BYTES;
 #pragma unroll
-          for (int ks = 0; ks < 12; ++ks) {
-            const uint64_t adv = (uint64_t)((ks & 3) * 2);
-            const uint32_t b = (uint32_t)(ks >> 2);
-            const uint64_t qh = umma_desc_sw128(q_hi + b * (128 * 128)) + adv, ql = umma_desc_sw128(q_lo + b * (128 * 128)) + adv;
-            const uint64_t kh = umma_desc_sw128(k_buf + (ks < 8 ? b : 4u) * ML_BOX) + adv;
-            umma_bf16(d, qh, kh, idesc_s, ks > 0 ? 1u : 0u);   // operand format (fp16) is in idesc
-            umma_bf16(d, ql, kh, idesc_s, 1u);
-            if (ks < 8) umma_bf16(d, qh, umma_desc_sw128(k_buf + (2 + b) * ML_BOX) + adv, idesc_s, 1u);   // (the rotary key is fp16 as cached)
-          }
-          umma_commit(smem_u32(&kempty));
-          umma_commit(smem_u32(&s_full[sb]));
+        for (int ks = 0; ks < 12; ++ks) {
+          const uint64_t adv = (uint64_t)((ks & 3) * 2);
+          const uint32_t b = (uint32_t)(ks >> 2);
+          const uint64_t qh = umma_desc_sw128(q_hi + b * (128 * 128)) + adv, ql = umma_desc_sw128(q_lo + b * (128 * 128)) + adv;
+          const uint64_t kh = umma_desc_sw128(k_buf + (ks < 8 ? b : 4u) * ML_BOX) + adv;
+          umma_bf16(d, qh, kh, idesc_s, ks > 0 ? 1u : 0u);   // operand format (fp16) is in idesc
+          umma_bf16(d, ql, kh, idesc_s, 1u);
+          if (ks < 8) umma_bf16(d, qh, umma_desc_sw128(k_buf + (2 + b) * ML_BOX) + adv, idesc_s, 1u);   // (the rotary key is fp16 as cached)
         }
-        if (j >= 1) {
-          const int i = j - 1, ob = i & 1;
-          if (!mbar_wait(smem_u32(&p_ready), (uint32_t)i & 1u, &abort_flag)) { failed = true; break; }
-          if (!mbar_wait(smem_u32(&vfull), (uint32_t)i & 1u, &abort_flag)) { failed = true; break; }
-          if (i >= 2 && !mbar_wait(smem_u32(&o_free[ob]), (uint32_t)((i >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
-          tc_fence_after();
-          const uint32_t d = tmem + 128 + (uint32_t)ob * 128;
+        umma_commit(smem_u32(&kempty[sb]));
+        umma_commit(smem_u32(&s_full[sb]));
+      };
+      scores(0);
+      if (n_blocks > 1 && !failed) scores(1);
+      for (int j = 0; j < n_blocks && !failed; ++j) {
+        const int b = j & 1;
+        if (!mbar_wait(smem_u32(&p_ready[b]), (uint32_t)(j >> 1) & 1u, &abort_flag)) { failed = true; break; }
+        if (!mbar_wait(smem_u32(&vfull), (uint32_t)j & 1u, &abort_flag)) { failed = true; break; }
+        if (j >= 2 && !mbar_wait(smem_u32(&o_free[b]), (uint32_t)((j >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
+        tc_fence_after();
+        const uint32_t p = tmem + (uint32_t)b * 64, d = tmem + 128 + (uint32_t)b * 128;
 #pragma unroll
-          for (int ks = 0; ks < ML_KEYS / 16; ++ks) {
-            const uint64_t ph = umma_desc_sw128(p_hi) + (uint64_t)(ks * 2), pl = umma_desc_sw128(p_lo) + (uint64_t)(ks * 2);
-            // values [128 dims x 16 tokens], MN-major: blocks of 64 dims a box apart, groups of 8 tokens 1 KiB apart
-            const uint64_t vh = umma_desc_sw128_mn(v_buf + (uint32_t)ks * 2048, ML_BOX, 1024u);
-            const uint64_t vl = umma_desc_sw128_mn(v_buf + 2 * ML_BOX + (uint32_t)ks * 2048, ML_BOX, 1024u);
-            umma_bf16(d, ph, vh, idesc_o, ks > 0 ? 1u : 0u);
-            umma_bf16(d, pl, vh, idesc_o, 1u);
-            umma_bf16(d, ph, vl, idesc_o, 1u);
-          }
-          umma_commit(smem_u32(&vempty));
-          umma_commit(smem_u32(&p_free));
-          umma_commit(smem_u32(&o_full[ob]));
+        for (int ks = 0; ks < ML_KEYS / 16; ++ks) {
+          const uint32_t ph = p + (uint32_t)(8 * ks), pl = ph + 32;   // 16 tokens of weights are 8 columns
+          // values [128 dims x 16 tokens], MN-major: blocks of 64 dims a box apart, groups of 8 tokens 1 KiB apart
+          const uint64_t vh = umma_desc_sw128_mn(v_buf + (uint32_t)ks * 2048, ML_BOX, 1024u);
+          const uint64_t vl = umma_desc_sw128_mn(v_buf + 2 * ML_BOX + (uint32_t)ks * 2048, ML_BOX, 1024u);
+          umma_f16_ts(d, ph, vh, idesc_o, ks > 0 ? 1u : 0u);
+          umma_f16_ts(d, pl, vh, idesc_o, 1u);
+          umma_f16_ts(d, ph, vl, idesc_o, 1u);
         }
+        umma_commit(smem_u32(&vempty));
+        umma_commit(smem_u32(&o_full[b]));
+        if (j + 2 < n_blocks) scores(j + 2);
       }
     }
   } else if (warp < 6) {
@@ -298,18 +303,11 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
 #pragma unroll
       for (int x = 0; x < 4; ++x) tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(sb * 64 + 16 * x), sv[x]);
       tmem_ld_wait();
-      tc_fence_before();
-      mbar_arrive(smem_u32(&s_free[sb]));
       const int lim = pos - j * ML_KEYS;            // keys 0 .. lim of the block are visible
-      float bm = -CUDART_INF_F;
-      if (lim >= ML_KEYS - 1) {
+      float m4[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
 #pragma unroll
-        for (int i = 0; i < ML_KEYS; ++i) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale);
-      } else {
-#pragma unroll
-        for (int i = 0; i < ML_KEYS; ++i)
-          if (i <= lim) bm = fmaxf(bm, __uint_as_float(sv[i >> 4][i & 15]) * scale);
-      }
+      for (int i = 0; i < ML_KEYS; ++i) m4[i & 3] = fmaxf(m4[i & 3], i <= lim ? __uint_as_float(sv[i >> 4][i & 15]) * scale : -CUDART_INF_F);
+      const float bm = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
       const float m_new = fmaxf(mx, bm), m_use = m_new == -CUDART_INF_F ? 0.f : m_new;   // (rows without a token: nothing visible)
       const float corr = ml_ex2(mx - m_use);
       mx = m_new;
@@ -321,22 +319,20 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
         acc[i & 3] += p[i];
       }
       l = l * corr + ((acc[0] + acc[1]) + (acc[2] + acc[3]));
-      corr_s[j & 3][tl] = corr;
-      if (j > 0) {
-        bool okp = mbar_wait(smem_u32(&p_free), (uint32_t)(j - 1) & 1u, &abort_flag);
-        okp = __all_sync(0xffffffffu, okp);
-        if (!okp) { failed = true; break; }
-      }
-      uint8_t *ph = base_ptr + (p_hi - base), *pl = base_ptr + (p_lo - base);
+      const uint32_t pt = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(sb * 64);
+      __syncwarp();
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        uint4 hi, lo;
-        ml_split8(&p[8 * c], hi, lo);
-        *reinterpret_cast<uint4 *>(ph + ml_swz(tl, c)) = hi;
-        *reinterpret_cast<uint4 *>(pl + ml_swz(tl, c)) = lo;
+      for (int c = 0; c < 4; ++c) {                 // (all scores of the row are in registers)
+        uint4 h0, l0, h1, l1;
+        ml_split8(&p[16 * c], h0, l0);
+        ml_split8(&p[16 * c + 8], h1, l1);
+        tmem_st8(pt + (uint32_t)(8 * c), {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w});
+        tmem_st8(pt + (uint32_t)(32 + 8 * c), {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w});
       }
-      fence_proxy_async();
-      mbar_arrive(smem_u32(&p_ready));
+      tmem_st_wait();
+      tc_fence_before();
+      mbar_arrive(smem_u32(&p_ready[sb]));
+      corr_s[j & 3][tl] = corr;                     // (block j - 4's has been read: its output was, before the scores of this block were issued)
       mbar_arrive(smem_u32(&c_ready[j & 3]));
     }
     l_s[tl] = l;
@@ -367,9 +363,10 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
     }
     bool ok = !failed && mbar_wait(smem_u32(&l_ready), 0u, &abort_flag);
     ok = __all_sync(0xffffffffu, ok);
-    if (ok && real) {
-      const float inv = 1.f / l_s[tl] / kvs.y;
-      const size_t at = ((size_t)(row0 + tl) * nh + h) * 128;
+    // bf16 hi / lo through the query tiles' shared memory (all MMAs have read them), then whole rows
+    auto at = [&](int row, int c) { return (uint32_t)(row * 256 + ((c ^ (row & 7)) << 4)); };
+    if (ok) {
+      const float inv = 1.f / l_s[tl] / kvs.y;      // (rows without a token: not stored)
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
         __nv_bfloat16 a[8], b[8];
@@ -379,8 +376,20 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
           a[i] = __float2bfloat16_rn(y);
           b[i] = __float2bfloat16_rn(y - __bfloat162float(a[i]));
         }
-        *reinterpret_cast<uint4 *>(ao_hi + at + 8 * q) = *reinterpret_cast<const uint4 *>(a);
-        *reinterpret_cast<uint4 *>(ao_lo + at + 8 * q) = *reinterpret_cast<const uint4 *>(b);
+        *reinterpret_cast<uint4 *>(base_ptr + at(tl, q)) = *reinterpret_cast<const uint4 *>(a);
+        *reinterpret_cast<uint4 *>(base_ptr + ML_Q_BYTES + at(tl, q)) = *reinterpret_cast<const uint4 *>(b);
+      }
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");  // warps 6-9 (whatever failed)
+    if (ok) {
+#pragma unroll 4
+      for (int k = 0; k < 16; ++k) {
+        const int u = k * 128 + tid - 192, row = u >> 4, c = u & 15;
+        if (row < n_rows) {
+          const size_t to = ((size_t)(row0 + row) * nh + h) * 128 + 8 * c;
+          *reinterpret_cast<uint4 *>(ao_hi + to) = *reinterpret_cast<const uint4 *>(base_ptr + at(row, c));
+          *reinterpret_cast<uint4 *>(ao_lo + to) = *reinterpret_cast<const uint4 *>(base_ptr + ML_Q_BYTES + at(row, c));
+        }
       }
     }
   }
