@@ -1095,9 +1095,12 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   const bool big_ok = !one_chunk_size &&
                       (!moe || (moe->n_experts % 8 == 0 && (2 * moe->expert_ffn) % GEMM_TILE_N == 0 && H % GEMM_TILE_N == 0 &&
                                 !getenv("CORUN_MOE_PREFILL_DENSE")));
-  // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG
+  // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG, and more
+  // than half of that only where one prompt can be longer: the buffers of twice the rows make an engine's creation longer (8 slots of
+  // 1024 tokens, 12 Qwen3-30B-A3B layers: 49 -> 94 ms)
   const long long big_rows = (long long)B * ((max_context + 127) / 128 * 128);
-  int big_cap = !big_ok ? 0 : big_rows < PREFILL_BIG ? (int)((big_rows + 255) / 256 * 256) : PREFILL_BIG;
+  const int big_most = std::min(PREFILL_BIG, std::max(PREFILL_BIG / 2, (max_context + 255) / 256 * 256));
+  int big_cap = !big_ok ? 0 : big_rows < big_most ? (int)((big_rows + 255) / 256 * 256) : big_most;
   const bool wide = e->wide = pad16(B) >= (moe ? 129 : WIDE_ROWS) && s.vocab % 8 == 0;   // (Program::wide)
   if (wide && gemm_encode_map(&e->tb_lm, w->lm_head, s.vocab, H, 128)) return fail(CORUN_EINVAL);
   e->tm_qkv.resize(s.n_layers);
