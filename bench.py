@@ -307,7 +307,7 @@ def run_corun(args, rank, world):
     if os.path.exists(tp) and args.workload == "qwen3_8b_b64":
         traffic = json.load(open(tp)).get("dram_bytes_per_launch_avg")
     roofline = {
-        "kernel": "gemm_streamk_kernel (all %d launches of a step)" % n_gemm, "bound": "hbm",
+        "kernel": "gemm_rows_kernel (all %d launches of a step)" % n_gemm, "bound": "hbm",
         "achieved": (w_step / n_gemm) / (gemm_ms / n_gemm * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
         "peak_source": which + " (MEASURED_PEAKS.json hbm_gbs)" if which == "measured" else "fallback 6650",
         "traffic": traffic, "bytes_per_launch_avg": w_step / n_gemm, "ms_per_launch_avg": gemm_ms / n_gemm,
