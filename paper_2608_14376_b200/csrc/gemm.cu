@@ -3,6 +3,8 @@
 
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <vector>
 
@@ -439,18 +441,34 @@ int gemm_plan_fill(GemmPlan *p, const void *W, int N, int K, const void *Xhi, co
   if (N <= 0 || K <= 0 || K % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > 256 || R < 1 || R > BN) return CORUN_EINVAL;
   p->N = N; p->K = K; p->R = R; p->BN = BN;
   p->tile_n = BN <= GEMM_NARROW_ROWS ? GEMM_TILE_N / 2 : GEMM_TILE_N;
-  p->n_tiles = (N + p->tile_n - 1) / p->tile_n;
   p->KB = K / GEMM_BLOCK_K;
-  const long long total = (long long)p->n_tiles * p->KB;
-  p->grid = (int)(total < num_sms ? total : num_sms);
   // With several CTAs per tile the ranges are cut tile by tile (the same number of CTAs for every tile, a few
   // SMs left out): no CTA then crosses a tile boundary, so none has two epilogues in a row, and above 128
   // rows -- where the two row blocks of a tile fill TMEM and the epilogue of a segment cannot overlap the MMAs
   // of the next -- none stops in the middle of its range.
   // At least four k-blocks per CTA: with fewer, the consumer's extra partials cost more than the shorter stream saves.
-  int per_tile = p->grid >= 2 * p->n_tiles ? p->grid / p->n_tiles : 0;
-  if (per_tile > 2 && per_tile > (p->KB + 3) / 4) per_tile = p->KB > 8 ? (p->KB + 3) / 4 : 2;
-  if (per_tile) p->grid = per_tile * p->n_tiles;
+  struct Cut { int n_tiles, grid, per_tile; };
+  auto cut = [&](int tile_n) {
+    Cut c{(N + tile_n - 1) / tile_n, 0, 0};
+    const long long total = (long long)c.n_tiles * p->KB;
+    c.grid = (int)(total < num_sms ? total : num_sms);
+    c.per_tile = c.grid >= 2 * c.n_tiles ? c.grid / c.n_tiles : 0;
+    if (c.per_tile > 2 && c.per_tile > (p->KB + 3) / 4) c.per_tile = p->KB > 8 ? (p->KB + 3) / 4 : 2;
+    if (c.per_tile) c.grid = c.per_tile * c.n_tiles;
+    return c;
+  };
+  const Cut own = cut(p->tile_n);
+  p->n_tiles = own.n_tiles;
+  p->grid = own.grid;
+  const int per_tile = own.per_tile;
+  const long long total = (long long)p->n_tiles * p->KB;
+  if (p->tile_n < GEMM_TILE_N) {
+    // as many accumulators as an accumulator of a wide tile goes into a CTA's share of K, one for K as a whole
+    const Cut wide = cut(GEMM_TILE_N);
+    auto longest = [&](const Cut &c) { return std::min((double)p->KB, c.per_tile ? (double)p->KB / c.per_tile : (double)c.n_tiles * p->KB / c.grid); };
+    const int runs = std::min(GEMM_MAX_RUNS, std::max(1, (int)std::ceil(longest(own) / longest(wide) - 1e-9)));
+    if (runs > 1) p->run_kb = ((int)std::ceil(longest(own)) + runs - 1) / runs;
+  }
   if (total * (long long)p->grid >= (1ll << 31)) return CORUN_EINVAL;
   p->direct = direct;
   p->ws = ws;

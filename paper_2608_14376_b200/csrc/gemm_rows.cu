@@ -14,11 +14,12 @@ namespace {
 constexpr int GR_THREADS = 320;                     // warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue
 constexpr int GR_MAX_STAGES = 11;
 constexpr uint32_t GR_W_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: what one MMA reads of the weights
+static_assert(GEMM_MAX_RUNS * 2 * GEMM_NARROW_ROWS <= 256, "a narrow tile's accumulators fit half of tensor memory");
 
 struct GemmRowsArgs {
   float *direct, *ws;
   const int *cta_start;
-  int N, KB, BN, R, stages, tile_n, w_rows;         // w_rows: weight rows per box (128; SWIGLU: gate rows = up rows of a tile)
+  int N, KB, BN, R, stages, tile_n, w_rows, run_kb; // w_rows: weight rows per box (128; SWIGLU: gate rows = up rows of a tile)
   uint32_t stage_bytes;
   const float *row_keep;
   int keep_pitch, keep_div;
@@ -45,6 +46,12 @@ struct GemmRowsArgs {
 // walk the range segment by segment (the part of the range that falls into one tile).  hi and lo have an accumulator each, added
 // at the end; K ascending.  A row's result depends neither on its place nor on the other rows.
 //
+// An accumulator cuts every sum off (gemm_pair.cu).  A narrow tile has half as many CTAs to share its K, so a segment of it is summed
+// in up to GEMM_MAX_RUNS accumulators of run_kb k-blocks, 64 columns (32 padded rows) apart, added in ascending order in fp32: none sums
+// more than one of a wide tile does.  Sums of positive products off 64 bits (N x K, wide tile / narrow with one accumulator / so):
+// 6144 x 4096 9.9e-7 / 2.5e-6 / 9.9e-7, 4096 x 4096 5.3e-7 / 1.5e-6 / 4.1e-7, 4096 x 12288 2.5e-6 / 7.9e-6 / 1.5e-6; normal products of
+// 4096 x 12288, with the activations' 2.5e-6, 2.8e-6 / 4.1e-6 / 2.6e-6.
+//
 // MASKED: row r of tile column n is stored only where row_keep[r * keep_pitch + (n / 256) / keep_div] != 0 (rows that no
 //   consumer will read are skipped).
 // SWIGLU: W is a gate / up matrix ([2F, K]); a tile is w_rows gate rows and the up rows of the same outputs as the two blocks
@@ -58,7 +65,9 @@ struct GemmRowsArgs {
 // SELECT (with GROUPED; the experts of up to 64 rows): the groups are the experts that at least one row selected, all rows of the
 //   step together.  group_tab holds keep_div ints, the selected experts of every row (< 0: none); every CTA makes the ascending
 //   list of them itself.  row_keep: routing weights [rows][keep_pitch]; only rows that selected the expert are stored.
-template <bool MASKED, bool GROUPED, bool SWIGLU, bool SELECT>
+// RUNS: several accumulators per segment.  An instantiation of its own: 8 rows of the Qwen3-8B QKV, O and down products 11.25 / 9.4 / 18.65
+//   us with one accumulator, 11.4 / 9.6 / 18.8 so.
+template <bool MASKED, bool GROUPED, bool SWIGLU, bool SELECT, bool RUNS = false>
 __global__ void __launch_bounds__(GR_THREADS, 1)
 gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ GemmXMaps tmX, const __grid_constant__ GemmRowsArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -278,24 +287,27 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         tc_fence_after();
         // kind::f16: D fp32 (bits 4-5 = 1), A and B bf16 (bits 7-9, 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_pad >> 2) << 17) | ((uint32_t)((m64 ? 64 : 128) >> 4) << 24);
-        const uint32_t d0 = tmem_base + mt_col(half, 0), d1 = tmem_base + mt_col(half, 1);
-        uint32_t more = 0;
-        for (int kb = kb_begin; kb < kb_end; ++kb) {
-          if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
-          if (g == k0 && kb == kb_begin) TRACE(4);
-          tc_fence_after();
-          const uint32_t st = base + (uint32_t)s * a.stage_bytes;
-          const uint64_t w0 = umma_desc_sw128(st), w1 = umma_desc_sw128(st + w_box), x = umma_desc_sw128(st + w_bytes);
+        const uint32_t d1 = tmem_base + mt_col(half, 1);
+        uint32_t d0 = tmem_base + mt_col(half, 0), more = 0;
+        for (int kb = kb_begin; kb < kb_end && !fail; d0 += 64, more = 0) {   // (RUNS) accumulator after accumulator
+          const int run_end = RUNS ? min(kb_end, kb + a.run_kb) : kb_end;
+          for (; kb < run_end; ++kb) {
+            if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
+            if (g == k0 && kb == kb_begin) TRACE(4);
+            tc_fence_after();
+            const uint32_t st = base + (uint32_t)s * a.stage_bytes;
+            const uint64_t w0 = umma_desc_sw128(st), w1 = umma_desc_sw128(st + w_box), x = umma_desc_sw128(st + w_bytes);
 #pragma unroll
-          for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
-            // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in 16-byte units
-            const uint64_t adv = (uint64_t)(k * 2);
-            umma_bf16(d0, w0 + adv, x + adv, idesc, more);
-            if (MT == 2) umma_bf16(d1, w1 + adv, x + adv, idesc, more);
-            more = 1u;
+            for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
+              // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in 16-byte units
+              const uint64_t adv = (uint64_t)(k * 2);
+              umma_bf16(d0, w0 + adv, x + adv, idesc, more);
+              if (MT == 2) umma_bf16(d1, w1 + adv, x + adv, idesc, more);
+              more = 1u;
+            }
+            umma_commit(smem_u32(&empty_bar[s]));   // frees the stage once these MMAs have read it
+            if (++s == a.stages) { s = 0; ph ^= 1u; }
           }
-          umma_commit(smem_u32(&empty_bar[s]));     // frees the stage once these MMAs have read it
-          if (++s == a.stages) { s = 0; ph ^= 1u; }
         }
         if (fail) break;
         for (int h = 0; h < 2; ++h)
@@ -400,12 +412,27 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           tmem_ld8(ta, h);
           tmem_ld8(ta + (uint32_t)n_pad, l);
           tmem_ld_wait();
+          float v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
+          if (RUNS) {
+            uint32_t at_run = ta;
+#pragma unroll 1
+            for (int left = kb_end - kb_begin - a.run_kb; left > 0; left -= a.run_kb) {   // (rolled: it runs once, from a cold instruction cache)
+              at_run += 64;
+              tmem_ld8(at_run, h);
+              tmem_ld8(at_run + (uint32_t)n_pad, l);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 8; ++j) v[j] += __uint_as_float(h[j]) + __uint_as_float(l[j]);
+            }
+          }
           uint32_t on = rows_on(c, SELECT ? g_id : MASKED ? n0 / GEMM_TILE_N / a.keep_div : 0);
           if (n0 + at >= N) on = 0;
           float *d = dst + (size_t)(8 * c) * pitch + at;
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            if ((on >> j) & 1u) d[(size_t)j * pitch] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
+            if ((on >> j) & 1u) d[(size_t)j * pitch] = v[j];
         }
       }
       tc_fence_before();
@@ -432,6 +459,8 @@ template <typename F>
 cudaError_t each_kernel(F f) {
   cudaError_t e = f(gemm_rows_kernel<false, false, false, false>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<true, false, false, false>);
+  if (e == cudaSuccess) e = f(gemm_rows_kernel<false, false, false, false, true>);
+  if (e == cudaSuccess) e = f(gemm_rows_kernel<true, false, false, false, true>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<false, false, true, false>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<true, false, true, false>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<false, true, false, false>);
@@ -473,7 +502,7 @@ cudaError_t gemm_rows_prepare() {
 
 cudaError_t gemm_rows_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int *d_status, cudaStream_t st, unsigned long long *trace,
                              bool pdl) {
-  const GemmRowsArgs a{p.direct, p.ws, p.d_cta_start, p.N, p.KB, p.BN, p.R, p.stages, p.tile_n, p.sw_half ? p.sw_half : 128, p.stage_bytes,
+  const GemmRowsArgs a{p.direct, p.ws, p.d_cta_start, p.N, p.KB, p.BN, p.R, p.stages, p.tile_n, p.sw_half ? p.sw_half : 128, p.run_kb, p.stage_bytes,
                        p.row_keep, p.keep_pitch, p.keep_div, p.group_tab, p.tiles_per_group, d_status, trace, p.sw_hi, p.sw_lo, p.row_blocks};
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(p.grid), dim3(GR_THREADS), p.smem_bytes, st, pdl, tmW_override ? *tmW_override : p.tmW, p.tmX, a);
@@ -482,6 +511,7 @@ cudaError_t gemm_rows_launch(const GemmPlan &p, const CUtensorMap *tmW_override,
   if (p.select) return p.sw_hi ? go(gemm_rows_kernel<false, true, true, true>) : go(gemm_rows_kernel<false, true, false, true>);
   if (p.group_tab) return p.sw_hi ? go(gemm_rows_kernel<false, true, true, false>) : go(gemm_rows_kernel<false, true, false, false>);
   if (p.sw_hi) return masked ? go(gemm_rows_kernel<true, false, true, false>) : go(gemm_rows_kernel<false, false, true, false>);
+  if (p.run_kb < p.KB) return masked ? go(gemm_rows_kernel<true, false, false, false, true>) : go(gemm_rows_kernel<false, false, false, false, true>);
   return masked ? go(gemm_rows_kernel<true, false, false, false>) : go(gemm_rows_kernel<false, false, false, false>);
 }
 

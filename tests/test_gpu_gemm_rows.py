@@ -21,6 +21,28 @@ def test_padded_row_counts(orc, R, N, K):
     assert np.abs(out - ref).max() <= tol
 
 
+@pytest.mark.parametrize("N,K", [(4096, 12288), (6144, 4096), (4096, 4096), (5120, 2048), (328, 1152), (20000, 1024)])
+def test_few_rows_are_no_further_off_than_many(N, K):
+    """The tensor core's accumulator cuts every sum off, so an error grows with the k-blocks that one accumulator takes.  Up to 32
+    rows a tile is half as wide and half as many CTAs share its K; what an accumulator sums stays no longer.  Positive products:
+    nothing of what is cut off cancels."""
+    import torch
+
+    from paper_2608_14376_b200 import corun
+
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    W = (torch.randn((N, K), generator=g, device="cuda") * 0.02).abs().bfloat16()
+    X = (torch.rand((48, K), generator=g, device="cuda") + 0.5).bfloat16().float()      # exact as it is: only the sums are off
+    want = X.double() @ W.double().T
+
+    def off(rows):
+        return float((corun.debug_gemm(W, X[:rows].contiguous()).double() - want[:rows]).norm() / want[:rows].norm())
+
+    wide = off(48)
+    for rows in (1, 16, 17, 32):
+        assert off(rows) <= 1.1 * wide + 3e-8, (rows, off(rows), wide)    # (3e-8: the result's own rounding to fp32)
+
+
 @pytest.mark.parametrize("B", [16, 40, 100, 128])
 def test_rows_of_a_step_are_counted(B):
     """A request's logits are the same bytes with any number of requests in the step: the padded rows follow the count."""
