@@ -6,9 +6,9 @@
 // to the tile's last token once:
 //   S[128 rows x 128 keys] = Q * K^T on tcgen05.mma (M = 128, N = 128, fp16, Q as a hi/lo pair: two MMAs per k-slice) into
 //     one of two TMEM buffers;
-//   softmax warps, a thread per row (TMEM lane = row): P = exp2(S - the block's own maximum) as fp16 into the first half of the
-//     scores' own buffer (causal mask: key position <= the row's own position), and the block's maximum and sum;
-//   O'[128 x hd] = P * V, P from tensor memory, one MMA per page, into one of two TMEM buffers;
+//   softmax warps, a thread per row (TMEM lane = row): P = exp2(S - the block's own maximum) as fp16 into one of two TMEM buffers
+//     of 64 columns (causal mask: key position <= the row's own position), and the block's maximum and sum;
+//   O'[128 x hd] = P * V, P from tensor memory, one MMA per page, into one of two (hd 128: the one) TMEM buffers;
 //   output warps, a thread per row and half of the dims: the factor between this block's scale and the earlier ones', O and O' to
 //     the larger of the two maxima and added, in registers; at the end O / sum -> bf16 hi/lo.
 // A block's largest weight is exactly 1 in fp16 and the factors are fp32, so the keys that carry a row have unrounded weights
@@ -19,7 +19,11 @@
 // 64 cycles per block, beside 1024 cycles of exponentials and 1650 of TMA: 16 boxes of 4 KB at 103).
 // Measured per layer of the Qwen3-8B shape, this kernel / one softmax group with weights through shared memory, a thread per row
 // for queries and results: 77 tokens 9.5 / 15.7 us, 1003 tokens 29.8 / 41.3, 6001 tokens 610 / 830.
-// The tensor pipe works in the order of issue: scores of block j + 2 after the values of block j, whose weights they overwrite.
+// MMAs on different accumulators may overtake one another, so none writes what another one may still read: a block's scores,
+// weights and output have places of their own.  Scores of block j + 2 overwrite those of block j, which the softmax has read when it
+// hands over its weights; the weights of block j + 2 are written behind the commit of its scores, which are issued behind the
+// values of block j and so complete no earlier; the one output buffer of hd 128 is read while the scores of block j + 2 are
+// multiplied.
 // Roles: warps 0-3 and 4-7 softmax, 8-11 and 12-15 output, warp 16 streams the keys and warp 17 the values with TMA (rings of two; one
 // 4-dimensional box per (page, head) tile), warp 18 issues the MMAs.
 //
@@ -58,6 +62,8 @@ struct PfLayout {
   static constexpr int Q_BYTES = NHALF * 128 * 128;           // one of hi / lo: [half][128 rows x 128 B]
   static constexpr int PAGE_BYTES = NHALF * KV_BLOCK * 128;   // one page's keys (values) of one head
   static constexpr int B_BYTES = PF_PAGES * PAGE_BYTES;       // a block of keys (values)
+  static constexpr int O_BUFS = HD == 64 ? 2 : 1;             // of the 512 columns: 2 x 128 scores, 2 x 64 weights, 128 output
+  static constexpr uint32_t P_COL = 256, O_COL = 384;
   static constexpr size_t SMEM = (size_t)2 * Q_BYTES + 2 * PF_RING * B_BYTES + 1024;
 };
 
@@ -67,10 +73,10 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
                     __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, int *status) {
   using L = PfLayout<HD>;
   constexpr int TPT = 128 / GROUP;                  // tokens per tile
-  constexpr int KSTEPS = HD / 16;
+  constexpr int KSTEPS = HD / 16, O_BUFS = L::O_BUFS;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t kfull[PF_RING], kempty[PF_RING], vfull[PF_RING], vempty[PF_RING], s_full[2], p_ready[2], o_full[2], o_free[2],
-      c_ready[4];
+  __shared__ __align__(8) uint64_t kfull[PF_RING], kempty[PF_RING], vfull[PF_RING], vempty[PF_RING], s_full[2], p_ready[2], o_full[O_BUFS],
+      o_free[O_BUFS], c_ready[4];
   __shared__ float max_s[4][128], sum_s[4][128];    // a block's maximum and sum per row, four blocks in turn
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
@@ -85,7 +91,9 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&s_full[i]), 1);           // scores in TMEM
-      mbar_init(smem_u32(&p_ready[i]), 128);        // every row thread has replaced them by its weights
+      mbar_init(smem_u32(&p_ready[i]), 128);        // every row thread has read them and written its weights
+    }
+    for (int i = 0; i < O_BUFS; ++i) {
       mbar_init(smem_u32(&o_full[i]), 1); mbar_init(smem_u32(&o_free[i]), 256);   // a block's output in TMEM / read by both groups
     }
     for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&c_ready[i]), 128);            // the rows' maxima and sums of a block
@@ -127,7 +135,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
                   (page * 2 * kv.n_kv + (keys ? 0 : kv.n_kv) + g) * (KV_BLOCK / 8), fb, l2_policy_evict_last());   // the tiles of the same request read the same cache rows
   };
   if (warp == 18) {
-    tmem_alloc(smem_u32(&tmem_base_s), 512);        // 2 x 128 columns of scores, 2 x 128 of output
+    tmem_alloc(smem_u32(&tmem_base_s), 512);        // (PfLayout)
     tmem_relinquish();
   } else if (warp >= 16) {
     page_next = lane < pages_of(0) ? table[lane] : 0;
@@ -198,17 +206,18 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
       scores(0);
       if (n_blocks > 1 && !failed) scores(1);
       for (int j = 0; j < n_blocks && !failed; ++j) {
-        const int buf = j % PF_RING, b = j & 1;
+        const int buf = j % PF_RING, b = j & 1, ob = j % O_BUFS;
         if (!mbar_wait(smem_u32(&p_ready[b]), (uint32_t)(j >> 1) & 1u, &abort_flag)) { failed = true; break; }
         if (!mbar_wait(smem_u32(&vfull[buf]), (uint32_t)(j / PF_RING) & 1u, &abort_flag)) { failed = true; break; }
-        if (j >= 2 && !mbar_wait(smem_u32(&o_free[b]), (uint32_t)((j >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
+        if (j >= O_BUFS && !mbar_wait(smem_u32(&o_free[ob]), (uint32_t)(j / O_BUFS - 1) & 1u, &abort_flag)) { failed = true; break; }
         tc_fence_after();
         const int n_pages = pages_of(j);
-        const uint32_t vt = v_ring + (uint32_t)(buf * L::B_BYTES), p = tmem + (uint32_t)b * 128, d = tmem + 256 + (uint32_t)b * 128;
+        const uint32_t vt = v_ring + (uint32_t)(buf * L::B_BYTES), p = tmem + L::P_COL + (uint32_t)b * 64,
+                       d = tmem + L::O_COL + (uint32_t)(ob * HD);
         for (int i = 0; i < n_pages; ++i)           // 16 tokens of weights are 8 columns
           umma_f16_ts(d, p + (uint32_t)(8 * i), umma_desc_sw128_mn(vt + (uint32_t)(i * L::PAGE_BYTES), 1024u, L::NHALF * 1024u), idesc_o, i > 0 ? 1u : 0u);
         umma_commit(smem_u32(&vempty[buf]));
-        umma_commit(smem_u32(&o_full[b]));
+        umma_commit(smem_u32(&o_full[ob]));
         if (j + 2 < n_blocks) scores(j + 2);
       }
     }
@@ -217,7 +226,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
     const int pos = real ? rows.pos[row0 + tl / GROUP] : -1;       // keys 0..pos are visible to this row
     const float sscale = (HD == 128 ? 0.08838834764831845f : 0.125f) * 1.4426950408889634f;   // log2(e)/sqrt(hd)
     const int sb = warp >> 2;
-    const uint32_t st = t_lane + (uint32_t)(sb * 128);
+    const uint32_t st = t_lane + (uint32_t)(sb * 128), pt = t_lane + L::P_COL + (uint32_t)(sb * 64);
     for (int j = sb; j < n_blocks; j += 2) {
       bool ok = mbar_wait(smem_u32(&s_full[sb]), (uint32_t)(j >> 1) & 1u, &abort_flag);
       ok = __all_sync(0xffffffffu, ok);
@@ -260,16 +269,16 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
             const __half2 h2 = __floats2half2_rn(p0, p1);
             w[i >> 1] = *reinterpret_cast<const uint32_t *>(&h2);
           }
-          tmem_st8(at, w);                          // (scores that have been read; the load in flight is of later columns)
+          tmem_st8(at, w);
         };
 #pragma unroll 1
         for (int c = 0; c < 8; c += 2) {
           tmem_ld_wait();
           tmem_ld16(st + (uint32_t)(16 * c + 16), v[1]);
-          weights(v[0], lim - 16 * c, st + (uint32_t)(8 * c));
+          weights(v[0], lim - 16 * c, pt + (uint32_t)(8 * c));
           tmem_ld_wait();
           tmem_ld16(st + (uint32_t)(c < 6 ? 16 * c + 32 : 112), v[0]);   // (the last one is not used)
-          weights(v[1], lim - 16 * c - 16, st + (uint32_t)(8 * c + 8));
+          weights(v[1], lim - 16 * c - 16, pt + (uint32_t)(8 * c + 8));
         }
         tmem_ld_wait();
       };
@@ -292,7 +301,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
 #pragma unroll
     for (int i = 0; i < HH; ++i) o[i] = 0.f;
     for (int j = 0; j < n_blocks; ++j) {
-      const int ob = j & 1;
+      const int ob = j % O_BUFS;
       bool ok = mbar_wait(smem_u32(&c_ready[j & 3]), (uint32_t)(j >> 2) & 1u, &abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) { failed = true; break; }
@@ -303,14 +312,14 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
       mx = fmaxf(mx, bm);
       l = up ? fmaf(l, factor, sum) : fmaf(sum, factor, l);
       const float f_old = up ? factor : 1.f, f_new = up ? 1.f : factor;
-      ok = mbar_wait(smem_u32(&o_full[ob]), (uint32_t)(j >> 1) & 1u, &abort_flag);
+      ok = mbar_wait(smem_u32(&o_full[ob]), (uint32_t)(j / O_BUFS) & 1u, &abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) { failed = true; break; }
       tc_fence_after();
 #pragma unroll
       for (int c = 0; c < HH / 16; ++c) {
         uint32_t v[16];
-        tmem_ld16(t_lane + (uint32_t)(256 + ob * 128 + dh * HH + 16 * c), v);
+        tmem_ld16(t_lane + L::O_COL + (uint32_t)(ob * HD + dh * HH + 16 * c), v);
         tmem_ld_wait();
 #pragma unroll
         for (int i = 0; i < 16; ++i) o[16 * c + i] = fmaf(o[16 * c + i], f_old, __uint_as_float(v[i]) * f_new);
