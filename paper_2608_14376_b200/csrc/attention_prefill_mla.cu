@@ -27,6 +27,7 @@ constexpr uint32_t ML_BOX = ML_KEYS * 128;          // [64 tokens x 64 dims] fp1
 constexpr uint32_t ML_Q_BYTES = 3 * 128 * 128;      // hi or lo: [3 blocks of 64 dims][128 rows x 128 B]
 constexpr uint32_t ML_K_BYTES = 5 * ML_BOX;         // hi, lo of the 128 no-rope dims, the rotary key
 constexpr uint32_t ML_V_BYTES = 4 * ML_BOX;         // hi, lo
+constexpr uint32_t ML_P_COL = 128, ML_O_COL = 256;  // tensor memory: scores, weights, outputs
 constexpr size_t ML_SMEM = 1024 + 2 * ML_Q_BYTES + 2 * ML_K_BYTES + ML_V_BYTES;
 
 __device__ __forceinline__ uint32_t ml_swz(int row, int chunk) { return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4)); }
@@ -114,11 +115,13 @@ mla_gather_kernel(const __grid_constant__ MlaSegs g, MlaCache cache, int rank, i
 
 // One CTA per (head, tile of 128 chunk rows = consecutive tokens of one request).  Per block of 64 keys:
 //   S[128 x 64] = Qhi Khi + Qlo Khi + Qhi Klo (12 k-slices) into one of two TMEM buffers;
-//   softmax warps, a thread per row: running maximum, P = exp2(S - max) as fp16 hi and lo in the scores' own columns, the factor by
-//     which the earlier sums shrink;
+//   softmax warps, a thread per row: running maximum, P = exp2(S - max) as fp16 hi and lo into one of two TMEM buffers, the factor
+//     by which the earlier sums shrink;
 //   O'[128 x 128] = Phi Vhi + Plo Vhi + Phi Vlo (4 k-slices), P from tensor memory, into one of two TMEM buffers;
 //   output warps, a thread per row: O = O * factor + O', in registers.
-// The tensor pipe works in the order of issue: scores of block j + 2 after the values of block j, whose weights they overwrite; the
+// MMAs on different accumulators may overtake one another, so none writes what another one may still read: scores of block j + 2
+// overwrite those of block j, which the softmax has read when it hands over its weights; the weights of block j + 2 are written
+// behind the commit of its scores, which are issued behind the values of block j and so complete no earlier.  The
 // keys of two blocks are in shared memory.  (One key buffer, weights through shared memory and one producer for keys and values, so that
 // a block's keys were requested behind the values before them, and queries and results by a thread per row: 2505 tokens of 16 heads
 // 160 us per layer, now 125.)  What bounds a block are its 32 MMAs of 48 and 12 of 64 cycles.
@@ -160,7 +163,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
     prefetch_tensormap(&tmR);
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&tmem_base_s), 512);        // scores 2 x 64 columns, outputs 2 x 128
+    tmem_alloc(smem_u32(&tmem_base_s), 512);        // scores 2 x 64 columns, weights (hi, lo) 2 x 64, outputs 2 x 128
     tmem_relinquish();
   }
   if (warp >= 2 && warp < 10) {
@@ -272,7 +275,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
         if (!mbar_wait(smem_u32(&vfull), (uint32_t)j & 1u, &abort_flag)) { failed = true; break; }
         if (j >= 2 && !mbar_wait(smem_u32(&o_free[b]), (uint32_t)((j >> 1) - 1) & 1u, &abort_flag)) { failed = true; break; }
         tc_fence_after();
-        const uint32_t p = tmem + (uint32_t)b * 64, d = tmem + 128 + (uint32_t)b * 128;
+        const uint32_t p = tmem + ML_P_COL + (uint32_t)b * 64, d = tmem + ML_O_COL + (uint32_t)b * 128;
 #pragma unroll
         for (int ks = 0; ks < ML_KEYS / 16; ++ks) {
           const uint32_t ph = p + (uint32_t)(8 * ks), pl = ph + 32;   // 16 tokens of weights are 8 columns
@@ -319,10 +322,10 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
         acc[i & 3] += p[i];
       }
       l = l * corr + ((acc[0] + acc[1]) + (acc[2] + acc[3]));
-      const uint32_t pt = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(sb * 64);
+      const uint32_t pt = tmem + ((uint32_t)(quad * 32) << 16) + ML_P_COL + (uint32_t)(sb * 64);
       __syncwarp();
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {                 // (all scores of the row are in registers)
+      for (int c = 0; c < 4; ++c) {
         uint4 h0, l0, h1, l1;
         ml_split8(&p[16 * c], h0, l0);
         ml_split8(&p[16 * c + 8], h1, l1);
@@ -353,7 +356,7 @@ mla_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_consta
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
         uint32_t v[8];
-        tmem_ld8(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(128 + ob * 128 + 8 * q), v);
+        tmem_ld8(tmem + ((uint32_t)(quad * 32) << 16) + ML_O_COL + (uint32_t)(ob * 128 + 8 * q), v);
         tmem_ld_wait();
 #pragma unroll
         for (int i = 0; i < 8; ++i) o[8 * q + i] = fmaf(o[8 * q + i], corr, __uint_as_float(v[i]));
