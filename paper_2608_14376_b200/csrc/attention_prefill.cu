@@ -102,6 +102,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap tmKV, const float *__res
     prefetch_tensormap(&tmKV);
   }
   griddep_wait();                                   // q and the chunk's own keys / values come from the kernel before
+  q = after_wait(q);
   // the tile's rows with a token are the first ones
   const int n_tok = __syncthreads_count(tid < TPT && row0 + tid < rows.R && rows.active[row0 + tid] != 0);
   griddep_launch_dependents();
