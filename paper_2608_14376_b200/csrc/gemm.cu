@@ -723,6 +723,7 @@ cudaError_t gemm_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int 
 
 int gemm_plan_rebase(GemmPlan *q, const GemmPlan &p, const void *Xhi, const void *Xlo, float *direct, __nv_bfloat16 *sw_hi,
                      __nv_bfloat16 *sw_lo, const int *row_blocks) {
+  if (p.BN > GEMM_MAX_ROWS) return CORUN_EINVAL;    // (the other kernel's maps have other boxes)
   *q = p;
   q->direct = direct;
   q->sw_hi = sw_hi;

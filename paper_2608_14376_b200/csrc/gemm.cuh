@@ -323,8 +323,8 @@ cudaError_t gemm_experts_launch(const GemmExpertsPlan &p, const CUtensorMap &tmW
 int tma_encode_store_2d(CUtensorMap *m, const void *base, int is_fp32, unsigned long long rows, int cols);
 // direct[r, n] = gemm_load(r, n) for every tile that has partials (makes `direct` a plain matrix).
 cudaError_t gemm_fixup_launch(const GemmPlan &p, cudaStream_t st, bool pdl = false, int rows = 0);   // rows: the first ones (0: p.R)
-// *q = p (gemm_plan_create or gemm_plan_create_swiglu) over other rows: activations, outputs and row_blocks of its own, the
-// tables shared with p (only p is destroyed).
+// *q = p (gemm_plan_create or gemm_plan_create_swiglu, up to GEMM_MAX_ROWS padded rows) over other rows: activations, outputs and
+// row_blocks of its own, the tables shared with p (only p is destroyed).
 int gemm_plan_rebase(GemmPlan *q, const GemmPlan &p, const void *Xhi, const void *Xlo, float *direct, __nv_bfloat16 *sw_hi,
                      __nv_bfloat16 *sw_lo, const int *row_blocks);
 
