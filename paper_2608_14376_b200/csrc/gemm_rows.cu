@@ -19,7 +19,7 @@ static_assert(GEMM_MAX_RUNS * 2 * GEMM_NARROW_ROWS <= 256, "a narrow tile's accu
 struct GemmRowsArgs {
   float *direct, *ws;
   const int *cta_start;
-  int N, KB, BN, R, stages, tile_n, w_rows, run_kb; // w_rows: weight rows per box (128; SWIGLU: gate rows = up rows of a tile)
+  int N, KB, BN, R, stages, tile_n, w_rows;         // w_rows: weight rows per box (128; SWIGLU: gate rows = up rows of a tile)
   uint32_t stage_bytes;
   const float *row_keep;
   int keep_pitch, keep_div;
@@ -29,6 +29,7 @@ struct GemmRowsArgs {
   unsigned long long *trace;
   __nv_bfloat16 *sw_hi, *sw_lo;
   const int *row_blocks;
+  int run_kb;
 };
 
 // out[r, n] = sum_k W[n, k] * (Xhi[r, k] + Xlo[r, k]).
@@ -65,8 +66,8 @@ struct GemmRowsArgs {
 // SELECT (with GROUPED; the experts of up to 64 rows): the groups are the experts that at least one row selected, all rows of the
 //   step together.  group_tab holds keep_div ints, the selected experts of every row (< 0: none); every CTA makes the ascending
 //   list of them itself.  row_keep: routing weights [rows][keep_pitch]; only rows that selected the expert are stored.
-// RUNS: several accumulators per segment.  An instantiation of its own: 8 rows of the Qwen3-8B QKV, O and down products 11.25 / 9.4 / 18.65
-//   us with one accumulator, 11.4 / 9.6 / 18.8 so.
+// RUNS: several accumulators per segment.  An instantiation of its own: 8 rows of the Qwen3-8B QKV, O and down products 11.1 / 9.4 / 18.6
+//   us with one accumulator, 11.25 / 9.5 / 18.8 so.
 template <bool MASKED, bool GROUPED, bool SWIGLU, bool SELECT, bool RUNS = false>
 __global__ void __launch_bounds__(GR_THREADS, 1)
 gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ GemmXMaps tmX, const __grid_constant__ GemmRowsArgs a) {
@@ -289,25 +290,31 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_pad >> 2) << 17) | ((uint32_t)((m64 ? 64 : 128) >> 4) << 24);
         const uint32_t d1 = tmem_base + mt_col(half, 1);
         uint32_t d0 = tmem_base + mt_col(half, 0), more = 0;
-        for (int kb = kb_begin; kb < kb_end && !fail; d0 += 64, more = 0) {   // (RUNS) accumulator after accumulator
-          const int run_end = RUNS ? min(kb_end, kb + a.run_kb) : kb_end;
-          for (; kb < run_end; ++kb) {
-            if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
-            if (g == k0 && kb == kb_begin) TRACE(4);
-            tc_fence_after();
-            const uint32_t st = base + (uint32_t)s * a.stage_bytes;
-            const uint64_t w0 = umma_desc_sw128(st), w1 = umma_desc_sw128(st + w_box), x = umma_desc_sw128(st + w_bytes);
-#pragma unroll
-            for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
-              // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in 16-byte units
-              const uint64_t adv = (uint64_t)(k * 2);
-              umma_bf16(d0, w0 + adv, x + adv, idesc, more);
-              if (MT == 2) umma_bf16(d1, w1 + adv, x + adv, idesc, more);
-              more = 1u;
+        int left = a.run_kb;
+        for (int kb = kb_begin; kb < kb_end; ++kb) {
+          if (RUNS) {                               // the next accumulator
+            if (left == 0) {
+              left = a.run_kb;
+              d0 += 64;
+              more = 0;
             }
-            umma_commit(smem_u32(&empty_bar[s]));   // frees the stage once these MMAs have read it
-            if (++s == a.stages) { s = 0; ph ^= 1u; }
+            --left;
           }
+          if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
+          if (g == k0 && kb == kb_begin) TRACE(4);
+          tc_fence_after();
+          const uint32_t st = base + (uint32_t)s * a.stage_bytes;
+          const uint64_t w0 = umma_desc_sw128(st), w1 = umma_desc_sw128(st + w_box), x = umma_desc_sw128(st + w_bytes);
+#pragma unroll
+          for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
+            // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in 16-byte units
+            const uint64_t adv = (uint64_t)(k * 2);
+            umma_bf16(d0, w0 + adv, x + adv, idesc, more);
+            if (MT == 2) umma_bf16(d1, w1 + adv, x + adv, idesc, more);
+            more = 1u;
+          }
+          umma_commit(smem_u32(&empty_bar[s]));     // frees the stage once these MMAs have read it
+          if (++s == a.stages) { s = 0; ph ^= 1u; }
         }
         if (fail) break;
         for (int h = 0; h < 2; ++h)
@@ -412,19 +419,20 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           tmem_ld8(ta, h);
           tmem_ld8(ta + (uint32_t)n_pad, l);
           tmem_ld_wait();
-          float v[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
-          if (RUNS) {
+          if (RUNS) {                               // (rolled: it runs once, from a cold instruction cache)
             uint32_t at_run = ta;
 #pragma unroll 1
-            for (int left = kb_end - kb_begin - a.run_kb; left > 0; left -= a.run_kb) {   // (rolled: it runs once, from a cold instruction cache)
+            for (int left = kb_end - kb_begin - a.run_kb; left > 0; left -= a.run_kb) {
+              uint32_t x[8], y[8];
               at_run += 64;
-              tmem_ld8(at_run, h);
-              tmem_ld8(at_run + (uint32_t)n_pad, l);
+              tmem_ld8(at_run, x);
+              tmem_ld8(at_run + (uint32_t)n_pad, y);
               tmem_ld_wait();
 #pragma unroll
-              for (int j = 0; j < 8; ++j) v[j] += __uint_as_float(h[j]) + __uint_as_float(l[j]);
+              for (int j = 0; j < 8; ++j) {         // h: the sum so far, l: the accumulator that is added next
+                h[j] = __float_as_uint(__uint_as_float(h[j]) + __uint_as_float(l[j]));
+                l[j] = __float_as_uint(__uint_as_float(x[j]) + __uint_as_float(y[j]));
+              }
             }
           }
           uint32_t on = rows_on(c, SELECT ? g_id : MASKED ? n0 / GEMM_TILE_N / a.keep_div : 0);
@@ -432,7 +440,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           float *d = dst + (size_t)(8 * c) * pitch + at;
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            if ((on >> j) & 1u) d[(size_t)j * pitch] = v[j];
+            if ((on >> j) & 1u) d[(size_t)j * pitch] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
         }
       }
       tc_fence_before();
@@ -502,8 +510,8 @@ cudaError_t gemm_rows_prepare() {
 
 cudaError_t gemm_rows_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int *d_status, cudaStream_t st, unsigned long long *trace,
                              bool pdl) {
-  const GemmRowsArgs a{p.direct, p.ws, p.d_cta_start, p.N, p.KB, p.BN, p.R, p.stages, p.tile_n, p.sw_half ? p.sw_half : 128, p.run_kb, p.stage_bytes,
-                       p.row_keep, p.keep_pitch, p.keep_div, p.group_tab, p.tiles_per_group, d_status, trace, p.sw_hi, p.sw_lo, p.row_blocks};
+  const GemmRowsArgs a{p.direct, p.ws, p.d_cta_start, p.N, p.KB, p.BN, p.R, p.stages, p.tile_n, p.sw_half ? p.sw_half : 128, p.stage_bytes,
+                       p.row_keep, p.keep_pitch, p.keep_div, p.group_tab, p.tiles_per_group, d_status, trace, p.sw_hi, p.sw_lo, p.row_blocks, p.run_kb};
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(p.grid), dim3(GR_THREADS), p.smem_bytes, st, pdl, tmW_override ? *tmW_override : p.tmW, p.tmX, a);
   };
