@@ -38,7 +38,7 @@ WORKLOADS = {
     # Mixture-of-Experts decoder (Qwen3-30B-A3B shape); no CPU baseline (the weights do not fit the host leg)
     "qwen3_30b_a3b_b64": (synth.QWEN3_30B_A3B, 64, 40, 512, 4096, 0.7, 0.95, 1.28),
 }
-PREFILL_ROWS, PREFILL_ROWS_EXPERTS = 2048, 4096   # rows of a long prompt's chunk (the layers' weights are streamed once per chunk)
+PREFILL_ROWS = 4096   # rows of a long prompt's chunk (the layers' weights are streamed once per chunk)
 MOE = {"qwen3_30b_a3b_b64": (synth.QWEN3_30B_A3B_MOE, synth.QWEN3_30B_A3B_EFF)}
 # Decoder with multi-head latent attention and expert layers (DeepSeek-V2-Lite shape): 128 slots, all active
 MLA = {"deepseek_v2_lite_b128": (synth.DEEPSEEK_V2_LITE, synth.DEEPSEEK_V2_LITE_MLA, synth.DEEPSEEK_V2_LITE_MOE, 128, 128, 512, 4096, 0.7, 0.95, 0.5)}
@@ -363,9 +363,8 @@ def run_corun(args, rank, world):
             w_exp = 2 * 3 * sh.hidden * mc["expert_ffn"] * sh.n_layers      # bytes of one expert over all layers
             w_mma = w_layers - (mc["n_experts"] - mc["top_k"]) * w_exp
         t_mma = t_hbm = 0.0
-        chunk = PREFILL_ROWS_EXPERTS if moe_cfg else PREFILL_ROWS
         while left > 0:
-            rows = min(chunk, left)
+            rows = min(PREFILL_ROWS, left)
             t_mma += 2 * 2 * (w_mma // 2) * rows / (tf_s * 1e12)
             t_hbm += w_layers / (hbm * 1e9)
             t_roof += max(2 * 2 * (w_mma // 2) * rows / (tf_s * 1e12), w_layers / (hbm * 1e9))
@@ -375,7 +374,7 @@ def run_corun(args, rank, world):
         t_alg = w_lm / (hbm * 1e9)
         left = n_pf
         while left > 0:
-            rows = min(chunk, left)
+            rows = min(PREFILL_ROWS, left)
             t_alg += max(2 * (w_mma // 2) * rows / (tf_s * 1e12), w_layers / (hbm * 1e9))
             left -= rows
         prefill = {"tokens": n_pf, "ms": dt * 1e3, "tok_per_s": n_pf / dt, "roofline_ms": t_alg * 1e3,
@@ -383,7 +382,7 @@ def run_corun(args, rank, world):
                    "bound": "tensor" if t_mma >= t_hbm else "hbm",
                    "note": "frac: per chunk of up to %d tokens the larger of the algorithmic MMA work (2 FLOPs per weight and token at "
                            "%.0f TFLOP/s sustained) and the layers' weights streamed once; frac_of_executed_work counts the "
-                           "two MMAs per weight tile that the bf16 hi/lo pair of the activations costs; attention not counted" % (chunk, tf_s)}
+                           "two MMAs per weight tile that the bf16 hi/lo pair of the activations costs; attention not counted" % (PREFILL_ROWS, tf_s)}
 
     # ---- the Mixture-of-Experts feed-forward block (DeepSeek-V2-Lite block shape, B = 128 padded rows): time per
     # call with CUDA events against the bytes of expert weights a call streams (rank 0, full-size workload only)
@@ -627,11 +626,11 @@ def run_corun_mla(args, rank, world):
         torch.cuda.synchronize()
         dt = time.perf_counter() - t0
         eng.release(s_pf)
-    chunks = -(-n_pf // PREFILL_ROWS_EXPERTS)
+    chunks = -(-n_pf // PREFILL_ROWS)
     prefill = {"tokens": n_pf, "ms": dt * 1e3, "tok_per_s": n_pf / dt,
                "weights_streamed_once_per_chunk_ms": chunks * (w_bytes - 2 * sh.vocab * sh.hidden) / (hbm * 1e9) * 1e3,
                "note": "chunks of up to %d rows; expert layers in their grouped form; keys and values decompressed once per "
-                       "chunk, attention in tiles of 128 query tokens" % PREFILL_ROWS_EXPERTS}
+                       "chunk, attention in tiles of 128 query tokens" % PREFILL_ROWS}
     eng.close()
     del eng, w_t, m_t, e_t
     torch.cuda.empty_cache()

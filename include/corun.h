@@ -249,7 +249,7 @@ int corun_prefill_geometry(corun_engine *e, int32_t *chunk_rows, int32_t *tile_r
 /* The same for prompts of n_tokens (>= 1), and their class: 0 up to 128 tokens, 1 above (0 for all where the engine has one
  * program for both).  Requests of different classes do not share a pass over the layers' weights: corun_prefill_batch runs
  * one class after the other.  chunk_rows is what a scheduler should count, not what the engine launches (up to 4096 rows of
- * class 1 with expert layers, 2048 without, for the rows there are); 256 rows are one row tile of class 1 and two blocks of class 0, each a pass over the
+ * class 1, for the rows there are); 256 rows are one row tile of class 1 and two blocks of class 0, each a pass over the
  * weights.  Any of the pointers may be NULL. */
 int corun_prefill_class(corun_engine *e, int32_t n_tokens, int32_t *prefill_class, int32_t *chunk_rows, int32_t *tile_rows);
 /* Number of kernel launches in one decode iteration. */

@@ -133,11 +133,10 @@ struct Program {
 // Prompts of up to PREFILL_SMALL tokens are short (Program::shorts), longer ones long.  Which one depends on the prompt's
 // own length only, so a prompt's values do not depend on what is prefilled with it.  Measured, GEMMs of the Qwen3-8B layer:
 // 64 rows 82 us and 128 rows 110 us in a block of SHORT_ROWS; 256 rows 179 us (two blocks: 220), 512 rows 299, 1024 rows
-// 543, 2048 rows 1049 on pairs of SMs (hence chunks as large as the buffers allow).  Chunks of up to PREFILL_BIG rows are for decoders
-// with expert layers, where a chunk is a pass over the experts (2048 rows -> 4096: 2505 tokens through 9 DeepSeek-V2-Lite layers
-// 12.1 -> 9.9 ms, 3000 tokens through 12 Qwen3-30B-A3B layers 15.1 -> 12.7); dense ones are bound by the tensor cores at PREFILL_DENSE
-// rows (12 Qwen3-8B layers: 3000 / 4096 / 6001 tokens 25.5 / 34.5 / 53.2 ms in chunks of 2048 rows, 25.4 / 34.3 / 53.4 in chunks of 4096).
-constexpr int PREFILL_SMALL = 128, PREFILL_DENSE = 2048, PREFILL_BIG = 4096;
+// 543, 2048 rows 1049 on pairs of SMs (hence chunks as large as the buffers allow; PREFILL_BIG 2048 -> 4096, that is one pass over
+// the experts and not two: 2505 tokens through 9 DeepSeek-V2-Lite layers 13.6 -> 10.9 ms; 6001 tokens through 12 Qwen3-8B layers
+// 54.3 -> 54.0, where the products are bound by the tensor cores).
+constexpr int PREFILL_SMALL = 128, PREFILL_BIG = 4096;
 // Rows of a long prompt's chunk that the latent attention takes at a time (its partial results are kept per row).
 constexpr int MLA_ROWS = 256;
 constexpr int SHORT_ROWS = 128;
@@ -1096,11 +1095,11 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   const bool big_ok = !one_chunk_size &&
                       (!moe || (moe->n_experts % 8 == 0 && (2 * moe->expert_ffn) % GEMM_TILE_N == 0 && H % GEMM_TILE_N == 0 &&
                                 !getenv("CORUN_MOE_PREFILL_DENSE")));
-  // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG (dense
-  // decoders: PREFILL_DENSE), and more than PREFILL_DENSE only where one prompt can be longer: the buffers of twice the rows make an
-  // engine's creation longer (8 slots of 1024 tokens, 12 Qwen3-30B-A3B layers: 49 -> 94 ms)
+  // rows of a chunk: as many as all slots' longest prompts could fill (pieces start on attention tiles), at most PREFILL_BIG, and more
+  // than half of that only where one prompt can be longer: the buffers of twice the rows make an engine's creation longer (8 slots of
+  // 1024 tokens, 12 Qwen3-30B-A3B layers: 49 -> 94 ms)
   const long long big_rows = (long long)B * ((max_context + 127) / 128 * 128);
-  const int big_most = moe ? std::min(PREFILL_BIG, std::max(PREFILL_DENSE, (max_context + 255) / 256 * 256)) : PREFILL_DENSE;
+  const int big_most = std::min(PREFILL_BIG, std::max(PREFILL_BIG / 2, (max_context + 255) / 256 * 256));
   int big_cap = !big_ok ? 0 : big_rows < big_most ? (int)((big_rows + 255) / 256 * 256) : big_most;
   const bool wide = e->wide = pad16(B) >= (moe ? 129 : WIDE_ROWS) && s.vocab % 8 == 0;   // (Program::wide)
   if (wide && gemm_encode_map(&e->tb_lm, w->lm_head, s.vocab, H, 128)) return fail(CORUN_EINVAL);

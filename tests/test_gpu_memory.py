@@ -39,26 +39,3 @@ def test_an_engine_fits_beside_what_is_left_and_gives_the_same_bytes():
     finally:
         del hog
         torch.cuda.empty_cache()
-
-
-def test_a_dense_decoders_chunks_stay_at_2048_rows():
-    """Longer chunks gain a dense decoder nothing: an engine for longer prompts takes its longer tables, not larger buffers."""
-    import torch
-
-    from paper_2608_14376_b200 import corun
-
-    sh = synth.ModelShape(1, 4096, 32, 8, 128, 12288, 4096, 1e-6, 10000.0)
-    w = synth.make_weights_torch(sh, seed=3)
-
-    def used(max_context):
-        gc.collect(); torch.cuda.empty_cache(); torch.cuda.synchronize()
-        free = torch.cuda.mem_get_info()[0]
-        eng = corun.Engine(sh, w, 8, max_context, kv_pool_blocks=64)
-        try:
-            return free - torch.cuda.mem_get_info()[0]
-        finally:
-            eng.close()
-
-    used(2048)                                        # (kernels are loaded)
-    # tables and partial results of twice the context: some 10 MB; 2048 more rows would be 300 MB
-    assert used(4096) - used(2048) <= 64 << 20
