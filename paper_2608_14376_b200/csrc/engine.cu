@@ -45,6 +45,18 @@ struct DevMem {
   char *cur = nullptr;
   size_t left = 0, next = (size_t)32 << 20;
   bool tight = false;                                // there was no room for a whole block
+  // Room for `bytes` in one block of that size, if there is as much: what follows fits it and leaves nothing over.
+  void reserve(size_t bytes) {
+    void *q = nullptr;
+    if (cudaMalloc(&q, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      tight = true;
+      return;
+    }
+    blocks.push_back(q);
+    cur = (char *)q;
+    left = bytes;
+  }
   void release() {
     for (void *p : blocks) cudaFree(p);
     blocks.clear();
@@ -282,7 +294,7 @@ int dmalloc(DevMem &m, T **p, size_t n, bool zero = true) {
 int pad16(int x) { return (x + 15) / 16 * 16; }
 
 void mla_group_table(std::vector<int> &t, int nh, int rows_per_head, int BG, int R, int w_rows, int count_at);
-int program_create_groups(corun_engine *e, Program &P, int R, int lg_rows);
+int program_create_groups(corun_engine *e, Program &P, int R, int lg_rows, char *room = nullptr);
 
 // fuse_swiglu: the gate / up GEMM writes silu(gate) * up itself (dense feed-forward, up to 128 padded rows: the
 // decode program while it is bound by the weight stream; whole tiles on fewer CTAs would cost a prefill chunk,
@@ -459,26 +471,39 @@ void mla_group_table(std::vector<int> &t, int nh, int rows_per_head, int BG, int
   t[count_at] = n;
 }
 
+// Slots of the experts' grouped form for up to R rows, and what their gathered rows, hidden activations and results take at `room`
+// (the results over the gathered rows, which only the gate / up product reads).
+size_t group_slots(const corun_engine *e, int R, int lg_rows) { return (size_t)moe_max_groups(R, e->moe_E, e->moe_S, e->moe_K, lg_rows) << lg_rows; }
+size_t group_room(const corun_engine *e, int R, int lg_rows) { return group_slots(e, R, lg_rows) * 4 * (size_t)(e->sh.hidden + e->moe_F); }
+
 // Buffers and plans of the experts' grouped form for up to R rows.
-int program_create_groups(corun_engine *e, Program &P, int R, int lg_rows) {
+int program_create_groups(corun_engine *e, Program &P, int R, int lg_rows, char *room) {
   const int Fm = e->moe_F, NB = e->moe_E + e->moe_S, H = e->sh.hidden;
   auto &A = P.allocs;
   MoeGroups &g = P.grp;
   g.lg_rows = lg_rows;
   g.n_groups_max = moe_max_groups(R, e->moe_E, e->moe_S, e->moe_K, lg_rows);
-  const size_t slots = (size_t)g.n_groups_max << lg_rows;
+  const size_t slots = group_slots(e, R, lg_rows);
   RC(dmalloc(A, &g.tab_up, (size_t)g.n_groups_max * 3 + 1));
   RC(dmalloc(A, &g.tab_down, (size_t)g.n_groups_max * 3 + 1));
   RC(dmalloc(A, &g.group_expert, (size_t)g.n_groups_max));
   RC(dmalloc(A, &g.slot_row, slots));
   RC(dmalloc(A, &g.slot_of, (size_t)R * NB));
   RC(dmalloc(A, &g.slot_w, slots));
-  RC(dmalloc(A, &P.xg_hi, slots * H));
-  RC(dmalloc(A, &P.xg_lo, slots * H));
-  RC(dmalloc(A, &P.hg_hi, slots * Fm));
-  RC(dmalloc(A, &P.hg_lo, slots * Fm));
-  RC(dmalloc(A, &P.yg_out, slots * H));
   P.grouped = true;
+  if (room) {
+    P.xg_hi = (bf16 *)room;
+    P.xg_lo = P.xg_hi + slots * H;
+    P.yg_out = (float *)room;
+    P.hg_hi = P.xg_lo + slots * H;
+    P.hg_lo = P.hg_hi + slots * Fm;
+  } else {
+    RC(dmalloc(A, &P.xg_hi, slots * H));
+    RC(dmalloc(A, &P.xg_lo, slots * H));
+    RC(dmalloc(A, &P.hg_hi, slots * Fm));
+    RC(dmalloc(A, &P.hg_lo, slots * Fm));
+    RC(dmalloc(A, &P.yg_out, slots * H));
+  }
   if (P.pair) {                                     // prompts: on pairs of SMs
     RC(gemm_experts_plan_create_swiglu(&P.x_gu, Fm, H, P.xg_hi, P.xg_lo, g.n_groups_max, P.hg_hi, P.hg_lo, g.slot_w, g.tab_up, e->num_sms));
     return gemm_experts_plan_create(&P.x_down, H, Fm, P.hg_hi, P.hg_lo, g.n_groups_max, P.yg_out, g.tab_down, e->num_sms);
@@ -511,14 +536,38 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   P.has_layers = true;
   auto &A = P.allocs;
   const size_t c = (size_t)cap;
+  // One piece of memory for what the attention half of a layer hands on (the projections, queries, latent queries and values) and what
+  // the feed-forward half does.  Each is written, for all rows of the chunk, before it is read, so nothing needs clearing.
+  const size_t hr = e->mla ? (size_t)md.nh * cap : 0;   // rows of the head-major matrices (cap is a multiple of 64)
+  const size_t attn_room = (c * (QKVN + (e->mla ? 0 : QD)) + hr * (md.rank + md.nope + md.vh)) * sizeof(float);
+  const size_t room_bytes = std::max(attn_room, std::max(c * F * 4, e->moe_E ? group_room(e, cap, 7) : (size_t)0));
+  // partial tiles of an unfilled wave: consumed by the next kernel of the stream, so one buffer serves all
+  size_t part = gemm_pair_part_floats(QKVN, H, cap, e->num_sms);
+  for (size_t x : {gemm_pair_part_floats(H, QD, cap, e->num_sms), F > 0 ? gemm_pair_part_floats(H, F, cap, e->num_sms) : 0,
+                   e->moe_E ? gemm_pair_part_floats(e->moe_E, H, cap, e->num_sms) : 0})
+    part = x > part ? x : part;
+  // at most one request of a chunk began in an earlier one: the others' tokens are rows of the chunk
+  if (e->big_mla_tiles) P.kv_cap = (e->max_ctx + cap + 64 * MLA_MAX_SEGS + 255) / 256 * 256;
+  // All of it in one block.  Engines with chunks of 2048 rows / of 4096, every buffer apart and cleared, in blocks of powers of two / so:
+  // 12 Qwen3-8B layers, 8 slots 2686 / 3038 / 2546 MiB, 12 Qwen3-30B-A3B layers, 64 slots 3882 / 4778 / 3704, 9 DeepSeek-V2-Lite layers, 128
+  // slots 6174 / 7264 / 5746; created in 19 / 20.5 / 18, 15 / 21 / 14.5 and 15.5 / 17.5 / 13.5 ms.
+  const int NB = e->moe_E + e->moe_S;
+  size_t all = c * 4 * (3 * (size_t)H + QD + 4) + room_bytes + (gemm_ws_floats(e->num_sms, SHORT_ROWS) + part) * sizeof(float) + (1 << 20);
+  if (e->mla)
+    all += hr * 4 * (size_t)(md.nope + md.rank + md.rope) + (size_t)P.kv_cap * (4 * md.rank + 128 + 1024 * (size_t)md.nh) +
+           ((size_t)mla_part_ml_floats(MLA_ROWS, md.nh, e->max_ctx) + mla_part_o_floats(MLA_ROWS, md.nh, md.rank, e->max_ctx)) * sizeof(float);
+  if (e->moe_E) all += c * 4 * (size_t)(2 * NB + e->moe_E) + group_slots(e, cap, 7) * 8 + (size_t)NB * (MOE_MANY_ROWS / 8);
+  A.reserve(all);
   RC(dmalloc(A, &P.xn_hi, c * H));
   RC(dmalloc(A, &P.xn_lo, c * H));
   RC(dmalloc(A, &P.row_token, 4 * c));              // token | position | active | slot, as many rows as the chunk at hand has
   RC(dmalloc(A, &P.row_blocks, c / SHORT_ROWS));
   RC(dmalloc(A, &P.h, c * H));
-  RC(dmalloc(A, &P.qkv_out, c * QKVN));
-  RC(dmalloc(A, &P.o_out, c * H));
   RC(dmalloc(A, &P.down_out, c * H));
+  P.o_out = P.down_out;                             // (the residual takes one up before the other is written)
+  char *room = nullptr;
+  RC(dmalloc(A, &room, room_bytes, false));
+  P.qkv_out = (float *)room;
   RC(dmalloc(A, &P.ao_hi, c * QD));
   RC(dmalloc(A, &P.ao_lo, c * QD));
   RC(dmalloc(A, &P.plain_tiles, (size_t)((QKVN > H ? QKVN : H) / GEMM_TILE_N + 1)));
@@ -527,17 +576,12 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
   for (auto *v : {&P.s_qkv, &P.s_o, &P.s_gu, &P.s_down}) v->resize((size_t)n_blk);
   RC(gemm_plan_create(&P.s_qkv[0], e->w0_qkv, QKVN, H, P.xn_hi, P.xn_lo, SHORT_ROWS, SHORT_ROWS, P.qkv_out, P.ws, e->num_sms));
   RC(gemm_plan_create(&P.s_o[0], e->w0_o, H, QD, P.ao_hi, P.ao_lo, SHORT_ROWS, SHORT_ROWS, P.o_out, P.ws, e->num_sms));
-  // partial tiles of an unfilled wave: consumed by the next kernel of the stream, so one buffer serves all
-  size_t part = gemm_pair_part_floats(QKVN, H, cap, e->num_sms);
-  for (size_t x : {gemm_pair_part_floats(H, QD, cap, e->num_sms), F > 0 ? gemm_pair_part_floats(H, F, cap, e->num_sms) : 0,
-                   e->moe_E ? gemm_pair_part_floats(e->moe_E, H, cap, e->num_sms) : 0})
-    part = x > part ? x : part;
   RC(dmalloc(A, &P.pair_part, part, false));
   RC(gemm_pair_plan_create(&P.b_qkv, QKVN, H, P.xn_hi, P.xn_lo, cap, P.qkv_out, P.pair_part, e->num_sms));
   RC(gemm_pair_plan_create(&P.b_o, H, QD, P.ao_hi, P.ao_lo, cap, P.o_out, P.pair_part, e->num_sms));
   if (F > 0) {
-    RC(dmalloc(A, &P.ff_hi, c * F));
-    RC(dmalloc(A, &P.ff_lo, c * F));
+    P.ff_hi = (bf16 *)room;
+    P.ff_lo = P.ff_hi + c * F;
     RC(gemm_plan_create_swiglu(&P.s_gu[0], e->moe_E ? e->w0_gu_d : e->w0_gu, F, H, P.xn_hi, P.xn_lo, SHORT_ROWS, SHORT_ROWS, P.ff_hi, P.ff_lo,
                                e->num_sms));
     RC(gemm_plan_create(&P.s_down[0], e->moe_E ? e->w0_down_d : e->w0_down, H, F, P.ff_hi, P.ff_lo, SHORT_ROWS, SHORT_ROWS, P.down_out, P.ws,
@@ -556,17 +600,16 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
     }
   }
   if (!e->mla) {
-    RC(dmalloc(A, &P.q, c * QD));
+    P.q = P.qkv_out + c * QKVN;
   } else {
-    const size_t hr = (size_t)md.nh * cap;          // rows of the head-major matrices (cap is a multiple of 64)
     const int n_groups = md.nh * (cap / 64);
     RC(dmalloc(A, &P.qn_hi, hr * md.nope));
     RC(dmalloc(A, &P.qn_lo, hr * md.nope));
-    RC(dmalloc(A, &P.q_lat, hr * md.rank));
+    P.q_lat = P.qkv_out + c * QKVN;
+    P.uv_out = P.q_lat + hr * md.rank;
     RC(dmalloc(A, &P.q_rope, c * md.nh * md.rope));
     RC(dmalloc(A, &P.ol_hi, hr * md.rank));
     RC(dmalloc(A, &P.ol_lo, hr * md.rank));
-    RC(dmalloc(A, &P.uv_out, hr * (md.nope + md.vh)));
     RC(dmalloc(A, &P.mla_ml, (size_t)mla_part_ml_floats(MLA_ROWS, md.nh, e->max_ctx) / 2));
     RC(dmalloc(A, &P.mla_po, (size_t)mla_part_o_floats(MLA_ROWS, md.nh, md.rank, e->max_ctx)));
     RC(dmalloc(A, &P.tab_uk, (size_t)n_groups * 3 + 1));
@@ -577,8 +620,6 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
                                 P.ol_lo, n_groups, 64, P.uv_out, P.tab_uv, e->num_sms));
     if (e->big_mla_tiles) {
       P.mla_tiles = true;
-      // at most one request of a chunk began in an earlier one: the others' tokens are rows of the chunk
-      P.kv_cap = (e->max_ctx + cap + 64 * MLA_MAX_SEGS + 255) / 256 * 256;
       const size_t kc = (size_t)P.kv_cap;
       RC(dmalloc(A, &P.c_hi, kc * md.rank));
       RC(dmalloc(A, &P.c_lo, kc * md.rank));
@@ -593,11 +634,11 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
     P.p_uk.keep_div = P.p_uv.keep_div = -1;         // the tables are copied ahead of a chunk's kernels (set_mla_rows)
   }
   if (e->moe_E) {
-    RC(dmalloc(A, &P.moe_w, c * (e->moe_E + e->moe_S)));
+    RC(dmalloc(A, &P.moe_w, c * NB));
     RC(dmalloc(A, &P.router_out, c * e->moe_E));
-    RC(dmalloc(A, &P.moe_mask, (size_t)(e->moe_E + e->moe_S) * (MOE_MANY_ROWS / 32)));
+    RC(dmalloc(A, &P.moe_mask, (size_t)NB * (MOE_MANY_ROWS / 32)));
     RC(gemm_pair_plan_create(&P.b_router, e->moe_E, H, P.xn_hi, P.xn_lo, cap, P.router_out, P.pair_part, e->num_sms));
-    RC(program_create_groups(e, P, cap, 7));
+    RC(program_create_groups(e, P, cap, 7, room));
   }
   return CORUN_OK;
 }

@@ -39,3 +39,35 @@ def test_an_engine_fits_beside_what_is_left_and_gives_the_same_bytes():
     finally:
         del hog
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("experts", [False, True])
+def test_chunks_of_more_rows_take_what_the_rows_need(experts):
+    """A chunk may have 4096 rows where a prompt can have more than 2048 tokens.  What one half of a layer hands on and what the other
+    does share memory, and so do an expert's gathered rows and its results."""
+    import torch
+
+    from paper_2608_14376_b200 import corun
+
+    H, nq, nkv, hd, E, K, Fx = 4096, 32, 8, 128, 128, 16, 512
+    F = 64 if experts else 12288
+    sh = synth.ModelShape(1, H, nq, nkv, hd, F, 4096, 1e-6, 10000.0)
+    w = synth.make_weights_torch(sh, seed=3, dense_ffn=not experts)
+    kw = dict(moe=synth.make_moe_torch(sh, seed=3, n_experts=E, top_k=K, expert_ffn=Fx, n_shared=0, renormalize=True)) if experts else {}
+
+    def used(max_context):
+        gc.collect(); torch.cuda.empty_cache(); torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        eng = corun.Engine(sh, w, 8, max_context, kv_pool_blocks=64, **kw)
+        try:
+            return free - torch.cuda.mem_get_info()[0]
+        finally:
+            eng.close()
+
+    used(2048)                                        # (kernels are loaded)
+    # a row's normalised pair, residual, attention output and output of half a layer; beside them the larger of the projections and
+    # queries, and of the feed-forward's hidden activations or K experts' rows (gathered, then results) with theirs
+    row = 4 * H + 4 * H + 4 * nq * hd + 4 * H + max(4 * (2 * nq + 2 * nkv) * hd, K * 4 * (H + Fx) if experts else 4 * F)
+    # (10 % for tables and partial tiles; apart, the buffers of a row take 1.5 and 1.9 times as much)
+    more = used(4096) - used(2048)
+    assert more <= 1.1 * 2048 * row + (32 << 20), (more, 2048 * row)
