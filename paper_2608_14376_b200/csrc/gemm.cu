@@ -33,25 +33,16 @@ constexpr uint32_t A_BLOCK_BYTES = GEMM_ROW_BLOCK * GEMM_BLOCK_K * 2;      // 16
 // per block of 128 activation rows.
 // MASKED: the optional store mask of the epilogue (a separate instantiation, so that the plain kernel is
 // exactly the code it was without it).
-// SWIGLU: W is a gate / up matrix ([2F, K]: F gate rows, then F up rows).  A tile is sw_half gate rows and the
-// sw_half up rows of the same outputs (two boxes of sw_half rows land in one stage; the MMA's N is 2 * sw_half),
-// every CTA owns whole tiles, and the epilogue writes silu(gate) * up as a bf16 hi/lo pair ([BN, F]) instead of
-// fp32 sums: no partials, no separate SwiGLU kernel.  tmW then has a box of sw_half rows.
-// SWIGLU with MASKED: W is a stack of keep_pitch such matrices (the experts of a Mixture-of-Experts layer: block e =
-// Fb gate rows, then Fb up rows, Fb = N / (2 * keep_pitch)), a tile belongs to one block (keep_div tiles per block),
-// and the epilogue writes row_keep[r, e] * silu(gate) * up, exact zeros where row r did not select block e, to
-// columns e * Fb .. of the bf16 hi/lo output [BN, N / 2].
 // *row_blocks (bit b: rows 128 b .. hold active rows; written by an earlier kernel of the step, or null = both) says which
 // blocks of 128 rows exist this step: an absent block is neither loaded nor multiplied nor stored (its output rows keep what
 // they held: nobody reads rows without a request); with one block left its two accumulator buffers alternate.  A row's value
 // does not depend on which blocks exist.
-template <bool MASKED, bool SWIGLU>
+template <bool MASKED>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmHi,
                     const __grid_constant__ CUtensorMap tmLo, float *__restrict__ direct, float *__restrict__ ws,
                     const int *__restrict__ cta_start, int N, int KB, int BN, int R, int stages, uint32_t idesc,
-                    const float *row_keep, int keep_pitch, int keep_div, int *status, unsigned long long *trace,
-                    __nv_bfloat16 *__restrict__ sw_hi, __nv_bfloat16 *__restrict__ sw_lo, int sw_half, const int *row_blocks) {
+                    const float *row_keep, int keep_pitch, int keep_div, int *status, unsigned long long *trace, const int *row_blocks) {
   extern __shared__ uint8_t smem_raw[];
   // optional per-CTA timeline (debug): 8 globaltimer stamps
 #define TRACE(i) do { if (trace) trace[(size_t)blockIdx.x * 8 + (i)] = globaltimer_ns(); } while (0)
@@ -69,10 +60,7 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   // the hi tiles of both blocks (128 rows each, whatever BN is), then the lo tiles
   const uint32_t lo_off = 2u * A_BLOCK_BYTES;
-  const uint32_t w_tile_bytes = SWIGLU ? (uint32_t)(2 * sw_half * GEMM_BLOCK_K * 2) : W_TILE_BYTES;
-  // SWIGLU: first gate row of a tile, and the distance to the up rows of the same outputs
-  const int sw_fb = (SWIGLU && MASKED) ? N / (2 * keep_pitch) : N / 2;
-  const uint32_t stage_bytes = w_tile_bytes + 4u * A_BLOCK_BYTES;
+  constexpr uint32_t stage_bytes = W_TILE_BYTES + 4u * A_BLOCK_BYTES;
   constexpr int n_rb = 2;                           // blocks of 128 activation rows
   int bmask = 3, n_acc = 1;
   uint32_t tx_bytes = 0;
@@ -80,7 +68,7 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     if (row_blocks) { griddep_wait(); bmask = *reinterpret_cast<const volatile int *>(row_blocks) & 3; }
     if (bmask == 0) bmask = 1;                      // a step without requests: block 0 is computed and ignored
     n_acc = bmask == 3 ? 1 : 2;
-    tx_bytes = w_tile_bytes + (uint32_t)__popc(bmask) * 2 * A_BLOCK_BYTES;
+    tx_bytes = W_TILE_BYTES + (uint32_t)__popc(bmask) * 2 * A_BLOCK_BYTES;
   };
   auto acc_col = [&](int acc, int b) { return (uint32_t)(n_acc == 2 ? acc : b) * GEMM_TILE_N; };
 
@@ -119,14 +107,8 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       const uint64_t pol_w = l2_policy_evict_first();   // weights are streamed once per step
       const uint64_t pol_x = l2_policy_evict_last();    // activations are re-read by every CTA
       auto load_w = [&](uint32_t dst, int tile, int kb, uint32_t fb) {
-        int row0 = tile * GEMM_TILE_N, row1 = row0 + 128;
-        if (SWIGLU) {
-          const int e = MASKED ? tile / keep_div : 0;
-          row0 = e * 2 * sw_fb + (MASKED ? tile - e * keep_div : tile) * sw_half;
-          row1 = row0 + sw_fb;
-        }
-        tma_load_2d(dst, &tmW, kb * GEMM_BLOCK_K, row0, fb, pol_w);
-        tma_load_2d(dst + w_tile_bytes / 2, &tmW, kb * GEMM_BLOCK_K, row1, fb, pol_w);
+        tma_load_2d(dst, &tmW, kb * GEMM_BLOCK_K, tile * GEMM_TILE_N, fb, pol_w);
+        tma_load_2d(dst + W_TILE_BYTES / 2, &tmW, kb * GEMM_BLOCK_K, tile * GEMM_TILE_N + GEMM_W_BOX, fb, pol_w);
       };
       // The weights depend on no earlier kernel: fill the ring with weight tiles first, then wait for
       // the predecessor (which produces the activations) and add the activation tiles to the same
@@ -135,7 +117,7 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       for (int it = 0; it < n_pre; ++it) {
         const int g = k0 + it, tile = g / KB, kb = g - tile * KB;
         const uint32_t fb = smem_u32(&full_bar[it]);
-        mbar_expect_tx(fb, w_tile_bytes);           // the activations' bytes and the arrival follow behind the wait
+        mbar_expect_tx(fb, W_TILE_BYTES);           // the activations' bytes and the arrival follow behind the wait
         load_w(tiles_base + (uint32_t)it * stage_bytes, tile, kb, fb);
         if (it == 0) TRACE(2);
       }
@@ -145,14 +127,14 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
 #pragma unroll
         for (int b = 0; b < 2; ++b)
           if ((bmask >> b) & 1) {
-            tma_load_2d(dst + w_tile_bytes + (uint32_t)b * A_BLOCK_BYTES, &tmHi, kb * GEMM_BLOCK_K, GEMM_ROW_BLOCK * b, fb, pol_x);
-            tma_load_2d(dst + w_tile_bytes + lo_off + (uint32_t)b * A_BLOCK_BYTES, &tmLo, kb * GEMM_BLOCK_K, GEMM_ROW_BLOCK * b, fb, pol_x);
+            tma_load_2d(dst + W_TILE_BYTES + (uint32_t)b * A_BLOCK_BYTES, &tmHi, kb * GEMM_BLOCK_K, GEMM_ROW_BLOCK * b, fb, pol_x);
+            tma_load_2d(dst + W_TILE_BYTES + lo_off + (uint32_t)b * A_BLOCK_BYTES, &tmLo, kb * GEMM_BLOCK_K, GEMM_ROW_BLOCK * b, fb, pol_x);
           }
       };
       for (int it = 0; it < n_pre; ++it) {
         const int g = k0 + it, kb = g % KB;
         const uint32_t fb = smem_u32(&full_bar[it]);
-        mbar_arrive_expect_tx(fb, tx_bytes - w_tile_bytes);
+        mbar_arrive_expect_tx(fb, tx_bytes - W_TILE_BYTES);
         load_x(tiles_base + (uint32_t)it * stage_bytes, kb, fb);
       }
       int it = n_pre;
@@ -191,8 +173,8 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
           const uint64_t w_desc = umma_desc_sw128(w_addr);
           for (int rb = 0; rb < n_rb; ++rb) {
             if (!((bmask >> rb) & 1)) continue;
-            const uint64_t hi_desc = umma_desc_sw128(w_addr + w_tile_bytes + (uint32_t)rb * A_BLOCK_BYTES);
-            const uint64_t lo_desc = umma_desc_sw128(w_addr + w_tile_bytes + lo_off + (uint32_t)rb * A_BLOCK_BYTES);
+            const uint64_t hi_desc = umma_desc_sw128(w_addr + W_TILE_BYTES + (uint32_t)rb * A_BLOCK_BYTES);
+            const uint64_t lo_desc = umma_desc_sw128(w_addr + W_TILE_BYTES + lo_off + (uint32_t)rb * A_BLOCK_BYTES);
             const uint32_t d_tmem = tmem_base + acc_col(acc, rb);
 #pragma unroll
             for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
@@ -229,44 +211,6 @@ gemm_streamk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       const int n0 = tile * GEMM_TILE_N;
       // optional: rows whose entry for this tile's column group is zero are not stored (nobody reads them)
       const float *keep = MASKED ? row_keep + tile / keep_div : nullptr;
-      if (SWIGLU) {
-        // accumulator columns 0 .. sw_half-1: gate sums of outputs tile * sw_half .., the next sw_half columns: the
-        // up sums of the same outputs; every tile is whole
-        const int HALF = sw_half;
-        // F: outputs per block (the whole matrix unless MASKED); f0: the tile's first output inside its block;
-        // o_base: its first column in the output row of N / 2 values; blk: the block (expert) of the tile
-        const int blk = MASKED ? tile / keep_div : 0;
-        const int F = sw_fb, f0 = (MASKED ? tile - blk * keep_div : tile) * HALF;
-        const int o_pitch = N / 2, o_base = blk * F + f0;
-        auto silu_mul = [](float gt, float up) { return __fdividef(gt, 1.f + __expf(-gt)) * up; };
-        for (int rb = 0; rb < n_rb; ++rb) {
-          if (!((bmask >> rb) & 1)) continue;
-          const int row_base = rb * GEMM_ROW_BLOCK + lane_base;
-          if (row_base >= R) continue;                 // warp-uniform
-          const int row = row_base + lane;
-          for (int c0 = 0; c0 < HALF; c0 += 8) {
-            if (f0 + c0 >= F) break;                   // F % 8 == 0
-            uint32_t vg[8], vu[8];
-            const uint32_t ta = tmem_base + ((uint32_t)lane_base << 16) + acc_col(acc, rb) + (uint32_t)c0;
-            tmem_ld8(ta, vg);
-            tmem_ld8(ta + HALF, vu);
-            tmem_ld_wait();
-            if (row >= R) continue;
-            const float wgt = MASKED ? row_keep[(size_t)row * keep_pitch + blk] : 1.f;
-            __nv_bfloat16 a[8], b[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              float y = silu_mul(__uint_as_float(vg[q]), __uint_as_float(vu[q]));
-              if (MASKED) y = wgt != 0.f ? wgt * y : 0.f;
-              a[q] = __float2bfloat16_rn(y);
-              b[q] = __float2bfloat16_rn(y - __bfloat162float(a[q]));
-            }
-            const size_t o = (size_t)row * o_pitch + o_base + c0;
-            *reinterpret_cast<uint4 *>(sw_hi + o) = *reinterpret_cast<const uint4 *>(a);
-            *reinterpret_cast<uint4 *>(sw_lo + o) = *reinterpret_cast<const uint4 *>(b);
-          }
-        }
-      } else
       for (int rb = 0; rb < n_rb; ++rb) {
         if (!((bmask >> rb) & 1)) continue;
         const int row_base = rb * GEMM_ROW_BLOCK + lane_base;
@@ -423,15 +367,14 @@ static int plan_operands(GemmPlan *p, const void *Xhi, const void *Xlo, unsigned
     if ((rc = gemm_rows_stages(p)) != 0) return rc;
     return gemm_encode_x(&p->tmX, Xhi, Xlo, x_rows, p->K);
   }
-  const int n = p->sw_half ? 2 * p->sw_half : GEMM_TILE_N;   // weight rows of a tile
-  const size_t stage = (size_t)n * GEMM_BLOCK_K * 2 + 4 * (size_t)A_BLOCK_BYTES;
+  const size_t stage = W_TILE_BYTES + 4 * (size_t)A_BLOCK_BYTES;
   const int stages = (int)((GEMM_MAX_DYN_SMEM - 1024) / stage);
   p->stages = stages < MAX_STAGES ? stages : MAX_STAGES;
   if (p->stages < 2) return CORUN_EINVAL;
   p->smem_bytes = stage * p->stages + 1024;
   // kind::f16 instruction descriptor: D fp32 (bits 4-5 = 1), A and B bf16 (bits 7-9, 10-12 = 1),
   // both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
-  p->idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GEMM_ROW_BLOCK >> 4) << 24);
+  p->idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GEMM_TILE_N >> 3) << 17) | ((uint32_t)(GEMM_ROW_BLOCK >> 4) << 24);
   if ((rc = gemm_encode_map(&p->tmX.hi[0], Xhi, (int)x_rows, p->K, GEMM_ROW_BLOCK)) != 0) return rc;
   return gemm_encode_map(&p->tmX.lo[0], Xlo, (int)x_rows, p->K, GEMM_ROW_BLOCK);
 }
@@ -530,7 +473,7 @@ int gemm_swiglu_half(int F, int num_sms) {
 
 int gemm_plan_create_swiglu(GemmPlan *p, const void *W, int F, int K, const void *Xhi, const void *Xlo, int R, int BN,
                             __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int num_sms) {
-  if (F <= 0 || F % 8 || K <= 0 || K % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > 256 || R < 1 || R > BN || !out_hi || !out_lo ||
+  if (F <= 0 || F % 8 || K <= 0 || K % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > GEMM_MAX_ROWS || R < 1 || R > BN || !out_hi || !out_lo ||
       num_sms < 1)
     return CORUN_EINVAL;
   // as many whole tiles as there are SMs, if the matrix is large enough: the narrowest tile (a multiple of 8 gate
@@ -581,7 +524,7 @@ int gemm_swiglu_blocks_half(int Fb, int n_blocks, int num_sms) {
 int gemm_plan_create_swiglu_blocks(GemmPlan *p, const void *W, int n_blocks, int Fb, int K, const void *Xhi, const void *Xlo,
                                    int R, int BN, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, const float *row_scale,
                                    int num_sms) {
-  if (n_blocks < 1 || Fb <= 0 || Fb % 8 || K <= 0 || K % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > 256 || R < 1 || R > BN ||
+  if (n_blocks < 1 || Fb <= 0 || Fb % 8 || K <= 0 || K % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > GEMM_MAX_ROWS || R < 1 || R > BN ||
       !out_hi || !out_lo || !row_scale || num_sms < 1)
     return CORUN_EINVAL;
   const int HALF = gemm_swiglu_blocks_half(Fb, n_blocks, num_sms);
@@ -634,15 +577,7 @@ int gemm_plan_create_grouped(GemmPlan *p, const void *W, long long w_rows, int w
   int rc;
   if ((rc = tma_encode_2d(&p->tmW, W, 0, (unsigned long long)w_rows, w_cols, GEMM_W_BOX, GEMM_BLOCK_K)) != 0) return rc;
   if ((rc = plan_operands(p, Xhi, Xlo, (unsigned long long)n_groups * BN)) != 0) return rc;
-  // every CTA's range is exactly one tile
-  std::vector<int> tab((size_t)p->grid + 1);
-  for (int c = 0; c <= p->grid; ++c) tab[(size_t)c] = c * p->KB;
-  int *d_tab = nullptr;
-  if (cudaMalloc(&d_tab, tab.size() * sizeof(int)) != cudaSuccess) return CORUN_ENOMEM;
-  cudaError_t me = cudaMemcpy(d_tab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice);
-  if (me != cudaSuccess) { g_last_cuda_error = (int)me; cudaFree(d_tab); return CORUN_ECUDA; }
-  p->d_cta_start = d_tab;
-  p->d_tile_first = p->d_tile_cend = p->d_split_tiles = nullptr;
+  p->d_cta_start = p->d_tile_first = p->d_tile_cend = p->d_split_tiles = nullptr;   // the kernel derives its tiles itself
   p->n_split_tiles = 0;
   cudaError_t ae = gemm_prepare_kernel();
   if (ae != cudaSuccess) { g_last_cuda_error = (int)ae; return CORUN_ECUDA; }
@@ -698,7 +633,7 @@ int gemm_plan_create_select_down(GemmPlan *p, const void *W, int NB, int N, int 
 
 cudaError_t gemm_prepare_kernel() {
   cudaError_t e = gemm_rows_prepare();
-  for (auto kernel : {gemm_streamk_kernel<false, false>, gemm_streamk_kernel<true, false>, gemm_streamk_kernel<false, true>, gemm_streamk_kernel<true, true>})
+  for (auto kernel : {gemm_streamk_kernel<false>, gemm_streamk_kernel<true>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_MAX_DYN_SMEM);
   return e;
 }
@@ -715,10 +650,9 @@ cudaError_t gemm_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int 
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(p.grid), dim3(GEMM_THREADS), p.smem_bytes, st, pdl, tmW_override ? *tmW_override : p.tmW, p.tmX.hi[0], p.tmX.lo[0],
                     p.direct, p.ws, p.d_cta_start, p.N, p.KB, p.BN, p.R, p.stages, p.idesc, p.row_keep, p.keep_pitch, p.keep_div, d_status, trace,
-                    p.sw_hi, p.sw_lo, p.sw_half, p.row_blocks);
+                    p.row_blocks);
   };
-  if (p.sw_hi) return masked ? go(gemm_streamk_kernel<true, true>) : go(gemm_streamk_kernel<false, true>);
-  return masked ? go(gemm_streamk_kernel<true, false>) : go(gemm_streamk_kernel<false, false>);
+  return masked ? go(gemm_streamk_kernel<true>) : go(gemm_streamk_kernel<false>);
 }
 
 int gemm_plan_rebase(GemmPlan *q, const GemmPlan &p, const void *Xhi, const void *Xlo, float *direct, __nv_bfloat16 *sw_hi,

@@ -213,7 +213,7 @@ int gemm_plan_create_select_up(GemmPlan *p, const void *W, int NB, int F, int K,
                                __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, const float *w, const int *sel, int n_sel, int num_sms);
 int gemm_plan_create_select_down(GemmPlan *p, const void *W, int NB, int N, int F, const void *Xhi, const void *Xlo, int R, int BN,
                                  float *direct, const float *w, const int *sel, int n_sel, int num_sms);
-// Gate / up GEMM with the SwiGLU in its epilogue: W is [2F, K] (F gate rows, then F up rows; F % 8 == 0);
+// Gate / up GEMM with the SwiGLU in its epilogue (BN <= GEMM_MAX_ROWS): W is [2F, K] (F gate rows, then F up rows; F % 8 == 0);
 // out_hi / out_lo [BN, F] receive silu(gate) * up of rows 0 .. R-1 as a bf16 hi/lo pair.  A tile is
 // gemm_swiglu_half(F, num_sms) gate rows with the up rows of the same outputs, and every CTA owns whole tiles
 // (one each when the SMs allow), so there are no partials; a tensor map that overrides the plan's at launch
