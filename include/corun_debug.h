@@ -71,9 +71,18 @@ int corun_debug_gemm(const void *W, int32_t N, int32_t K, const float *X, int32_
  *   form 2  N = 256 heads (per head 128 key rows, then 128 value rows): out [R, N] = X W^T by way of the fp16 hi / lo pairs
  *           that the latent prefill attention reads
  *   form 3, 4  as 0, 1 in the form of a decode step (R <= 256; up to 128 rows: that of a step without requests beyond them)
- * (forms 1, 2 and 4: the sum of the stored pair).  1 <= R <= 2048, K % 64 == 0; pointers as above. */
+ * (forms 1, 2 and 4: the sum of the stored pair).  1 <= R <= 4096, K % 64 == 0; pointers as above. */
 int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, const float *X, int32_t R, float *out,
                           void *cuda_stream);
+/* Stand-alone run of the GEMMs of a prompt's experts: rows[e] rows of X (host array; 0 .. 4096 each, one at least in all) go through
+ * expert e, expert after expert:
+ *   form 0  W [N, n_experts K], N % 128 == 0: out[r, n] = sum_k W[n, e K + k] X[r, k]
+ *   form 1  W [n_experts N, K], N = 2F % 16 == 0: out[r, f] = row_w[r] silu(X Wg^T) (X Wu^T), the sum of the stored bf16 pair; Wg the
+ *           first F rows of the expert's N, Wu the others
+ * X fp32 [rows, K], row_w fp32 [rows] (form 1, else NULL), out fp32 (all device), K % 64 == 0, W on a 16-byte boundary, the others on a
+ * 4-byte one.  What the kernel's blocks of rows hold beyond an expert's rows is NaN. */
+int corun_debug_gemm_experts(int32_t form, const void *W, int32_t n_experts, int32_t N, int32_t K, const int32_t *rows, const float *X,
+                             const float *row_w, float *out, void *cuda_stream);
 /* The attention kernel of long prompts for n query rows at positions pos0 .. pos0 + n - 1 of an occupied slot, over the layer's
  * cached positions 0 .. pos0 + n - 1 (host arrays): q fp32 [n][n_q_heads][head_dim], latent attention [n][n_q_heads][qk_nope +
  * qk_rope], both rotated; out fp32 [n][n_q_heads][head_dim (v_head)], the sum of the stored bf16 pair.  EINVAL where the engine

@@ -20,7 +20,7 @@ EXPORTS = [
     "corun_init", "corun_init_moe", "corun_init_mla", "corun_prefill", "corun_prefill_batch", "corun_decode_step", "corun_decode_enqueue", "corun_decode_wait",
     "corun_release", "corun_destroy", "corun_get_logits", "corun_force_token", "corun_context_len",
     "corun_free_blocks", "corun_debug_kv_read", "corun_debug_kv_write", "corun_debug_adopt",
-    "corun_debug_set_eager", "corun_debug_read", "corun_debug_kv_fill", "corun_debug_time_kernel", "corun_decode_launches", "corun_debug_gemm", "corun_debug_gemm_pair", "corun_debug_prefill_attention", "corun_debug_variate",
+    "corun_debug_set_eager", "corun_debug_read", "corun_debug_kv_fill", "corun_debug_time_kernel", "corun_decode_launches", "corun_debug_gemm", "corun_debug_gemm_pair", "corun_debug_gemm_experts", "corun_debug_prefill_attention", "corun_debug_variate",
     "corun_debug_sample", "corun_debug_wait_probe", "corun_debug_microbench", "corun_debug_check_index", "corun_gemm_static", "corun_strerror", "corun_last_cuda_error", "corun_engine_info",
     "corun_sched_create", "corun_sched_create_for_engine", "corun_sched_destroy", "corun_sched_submit",
     "corun_sched_step", "corun_sched_poll", "corun_sched_slot_of", "corun_sched_counts",
@@ -143,6 +143,7 @@ def lib():
         L.corun_debug_gemm.argtypes = [vp, i32, i32, vp, i32, vp, vp]
         L.corun_prefill_class.argtypes = [vp, i32, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32)]
         L.corun_debug_gemm_pair.argtypes = [i32, vp, i32, i32, vp, i32, vp, vp]
+        L.corun_debug_gemm_experts.argtypes = [i32, vp, i32, i32, i32, vp, vp, vp, vp, vp]
         L.corun_debug_prefill_attention.argtypes = [vp, i32, i32, i32, i32, vp, vp]
         L.corun_debug_variate.argtypes = [u64, u64, C.POINTER(C.c_uint32)]
         L.corun_debug_sample.argtypes = [vp, i32, i32, C.POINTER(Sampling), vp, vp]
@@ -506,6 +507,21 @@ def debug_gemm_pair(form, W, X):
     out = torch.empty((R, N // 2 if form in (1, 4) else N), dtype=torch.float32, device=X.device)
     torch.cuda.synchronize()
     _check(lib().corun_debug_gemm_pair(form, W.data_ptr(), N, K, X.data_ptr(), R, out.data_ptr(), None), "corun_debug_gemm_pair")
+    return out
+
+
+def debug_gemm_experts(form, W, rows, X, row_w=None):
+    """The GEMMs of a prompt's experts (``corun_debug_gemm_experts``), rows[e] rows of X through expert e: form 0 W [N, E K], 1 gate / up
+    with SwiGLU, W [E, 2F, K]."""
+    import torch
+
+    E, K = len(rows), X.shape[1]
+    N = W.shape[1] if form else W.shape[0]
+    out = torch.empty((X.shape[0], N // 2 if form else N), dtype=torch.float32, device=X.device)
+    counts = np.asarray(rows, np.int32)
+    torch.cuda.synchronize()
+    _check(lib().corun_debug_gemm_experts(form, W.data_ptr(), E, N, K, counts.ctypes.data, X.data_ptr(),
+                                          row_w.data_ptr() if row_w is not None else None, out.data_ptr(), None), "corun_debug_gemm_experts")
     return out
 
 

@@ -2179,6 +2179,72 @@ int corun_debug_gemm_pair(int32_t form, const void *W, int32_t N, int32_t K, con
   return rc;
 }
 
+int corun_debug_gemm_experts(int32_t form, const void *W, int32_t n_experts, int32_t N, int32_t K, const int32_t *rows, const float *X,
+                             const float *row_w, float *out, void *cuda_stream) {
+  if (form < 0 || form > 1 || !W || n_experts < 1 || n_experts > 256 || N < 128 || N % (form ? 16 : 128) || K < 64 || K % 64 || !rows || !X || !out ||
+      (form && !row_w))
+    return CORUN_EINVAL;
+  if (((uintptr_t)W & 15u) || ((uintptr_t)X & 3u) || ((uintptr_t)out & 3u) || ((uintptr_t)row_w & 3u)) return CORUN_EINVAL;
+  std::vector<int> tab;                              // per group: first weight row, first weight k-block, rows
+  for (int x = 0; x < n_experts; ++x) {
+    if (rows[x] < 0 || rows[x] > PREFILL_BIG) return CORUN_EINVAL;
+    for (int r = 0; r < rows[x]; r += 128)
+      for (int v : {form ? x * N : 0, form ? 0 : x * (K / GEMM_BLOCK_K), std::min(128, rows[x] - r)}) tab.push_back(v);
+  }
+  const int used = (int)tab.size() / 3, n_groups = used + 1, F = N / 2;   // (one group more than there are)
+  if (!used) return CORUN_EINVAL;
+  tab.insert(tab.end(), {0, 0, 0, used});
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  int dev = 0, sms = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const size_t slots = (size_t)n_groups * 128;
+  std::vector<void *> keep;
+  bf16 *hi = nullptr, *lo = nullptr, *ohi = nullptr, *olo = nullptr;
+  float *full = nullptr, *w = nullptr;
+  int *status = nullptr, *d_tab = nullptr, rc = CORUN_OK;
+  GemmExpertsPlan p;
+  CUtensorMap tw;
+  auto ok = [&](int r) { return (rc = r) == CORUN_OK; };
+  if (ok(dmalloc(keep, &hi, slots * K, false)) && ok(dmalloc(keep, &lo, slots * K, false)) && ok(dmalloc(keep, &w, slots, false)) &&
+      ok(dmalloc(keep, &d_tab, tab.size(), false)) && ok(dmalloc(keep, &status, 1)) &&
+      ok(tma_encode_2d(&tw, W, 0, (unsigned long long)(form ? (long long)n_experts * N : N), form ? K : n_experts * K, GEMM_W_BOX, GEMM_BLOCK_K))) {
+    if (form)
+      ok(dmalloc(keep, &ohi, slots * F)) && ok(dmalloc(keep, &olo, slots * F)) &&
+          ok(gemm_experts_plan_create_swiglu(&p, F, K, hi, lo, n_groups, ohi, olo, w, d_tab, sms));
+    else
+      ok(dmalloc(keep, &full, slots * N)) && ok(gemm_experts_plan_create(&p, N, K, hi, lo, n_groups, full, d_tab, sms));
+  }
+  if (rc == CORUN_OK) {
+    // what a group has no row for is never more than its own column of a product: NaN here
+    cudaError_t ce = cudaMemset(hi, 0xff, slots * K * sizeof(bf16));
+    if (ce == cudaSuccess) ce = cudaMemset(lo, 0xff, slots * K * sizeof(bf16));
+    if (ce == cudaSuccess) ce = cudaMemset(w, 0xff, slots * sizeof(float));
+    if (ce == cudaSuccess) ce = cudaMemcpy(d_tab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess) ce = cudaDeviceSynchronize();   // (all of it through the legacy stream)
+    size_t at = 0;
+    for (int g = 0; g < used && ce == cudaSuccess; at += tab[3 * g++ + 2]) {
+      const int n = tab[3 * g + 2];
+      ce = launch_split(X + at * K, n, K, hi + (size_t)g * 128 * K, lo + (size_t)g * 128 * K, st);
+      if (ce == cudaSuccess && form) ce = cudaMemcpyAsync(w + (size_t)g * 128, row_w + at, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, st);
+    }
+    if (ce == cudaSuccess) ce = gemm_experts_launch(p, tw, status, st);
+    at = 0;
+    for (int g = 0; g < used && ce == cudaSuccess; at += tab[3 * g++ + 2]) {
+      const int n = tab[3 * g + 2];
+      ce = form ? launch_join(ohi + (size_t)g * 128 * F, olo + (size_t)g * 128 * F, false, n, F, out + at * F, F, st)
+                : cudaMemcpyAsync(out + at * N, full + (size_t)g * 128 * N, (size_t)n * N * sizeof(float), cudaMemcpyDeviceToDevice, st);
+    }
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+    int hs = 0;
+    if (ce == cudaSuccess) ce = cudaMemcpy(&hs, status, sizeof(int), cudaMemcpyDeviceToHost);
+    if (ce != cudaSuccess) { g_last_cuda_error = (int)ce; rc = CORUN_ECUDA; }
+    else if (hs != 0) rc = CORUN_ETIMEOUT;
+  }
+  for (void *q : keep) cudaFree(q);
+  return rc;
+}
+
 int corun_debug_prefill_attention(corun_engine *e, int32_t slot, int32_t layer, int32_t pos0, int32_t n, const float *q, float *out) {
   if (!e || !q || !out || pos0 < 0 || n < 1 || layer < 0 || layer >= e->sh.n_layers) return CORUN_EINVAL;
   if (!slot_ok(e, slot) || !e->in_use[slot]) return CORUN_ESLOT;

@@ -142,6 +142,43 @@ def test_decode_pair_gemm_gives_a_row_the_same_bytes_in_both_forms(form, N, K):
     assert torch.equal(corun.debug_gemm_pair(form, W, X[100:200].contiguous()), full[100:200])
 
 
+# rows per expert at the edges of the padded counts (16, 32, 48, 64: two tiles in tensor memory; 80, 96, 128: one), experts of several
+# groups, some without a row.  Weight rows of a tile: 256 in each SM, or 128 gate and their up rows: N and F that end in the first
+# SM of a later tile, inside the second one, and in between
+GROUPS = [[1, 16, 17, 0, 64, 65, 80], [81, 96, 97, 112, 128, 129, 200], [128, 1, 128, 31, 256, 5, 127], [0, 0, 48, 0, 0, 0, 300]]
+
+
+@pytest.mark.parametrize("rows", GROUPS, ids=["few", "many", "mixed", "empty"])
+@pytest.mark.parametrize("form,N,K", [(0, 128, 64), (0, 512, 384), (0, 768, 1408), (0, 896, 192), (0, 2048, 768), (1, 2 * 64, 64), (1, 2 * 200, 256),
+                                      (1, 2 * 384, 768), (1, 2 * 456, 192), (1, 2 * 1408, 2048)])
+def test_experts_of_a_prompt_match_fp64(form, N, K, rows):
+    import torch
+
+    from paper_2608_14376_b200 import corun
+
+    g = torch.Generator(device="cuda").manual_seed(N + K + sum(rows))
+    E, n = len(rows), sum(rows)
+    W = (torch.randn((E, N, K), generator=g, device="cuda") * 0.02).bfloat16()
+    X = torch.randn((n, K), generator=g, device="cuda")
+    row_w = torch.rand((n,), generator=g, device="cuda") + 0.1
+    flat = W if form else W.permute(1, 0, 2).reshape(N, E * K).contiguous()
+    got = corun.debug_gemm_experts(form, flat, rows, X, row_w if form else None)
+    # 16 significand bits of the activations (2.5e-6), sums cut off at each of 4 MMAs per k-block (1.7e-8); with SwiGLU a product of
+    # two such sums, stored as a bf16 pair (2e-6)
+    bound = (2.5e-6 + 4 * 1.7e-8 * K / 64) * (2 if form else 1) + (2e-6 if form else 0) + 5e-7
+    at = 0
+    for e, m in enumerate(rows):                      # expert by expert: a row's error is not hidden among the others'
+        if m == 0:
+            continue
+        y = X[at:at + m].double() @ W[e].double().T
+        if form:
+            y = row_w[at:at + m, None].double() * torch.nn.functional.silu(y[:, :N // 2]) * y[:, N // 2:]
+        off = ((got[at:at + m].double() - y).norm(dim=1) / y.norm(dim=1)).max()
+        assert off <= 2.5 * bound, (e, float(off), bound)       # the worst row: of K = 64 products only, some 1.6 times the mean's error
+        assert float((got[at:at + m].double() - y).norm() / y.norm()) <= bound, e
+        at += m
+
+
 MLA = dict(kv_lora_rank=256, qk_nope=128, qk_rope=32, v_head=128, first_dense=2)
 
 
