@@ -10,10 +10,11 @@ TOL = 3e-3          # as in test_gpu_long_prompt
 
 
 @pytest.mark.parametrize("arch,lens", [("dense", [300, 4096]), ("dense", [4097, 129]), ("moe", [300, 4097]), ("moe", [4500, 140]),
-                                       ("mla", [140, 4097]), ("mla", [129] * 17 + [200])])
+                                       ("mla", [140, 4097]), ("mla", [129] * 17 + [200]), ("mla", [4096 + 100] + [129] * 15 + [200])])
 def test_where_a_chunk_ends_changes_no_byte(orc, arch, lens):
-    """Expert layers: an expert's rows over a whole chunk, more than 64 words of row masks.  Latent attention: as many requests in a
-    chunk as it can hold (129 tokens begin on two tiles of 128 rows)."""
+    """Expert layers: an expert's rows over a whole chunk, more than 64 words of row masks.  Latent attention: chunks
+    full of requests (129 tokens take two tiles of 128 rows), 8 in one of 2048 rows; and as many as 4096 rows can hold, 17: the end of a
+    longer prompt on one tile, 15 on two each, and the beginning of one on the last tile."""
     from paper_2608_14376_b200 import corun
 
     mla = dict(kv_lora_rank=256, qk_nope=128, qk_rope=32, v_head=128, first_dense=1)
@@ -39,6 +40,11 @@ def test_where_a_chunk_ends_changes_no_byte(orc, arch, lens):
     try:
         for s in slots:
             e.prefill(s, prompts[s], res[s])
+        if arch == "mla" and lens[0] > 4096:          # the chunk has 4096 rows: its attention takes that many and no more
+            q = np.zeros((4097, 4, 160), np.float32)
+            e.prefill_attention(0, 0, 0, q[:4096])
+            with pytest.raises(corun.CorunError):
+                e.prefill_attention(0, 0, 0, q)
         for s in slots:
             if lens[s] <= 300 and s < 3:
                 r = orc.Request(model, prompts[s], 1, max_T=lens[s] + 2)

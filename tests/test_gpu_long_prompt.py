@@ -1,5 +1,5 @@
-"""Prefill of prompts beyond the small chunk: the projections on pairs of SMs, chunks of up to 2048 rows, at the edges of
-their tiles (256 rows, 128 per SM, 32 per store) and of the chunk."""
+"""Prefill of prompts beyond the small chunk: the projections on pairs of SMs, at the edges of their tiles (256 rows,
+128 per SM, 32 per store).  The chunks have 2048 rows, 2304 where a prompt has 2049 tokens (test_gpu_chunk_edges: 4096)."""
 import numpy as np
 import pytest
 
@@ -61,7 +61,7 @@ def test_long_prompts_alone_and_sharing_chunks(tiny, lens):
 @pytest.mark.parametrize("lens", [[257, 30, 383], [2049, 300]])
 def test_long_prompts_through_expert_layers(orc, arch, lens):
     """The same for decoders with expert layers (rows grouped by expert over a whole chunk; 2049 tokens: several groups of an
-    expert, and a chunk of one row behind a full one) and for latent attention (blocks of 64 rows per head)."""
+    expert, one row on a tile of its own) and for latent attention (blocks of 64 rows per head)."""
     from paper_2608_14376_b200 import corun
 
     B = 4
