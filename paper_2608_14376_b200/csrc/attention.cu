@@ -60,20 +60,20 @@ __device__ __forceinline__ void split_half(float x, __half &hi, __half &lo) {
   lo = __float2half_rn(x - __half2float(hi));
 }
 
-// Combines the splits of 64 output dims (the d0-th and on) of one (row, head) by one warp.  Lanes first hold one split each (max by
+// Combines the splits of 64 output dims (the dim0-th and on) of one (row, head) by one warp.  Lanes first hold one split each (max by
 // butterfly, which is exact; the denominator by a fixed butterfly over at most 32 lanes, then
 // ascending chunks of 32), then every lane owns two output dims and adds the splits' weighted
 // partial outputs in ascending split order, 32 of them in flight.  Output: bf16 hi/lo pair for the O projection.
 // The partials may come from other SMs: they are read past the L1 cache.
 template <int HD>
-__device__ __forceinline__ void attn_combine_pair(int r, int j, int d0, int nsplit, int nq, int max_splits,
+__device__ __forceinline__ void attn_combine_pair(int r, int j, int dim0, int nsplit, int nq, int max_splits,
                                                   const float *__restrict__ part_acc, const float *__restrict__ part_ml,
                                                   __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo,
                                                   int lane) {
   constexpr int FLY = 32;                        // partial outputs in flight
   float o[2] = {0.f, 0.f};
   const float2 *ml = reinterpret_cast<const float2 *>(part_ml) + ((size_t)r * nq + j) * max_splits;
-  const float *pa = part_acc + ((size_t)r * nq + j) * max_splits * HD + d0 + lane * 2;
+  const float *pa = part_acc + ((size_t)r * nq + j) * max_splits * HD + dim0 + lane * 2;
   auto load_acc = [&](int s) { return s < nsplit ? __ldcg(reinterpret_cast<const float2 *>(pa + (size_t)s * HD)) : make_float2(0.f, 0.f); };
   auto add_acc = [&](const float2 &a, float ws) { o[0] = fmaf(a.x, ws, o[0]); o[1] = fmaf(a.y, ws, o[1]); };
   float den = 0.f;
@@ -135,7 +135,7 @@ __device__ __forceinline__ void attn_combine_pair(int r, int j, int d0, int nspl
     }
   }
   const float y0 = o[0] / den, y1 = o[1] / den;
-  const size_t idx = (size_t)r * nq * HD + (size_t)j * HD + d0 + lane * 2;
+  const size_t idx = (size_t)r * nq * HD + (size_t)j * HD + dim0 + lane * 2;
   const __nv_bfloat16 h0 = __float2bfloat16_rn(y0), h1 = __float2bfloat16_rn(y1);
   *reinterpret_cast<__nv_bfloat162 *>(out_hi + idx) = __halves2bfloat162(h0, h1);
   *reinterpret_cast<__nv_bfloat162 *>(out_lo + idx) =

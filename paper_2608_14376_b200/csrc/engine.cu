@@ -85,8 +85,8 @@ struct Program {
   RouterScratch router_rs{};
   // selected-experts form (decode up to 64 rows): only the experts that a row selected are streamed; p_gug / p_dng are its
   // GEMMs, hg / yg hold [expert][BN] rows, moe_sel every row's experts.  Measured per step, 12 layers of the Qwen3-30B-A3B
-  // shape, against every row through every expert: 1 row of 1 3.15 -> 1.24 ms, 16 of 32 3.54 -> 2.72, 40 of 64
-  // 3.94 -> 3.87, 64 of 64 (nearly all experts selected) 4.26 -> 4.28.
+  // shape, against every row through every expert: 1 row of 1 2.84 -> 0.99 ms, 8 of 8 2.95 -> 1.72, 16 of 32 3.05 -> 2.38, 20 of 64
+  // 3.28 -> 2.60, 40 of 64 3.50 -> 3.44, 64 of 64 (nearly all experts selected) 3.76 -> 3.95.
   bool select = false;
   int *moe_sel = nullptr;
   // grouped form of the experts' GEMMs: the rows of an expert gathered into blocks of 64 (prompts: of 128, on pairs of SMs)
@@ -143,11 +143,12 @@ struct Program {
 };
 
 // Prompts of up to PREFILL_SMALL tokens are short (Program::shorts), longer ones long.  Which one depends on the prompt's
-// own length only, so a prompt's values do not depend on what is prefilled with it.  Measured, GEMMs of the Qwen3-8B layer:
-// 64 rows 82 us and 128 rows 110 us in a block of SHORT_ROWS; 256 rows 179 us (two blocks: 220), 512 rows 299, 1024 rows
-// 543, 2048 rows 1049 on pairs of SMs (hence chunks as large as the buffers allow; PREFILL_BIG 2048 -> 4096, that is one pass over
-// the experts and not two: 2505 tokens through 9 DeepSeek-V2-Lite layers 13.6 -> 10.9 ms; 6001 tokens through 12 Qwen3-8B layers
-// 54.3 -> 54.0, where the products are bound by the tensor cores).
+// own length only, so a prompt's values do not depend on what is prefilled with it.  Prompts of 65 / 96 / 128 / 160 / 192 / 256 tokens
+// through 12 Qwen3-8B layers: 1.63 / 1.75 / 2.0 / 3.1 / 3.25 / 3.75 ms in blocks of SHORT_ROWS, 2.55 / 2.43 / 2.56 / 2.6 / 2.7 / 2.8 on
+// pairs of SMs.  There GEMMs of a Qwen3-8B layer take 299 us for 512 rows, 543 for 1024 and 1049 for 2048, hence chunks as large as the
+// buffers allow.  PREFILL_BIG 2048 -> 4096: 3000 tokens through 12 Qwen3-30B-A3B layers 15.1 -> 12.7 ms, 2505 through 9 DeepSeek-V2-Lite
+// layers 12.1 -> 9.9 (one pass over the experts and not two); prompts one behind the other through 12 Qwen3-8B layers, 2500 / 4096 /
+// 6001 tokens 21.9 / 34.5 / 53.3 -> 20.3 / 33.8 / 52.7.
 constexpr int PREFILL_SMALL = 128, PREFILL_BIG = 4096;
 // Rows of a long prompt's chunk that the latent attention takes at a time (its partial results are kept per row).
 constexpr int MLA_ROWS = 256;
@@ -638,7 +639,7 @@ int program_create_big(corun_engine *e, Program &P, int cap) {
     RC(dmalloc(A, &P.router_out, c * e->moe_E));
     RC(dmalloc(A, &P.moe_mask, (size_t)NB * (MOE_MANY_ROWS / 32)));
     RC(gemm_pair_plan_create(&P.b_router, e->moe_E, H, P.xn_hi, P.xn_lo, cap, P.router_out, P.pair_part, e->num_sms));
-    RC(program_create_groups(e, P, cap, 7, room));
+    RC(program_create_groups(e, P, cap, 7, room));  // (groups of 128 rows: an expert with fewer pays for those it has)
   }
   return CORUN_OK;
 }
@@ -1318,9 +1319,8 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   }
 #endif
   // expert layers of the decode program: above 64 padded rows the grouped form (an expert's rows gathered into blocks of
-  // 64: one MMA per k-slice covers the hi and lo halves of a block, where every row through every expert costs two on
-  // 128 rows and keeps the tensor pipe as busy as the weight stream); up to 64 rows the experts that a row
-  // selected (Program::select), each for all rows of the step
+  // 64, of which as many are multiplied as there are, where every row through every expert keeps the tensor pipe as busy as the
+  // weight stream); up to 64 rows the experts that a row selected (Program::select), each for all rows of the step
   const bool dec_grouped = e->moe_E > 0 && pad16(B) > 64 && !getenv("CORUN_MOE_DECODE_DENSE");
   if ((rc = program_create(e, e->dec, B, true, true, dec_grouped, true))) return fail(rc);
   // the decode step's first kernel says which blocks of rows hold a request (64 rows each up to 128 padded rows, 128

@@ -1,11 +1,11 @@
-// Decode / prefill-chunk GEMM  out[r, n] = sum_k W[n, k] * (Xhi[r, k] + Xlo[r, k]).
+// GEMMs of decode steps and prefill chunks  out[r, n] = sum_k W[n, k] * (Xhi[r, k] + Xlo[r, k]).
 //
-// The rows of activations (up to 256, in blocks of 128) are the M operand of
-// the MMA and a tile of 256 weight rows is its N operand, so every tcgen05.mma
-// is a full-size 128 x 256 x 16 instruction whatever the row count; one fixed
-// tiling serves every row count.  The flat space of (weight tile, 64-wide k-block) pairs is cut
-// into one contiguous, equally sized range per CTA; the cut depends on the
-// shape (N, K) and the grid only, never on which rows are occupied.  A tile
+// Up to GEMM_MAX_ROWS padded rows (gemm_rows.cu) a tile of 128 or 256 weight rows is the M operand of the MMAs and the rows there are
+// (hi, then lo) the N operand; above (gemm.cu) blocks of 128 rows are the M operand and a tile of 256 weight rows the N operand;
+// prompts and decode steps of many slots run on pairs of SMs (gemm_pair.cu, gemm_experts.cu, below).
+//
+// The flat space of (weight tile, 64-wide k-block) pairs is cut into one contiguous range per CTA.  The cut depends on the shape
+// (N, K), on the padded rows by way of the tile's width, and on the SM count, never on which rows are occupied.  A tile
 // whose k-blocks all belong to one CTA is written straight to `direct`;
 // otherwise each CTA writes a partial to its workspace slot and the consumer
 // adds the partials in ascending CTA order (gemm_load).  No atomics anywhere.
@@ -20,8 +20,8 @@ namespace corun {
 // Last CUDA runtime error (cudaError_t), or 100000 + CUresult for driver calls.
 extern int g_last_cuda_error;
 
-constexpr int GEMM_TILE_N = 256;   // weight rows per tile (the MMA's N)
-constexpr int GEMM_ROW_BLOCK = 128; // activation rows per MMA (the MMA's M)
+constexpr int GEMM_TILE_N = 256;   // weight rows per tile (up to GEMM_NARROW_ROWS padded rows: half)
+constexpr int GEMM_ROW_BLOCK = 128; // (above GEMM_MAX_ROWS) activation rows per MMA (the MMA's M)
 constexpr int GEMM_BLOCK_K = 64;   // bf16 elements per k-block (= one 128-byte swizzle row)
 constexpr int GEMM_MAX_SELECT = 288;  // experts of a selected-experts GEMM
 constexpr int GEMM_W_BOX = 128;    // weight rows per TMA box
@@ -34,14 +34,14 @@ constexpr int GEMM_THREADS = 192;  // (above GEMM_MAX_ROWS) warp 0 TMA producer,
 // What a consumer kernel needs to read a GEMM result.
 struct GemmOut {
   const float *direct;   // [rows, N]; valid for tiles owned by one CTA
-  const float *ws;       // [(cta*2 + slot), BN, 256] partials
+  const float *ws;       // [(cta*2 + slot), BN, 1 << tile_shift] partials
   const int *tile_first; // [n_tiles] 2 * (first CTA touching the tile) + (the slot that CTA used for it)
   const int *tile_cend;  // [n_tiles] last CTA touching the tile (every later CTA used slot 0)
   int N, KB, BN;
   // Result of gemm_pair.cu (row_tiles > 0): tiles [256 rows x 256 columns], row tiles fastest; the first `whole` are in
   // `direct`, the others in `ws`, tile after tile as `slices` partial tiles [256][256].
   int row_tiles, whole, slices;
-  int tile_shift = 8;    // log2 of the tile's columns: partials are [(cta*2 + slot), BN, 1 << tile_shift]
+  int tile_shift = 8;    // log2 of the tile's columns
 };
 
 // Values of a gemm_pair.cu result, the slices added in ascending order.
@@ -158,7 +158,7 @@ struct GemmPlan {
   // row_keep[r * keep_pitch + t / keep_div] != 0 (rows that no consumer will read are skipped).
   const float *row_keep = nullptr;
   int keep_pitch = 0, keep_div = 1;
-  // Grouped mode (gemm_plan_create_grouped): the CTAs take the (group, weight tile) pairs in turn; see gemm.cu.
+  // Grouped mode (gemm_plan_create_grouped): the CTAs take the (group, weight tile) pairs in turn; see gemm_rows.cu.
   const int *group_tab = nullptr;    // device, not owned: per group (first weight row, first weight k-block, rows),
                                      // then ONE more int: the number of groups in use (the first ones);
                                      // keep_div = -1 tells the kernel that no kernel of the same stream writes it

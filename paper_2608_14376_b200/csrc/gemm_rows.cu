@@ -57,7 +57,8 @@ struct GemmRowsArgs {
 //   consumer will read are skipped).
 // SWIGLU: W is a gate / up matrix ([2F, K]); a tile is w_rows gate rows and the up rows of the same outputs as the two blocks
 //   (fewer than 128, or 64, rows are loaded of each: the other lanes hold meaningless values that are never read back; up to 64 rows the
-//   MMAs read 64, half the shared memory that bounds them at few activation rows), every CTA owns whole tiles, and the epilogue writes silu(gate) * up as a bf16 hi / lo pair.
+//   MMAs read 64, half the shared memory that bounds them at few activation rows), every CTA owns whole tiles, and the epilogue writes
+//   silu(gate) * up as a bf16 hi / lo pair.
 // SWIGLU with MASKED: a stack of keep_pitch such matrices (keep_div tiles each); times row_keep[r, block], exact zeros where it is zero.
 // GROUPED: a tile belongs to one group: group_tab holds, per group, the first weight row, the first weight k-block and the rows
 //   in use, and behind its keep_pitch entries the number of groups in use (the first ones); the CTAs take the tiles of those
@@ -363,7 +364,8 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const int blk = MASKED ? tile / a.keep_div : 0;
         const int f0 = (GROUPED ? g_j : MASKED ? tile - blk * a.keep_div : tile) * a.w_rows;
         const int w0 = m64 ? lane_base / 2 : lane_base, f = f0 + w0 + lane, o_pitch = N / 2, col = blk * sw_fb + f;   // w0: this warp's first weight row
-        const bool f_ok = w0 + lane < a.w_rows && f < sw_fb && (!m64 || lane < 16);   // (F, the matrix and w_rows are multiples of 8: the same for both lanes of a pair)
+        // (F, the matrix and w_rows are multiples of 8: the same for both lanes of a pair)
+        const bool f_ok = w0 + lane < a.w_rows && f < sw_fb && (!m64 || lane < 16);
         const int row0 = GROUPED ? g_id * BN : 0;
         const uint32_t tg = t_lane + mt_col(half, 0), tu = t_lane + mt_col(half, 1);
         if (w0 < a.w_rows) {

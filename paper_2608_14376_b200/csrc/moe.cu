@@ -724,9 +724,9 @@ int corun_moe_create(const corun_moe_shape *shape, const void *router, const voi
     m->p_gu.keep_pitch = NB;
     m->p_gu.keep_div = 2 * F / GEMM_TILE_N;
   }
-  // above 64 padded rows: the grouped form (one MMA per k-slice covers the hi and lo halves of a block of 64 rows,
-  // where every row through every expert costs two on 128 rows), with the routing weight and the SwiGLU in the
-  // per-group gate / up GEMM's epilogue
+  // above 64 padded rows: the grouped form (an expert's rows gathered into blocks of 64, of which as many are multiplied as there
+  // are; every row through every expert would be (E + S) / (top_k + S) times the MMA work), with the routing weight and the SwiGLU in
+  // the per-group gate / up GEMM's epilogue
   const int g_half = gemm_swiglu_blocks_half(F, NB, m->num_sms);
   if (m->BN > 64 && g_half > 0 && H % GEMM_TILE_N == 0 && !getenv("CORUN_MOE_DECODE_DENSE")) {
     MoeGroups &g = m->grp;

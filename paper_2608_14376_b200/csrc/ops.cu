@@ -1035,7 +1035,7 @@ cudaError_t launch_resid_norm(float *h, int H, const __nv_bfloat16 *embed, const
                               cudaStream_t st, bool many) {
   GemmOut g{};
   if (prev) g = *prev;
-  if (many && H <= 16 * NORM_MANY_THREADS) {
+  if (many && H <= 16 * NORM_MANY_THREADS) {         // (what the 64 registers a thread of four CTAs per SM hold: 16 values and 16 to add)
     const int V = (H + 4 * NORM_MANY_THREADS - 1) / (4 * NORM_MANY_THREADS);
     auto go = [&](auto kernel) {
       return launch_k(kernel, dim3(rows.R), dim3(NORM_MANY_THREADS), 0, st, true, h, H, embed, rows, g, prev ? 0 : 1, gains, eps, out_hi, out_lo);
