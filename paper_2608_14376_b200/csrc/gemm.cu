@@ -4,7 +4,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <cmath>
 #include <cstdlib>
 #include <vector>
 
@@ -385,16 +384,15 @@ int gemm_plan_fill(GemmPlan *p, const void *W, int N, int K, const void *Xhi, co
                    float *direct, float *ws, int num_sms, int *tab, int tab_cap, int *tab_ints) {
   if (N <= 0 || K <= 0 || K % GEMM_BLOCK_K || BN % 16 || BN < 16 || BN > 256 || R < 1 || R > BN) return CORUN_EINVAL;
   p->N = N; p->K = K; p->R = R; p->BN = BN;
-  p->tile_n = BN <= GEMM_NARROW_ROWS ? GEMM_TILE_N / 2 : GEMM_TILE_N;
   p->KB = K / GEMM_BLOCK_K;
   // With several CTAs per tile the ranges are cut tile by tile (the same number of CTAs for every tile, a few
   // SMs left out): no CTA then crosses a tile boundary, so none has two epilogues in a row, and above 128
   // rows -- where the two row blocks of a tile fill TMEM and the epilogue of a segment cannot overlap the MMAs
   // of the next -- none stops in the middle of its range.
   // At least four k-blocks per CTA: with fewer, the consumer's extra partials cost more than the shorter stream saves.
-  struct Cut { int n_tiles, grid, per_tile; };
+  struct Cut { int tile_n, n_tiles, grid, per_tile; };
   auto cut = [&](int tile_n) {
-    Cut c{(N + tile_n - 1) / tile_n, 0, 0};
+    Cut c{tile_n, (N + tile_n - 1) / tile_n, 0, 0};
     const long long total = (long long)c.n_tiles * p->KB;
     c.grid = (int)(total < num_sms ? total : num_sms);
     c.per_tile = c.grid >= 2 * c.n_tiles ? c.grid / c.n_tiles : 0;
@@ -402,18 +400,19 @@ int gemm_plan_fill(GemmPlan *p, const void *W, int N, int K, const void *Xhi, co
     if (c.per_tile) c.grid = c.per_tile * c.n_tiles;
     return c;
   };
-  const Cut own = cut(p->tile_n);
+  // Up to GEMM_NARROW_ROWS rows a tile is half as wide where a CTA's share of K does not grow with it: whole tiles, and matrices so small
+  // that the four k-blocks bound it, which twice the CTAs then stream (a step of one row of a decoder of width 1024 483 us, 489 in wide
+  // tiles).  Elsewhere half as many CTAs would share a tile's K and an accumulator sum twice the k-blocks, and it cuts every sum off
+  // (gemm_pair.cu): sums of positive products of 6144 x 4096 / 4096 x 12288 2.5e-6 / 7.9e-6 off 64 bits instead of 9.9e-7 / 2.5e-6.  Nor is
+  // that faster: 8 rows of Qwen3-8B's QKV, O and down 11.15 / 9.4 / 18.65 us in narrow tiles, 9.85 / 8.05 / 16.95 in wide ones.
+  const Cut wide = cut(GEMM_TILE_N), narrow = cut(GEMM_TILE_N / 2);
+  auto share = [&](const Cut &c) { return std::min((double)p->KB, c.per_tile ? (double)p->KB / c.per_tile : (double)c.n_tiles * p->KB / c.grid); };
+  const Cut own = BN <= GEMM_NARROW_ROWS && share(narrow) <= share(wide) ? narrow : wide;
+  p->tile_n = own.tile_n;
   p->n_tiles = own.n_tiles;
   p->grid = own.grid;
   const int per_tile = own.per_tile;
   const long long total = (long long)p->n_tiles * p->KB;
-  if (p->tile_n < GEMM_TILE_N) {
-    // as many accumulators as an accumulator of a wide tile goes into a CTA's share of K, one for K as a whole
-    const Cut wide = cut(GEMM_TILE_N);
-    auto longest = [&](const Cut &c) { return std::min((double)p->KB, c.per_tile ? (double)p->KB / c.per_tile : (double)c.n_tiles * p->KB / c.grid); };
-    const int runs = std::min(GEMM_MAX_RUNS, std::max(1, (int)std::ceil(longest(own) / longest(wide) - 1e-9)));
-    if (runs > 1) p->run_kb = ((int)std::ceil(longest(own)) + runs - 1) / runs;
-  }
   if (total * (long long)p->grid >= (1ll << 31)) return CORUN_EINVAL;
   p->direct = direct;
   p->ws = ws;

@@ -20,14 +20,13 @@ namespace corun {
 // Last CUDA runtime error (cudaError_t), or 100000 + CUresult for driver calls.
 extern int g_last_cuda_error;
 
-constexpr int GEMM_TILE_N = 256;   // weight rows per tile (up to GEMM_NARROW_ROWS padded rows: half)
+constexpr int GEMM_TILE_N = 256;   // weight rows per tile (up to GEMM_NARROW_ROWS padded rows: or half)
 constexpr int GEMM_ROW_BLOCK = 128; // (above GEMM_MAX_ROWS) activation rows per MMA (the MMA's M)
 constexpr int GEMM_BLOCK_K = 64;   // bf16 elements per k-block (= one 128-byte swizzle row)
 constexpr int GEMM_MAX_SELECT = 288;  // experts of a selected-experts GEMM
 constexpr int GEMM_W_BOX = 128;    // weight rows per TMA box
 constexpr int GEMM_MAX_ROWS = 128; // padded rows up to which gemm_rows.cu has the kernel
-constexpr int GEMM_NARROW_ROWS = 32;  // padded rows up to which a tile is 128 weight rows
-constexpr int GEMM_MAX_RUNS = 4;   // accumulators of a narrow tile's segment
+constexpr int GEMM_NARROW_ROWS = 32;  // padded rows up to which a tile may be 128 weight rows
 constexpr int GEMM_ROWS_MAX_SMEM = 224 * 1024;
 constexpr int GEMM_THREADS = 192;  // (above GEMM_MAX_ROWS) warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue
 
@@ -146,7 +145,6 @@ struct GemmPlan {
   int N = 0, K = 0, R = 0, BN = 0;   // weight rows, reduction length, real rows, padded rows
   int tile_n = GEMM_TILE_N;          // weight rows per tile (without SwiGLU)
   int n_tiles = 0, KB = 0, grid = 0, stages = 0;
-  int run_kb = 1 << 30;              // k-blocks that one accumulator sums (narrow tiles whose CTAs' shares are longer than a wide tile's)
   uint32_t idesc = 0, stage_bytes = 0;
   size_t smem_bytes = 0;
   float *direct = nullptr;           // not owned

@@ -14,7 +14,6 @@ namespace {
 constexpr int GR_THREADS = 320;                     // warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue
 constexpr int GR_MAX_STAGES = 11;
 constexpr uint32_t GR_W_BYTES = 128 * GEMM_BLOCK_K * 2;      // 16 KiB: what one MMA reads of the weights
-static_assert(GEMM_MAX_RUNS * 2 * GEMM_NARROW_ROWS <= 256, "a narrow tile's accumulators fit half of tensor memory");
 
 struct GemmRowsArgs {
   float *direct, *ws;
@@ -29,7 +28,6 @@ struct GemmRowsArgs {
   unsigned long long *trace;
   __nv_bfloat16 *sw_hi, *sw_lo;
   const int *row_blocks;
-  int run_kb;
 };
 
 // out[r, n] = sum_k W[n, k] * (Xhi[r, k] + Xlo[r, k]).
@@ -41,17 +39,11 @@ struct GemmRowsArgs {
 // proportional to the rows there are: they are counted on the device (row_blocks bits 8 .., or the group's rows).  With the
 // rows as the M operand (128 lanes whatever there is, and a tile's end of 256 columns through shared memory) the end of a tile took
 // 2.9 us at 8 rows of 16; here a warp stores its 32 weight rows' value of one activation row as one 128-byte segment.
-// tile_n = 128 up to 32 padded rows: half as many partial sums per output for the same number of CTAs.
+// tile_n = 128 up to 32 padded rows where that leaves a CTA's share of K as it is (gemm_plan_fill).
 //
 // The flat space of (tile, k-block) pairs is cut into one contiguous range per CTA, a function of (N, K, SM count); role loops
 // walk the range segment by segment (the part of the range that falls into one tile).  hi and lo have an accumulator each, added
 // at the end; K ascending.  A row's result depends neither on its place nor on the other rows.
-//
-// An accumulator cuts every sum off (gemm_pair.cu).  A narrow tile has half as many CTAs to share its K, so a segment of it is summed
-// in up to GEMM_MAX_RUNS accumulators of run_kb k-blocks, 64 columns (32 padded rows) apart, added in ascending order in fp32: none sums
-// more than one of a wide tile does.  Sums of positive products off 64 bits (N x K, wide tile / narrow with one accumulator / so):
-// 6144 x 4096 9.9e-7 / 2.5e-6 / 9.9e-7, 4096 x 4096 5.3e-7 / 1.5e-6 / 4.1e-7, 4096 x 12288 2.5e-6 / 7.9e-6 / 1.5e-6; normal products of
-// 4096 x 12288, with the activations' 2.5e-6, 2.8e-6 / 4.1e-6 / 2.6e-6.
 //
 // MASKED: row r of tile column n is stored only where row_keep[r * keep_pitch + (n / 256) / keep_div] != 0 (rows that no
 //   consumer will read are skipped).
@@ -67,9 +59,7 @@ struct GemmRowsArgs {
 // SELECT (with GROUPED; the experts of up to 64 rows): the groups are the experts that at least one row selected, all rows of the
 //   step together.  group_tab holds keep_div ints, the selected experts of every row (< 0: none); every CTA makes the ascending
 //   list of them itself.  row_keep: routing weights [rows][keep_pitch]; only rows that selected the expert are stored.
-// RUNS: several accumulators per segment.  An instantiation of its own: 8 rows of the Qwen3-8B QKV, O and down products 11.1 / 9.4 / 18.6
-//   us with one accumulator, 11.25 / 9.5 / 18.8 so.
-template <bool MASKED, bool GROUPED, bool SWIGLU, bool SELECT, bool RUNS = false>
+template <bool MASKED, bool GROUPED, bool SWIGLU, bool SELECT>
 __global__ void __launch_bounds__(GR_THREADS, 1)
 gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ GemmXMaps tmX, const __grid_constant__ GemmRowsArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -289,18 +279,9 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         tc_fence_after();
         // kind::f16: D fp32 (bits 4-5 = 1), A and B bf16 (bits 7-9, 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_pad >> 2) << 17) | ((uint32_t)((m64 ? 64 : 128) >> 4) << 24);
-        const uint32_t d1 = tmem_base + mt_col(half, 1);
-        uint32_t d0 = tmem_base + mt_col(half, 0), more = 0;
-        int left = a.run_kb;
+        const uint32_t d0 = tmem_base + mt_col(half, 0), d1 = tmem_base + mt_col(half, 1);
+        uint32_t more = 0;
         for (int kb = kb_begin; kb < kb_end; ++kb) {
-          if (RUNS) {                               // the next accumulator
-            if (left == 0) {
-              left = a.run_kb;
-              d0 += 64;
-              more = 0;
-            }
-            --left;
-          }
           if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_p)) { fail = DEV_TIMEOUT_MMA; break; }
           if (g == k0 && kb == kb_begin) TRACE(4);
           tc_fence_after();
@@ -421,22 +402,6 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           tmem_ld8(ta, h);
           tmem_ld8(ta + (uint32_t)n_pad, l);
           tmem_ld_wait();
-          if (RUNS) {                               // (rolled: it runs once, from a cold instruction cache)
-            uint32_t at_run = ta;
-#pragma unroll 1
-            for (int left = kb_end - kb_begin - a.run_kb; left > 0; left -= a.run_kb) {
-              uint32_t x[8], y[8];
-              at_run += 64;
-              tmem_ld8(at_run, x);
-              tmem_ld8(at_run + (uint32_t)n_pad, y);
-              tmem_ld_wait();
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {         // h: the sum so far, l: the accumulator that is added next
-                h[j] = __float_as_uint(__uint_as_float(h[j]) + __uint_as_float(l[j]));
-                l[j] = __float_as_uint(__uint_as_float(x[j]) + __uint_as_float(y[j]));
-              }
-            }
-          }
           uint32_t on = rows_on(c, SELECT ? g_id : MASKED ? n0 / GEMM_TILE_N / a.keep_div : 0);
           if (n0 + at >= N) on = 0;
           float *d = dst + (size_t)(8 * c) * pitch + at;
@@ -469,8 +434,6 @@ template <typename F>
 cudaError_t each_kernel(F f) {
   cudaError_t e = f(gemm_rows_kernel<false, false, false, false>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<true, false, false, false>);
-  if (e == cudaSuccess) e = f(gemm_rows_kernel<false, false, false, false, true>);
-  if (e == cudaSuccess) e = f(gemm_rows_kernel<true, false, false, false, true>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<false, false, true, false>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<true, false, true, false>);
   if (e == cudaSuccess) e = f(gemm_rows_kernel<false, true, false, false>);
@@ -513,7 +476,7 @@ cudaError_t gemm_rows_prepare() {
 cudaError_t gemm_rows_launch(const GemmPlan &p, const CUtensorMap *tmW_override, int *d_status, cudaStream_t st, unsigned long long *trace,
                              bool pdl) {
   const GemmRowsArgs a{p.direct, p.ws, p.d_cta_start, p.N, p.KB, p.BN, p.R, p.stages, p.tile_n, p.sw_half ? p.sw_half : 128, p.stage_bytes,
-                       p.row_keep, p.keep_pitch, p.keep_div, p.group_tab, p.tiles_per_group, d_status, trace, p.sw_hi, p.sw_lo, p.row_blocks, p.run_kb};
+                       p.row_keep, p.keep_pitch, p.keep_div, p.group_tab, p.tiles_per_group, d_status, trace, p.sw_hi, p.sw_lo, p.row_blocks};
   auto go = [&](auto kernel) {
     return launch_k(kernel, dim3(p.grid), dim3(GR_THREADS), p.smem_bytes, st, pdl, tmW_override ? *tmW_override : p.tmW, p.tmX, a);
   };
@@ -521,7 +484,6 @@ cudaError_t gemm_rows_launch(const GemmPlan &p, const CUtensorMap *tmW_override,
   if (p.select) return p.sw_hi ? go(gemm_rows_kernel<false, true, true, true>) : go(gemm_rows_kernel<false, true, false, true>);
   if (p.group_tab) return p.sw_hi ? go(gemm_rows_kernel<false, true, true, false>) : go(gemm_rows_kernel<false, true, false, false>);
   if (p.sw_hi) return masked ? go(gemm_rows_kernel<true, false, true, false>) : go(gemm_rows_kernel<false, false, true, false>);
-  if (p.run_kb < p.KB) return masked ? go(gemm_rows_kernel<true, false, false, false, true>) : go(gemm_rows_kernel<false, false, false, false, true>);
   return masked ? go(gemm_rows_kernel<true, false, false, false>) : go(gemm_rows_kernel<false, false, false, false>);
 }
 
