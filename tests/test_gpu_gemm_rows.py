@@ -24,8 +24,8 @@ def test_padded_row_counts(orc, R, N, K):
 @pytest.mark.parametrize("N,K", [(4096, 12288), (6144, 4096), (4096, 4096), (5120, 2048), (328, 1152), (20000, 1024)])
 def test_few_rows_are_no_further_off_than_many(N, K):
     """The tensor core's accumulator cuts every sum off, so an error grows with the k-blocks that one accumulator takes.  Up to 32
-    rows a tile is half as wide and half as many CTAs share its K; what an accumulator sums stays no longer.  Positive products:
-    nothing of what is cut off cancels."""
+    rows a tile may be half as wide, but not where half as many CTAs would then share its K.  Positive products: nothing of what is
+    cut off cancels."""
     import torch
 
     from paper_2608_14376_b200 import corun
