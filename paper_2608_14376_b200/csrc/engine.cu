@@ -44,13 +44,11 @@ struct DevMem {
   std::vector<void *> blocks;
   char *cur = nullptr;
   size_t left = 0, next = (size_t)32 << 20;
-  bool tight = false;                                // there was no room for a whole block
   // Room for `bytes` in one block of that size, if there is as much: what follows fits it and leaves nothing over.
   void reserve(size_t bytes) {
     void *q = nullptr;
     if (cudaMalloc(&q, bytes) != cudaSuccess) {
       cudaGetLastError();
-      tight = true;
       return;
     }
     blocks.push_back(q);
@@ -270,7 +268,7 @@ int dmalloc(DevMem &m, T **p, size_t n, bool zero = true) {
     else if (m.next < ((size_t)256 << 20)) m.next *= 2;
     void *q = nullptr;
     cudaError_t e = cudaMalloc(&q, want);
-    if (e != cudaSuccess && want > bytes) { cudaGetLastError(); m.tight = true; e = cudaMalloc(&q, want = bytes); }
+    if (e != cudaSuccess && want > bytes) { cudaGetLastError(); e = cudaMalloc(&q, want = bytes); }
     if (e != cudaSuccess) {
       cudaGetLastError();
       g_last_cuda_error = (int)e;
@@ -1336,7 +1334,7 @@ static int engine_create(const corun_shape *shape, const corun_weights *w, const
   while (big_cap) {
     size_t free_b = 0;
     rc = program_create_big(e, e->big, big_cap);
-    if (rc == CORUN_OK && big_cap > 256 && e->big.allocs.tight && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b < (size_t)128 << 20) rc = CORUN_ENOMEM;
+    if (rc == CORUN_OK && big_cap > 256 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b < (size_t)128 << 20) rc = CORUN_ENOMEM;
     if (rc != CORUN_ENOMEM) break;
     program_destroy(e->big);
     e->big = Program();

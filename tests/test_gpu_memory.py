@@ -41,6 +41,38 @@ def test_an_engine_fits_beside_what_is_left_and_gives_the_same_bytes():
         torch.cuda.empty_cache()
 
 
+def test_an_engine_leaves_room_for_its_step():
+    """The buffers of the largest chunks would fit and leave next to nothing: smaller ones are taken, 128 MiB stay free."""
+    import torch
+
+    from paper_2608_14376_b200 import corun
+
+    sh = synth.ModelShape(2, 2048, 16, 4, 128, 8192, 4096, 1e-6, 10000.0)
+    w = synth.make_weights_torch(sh, seed=3)
+    prompts = synth.make_prompts(sh.vocab, [1900, 60], seed=4)
+
+    def run():
+        eng = corun.Engine(sh, w, 8, 2048, kv_pool_blocks=3 * 128)
+        try:
+            free = torch.cuda.mem_get_info()[0]
+            eng.prefill_batch([1, 6], prompts, [len(p) + 8 for p in prompts])
+            return free, [eng.logits(s).tobytes() for s in (1, 6)]
+        finally:
+            eng.close()
+
+    run()                                             # (every kernel is loaded)
+    gc.collect(); torch.cuda.empty_cache(); torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    free, want = run()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (before - free) - (32 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        free, got = run()
+        assert got == want and free >= 100 << 20      # (what was left, but for the step's graph)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+
+
 @pytest.mark.parametrize("experts", [False, True])
 def test_chunks_of_more_rows_take_what_the_rows_need(experts):
     """A chunk may have 4096 rows where a prompt can have more than 2048 tokens.  What one half of a layer hands on and what the other
